@@ -23,9 +23,14 @@
 // the cached length requests that tile before it waits for the preceding kernel: those rows
 // were written by earlier steps.  Every wait is bounded (2 s by default): on expiry the CTA flags
 // CS_DEV_TIMEOUT, drains its copies, frees its TMEM and returns.
+//
+// Bound by latency (one tile per CTA at 4k keys: 10.2 us a layer, 10.6 before the MMAs were issued with
+// uniform operands) and, where a block fills the M rows, by the tensor pipe on two-term operands (256
+// rows over 3,840 keys: 102 us, 119 before).
 #include <stdlib.h>
 
 #include "cs_common.cuh"
+#include "cs_tcgen.cuh"
 
 namespace {
 
@@ -50,70 +55,6 @@ struct AttnArgs {
   unsigned long long* stamp;    // step timeline slot of this launch, or NULL
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                       unsigned long long limit_ns) {
-  unsigned long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u) {
-      if (*abort_flag) return false;
-      const unsigned long long now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) return false;
-    }
-  }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-// operand descriptors, 128-byte swizzle.  K-major: rows of 128 bytes, 8-row groups 1024 bytes
-// apart.  MN-major: rows (one per K index) of 128 bytes holding 64 contiguous MN elements,
-// 8-row groups 1024 bytes apart (stride field), the next 64 MN elements `lbo` bytes further.
-__device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t saddr, uint32_t lbo) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
@@ -217,7 +158,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
                  b_vfree = smem_u32(bars + 6), b_qfull = smem_u32(bars + 8), b_sready = smem_u32(bars + 9),
                  b_pready = smem_u32(bars + 10), b_odone = smem_u32(bars + 11), b_pair = smem_u32(bars + 12);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int b = blockIdx.x / a.Hkv, kvh = blockIdx.x % a.Hkv, split = blockIdx.y;
   const int nact = (nq + 31) >> 5;                     // softmax warps that own real rows
   constexpr uint32_t kTmemCols = 256, kOCol = 128;     // S in columns 0..127, O in 128..255
@@ -244,7 +185,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = uniform(*tmem_slot);
   // Slice `split` works on key tiles split, split + nsplit, ...: its first tile is known before
   // the key range is, so the queries and that tile are requested while the range is worked out
   // (a slice beyond the range only has to let them land).
@@ -252,10 +193,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
   const long long vrow = ((((long long)a.layer * 2 + 1) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
   const int key_first = split * kTileKeys;
   bool early = false;
-  if (warp == kProdWarp && lane == 0 && a.kv_len_early != nullptr) {
+  if (warp == kProdWarp && a.kv_len_early != nullptr) {
     // a tile of cached keys only: nothing in flight writes it, so it need not wait
-    if (key_first + kTileKeys <= min(a.kv_len_early[b], a.max_seq)) {
-      early = true;
+    early = uniform(key_first + kTileKeys <= min(a.kv_len_early[b], a.max_seq) ? 1u : 0u) != 0;
+    if (early && elect_one()) {
       const uint32_t dk = smem_u32(sK), dv = smem_u32(sV);
       mbar_expect_tx(b_kfull, 2u * kHalfBytes);
       tma_load_2d(dk, &tmKV, b_kfull, 0, (int)(krow + key_first));
@@ -273,7 +214,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
     lm = __reduce_max_sync(0xffffffffu, lm);
     if (lane == 0 && lm > 0) atomicMax(s_lmax, lm);
   }
-  if (warp == kProdWarp && lane == 0) {
+  if (warp == kProdWarp && elect_one()) {
     // K first (it comes from HBM and the first product waits for it), then the queries (fresh in
     // L2), V last: it is not needed before the softmax of the tile is done
     const uint32_t dk = smem_u32(sK), dv = smem_u32(sV);
@@ -294,80 +235,92 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
     }
   }
   __syncthreads();
-  const int lmax = *s_lmax;
+  const int lmax = (int)uniform((uint32_t)*s_lmax);
   const int ntiles = (lmax + kTileKeys - 1) / kTileKeys;
   const int ntl = (ntiles > split) ? (ntiles - split + a.nsplit - 1) / a.nsplit : 0;
 
   if (warp == kProdWarp) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int ik = 1, iv = 1;   // K and V tiles requested so far (tile 0 of this slice is already on its way)
-      bool ok = true;
-      for (int i = 1; i < ntl; ++i) {
-        const int s = i % stages;
-        const uint32_t ph = (uint32_t)(i / stages) & 1u;
-        const int key0 = (split + i * a.nsplit) * kTileKeys;
-        const uint32_t dk = smem_u32(sK + (size_t)s * 2 * kHalfBytes), dv = smem_u32(sV + (size_t)s * 2 * kHalfBytes);
-        if (!mbar_wait(b_kfree + 8 * s, ph ^ 1u, s_abort, a.wait_ns)) { ok = false; break; }
+    int ik = 1, iv = 1;     // K and V tiles requested so far (tile 0 of this slice is already on its way)
+    int s = stages > 1 ? 1 : 0;
+    uint32_t ph = stages > 1 ? 0u : 1u;
+    bool ok = true;
+    for (int i = 1; i < ntl; ++i) {
+      const int key0 = (split + i * a.nsplit) * kTileKeys;
+      const uint32_t dk = smem_u32(sK) + (uint32_t)(s * 2 * kHalfBytes), dv = smem_u32(sV) + (uint32_t)(s * 2 * kHalfBytes);
+      ok = mbar_wait_warp(b_kfree + 8 * s, ph ^ 1u, s_abort, a.wait_ns);
+      if (!ok) break;
+      if (elect_one()) {
         mbar_expect_tx(b_kfull + 8 * s, 2u * kHalfBytes);
         tma_load_2d(dk, &tmKV, b_kfull + 8 * s, 0, (int)(krow + key0));
         tma_load_2d(dk + kHalfBytes, &tmKV, b_kfull + 8 * s, 64, (int)(krow + key0));
-        ik = i + 1;
-        if (!mbar_wait(b_vfree + 8 * s, ph ^ 1u, s_abort, a.wait_ns)) { ok = false; break; }
+      }
+      ik = i + 1;
+      ok = mbar_wait_warp(b_vfree + 8 * s, ph ^ 1u, s_abort, a.wait_ns);
+      if (!ok) break;
+      if (elect_one()) {
         mbar_expect_tx(b_vfull + 8 * s, 2u * kHalfBytes);
         tma_load_2d(dv, &tmKV, b_vfull + 8 * s, 0, (int)(vrow + key0));
         tma_load_2d(dv + kHalfBytes, &tmKV, b_vfull + 8 * s, 64, (int)(vrow + key0));
-        iv = i + 1;
       }
-      if (!ok) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
-      if (*s_abort || ntl == 0) {   // let the copies land before the shared memory goes away
-        mbar_wait(b_qfull, 0, s_never, a.wait_ns);
-        for (int j = max(0, ik - stages); j < ik; ++j) mbar_wait(b_kfull + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, a.wait_ns);
-        for (int j = max(0, iv - stages); j < iv; ++j) mbar_wait(b_vfull + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, a.wait_ns);
-      }
+      iv = i + 1;
+      if (++s == stages) { s = 0; ph ^= 1u; }
+    }
+    if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
+    __syncwarp();
+    if ((*s_abort || ntl == 0) && lane == 0) {   // let the copies land before the shared memory goes away
+      mbar_wait(b_qfull, 0, s_never, a.wait_ns);
+      for (int j = max(0, ik - stages); j < ik; ++j) mbar_wait(b_kfull + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, a.wait_ns);
+      for (int j = max(0, iv - stages); j < iv; ++j) mbar_wait(b_vfull + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, a.wait_ns);
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && ntl > 0) {
+    if (ntl > 0) {
       const uint32_t idesc1 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
       const uint32_t idesc2 = idesc1 | (1u << 16);      // B (= V) is MN-major
-      const uint32_t aq = smem_u32(sQ), ap = smem_u32(sP);
-      // S of tile i: issued behind the P V product of tile i - 1, so one commit covers both
-      auto issue_scores = [&](int i) -> bool {
-        const int s = i % stages;
-        if (!mbar_wait(b_kfull + 8 * s, (uint32_t)(i / stages) & 1u, s_abort, a.wait_ns)) return false;
+      const uint64_t dq = desc_kmajor(smem_u32(sQ)), dp = desc_kmajor(smem_u32(sP));
+      const uint64_t dk0 = desc_kmajor(smem_u32(sK)), dv0 = desc_mnmajor(smem_u32(sV), kHalfBytes);
+      int s = 0;                                         // stage of tile i, and of tile i + 1's scores
+      uint32_t ph = 0;
+      // S of the tile in stage `st`: issued behind the P V product of the tile before, so one commit covers both
+      auto issue_scores = [&](int st, uint32_t phase) -> bool {
+        if (!mbar_wait_warp(b_kfull + 8 * st, phase, s_abort, a.wait_ns)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t ak = smem_u32(sK + (size_t)s * 2 * kHalfBytes);
+        if (elect_one()) {
+          const uint64_t dk = dk0 + (uint64_t)(uint32_t)(st * (2 * kHalfBytes >> 4));
 #pragma unroll
-        for (int term = 0; term < 2; ++term)
+          for (int term = 0; term < 2; ++term)
 #pragma unroll
-          for (int dh = 0; dh < 2; ++dh)
+            for (int dh = 0; dh < 2; ++dh)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16(tmem_base, desc_kmajor(aq + term * qterm + dh * qhalf) + 2 * kk, desc_kmajor(ak + dh * kHalfBytes) + 2 * kk,
-                        idesc1, (term | dh | kk) ? 1u : 0u);
-        umma_commit(b_kfree + 8 * s);
-        umma_commit(b_sready);
+              for (int kk = 0; kk < 4; ++kk)
+                umma_bf16(tmem_base, dq + (uint64_t)((term * qterm + dh * qhalf) >> 4) + 2 * kk, dk + dh * (kHalfBytes >> 4) + 2 * kk,
+                          idesc1, (term | dh | kk) ? 1u : 0u);
+          umma_commit(b_kfree + 8 * st);
+          umma_commit(b_sready);
+        }
         return true;
       };
-      bool ok = mbar_wait(b_qfull, 0, s_abort, a.wait_ns) && issue_scores(0);
+      bool ok = mbar_wait_warp(b_qfull, 0, s_abort, a.wait_ns) && issue_scores(0, 0);
       for (int i = 0; i < ntl && ok; ++i) {
-        const int s = i % stages;
-        const uint32_t ph = (uint32_t)(i / stages) & 1u;
-        if (!mbar_wait(b_pready, (uint32_t)i & 1u, s_abort, a.wait_ns) || !mbar_wait(b_vfull + 8 * s, ph, s_abort, a.wait_ns)) { ok = false; break; }
+        ok = mbar_wait_warp(b_pready, (uint32_t)i & 1u, s_abort, a.wait_ns) && mbar_wait_warp(b_vfull + 8 * s, ph, s_abort, a.wait_ns);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t av = smem_u32(sV + (size_t)s * 2 * kHalfBytes);
+        if (elect_one()) {
+          const uint64_t dv = dv0 + (uint64_t)(uint32_t)(s * (2 * kHalfBytes >> 4));
 #pragma unroll
-        for (int term = 0; term < 2; ++term)
+          for (int term = 0; term < 2; ++term)
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk)   // 16 keys per instruction
-            umma_bf16(tmem_base + kOCol, desc_kmajor(ap + term * qterm + (kk >> 2) * qhalf) + 2 * (kk & 3),
-                      desc_mnmajor(av + kk * 2048, kHalfBytes), idesc2, (i > 0 || term > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(b_vfree + 8 * s);
-        umma_commit(b_odone);
-        if (i + 1 < ntl && !issue_scores(i + 1)) { ok = false; break; }
+            for (int kk = 0; kk < 8; ++kk)   // 16 keys per instruction
+              umma_bf16(tmem_base + kOCol, dp + (uint64_t)((term * qterm + (kk >> 2) * qhalf) >> 4) + 2 * (kk & 3),
+                        dv + kk * (2048 >> 4), idesc2, (i > 0 || term > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(b_vfree + 8 * s);
+          umma_commit(b_odone);
+        }
+        if (++s == stages) { s = 0; ph ^= 1u; }
+        if (i + 1 < ntl) ok = issue_scores(s, ph);
       }
-      if (!ok) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
+      if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
     }
   } else if ((warp & 3) < nact) {
     // ------------------------------------------------------------------ softmax + epilogue (two threads per query row)

@@ -10,11 +10,10 @@
 //     O^T [128 dims x NQ]  = V_tile^T P_hi^T + V_tile^T P_lo^T (A = V tile, MN-major straight from the
 //                                                               cache layout; B = P^T, MN-major)
 // Queries and softmax weights enter as two bf16 terms each, so they are fp32-equivalent and only
-// K and V - which the cache stores in bf16 - are rounded.  A tcgen05.mma of these shapes keeps
-// its issuer busy for about 114 cycles whatever N is (measured for N from 32 to 192), so the
+// K and V - which the cache stores in bf16 - are rounded.  The
 // two terms of the second operand are laid side by side along N - [Q_hi; Q_lo] as one operand of
 // 2 NQ rows, [P_hi^T | P_lo^T] as one of 2 NQ columns - and one instruction per 16 K-elements
-// does the work of two; the two halves of the accumulator are added where it is read (S^T keeps
+// does the work of two, reading the K or V tile once; the two halves of the accumulator are added where it is read (S^T keeps
 // one NQ-wide accumulator and two instructions when TMEM has no room for 2 NQ columns twice).
 // TMEM lane = key (S^T) or head dim (O^T), column = query row.  Softmax: twelve warps in three
 // column groups; thread t of a lane quarter owns key t of the tile and a third of the query
@@ -41,9 +40,15 @@
 // steps.  Every wait is bounded (2 s by default): on expiry the CTA flags CS_DEV_TIMEOUT, drains
 // its copies, frees its TMEM and returns; the decision to give up is made uniform across the
 // softmax threads by a predicate-reducing barrier, so no thread is left behind at a barrier.
+//
+// Bound by the softmax warps' issue slots and, at batch 16, by HBM.  Measured per layer (8B shape, issue
+// by an elected lane with uniform operands, before that from one lane): 176 rows over 16 x 8,192 keys
+// 120.6 -> 93.6 us (0.54 GB: 5.8 TB/s), 16 rows over the same 114.2 -> 83.2 us, 168 rows over
+// 8 x 16,384 keys 159.8 -> 136.7 us, 11 rows over 30,720 keys 33.8 -> 29.2 us.
 #include <stdlib.h>
 
 #include "cs_common.cuh"
+#include "cs_tcgen.cuh"
 
 namespace {
 
@@ -71,70 +76,6 @@ struct AttnArgs {
   unsigned long long* stamp;    // step timeline slot of this launch, or NULL
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                       unsigned long long limit_ns) {
-  unsigned long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u) {
-      if (*abort_flag) return false;
-      const unsigned long long now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) return false;
-    }
-  }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-// operand descriptors, 128-byte swizzle.  K-major: rows of 128 bytes, 8-row groups 1024 bytes
-// apart.  MN-major: rows (one per K index) of 128 bytes holding 64 contiguous MN elements,
-// 8-row groups 1024 bytes apart (stride field), the next 64 MN elements `lbo` bytes further.
-__device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ uint64_t desc_mnmajor(uint32_t saddr, uint32_t lbo) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
 // eight accumulator columns of this thread's lane (no wait: several loads share one wait)
 __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, float* v) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -258,7 +199,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
                  b_vfree = smem_u32(bars + 6), b_qfull = smem_u32(bars + 8), b_sready = smem_u32(bars + 16),   // b_sready: one per S^T buffer (bars 16-19)
                  b_pready = smem_u32(bars + 14), b_odone = smem_u32(bars + 12);   // b_pready (bars 14, 15) and b_odone: two barriers each, by tile parity
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int b = blockIdx.x / a.Hkv, kvh = blockIdx.x % a.Hkv, split = blockIdx.y;
   // TMEM columns: S^T of even tiles, S^T of odd tiles (each NQ wide, or 2 NQ when the two query terms
   // are kept apart), then O^T, 2 NQ wide: the leading and the trailing weight terms' shares
@@ -288,34 +229,30 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = uniform(*tmem_slot);
   // Slice `split` works on key tiles split, split + nsplit, ...  Its first tiles are known before
   // the key range is, so they are requested while the range is worked out (a slice beyond the
   // range only has to let them land).
   const long long krow = ((((long long)a.layer * 2 + 0) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
   const long long vrow = ((((long long)a.layer * 2 + 1) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
-  auto load_k = [&](int i) {
-    const int s = i & 1, key0 = (split + i * a.nsplit) * kTileKeys;
-    const uint32_t dk = smem_u32(sK + (size_t)s * 2 * kHalfBytes);
-    mbar_expect_tx(b_kfull + 8 * s, 2u * kHalfBytes);
-    tma_load_2d(dk, &tmKV, b_kfull + 8 * s, 0, (int)(krow + key0));
-    tma_load_2d(dk + kHalfBytes, &tmKV, b_kfull + 8 * s, 64, (int)(krow + key0));
+  auto load_tile = [&](uint32_t buf, uint32_t bar, long long first, int i) {   // tile i of this slice (by the elected lane)
+    const int key0 = (split + i * a.nsplit) * kTileKeys;
+    mbar_expect_tx(bar, 2u * kHalfBytes);
+    tma_load_2d(buf, &tmKV, bar, 0, (int)(first + key0));
+    tma_load_2d(buf + kHalfBytes, &tmKV, bar, 64, (int)(first + key0));
   };
-  auto load_v = [&](int i) {
-    const int s = i % vstages, key0 = (split + i * a.nsplit) * kTileKeys;
-    const uint32_t dv = smem_u32(sV + (size_t)s * 2 * kHalfBytes);
-    mbar_expect_tx(b_vfull + 8 * s, 2u * kHalfBytes);
-    tma_load_2d(dv, &tmKV, b_vfull + 8 * s, 0, (int)(vrow + key0));
-    tma_load_2d(dv + kHalfBytes, &tmKV, b_vfull + 8 * s, 64, (int)(vrow + key0));
-  };
+  // one producer warp feeds K, one feeds V
+  const bool is_k = warp == kProdWarp, is_prod = is_k || warp == kVProdWarp;
+  const int st = is_k ? 2 : vstages;
+  const uint32_t ring = smem_u32(is_k ? sK : sV), bfree = is_k ? b_kfree : b_vfree, bfull = is_k ? b_kfull : b_vfull;
+  const long long first_row = is_k ? krow : vrow;
   // tiles of cached keys only: nothing in flight writes them, so they need not wait for the
-  // preceding kernel.  n_early = tiles of this slice this producer lane requested before the wait.
+  // preceding kernel.  n_early = tiles of this slice this producer requested before the wait.
   int n_early = 0;
-  if ((warp == kProdWarp || warp == kVProdWarp) && lane == 0 && a.kv_len_early != nullptr) {
-    const int cached = min(a.kv_len_early[b], a.max_seq);
-    const int want = (warp == kProdWarp) ? 2 : vstages;
-    while (n_early < want && (split + n_early * a.nsplit + 1) * kTileKeys <= cached) {
-      if (warp == kProdWarp) load_k(n_early); else load_v(n_early);
+  if (is_prod && a.kv_len_early != nullptr) {
+    const int cached = (int)uniform((uint32_t)min(a.kv_len_early[b], a.max_seq));
+    while (n_early < st && (split + n_early * a.nsplit + 1) * kTileKeys <= cached) {
+      if (elect_one()) load_tile(ring + (uint32_t)(n_early * 2 * kHalfBytes), bfull + 8 * n_early, first_row, n_early);
       ++n_early;
     }
   }
@@ -336,106 +273,111 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
       s_lim[q] = (q < nq) ? a.row_lim[b * R + r0 + q / G] : 0;
     }
   }
-  if (warp == kProdWarp && lane == 0) {
-    // tile 0 of K first (the first product waits for it), then the queries (fresh in L2)
-    if (n_early < 1) load_k(0);
+  // tile 0 of K first (the first product waits for it), then the queries (fresh in L2)
+  if (is_prod && n_early < 1 && elect_one()) load_tile(ring, bfull, first_row, 0);
+  if (warp == kProdWarp && elect_one()) {
     mbar_expect_tx(b_qfull, (uint32_t)(4 * nq_box * 128));
     for (int term = 0; term < 2; ++term)
       for (int dh = 0; dh < 2; ++dh)
         tma_load_3d(smem_u32(sQ + (2 * dh + term) * qhalf), &tmQ, b_qfull, dh * 64, kvh * G,
                     term * CS_MAX_ROWS + b * R + r0);   // the box is always Rg rows tall; rows past the group are never used
   }
-  if (warp == kVProdWarp && lane == 0 && n_early < 1) load_v(0);
   __syncthreads();
-  const int lmax = *s_lmax;
+  const int lmax = (int)uniform((uint32_t)*s_lmax);
   const int ntiles = (lmax + kTileKeys - 1) / kTileKeys;
   const int ntl = (ntiles > split) ? (ntiles - split + a.nsplit - 1) / a.nsplit : 0;
 
-  if (warp == kProdWarp || warp == kVProdWarp) {
-    // ------------------------------------------------------------------ TMA producers: one warp feeds K, one feeds V
-    if (lane == 0) {
-      const bool is_k = warp == kProdWarp;
-      const int st = is_k ? 2 : vstages;
-      const uint32_t bfree = is_k ? b_kfree : b_vfree, bfull = is_k ? b_kfull : b_vfull;
-      int issued = max(1, n_early);                     // tiles requested so far (tile 0 always is)
-      bool ok = true;
-      for (int i = issued; i < ntl; ++i) {
-        const int s = i % st;
-        if (i >= st && !mbar_wait(bfree + 8 * s, (uint32_t)(i / st - 1) & 1u, s_abort, a.wait_ns)) { ok = false; break; }
-        if (is_k) load_k(i); else load_v(i);
-        issued = i + 1;
-      }
-      if (!ok) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
-      // copies that nobody will consume (the CTA gave up, or tiles requested early beyond the key
-      // range) must land before the shared memory goes away
-      if (*s_abort || issued > ntl) {
-        if (is_k) mbar_wait(b_qfull, 0, s_never, a.wait_ns);
-        for (int j = max(0, issued - st); j < issued; ++j) mbar_wait(bfull + 8 * (j % st), (uint32_t)(j / st) & 1u, s_never, a.wait_ns);
-      }
+  if (is_prod) {
+    // ------------------------------------------------------------------ TMA producers
+    int issued = max(1, n_early);                       // tiles requested so far (tile 0 always is)
+    int s = issued == st ? 0 : issued;
+    uint32_t ph = issued == st ? 0u : 1u;
+    bool ok = true;
+    for (int i = issued; i < ntl; ++i) {
+      if (i >= st) ok = mbar_wait_warp(bfree + 8 * s, ph, s_abort, a.wait_ns);
+      if (!ok) break;
+      if (elect_one()) load_tile(ring + (uint32_t)(s * 2 * kHalfBytes), bfull + 8 * s, first_row, i);
+      issued = i + 1;
+      if (++s == st) { s = 0; ph ^= 1u; }
+    }
+    if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
+    __syncwarp();
+    // copies that nobody will consume (the CTA gave up, or tiles requested early beyond the key
+    // range) must land before the shared memory goes away
+    if ((*s_abort || issued > ntl) && lane == 0) {
+      if (is_k) mbar_wait(b_qfull, 0, s_never, a.wait_ns);
+      for (int j = max(0, issued - st); j < issued; ++j) mbar_wait(bfull + 8 * (j % st), (uint32_t)(j / st) & 1u, s_never, a.wait_ns);
     }
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0 && ntl > 0) {
-      // bf16 x bf16 -> fp32, M = 128.  An instruction costs about the same for any N up to 200, so
-      // the two bf16 terms of the second operand sit side by side along N wherever TMEM has the
-      // columns: one instruction then does the work of two, and the two halves of the result are
-      // added when they are read.
+    if (ntl > 0) {
+      // bf16 x bf16 -> fp32, M = 128.  The two bf16 terms of the second operand sit side by side along N
+      // wherever TMEM has the columns: one instruction then does the work of two, and the two halves
+      // of the result are added when they are read.
       auto idesc = [](int n) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24); };
       const uint32_t idesc_s = idesc(a.qstack ? 2 * NQ : NQ);
       const uint32_t idesc_o = idesc(2 * NQ) | (1u << 15) | (1u << 16);   // A (= V) and B (= P^T) are MN-major
-      const uint32_t aq = smem_u32(sQ), ap = smem_u32(sP);
+      const uint64_t dq = desc_kmajor(smem_u32(sQ)), dp0 = desc_mnmajor(smem_u32(sP), kHalfBytes);
+      const uint64_t dk0 = desc_kmajor(smem_u32(sK)), dv0 = desc_mnmajor(smem_u32(sV), kHalfBytes);
       auto issue_scores = [&](int i) -> bool {
         const int s = i & 1, sb = i & (NSB - 1);           // K stage, S^T buffer
-        if (!mbar_wait(b_kfull + 8 * s, (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns)) return false;
+        if (!mbar_wait_warp(b_kfull + 8 * s, (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t ak = smem_u32(sK + (size_t)s * 2 * kHalfBytes);
-        const uint32_t acc = tmem_base + (uint32_t)sb * cstride;
-        if (a.qstack) {
-#pragma unroll
-          for (int dh = 0; dh < 2; ++dh)
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              umma_bf16(acc, desc_kmajor(ak + dh * kHalfBytes) + 2 * kk, desc_kmajor(aq + dh * 2 * qhalf) + 2 * kk, idesc_s,
-                        (dh | kk) ? 1u : 0u);
-        } else {
-#pragma unroll
-          for (int term = 0; term < 2; ++term)
+        if (elect_one()) {
+          const uint64_t dk = dk0 + (uint64_t)(uint32_t)(s * (2 * kHalfBytes >> 4));
+          const uint32_t acc = tmem_base + (uint32_t)sb * cstride;
+          if (a.qstack) {
 #pragma unroll
             for (int dh = 0; dh < 2; ++dh)
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
-                umma_bf16(acc, desc_kmajor(ak + dh * kHalfBytes) + 2 * kk, desc_kmajor(aq + (2 * dh + term) * qhalf) + 2 * kk,
-                          idesc_s, (term | dh | kk) ? 1u : 0u);
+                umma_bf16(acc, dk + dh * (kHalfBytes >> 4) + 2 * kk, dq + (uint64_t)((dh * 2 * qhalf) >> 4) + 2 * kk, idesc_s,
+                          (dh | kk) ? 1u : 0u);
+          } else {
+#pragma unroll
+            for (int term = 0; term < 2; ++term)
+#pragma unroll
+              for (int dh = 0; dh < 2; ++dh)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                  umma_bf16(acc, dk + dh * (kHalfBytes >> 4) + 2 * kk, dq + (uint64_t)(((2 * dh + term) * qhalf) >> 4) + 2 * kk,
+                            idesc_s, (term | dh | kk) ? 1u : 0u);
+          }
+          umma_commit(b_kfree + 8 * s);
+          umma_commit(b_sready + 8 * sb);
         }
-        umma_commit(b_kfree + 8 * s);
-        umma_commit(b_sready + 8 * sb);
         return true;
       };
-      bool ok = mbar_wait(b_qfull, 0, s_abort, a.wait_ns);
+      bool ok = mbar_wait_warp(b_qfull, 0, s_abort, a.wait_ns);
       int qk = 0;                                          // score products issued so far
+      int s = 0, pb = 0;                                   // V stage and P^T buffer of tile i
+      uint32_t ph = 0;
       for (int i = 0; i < ntl && ok; ++i) {
         // The scores of the next tiles go first: they run during this tile's softmax.  The S^T buffer
         // of tile t was last read by the softmax of tile t - NSB, which had finished before P^T of
-        // that tile was signalled - and this thread has waited for the P^T of every tile before i.
+        // that tile was signalled - and this warp has waited for the P^T of every tile before i.
         // A column group whose tiles are quick - all its rows masked - can therefore be a tile ahead
         // of the others, which is why "P^T written" has a barrier per tile parity: it cannot be two
         // ahead, because the scores of tile i + 2 are only issued after P^T of tile i (with four
         // buffers the softmax hands tiles over in pairs, odd after even, so parity still tells them apart).
         while (qk < ntl && qk < i + NSB && ok) { ok = issue_scores(qk); ++qk; }
         if (!ok) break;
-        const int s = i % vstages;
-        if (!mbar_wait(b_pready + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns) ||
-            !mbar_wait(b_vfull + 8 * s, (uint32_t)(i / vstages) & 1u, s_abort, a.wait_ns)) { ok = false; break; }
+        ok = mbar_wait_warp(b_pready + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns) &&
+             mbar_wait_warp(b_vfull + 8 * s, ph, s_abort, a.wait_ns);
+        if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t av = smem_u32(sV + (size_t)s * 2 * kHalfBytes);
+        if (elect_one()) {
+          const uint64_t dv = dv0 + (uint64_t)(uint32_t)(s * (2 * kHalfBytes >> 4)), dp = dp0 + (uint64_t)(pb ? pbuf >> 4 : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk)   // 16 keys per instruction
-          umma_bf16(tmem_base + ocol, desc_mnmajor(av + kk * 2048, kHalfBytes),
-                    desc_mnmajor(ap + (uint32_t)(i % a.pbufs) * pbuf + kk * 2048, kHalfBytes), idesc_o, (i > 0 || kk > 0) ? 1u : 0u);
-        umma_commit(b_vfree + 8 * s);
-        umma_commit(b_odone + 8 * (i & 1));
+          for (int kk = 0; kk < 8; ++kk)   // 16 keys per instruction
+            umma_bf16(tmem_base + ocol, dv + kk * (2048 >> 4), dp + kk * (2048 >> 4), idesc_o, (i > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(b_vfree + 8 * s);
+          umma_commit(b_odone + 8 * (i & 1));
+        }
+        if (++s == vstages) { s = 0; ph ^= 1u; }
+        if (++pb == a.pbufs) pb = 0;
       }
-      if (!ok) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
+      if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue

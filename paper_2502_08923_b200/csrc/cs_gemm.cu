@@ -29,6 +29,11 @@
 // predecessor drains, fills its pipeline with weight tiles (which depend on nothing) and
 // only then waits for the predecessor before touching activations.
 //
+// Copies and MMAs are issued by an elected lane with uniform operands (cs_tcgen.cuh): a stage goes
+// back to the producer some 800 clocks sooner than when one lane issued the eight MMAs of a K block.
+// Measured on an 11-row block of the 8B shape, before and after: QKV 12.4 -> 12.1 us, attention output
+// 11.0 -> 9.8, gate/up 44.4 -> 42.2, down 23.7 -> 22.2, LM head 186 -> 170 us (6.2 TB/s).
+//
 // Every wait is bounded: when it runs out the CTA records CS_DEV_TIMEOUT, drains its
 // copies, still takes part in the cluster barriers, frees its TMEM and returns.
 #include <stdlib.h>
@@ -37,6 +42,7 @@
 #include <type_traits>
 
 #include "cs_common.cuh"
+#include "cs_tcgen.cuh"
 
 using std::max;
 using std::min;
@@ -67,75 +73,6 @@ struct GemmArgs {
   unsigned long long* stamp;    // step timeline slot of this launch, or NULL
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait.  Returns false when another role of this CTA gave up or `limit_ns` passed.
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                       unsigned long long limit_ns) {
-  unsigned long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 1023u) {
-      if (*abort_flag) return false;
-      const unsigned long long now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) return false;
-    }
-  }
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0,
-                                            int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-// K-major operand tile, 128-byte swizzle: rows of 128 bytes, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);   // start address / 16
-  d |= (uint64_t)1 << 16;                      // leading-dimension offset (unused here)
-  d |= (uint64_t)(1024 >> 4) << 32;            // stride between 8-row groups / 16
-  d |= (uint64_t)1 << 46;                      // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;                      // 128-byte swizzle
-  return d;
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -157,11 +94,6 @@ __device__ __forceinline__ void cluster_arrive() {
 __device__ __forceinline__ void cluster_wait() {
   __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %cluster_ctarank;" : "=r"(r));
-  return r;
 }
 // Four consecutive floats of every rank's parked tile, summed in rank order.  All loads are
 // issued before the first add so that their latencies overlap.
@@ -218,9 +150,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     return;
   }
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int cta_tile = blockIdx.x;
-  const int split = (a.splits > 1) ? (int)cluster_rank() : 0;
+  const int split = (int)blockIdx.y;             // = the rank in the cluster of (1, splits, 1)
   const int cta_n0 = cta_tile * MT * CS_GEMM_BM;
   const int kb0 = split * a.kb_per_split;
   const int kb1 = min(a.num_kb, kb0 + a.kb_per_split);
@@ -251,85 +183,84 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = uniform(*tmem_slot);
   bool ok = true;
 
   if (warp == 4) {
     // ------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      // weights depend on nothing: fill the ring with them before waiting for the predecessor
-      const int npre = min(nkb, a.stages);
-      for (int i = 0; i < npre; ++i) {
-        if (i == a.drop_kb) continue;   // (test hook: this stage never fills, the consumer's wait runs out)
-        mbar_expect_tx(bar_full + 8 * i, (uint32_t)stage_bytes);
+    const uint32_t ring = smem_u32(smem);
+    auto load_w = [&](int i, int s) {            // (by the elected lane)
+      mbar_expect_tx(bar_full + 8 * s, (uint32_t)stage_bytes);
 #pragma unroll
-        for (int m = 0; m < MT; ++m)
-          tma_load_2d(smem_u32(smem + (size_t)i * stage_bytes) + m * kTileABytes, &tmW, bar_full + 8 * i,
-                      (kb0 + i) * CS_GEMM_BK, cta_n0 + m * CS_GEMM_BM);
-      }
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      for (int i = 0; i < npre; ++i)
-      {
-        if (i == a.drop_kb) continue;
-        const uint32_t sx = smem_u32(smem + (size_t)i * stage_bytes) + wbytes;
-        tma_load_2d(sx, &tmX, bar_full + 8 * i, (kb0 + i) * CS_GEMM_BK, 0);
-        if (two) tma_load_2d(sx + xtile, &tmX, bar_full + 8 * i, (kb0 + i) * CS_GEMM_BK, a.lo_row);
-      }
-      int i = npre;
-      for (; i < nkb; ++i) {
-        const int s = i % a.stages;
-        const uint32_t ph = (uint32_t)(i / a.stages) & 1u;
-        if (!mbar_wait(bar_empty + 8 * s, ph ^ 1u, s_abort, a.wait_ns)) { ok = false; break; }
-        const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-        if (i == a.drop_kb) continue;
-        mbar_expect_tx(bar_full + 8 * s, (uint32_t)stage_bytes);
-#pragma unroll
-        for (int m = 0; m < MT; ++m)
-          tma_load_2d(sa + m * kTileABytes, &tmW, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, cta_n0 + m * CS_GEMM_BM);
-        tma_load_2d(sa + wbytes, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, 0);
-        if (two) tma_load_2d(sa + wbytes + xtile, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, a.lo_row);
-      }
-      if (!ok) {
-        *s_abort = 1;
-        atomicOr(a.status, CS_DEV_TIMEOUT);
-      }
-      if (*s_abort) {
-        // copies still in flight must land before this CTA's shared memory is reused or released
-        for (int j = max(0, i - a.stages); j < i; ++j)
-          if (j != a.drop_kb) mbar_wait(bar_full + 8 * (j % a.stages), (uint32_t)(j / a.stages) & 1u, s_never, a.wait_ns);
-      }
+      for (int m = 0; m < MT; ++m)
+        tma_load_2d(ring + (uint32_t)(s * stage_bytes + m * kTileABytes), &tmW, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK,
+                    cta_n0 + m * CS_GEMM_BM);
+    };
+    auto load_x = [&](int i, int s) {
+      const uint32_t sx = ring + (uint32_t)(s * stage_bytes + wbytes);
+      tma_load_2d(sx, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, 0);
+      if (two) tma_load_2d(sx + xtile, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, a.lo_row);
+    };
+    // weights depend on nothing: fill the ring with them before waiting for the predecessor
+    // (drop_kb is a test hook: that stage never fills and the consumer's wait runs out)
+    const int npre = min(nkb, a.stages);
+    for (int i = 0; i < npre; ++i)
+      if (i != a.drop_kb && elect_one()) load_w(i, i);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int i = 0; i < npre; ++i)
+      if (i != a.drop_kb && elect_one()) load_x(i, i);
+    int i = npre, s = 0;
+    uint32_t ph = 0;
+    for (; i < nkb; ++i) {
+      ok = mbar_wait_warp(bar_empty + 8 * s, ph, s_abort, a.wait_ns);
+      if (!ok) break;
+      if (i != a.drop_kb && elect_one()) { load_w(i, s); load_x(i, s); }
+      if (++s == a.stages) { s = 0; ph ^= 1u; }
+    }
+    if (!ok && lane == 0) {
+      *s_abort = 1;
+      atomicOr(a.status, CS_DEV_TIMEOUT);
+    }
+    __syncwarp();
+    if (*s_abort && lane == 0) {
+      // copies still in flight must land before this CTA's shared memory is reused or released
+      for (int j = max(0, i - a.stages); j < i; ++j)
+        if (j != a.drop_kb) mbar_wait(bar_full + 8 * (j % a.stages), (uint32_t)(j / a.stages) & 1u, s_never, a.wait_ns);
     }
   } else if (warp == 5) {
     // ------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      // bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n_tok
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.n_tok >> 3) << 17) |
-                             ((uint32_t)(CS_GEMM_BM >> 4) << 24);
-      for (int i = 0; i < nkb; ++i) {
-        const int s = i % a.stages;
-        const uint32_t ph = (uint32_t)(i / a.stages) & 1u;
-        if (!mbar_wait(bar_full + 8 * s, ph, s_abort, a.wait_ns)) { ok = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = smem_u32(smem + (size_t)s * stage_bytes);
-        const uint64_t db = umma_desc(sa + wbytes), dl = umma_desc(sa + wbytes + xtile);
+    // bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n_tok
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.n_tok >> 3) << 17) |
+                           ((uint32_t)(CS_GEMM_BM >> 4) << 24);
+    const uint64_t desc0 = desc_kmajor(smem_u32(smem));
+    const uint64_t x_off = (uint64_t)(wbytes >> 4), lo_off = (uint64_t)((wbytes + xtile) >> 4);
+    int s = 0;
+    uint32_t ph = 0;
+    for (int i = 0; i < nkb; ++i) {
+      ok = mbar_wait_warp(bar_full + 8 * s, ph, s_abort, a.wait_ns);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (elect_one()) {
+        const uint64_t d = desc0 + (uint64_t)(uint32_t)(s * (stage_bytes >> 4));
 #pragma unroll
         for (int m = 0; m < MT; ++m) {                   // every sub-tile against the same activation tile
-          const uint64_t da = umma_desc(sa + m * kTileABytes);
+          const uint64_t da = d + (uint64_t)(m * (kTileABytes >> 4));
           const uint32_t acc = tmem_base + (uint32_t)(m * a.n_tok);
 #pragma unroll
           for (int kk = 0; kk < CS_GEMM_BK / 16; ++kk) {   // 16 K-elements = 32 bytes per instruction
-            umma_bf16(acc, da + 2 * kk, db + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
-            if (two) umma_bf16(acc, da + 2 * kk, dl + 2 * kk, idesc, 1u);   // x = hi + lo
+            umma_bf16(acc, da + 2 * kk, d + x_off + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+            if (two) umma_bf16(acc, da + 2 * kk, d + lo_off + 2 * kk, idesc, 1u);   // x = hi + lo
           }
         }
         umma_commit(bar_empty + 8 * s);
       }
-      if (!ok) {
-        *s_abort = 1;
-        atomicOr(a.status, CS_DEV_TIMEOUT);
-      }
-      umma_commit(bar_acc);
+      if (++s == a.stages) { s = 0; ph ^= 1u; }
     }
+    if (!ok && lane == 0) {
+      *s_abort = 1;
+      atomicOr(a.status, CS_DEV_TIMEOUT);
+    }
+    if (elect_one()) umma_commit(bar_acc);
   } else {
     // ------------------------------------------------------------- epilogue warps 0-3: wait for the accumulators
     asm volatile("griddepcontrol.wait;" ::: "memory");
