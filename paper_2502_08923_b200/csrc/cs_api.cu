@@ -13,7 +13,7 @@ namespace {
 
 struct WsLayout {
   size_t x, xn, attn_out, act, qbuf, partial, attn_o, attn_ml, ssq, rope_cs, inv_freq, tile_max, tile_idx,
-      row_tok, row_pos, row_lim, row_write, seq_ok, status, loop_last, loop_draft, loop_dlen, loop_mpos,
+      row_tok, row_pos, row_lim, row_write, seq_ok, pair_part, pair_flag, status, loop_last, loop_draft, loop_dlen, loop_mpos,
       loop_emitted, loop_done, loop_accept, loop_out, loop_argmax, loop_stats, total;
   size_t qkv_elems;
   int attn_splits;
@@ -66,6 +66,8 @@ WsLayout ws_layout(const cs_model_config* c) {
   L.row_lim = take(&off, rows * 4);
   L.row_write = take(&off, rows * 4);
   L.seq_ok = take(&off, rows * 4);
+  L.pair_part = take(&off, (size_t)CS_MAX_PAIRS * 2 * CS_MAX_ROWS * CS_GEMM_BM * 4);
+  L.pair_flag = take(&off, CS_MAX_PAIRS * 2 * 4);
   L.status = take(&off, 256);
   L.loop_last = take(&off, rows * 4);
   L.loop_draft = take(&off, rows * 4);
@@ -89,15 +91,16 @@ cs_status fail(cs_ctx* ctx, cs_status s, const char* msg) {
   return s;
 }
 
-cs_status ensure_act_maps(cs_ctx* ctx, int n_tok) {
-  if (ctx->act_ntok == n_tok) return CS_OK;
+cs_status ensure_act_maps(cs_ctx* ctx, int rows) {
+  const int box = cs_gemm_act_box(CS_EPI_RESIDUAL, rows, true);
+  if (ctx->act_box == box) return CS_OK;
   const cs_model_config& c = ctx->cfg;
   cs_status s;
-  if ((s = cs_make_act_map(ctx, &ctx->tmXn, ctx->xn, 2 * CS_MAX_ROWS, c.d_model, n_tok)) != CS_OK) return s;
-  if ((s = cs_make_act_map(ctx, &ctx->tmAttn, ctx->attn_out, 2 * CS_MAX_ROWS, c.n_heads * c.head_dim, n_tok)) != CS_OK)
+  if ((s = cs_make_act_map(ctx, &ctx->tmXn, ctx->xn, 2 * CS_MAX_ROWS, c.d_model, box)) != CS_OK) return s;
+  if ((s = cs_make_act_map(ctx, &ctx->tmAttn, ctx->attn_out, 2 * CS_MAX_ROWS, c.n_heads * c.head_dim, box)) != CS_OK)
     return s;
-  if ((s = cs_make_act_map(ctx, &ctx->tmAct, ctx->act, 2 * CS_MAX_ROWS, c.d_ffn, n_tok)) != CS_OK) return s;
-  ctx->act_ntok = n_tok;
+  if ((s = cs_make_act_map(ctx, &ctx->tmAct, ctx->act, 2 * CS_MAX_ROWS, c.d_ffn, box)) != CS_OK) return s;
+  ctx->act_box = box;
   return CS_OK;
 }
 
@@ -107,10 +110,8 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
                           cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
   const int rows = B * R;
-  // second bf16 term of every activation operand (row offset in the operand maps), or -1 when the
-  // caller settles for the leading term
-  const int lo_row = ctx->one_term ? -1 : CS_MAX_ROWS;
-  cs_status s = ensure_act_maps(ctx, cs_ceil_div(rows, 16) * 16);
+  const int lo_row = CS_MAX_ROWS;      // second bf16 term of every activation operand: row offset in the operand maps
+  cs_status s = ensure_act_maps(ctx, rows);
   if (s != CS_OK) return s;
   // Only the first RMSNorm runs as a kernel.  Every later one is folded into the GEMMs around
   // it: the residual GEMM before it writes gain * x (two bf16 terms) and sums of squares, the
@@ -137,11 +138,7 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     if (s != CS_OK) return s;
     take_norm = NormFuse{};
     take_norm.ssq_in = ctx->ssq;
-    {
-      GemmShape sh;
-      if (cs_gemm_shape(ctx, &L.o, rows, lo_row >= 0, &sh) != CS_OK) return fail(ctx, CS_ERR_UNSUPPORTED, "no launch shape for the attention-output GEMM");
-      take_norm.slots_in = cs_ceil_div(L.o.N, CS_GEMM_BM) * sh.splits;
-    }
+    take_norm.slots_in = cs_ceil_div(L.o.N, CS_GEMM_BM) * cs_gemm_splits(ctx, &L.o, CS_EPI_RESIDUAL, rows, true);
     take_norm.slot_stride = ctx->ssq_stride;
     take_norm.inv_d = 1.f / (float)c.d_model;
     take_norm.eps = c.rms_eps;
@@ -154,11 +151,7 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     s = cs_launch_gemm(ctx, &L.down, &ctx->tmAct, lo_row, rows, CS_EPI_RESIDUAL, ctx->x, nullptr, nullptr, 0, nullptr,
                        &give, st);
     if (s != CS_OK) return s;
-    {
-      GemmShape sh;
-      if (cs_gemm_shape(ctx, &L.down, rows, lo_row >= 0, &sh) != CS_OK) return fail(ctx, CS_ERR_UNSUPPORTED, "no launch shape for the down GEMM");
-      take_norm.slots_in = cs_ceil_div(L.down.N, CS_GEMM_BM) * sh.splits;
-    }
+    take_norm.slots_in = cs_ceil_div(L.down.N, CS_GEMM_BM) * cs_gemm_splits(ctx, &L.down, CS_EPI_RESIDUAL, rows, true);
   }
   if (with_lm) {
     s = cs_launch_gemm(ctx, &ctx->lm, &ctx->tmXn, lo_row, rows, CS_EPI_ARGMAX, logits, nullptr, nullptr, 0, nullptr,
@@ -305,6 +298,8 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   ctx->row_lim = reinterpret_cast<int*>(base + L.row_lim);
   ctx->row_write = reinterpret_cast<int*>(base + L.row_write);
   ctx->seq_ok = reinterpret_cast<int*>(base + L.seq_ok);
+  ctx->pair_part = reinterpret_cast<float*>(base + L.pair_part);
+  ctx->pair_flag = reinterpret_cast<int*>(base + L.pair_flag);
   ctx->d_status = reinterpret_cast<int*>(base + L.status);
   ctx->loop_last = reinterpret_cast<int*>(base + L.loop_last);
   ctx->loop_draft = reinterpret_cast<int*>(base + L.loop_draft);
@@ -373,6 +368,8 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream) {
   CS_CUDA_OK(ctx, cudaMemcpyAsync(&bits, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   CS_CUDA_OK(ctx, cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st));
   CS_CUDA_OK(ctx, cudaStreamSynchronize(st));
+  // a wait that ran out may have left a hand-over flag of the two-SM GEMM raised
+  if (bits & CS_DEV_TIMEOUT) CS_CUDA_OK(ctx, cudaMemsetAsync(ctx->pair_flag, 0, CS_MAX_PAIRS * 2 * sizeof(int), st));
   return status_from_bits(ctx, bits);
 }
 
@@ -436,7 +433,7 @@ cs_status cs_verify_step_cached(cs_ctx* ctx, const int32_t* last_tok, const int3
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
     *g = VerifyGraph{};
-    cs_status s = ensure_act_maps(ctx, cs_ceil_div(B * (k + 1), 16) * 16);   // host work that must precede capture
+    cs_status s = ensure_act_maps(ctx, B * (k + 1));   // host work that must precede capture
     if (s != CS_OK) return s;
     CS_CUDA_OK(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed));
     ctx->stamp_n = 0;
@@ -532,7 +529,7 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
       if (G.exec) cudaGraphExecDestroy(G.exec);
       if (G.graph) cudaGraphDestroy(G.graph);
       G.exec = nullptr; G.graph = nullptr;
-      s = ensure_act_maps(ctx, cs_ceil_div(B * (k + 1), 16) * 16);   // host work that must precede capture
+      s = ensure_act_maps(ctx, B * (k + 1));   // host work that must precede capture
       if (s != CS_OK) return s;
       CS_CUDA_OK(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed));
       s = enqueue(ctx->cap_stream);
@@ -598,9 +595,8 @@ cs_status cs_prefill(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, 
     ctx->stamp_n = 0;
     cs_launch_prefill_setup(ctx, hist, hist_len, B, stride, start, r, st);
     cs_status s = enqueue_forward(ctx, B, r, kv_cache, false, nullptr, st);
-    if (s != CS_OK) { ctx->one_term = false; return s; }
+    if (s != CS_OK) return s;
   }
-  ctx->one_term = false;
   if (total <= 0) cs_launch_prefill_setup(ctx, hist, hist_len, B, stride, 0, 1, st);   // sets seq_ok
   cs_launch_prefill_finish(ctx, hist_len, kv_len, B, st);
   CS_CUDA_OK(ctx, cudaGetLastError());
@@ -635,7 +631,7 @@ cs_status cs_loop_begin(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, in
   cs_launch_loop_init(ctx, hist_len, kv_len, B, stride, max_new, k, st);
   CS_CUDA_OK(ctx, cudaGetLastError());
   // the activation maps must exist before capture (encoding them is host work)
-  cs_status s = ensure_act_maps(ctx, cs_ceil_div(B * (k + 1), 16) * 16);
+  cs_status s = ensure_act_maps(ctx, B * (k + 1));
   if (s != CS_OK) return s;
   if (L.use_graph) {
     // captured on the context's own stream (the legacy default stream cannot capture),
@@ -805,7 +801,7 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
   if (s != CS_OK) return s;
   const int n_tok = cs_ceil_div(rows, 16) * 16;
   CUtensorMap tmX;
-  if ((s = cs_make_act_map(ctx, &tmX, X, n_tok, K, n_tok)) != CS_OK) return s;
+  if ((s = cs_make_act_map(ctx, &tmX, X, n_tok, K, cs_gemm_act_box(CS_EPI_STORE, rows, false))) != CS_OK) return s;
   return cs_launch_gemm(ctx, &g, &tmX, -1, rows, CS_EPI_STORE, Y, nullptr, nullptr, 0, nullptr, nullptr, st);
 }
 
@@ -815,7 +811,7 @@ cs_status cs_lm_head(cs_ctx* ctx, const void* X, int rows, int32_t* ids, float* 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int n_tok = cs_ceil_div(rows, 16) * 16;
   CUtensorMap tmX;
-  cs_status s = cs_make_act_map(ctx, &tmX, X, n_tok, ctx->cfg.d_model, n_tok);
+  cs_status s = cs_make_act_map(ctx, &tmX, X, n_tok, ctx->cfg.d_model, cs_gemm_act_box(CS_EPI_ARGMAX, rows, false));
   if (s != CS_OK) return s;
   if ((s = cs_launch_gemm(ctx, &ctx->lm, &tmX, -1, rows, CS_EPI_ARGMAX, logits_dbg, nullptr, nullptr, 0, nullptr, nullptr, st)) != CS_OK) return s;
   cs_launch_tile_reduce(ctx, rows, ids, st);

@@ -27,6 +27,8 @@ static constexpr int CS_GEMM_BK = 64;     // K elements per stage (one 128-byte 
 static constexpr int CS_MAX_GAMMA = 8;
 static constexpr int CS_MAX_SPLITS = 8;   // split-K factor limit (portable cluster size)
 static constexpr int CS_SPLIT_TILE_CAP = 640;  // tiles * splits never exceeds this (unless splits == 1)
+static constexpr int CS_PAIR_MAX_SPLITS = 4;   // split-K factor limit of the two-SM GEMM (its clusters hold 2 x splits CTAs)
+static constexpr int CS_MAX_PAIRS = 80;        // persistent SM pairs of its stream form, at most
 
 struct GemmPlan {
   CUtensorMap tmW;      // weights [N][K], box 128 x 64, 128-byte swizzle
@@ -35,13 +37,6 @@ struct GemmPlan {
   int splits;           // split-K factor
   int kb_per_split;     // 64-wide K blocks per split
   bool allow_split;
-};
-
-// how one GEMM is launched for a given block height
-struct GemmShape {
-  int n_tok;            // token rows rounded up to 16 (UMMA N)
-  int mt;               // 128-feature sub-tiles per CTA
-  int splits, kb_per_split, stages, stage_bytes, smem;
 };
 
 struct LayerPlan {
@@ -132,6 +127,8 @@ struct cs_ctx {
   int* row_lim;              // number of keys a row attends to (0 = dead row)
   int* row_write;            // 1 = this row's K/V go into the cache
   int* seq_ok;               // per sequence: 1 = takes part in this step
+  float* pair_part;          // two-SM GEMM: sums of tiles cut between pairs [CS_MAX_PAIRS][2][CS_MAX_ROWS][128]
+  int* pair_flag;            // and their "written" flags [CS_MAX_PAIRS][2], 0 between launches
   int* d_status;             // device status word
   // loop state, all [max_batch] unless noted
   int* loop_last;
@@ -146,7 +143,7 @@ struct cs_ctx {
   unsigned long long* loop_stats;  // image of cs_stats
 
   // activation operand maps, rebuilt when the block height changes
-  int act_ntok;
+  int act_box;               // token rows per copy
   CUtensorMap tmXn, tmAttn, tmAct;
 
   // tensor-core attention: maps over the whole KV cache (rebuilt when the cache pointer
@@ -161,12 +158,11 @@ struct cs_ctx {
   const int* kv_len_early;
   // shared-memory opt-ins already made for this context's device (per context, not per
   // process: another context may live on another GPU)
-  bool gemm_attr_set;
-  int tall_clusters[3][CS_MAX_SPLITS + 1];   // clusters of a tall GEMM launch that can run at once, by sub-tile count and cluster size (0 = not asked yet)
+  bool gemm_attr_set, pair_attr_set;
+  int pair_clusters[CS_PAIR_MAX_SPLITS + 1];   // clusters of 2 x S CTAs that can run at once, by S (0 = not asked yet)
   unsigned attn_mma_attr_set;   // bit DH/32 per head size
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
-  bool one_term;             // the forward being enqueued feeds its GEMMs the leading bf16 term only
   bool no_graph;             // CS_NO_GRAPH=1 at creation: steps are enqueued kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
@@ -287,7 +283,6 @@ cs_status cs_launch_gram_update(void* index, int B, int capacity_tokens, const i
                                 int stride, int gamma, int max_chunks, int* status, cudaStream_t st);
 // cs_gemm.cu
 cs_status cs_gemm_plan(cs_ctx* ctx, GemmPlan* g, const void* w, int N, int K, bool allow_split);
-cs_status cs_gemm_shape(const cs_ctx* ctx, const GemmPlan* g, int rows, bool two_terms, GemmShape* out);
 cs_status cs_make_act_map(cs_ctx* ctx, CUtensorMap* tm, const void* base, int rows_total, int K,
                           int box_rows);
 // mode = CS_EPI_*: `out` is the fp32 destination (STORE, RESIDUAL) or the optional logits dump
@@ -296,6 +291,21 @@ cs_status cs_make_act_map(cs_ctx* ctx, CUtensorMap* tm, const void* base, int ro
 cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode,
                          float* out, __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
                          cudaStream_t st);
+// cs_gemm_pair.cu
+// Which GEMMs run on pairs of SMs: the gate/up and LM-head projections of every block - a persistent
+// stream over all tiles, 40.1 us against 41.0 and 153 against 168 us already at 11 rows - and the
+// others from 33 rows on: at 44 rows QKV takes 14.5 against 16.3 us, attention output 13.5 / 14.1,
+// down 26.6 / 27.0; at 22 rows the cluster of one-SM tiles is ahead (12.7 / 12.9, 11.1 / 11.0, 24.8 / 22.9).
+static inline bool cs_gemm_on_pairs(int mode, int rows) { return mode == CS_EPI_SWIGLU || mode == CS_EPI_ARGMAX || rows > 32; }
+// token rows per copy of the activations (two terms of at most 128 rows: a term per copy, in both kernels)
+static inline int cs_gemm_act_box(int mode, int rows, bool two_terms) {
+  const int n_tok = cs_ceil_div(rows, 16) * 16;
+  return !cs_gemm_on_pairs(mode, rows) || (two_terms && n_tok <= 128) ? n_tok : n_tok / 2;
+}
+int cs_gemm_splits(const cs_ctx* ctx, const GemmPlan* g, int mode, int rows, bool two_terms);   // split-K factor of a launch
+cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode, float* out,
+                              __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
+                              cudaStream_t st);
 // cs_layers.cu
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip,

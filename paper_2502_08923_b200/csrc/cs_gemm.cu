@@ -1,5 +1,6 @@
 // Skinny bf16 projections of the verification forward (Sec. 3.2): Y = X W^T with at most
-// 256 token rows and a large weight matrix that is streamed from HBM exactly once.
+// 32 token rows and a large weight matrix that is streamed from HBM exactly once.  (Taller blocks,
+// and the gate/up and LM-head projections of any height, are in cs_gemm_pair.cu.)
 //
 // The weight matrix is the M operand of the tensor-core instruction ("swap A/B"): one CTA
 // owns 128 output features (UMMA M = 128) and all token rows (UMMA N = rows rounded up to
@@ -20,10 +21,8 @@
 //   QKV       rotates q and k (RoPE), writes q as the attention operand and appends the new
 //             K/V rows to the bf16 cache            (QKV projection)
 //   RESIDUAL  x[row][n]   += y                      (attention output and FFN down projections)
-//   SWIGLU    act[row][j]  = bf16(silu(gate_j) * up_j), the tile holding 64 gate rows and the
-//             64 matching up rows                   (FFN gate/up projection)
 //   ARGMAX    per 128-feature tile (max logit, lowest token id) per row; logits are only
-//             written when a debug buffer is given   (LM head)
+//             written when a debug buffer is given   (cs_lm_head_static, which has no workspace)
 //
 // The kernel is launched with programmatic dependent launch: it starts while its
 // predecessor drains, fills its pipeline with weight tiles (which depend on nothing) and
@@ -32,14 +31,13 @@
 // Copies and MMAs are issued by an elected lane with uniform operands (cs_tcgen.cuh): a stage goes
 // back to the producer some 800 clocks sooner than when one lane issued the eight MMAs of a K block.
 // Measured on an 11-row block of the 8B shape, before and after: QKV 12.4 -> 12.1 us, attention output
-// 11.0 -> 9.8, gate/up 44.4 -> 42.2, down 23.7 -> 22.2, LM head 186 -> 170 us (6.2 TB/s).
+// 11.0 -> 9.8, down 23.7 -> 22.2.
 //
 // Every wait is bounded: when it runs out the CTA records CS_DEV_TIMEOUT, drains its
 // copies, still takes part in the cluster barriers, frees its TMEM and returns.
 #include <stdlib.h>
 
 #include <algorithm>
-#include <type_traits>
 
 #include "cs_common.cuh"
 #include "cs_tcgen.cuh"
@@ -57,10 +55,7 @@ struct GemmArgs {
   int rows, n_tok, N, K;
   int num_kb, kb_per_split, splits, stages, mode;
   float* out;            // STORE / RESIDUAL: [rows][N] fp32; ARGMAX: optional logits [rows][N]
-  __nv_bfloat16* act;    // SWIGLU: [rows][F] bf16 (leading term)
-  __nv_bfloat16* act_lo; // SWIGLU: second bf16 term of the same values, or NULL
   int lo_row;            // row coordinate of the activation operand's second bf16 term, -1 = none
-  int F;
   QkvEpi q;              // QKV: where the rotated queries and the new K/V rows go
   NormFuse nf;           // RMSNorm folded into this GEMM's read-out (consumer) or residual update (producer)
   float* tile_max;       // ARGMAX: [rows][tile_stride] (a row's tile maxima are contiguous: the reduction reads them coalesced)
@@ -122,9 +117,6 @@ __device__ __forceinline__ void keep_alive(const float4& p, const float4& q) {
   asm volatile("" ::"f"(p.x), "f"(p.y), "f"(p.z), "f"(p.w), "f"(q.x), "f"(q.y), "f"(q.z), "f"(q.w) : "memory");
 }
 
-// MT = 128-feature sub-tiles per CTA (compile-time, so that the one-tile kernel of the short blocks
-// carries no loop overhead in its issue paths: its ring is latency-bound)
-template <int MT>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, GemmArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -133,8 +125,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   uint8_t* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);   // operand tiles need 1024-byte alignment
   const int xtile = a.n_tok * 128;                 // one activation tile
   const bool two = a.lo_row >= 0;                   // activations come as two bf16 terms
-  const int wbytes = MT * kTileABytes;            // the CTA's weight sub-tiles of one K block
-  const int stage_bytes = wbytes + (two ? 2 : 1) * xtile;
+  const int stage_bytes = kTileABytes + (two ? 2 : 1) * xtile;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)a.stages * stage_bytes);
   // bars[0..stages) = tile landed, bars[stages..2*stages) = tile consumed, bars[2*stages] = accumulator done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * a.stages + 1);
@@ -151,14 +142,13 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   }
 
   const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int cta_tile = blockIdx.x;
+  const int tile = blockIdx.x, n0 = tile * CS_GEMM_BM;
   const int split = (int)blockIdx.y;             // = the rank in the cluster of (1, splits, 1)
-  const int cta_n0 = cta_tile * MT * CS_GEMM_BM;
   const int kb0 = split * a.kb_per_split;
   const int kb1 = min(a.num_kb, kb0 + a.kb_per_split);
   const int nkb = max(0, kb1 - kb0);
   uint32_t tmem_cols = 32;
-  while ((int)tmem_cols < MT * a.n_tok) tmem_cols <<= 1;   // one accumulator of n_tok columns per sub-tile
+  while ((int)tmem_cols < a.n_tok) tmem_cols <<= 1;
 
   const uint32_t bar_full = smem_u32(bars), bar_empty = smem_u32(bars + a.stages),
                  bar_acc = smem_u32(bars + 2 * a.stages);
@@ -191,13 +181,10 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     const uint32_t ring = smem_u32(smem);
     auto load_w = [&](int i, int s) {            // (by the elected lane)
       mbar_expect_tx(bar_full + 8 * s, (uint32_t)stage_bytes);
-#pragma unroll
-      for (int m = 0; m < MT; ++m)
-        tma_load_2d(ring + (uint32_t)(s * stage_bytes + m * kTileABytes), &tmW, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK,
-                    cta_n0 + m * CS_GEMM_BM);
+      tma_load_2d(ring + (uint32_t)(s * stage_bytes), &tmW, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, n0);
     };
     auto load_x = [&](int i, int s) {
-      const uint32_t sx = ring + (uint32_t)(s * stage_bytes + wbytes);
+      const uint32_t sx = ring + (uint32_t)(s * stage_bytes + kTileABytes);
       tma_load_2d(sx, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, 0);
       if (two) tma_load_2d(sx + xtile, &tmX, bar_full + 8 * s, (kb0 + i) * CS_GEMM_BK, a.lo_row);
     };
@@ -233,7 +220,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.n_tok >> 3) << 17) |
                            ((uint32_t)(CS_GEMM_BM >> 4) << 24);
     const uint64_t desc0 = desc_kmajor(smem_u32(smem));
-    const uint64_t x_off = (uint64_t)(wbytes >> 4), lo_off = (uint64_t)((wbytes + xtile) >> 4);
+    const uint64_t x_off = kTileABytes >> 4, lo_off = (uint64_t)(uint32_t)((kTileABytes + xtile) >> 4);
     int s = 0;
     uint32_t ph = 0;
     for (int i = 0; i < nkb; ++i) {
@@ -243,14 +230,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
       if (elect_one()) {
         const uint64_t d = desc0 + (uint64_t)(uint32_t)(s * (stage_bytes >> 4));
 #pragma unroll
-        for (int m = 0; m < MT; ++m) {                   // every sub-tile against the same activation tile
-          const uint64_t da = d + (uint64_t)(m * (kTileABytes >> 4));
-          const uint32_t acc = tmem_base + (uint32_t)(m * a.n_tok);
-#pragma unroll
-          for (int kk = 0; kk < CS_GEMM_BK / 16; ++kk) {   // 16 K-elements = 32 bytes per instruction
-            umma_bf16(acc, da + 2 * kk, d + x_off + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
-            if (two) umma_bf16(acc, da + 2 * kk, d + lo_off + 2 * kk, idesc, 1u);   // x = hi + lo
-          }
+        for (int kk = 0; kk < CS_GEMM_BK / 16; ++kk) {   // 16 K-elements = 32 bytes per instruction
+          umma_bf16(tmem_base, d + 2 * kk, d + x_off + 2 * kk, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+          if (two) umma_bf16(tmem_base, d + 2 * kk, d + lo_off + 2 * kk, idesc, 1u);   // x = hi + lo
         }
         umma_commit(bar_empty + 8 * s);
       }
@@ -292,13 +274,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   }
   if (warp >= 4) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  // One pass per 128-feature sub-tile: read its accumulator out, then (all but ARGMAX) the split-K
-  // reduction and the epilogue.  Every CTA of a cluster takes the same number of passes.
-#pragma unroll 1
-  for (int m = 0; m < MT; ++m) {
-  const int tile = cta_tile * MT + m;
-  const int n0 = cta_n0 + m * CS_GEMM_BM;
-  if (n0 >= a.N) break;
   if (warp < 4) {
     // ------------------------------------------------------------- accumulator read-out (warps 0-3)
     const int feat = n0 + warp * 32 + lane;
@@ -306,7 +281,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     for (int c0 = 0; c0 < a.n_tok && c0 < a.rows; c0 += 16) {
       uint32_t v[16];
       if (nkb > 0 && ok) {
-        tmem_ld16(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(m * a.n_tok + c0), v);
+        tmem_ld16(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
       } else {
 #pragma unroll
         for (int j = 0; j < 16; ++j) v[j] = 0u;
@@ -353,7 +328,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
           a.tile_idx[(size_t)tok * a.tile_stride + tile] = idx;
         }
       }
-      if (MT > 1) asm volatile("bar.sync 1, 128;" ::: "memory");   // the scratch rows are reused by the next pass
     }
   }
 
@@ -447,55 +421,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
             *reinterpret_cast<uint2*>(dst + half) = *reinterpret_cast<const uint2*>(h1);
           }
         }
-      } else if (a.mode == CS_EPI_SWIGLU) {
-        // features 0..63 of the tile are gate rows, 64..127 the matching up rows; each rank
-        // finishes a slice of j (a multiple of 4 wide), four consecutive j per thread
-        const int js = ((64 + a.splits - 1) / a.splits + 3) & ~3;
-        const int j_lo = split * js, j_n = max(0, min(64, j_lo + js) - j_lo);
-        const int per_tok = j_n >> 2;
-        const int total = per_tok * a.rows, iters = (total + 127) >> 7;
-        for (int it = 0; it < iters; ++it) {
-          const int idx = e + (it << 7);
-          const bool act = idx < total;
-          const int idc = act ? idx : 0;
-          const int j = j_lo + 4 * (idc % per_tok), tok = idc / per_tok;
-          float4 g = make_float4(0.f, 0.f, 0.f, 0.f), u = g;
-          if (a.splits > 1) {
-            if (act) {
-              g = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok * CS_GEMM_BM + j), a.splits);
-              u = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok * CS_GEMM_BM + 64 + j), a.splits);
-            }
-            if (it == iters - 1) { keep_alive(g, u); cluster_arrive(); arrived = true; }
-          } else if (act) {
-            g = *reinterpret_cast<const float4*>(dump + tok * CS_GEMM_BM + j);
-            u = *reinterpret_cast<const float4*>(dump + tok * CS_GEMM_BM + 64 + j);
-          }
-          if (!act) continue;
-          const float gv[4] = {g.x, g.y, g.z, g.w}, uv[4] = {u.x, u.y, u.z, u.w};
-          const int jj0 = tile * 64 + j;
-          if ((a.F & 3) == 0 && jj0 + 3 < a.F) {
-            float v4[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v4[i] = __fdividef(gv[i], 1.f + __expf(-gv[i])) * uv[i];
-            __nv_bfloat162 h[2], l[2];
-            h[0] = __floats2bfloat162_rn(v4[0], v4[1]); h[1] = __floats2bfloat162_rn(v4[2], v4[3]);
-            const float2 h0 = __bfloat1622float2(h[0]), h1 = __bfloat1622float2(h[1]);
-            l[0] = __floats2bfloat162_rn(v4[0] - h0.x, v4[1] - h0.y); l[1] = __floats2bfloat162_rn(v4[2] - h1.x, v4[3] - h1.y);
-            *reinterpret_cast<uint2*>(a.act + (size_t)tok * a.F + jj0) = *reinterpret_cast<const uint2*>(h);
-            if (a.act_lo != nullptr) *reinterpret_cast<uint2*>(a.act_lo + (size_t)tok * a.F + jj0) = *reinterpret_cast<const uint2*>(l);
-            continue;
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int jj = tile * 64 + j + i;
-            if (jj < a.F) {
-              const float v = __fdividef(gv[i], 1.f + __expf(-gv[i])) * uv[i];
-              const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-              a.act[(size_t)tok * a.F + jj] = hi;
-              if (a.act_lo != nullptr) a.act_lo[(size_t)tok * a.F + jj] = __float2bfloat16_rn(v - __bfloat162float(hi));
-            }
-          }
-        }
       } else {
         const int fs = ((CS_GEMM_BM + a.splits - 1) / a.splits + 3) & ~3;
         const int f_lo = split * fs, f_n = max(0, min(CS_GEMM_BM, f_lo + fs) - f_lo);
@@ -504,77 +429,47 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
         float* part = dump + a.n_tok * CS_GEMM_BM;   // [rows][32] sums of squares, behind the parked tile
         const int total = per_tok * a.rows, iters = (total + 127) >> 7;
         const bool vec_n = (a.N & 3) == 0;
-        // Tall blocks take two items per turn: the remote reads and the residual reads of both are
-        // requested before either is finished, so a dozen turns per thread overlap pairwise (128
-        // threads on an otherwise idle SM have nothing else to hide those latencies behind).  Short
-        // blocks have one turn and take it without the second item's bookkeeping.
-        auto turns = [&](auto per_turn) {
-        constexpr int NU = decltype(per_turn)::value;
-        for (int it = 0; it < iters; it += NU) {
-          int idx[NU], f[NU], tok[NU];
-          bool act[NU], vec[NU];
-          float4 y[NU], x[NU];
-#pragma unroll
-          for (int u = 0; u < NU; ++u) {
-            idx[u] = e + ((it + u) << 7);
-            act[u] = it + u < iters && idx[u] < total;
-            const int idc = act[u] ? idx[u] : 0;
-            f[u] = f_lo + 4 * (idc % per_tok);
-            tok[u] = idc / per_tok;
-            vec[u] = vec_n && n0 + f[u] + 3 < a.N;
-            y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            x[u] = y[u];
+        for (int it = 0; it < iters; ++it) {
+          const int idx = e + (it << 7);
+          const bool act = idx < total;
+          const int idc = act ? idx : 0;
+          const int f = f_lo + 4 * (idc % per_tok), tok = idc / per_tok;
+          const bool vec = vec_n && n0 + f + 3 < a.N;
+          float4 y = make_float4(0.f, 0.f, 0.f, 0.f), x = y;
+          if (act) {
+            if (a.splits > 1) y = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok * CS_GEMM_BM + f), a.splits);
+            else y = *reinterpret_cast<const float4*>(dump + tok * CS_GEMM_BM + f);
+            if (a.mode == CS_EPI_RESIDUAL && vec)
+              x = (it == 0) ? x_pre : *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
           }
-          if (a.splits > 1) {
-#pragma unroll
-            for (int u = 0; u < NU; ++u)
-              if (act[u]) y[u] = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok[u] * CS_GEMM_BM + f[u]), a.splits);
-          } else {
-#pragma unroll
-            for (int u = 0; u < NU; ++u)
-              if (act[u]) y[u] = *reinterpret_cast<const float4*>(dump + tok[u] * CS_GEMM_BM + f[u]);
-          }
-          if (a.mode == CS_EPI_RESIDUAL) {
-#pragma unroll
-            for (int u = 0; u < NU; ++u)
-              if (act[u] && vec[u])
-                x[u] = (it + u == 0) ? x_pre : *reinterpret_cast<const float4*>(a.out + (size_t)tok[u] * a.N + n0 + f[u]);
-          }
-          if (a.splits > 1 && it + NU >= iters) { keep_alive(y[0], y[NU - 1]); cluster_arrive(); arrived = true; }
-#pragma unroll
-          for (int u = 0; u < NU; ++u) {
-            if (!act[u]) continue;
-            if (feeds_norm) part[tok[u] * 32 + idx[u] % per_tok] = 0.f;
-            float* dst = a.out + (size_t)tok[u] * a.N + n0 + f[u];
-            if (vec[u]) {
-              float4 o = y[u];
-              o.x += x[u].x; o.y += x[u].y; o.z += x[u].z; o.w += x[u].w;   // (x stays 0 unless this is a residual update)
-              *reinterpret_cast<float4*>(dst) = o;
-              if (feeds_norm) {
-                const uint2 gw = *reinterpret_cast<const uint2*>(a.nf.gain_out + n0 + f[u]);
-                const float2 g01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.x));
-                const float2 g23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.y));
-                const float w0 = o.x * g01.x, w1 = o.y * g01.y, w2 = o.z * g23.x, w3 = o.w * g23.y;
-                __nv_bfloat162 h[2], l[2];
-                h[0] = __floats2bfloat162_rn(w0, w1); h[1] = __floats2bfloat162_rn(w2, w3);
-                const float2 h0 = __bfloat1622float2(h[0]), h1 = __bfloat1622float2(h[1]);
-                l[0] = __floats2bfloat162_rn(w0 - h0.x, w1 - h0.y); l[1] = __floats2bfloat162_rn(w2 - h1.x, w3 - h1.y);
-                __nv_bfloat16* xo = a.nf.xn_out + (size_t)tok[u] * a.N + n0 + f[u];
-                *reinterpret_cast<uint2*>(xo) = *reinterpret_cast<const uint2*>(h);
-                *reinterpret_cast<uint2*>(xo + (size_t)CS_MAX_ROWS * a.N) = *reinterpret_cast<const uint2*>(l);
-                part[tok[u] * 32 + idx[u] % per_tok] = (o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w);
-              }
-            } else {
-              const float yv[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
-#pragma unroll
-              for (int i = 0; i < 4; ++i)
-                if (n0 + f[u] + i < a.N) dst[i] = (a.mode == CS_EPI_RESIDUAL) ? dst[i] + yv[i] : yv[i];
+          if (a.splits > 1 && it == iters - 1) { keep_alive(y, y); cluster_arrive(); arrived = true; }
+          if (!act) continue;
+          if (feeds_norm) part[tok * 32 + idx % per_tok] = 0.f;
+          float* dst = a.out + (size_t)tok * a.N + n0 + f;
+          if (vec) {
+            const float4 o = make_float4(y.x + x.x, y.y + x.y, y.z + x.z, y.w + x.w);   // (x stays 0 unless this is a residual update)
+            *reinterpret_cast<float4*>(dst) = o;
+            if (feeds_norm) {
+              const uint2 gw = *reinterpret_cast<const uint2*>(a.nf.gain_out + n0 + f);
+              const float2 g01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.x));
+              const float2 g23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.y));
+              const float w0 = o.x * g01.x, w1 = o.y * g01.y, w2 = o.z * g23.x, w3 = o.w * g23.y;
+              __nv_bfloat162 h[2], l[2];
+              h[0] = __floats2bfloat162_rn(w0, w1); h[1] = __floats2bfloat162_rn(w2, w3);
+              const float2 h0 = __bfloat1622float2(h[0]), h1 = __bfloat1622float2(h[1]);
+              l[0] = __floats2bfloat162_rn(w0 - h0.x, w1 - h0.y); l[1] = __floats2bfloat162_rn(w2 - h1.x, w3 - h1.y);
+              __nv_bfloat16* xo = a.nf.xn_out + (size_t)tok * a.N + n0 + f;
+              *reinterpret_cast<uint2*>(xo) = *reinterpret_cast<const uint2*>(h);
+              *reinterpret_cast<uint2*>(xo + (size_t)CS_MAX_ROWS * a.N) = *reinterpret_cast<const uint2*>(l);
+              part[tok * 32 + idx % per_tok] = (o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w);
             }
+          } else {
+            const float yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (n0 + f + i < a.N) dst[i] = (a.mode == CS_EPI_RESIDUAL) ? dst[i] + yv[i] : yv[i];
           }
         }
-        };
-        if (iters > 1) turns(std::integral_constant<int, 2>{});
-        else turns(std::integral_constant<int, 1>{});
         if (feeds_norm) {
           asm volatile("bar.sync 1, 128;" ::: "memory");
           for (int tok = e; tok < a.rows; tok += 128) {
@@ -587,12 +482,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     }
     if (a.splits > 1) {
       if (!arrived) cluster_arrive();
-      cluster_wait();                              // nobody leaves (or parks its next tile) while a peer still reads this one
-    } else if (MT > 1) {
-      __syncthreads();                             // the parked tile is read out before the next one is parked
+      cluster_wait();                              // nobody leaves while a peer still reads its tile
     }
   }
-  }   // sub-tile passes
   // ---------------------------------------------------------------- teardown
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -622,6 +514,10 @@ EncodeTiledFn get_encode() {
   }
   return fn;
 }
+
+// what a CTA needs behind the ring: alignment slack, up to 2 * 8 + 1 barriers, the TMEM slot and flags, the
+// ARGMAX scratch and 1/rms
+int gemm_fixed_bytes(int n_tok) { return 1024 + (2 * 8 + 1) * 8 + 16 + 9 * n_tok * 4; }
 
 // [rows][K] bf16 row-major, tiles of box_rows x 64 elements, 128-byte swizzle, zero fill
 cs_status encode_2d(cs_ctx* ctx, CUtensorMap* tm, const void* base, int rows, int K, int box_rows,
@@ -704,107 +600,9 @@ cs_status cs_gemm_plan(cs_ctx* ctx, GemmPlan* g, const void* w, int N, int K, bo
 
 static cs_status ensure_gemm_attrs(cs_ctx* ctx) {
   if (!ctx->gemm_attr_set) {
-    CS_CUDA_OK(ctx, cudaFuncSetAttribute(k_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    CS_CUDA_OK(ctx, cudaFuncSetAttribute(k_gemm_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-    CS_CUDA_OK(ctx, cudaFuncSetAttribute(k_gemm_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    CS_CUDA_OK(ctx, cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     ctx->gemm_attr_set = true;
   }
-  return CS_OK;
-}
-
-// How many clusters of `spl` one-CTA-per-SM CTAs the device runs at once.  A cluster has to find
-// all its CTAs inside one GPC, so this can be well below SMs / spl: 48 clusters of 3 do not fit
-// on 148 SMs, and a launch that needs them takes two waves.  Asked of the runtime once per shape.
-static int tall_clusters_at_once(const cs_ctx* cctx, int mt, int spl, int smem) {
-  cs_ctx* ctx = const_cast<cs_ctx*>(cctx);
-  if (spl <= 1) return ctx->num_sms;
-  int& slot = ctx->tall_clusters[mt == 4 ? 2 : (mt == 2 ? 1 : 0)][spl];
-  if (slot == 0) {
-    int n = 0;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(ctx->num_sms, spl, 1);
-    lc.blockDim = dim3(kThreads, 1, 1);
-    lc.dynamicSmemBytes = (size_t)smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = spl; at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    void (*kernel)(const CUtensorMap, const CUtensorMap, GemmArgs) = mt == 4 ? k_gemm_tc<4> : (mt == 2 ? k_gemm_tc<2> : k_gemm_tc<1>);
-    if (ensure_gemm_attrs(ctx) == CS_OK && cudaOccupancyMaxActiveClusters(&n, kernel, &lc) == cudaSuccess && n > 0) slot = n;
-    else { (void)cudaGetLastError(); slot = max(1, ctx->num_sms * 85 / 100 / spl); }   // no answer: the planner's allowance
-  }
-  return slot;
-}
-
-// Launch shape of one GEMM for a block of `rows` token rows.
-//  - Short blocks (two CTAs fit on an SM): one 128-feature tile per CTA and the plan's split-K
-//    factor, made for two CTAs per SM - the HBM-bound regime of 11-row blocks.
-//  - Tall blocks (one CTA per SM): every CTA re-reads its K range of the activations from L2,
-//    which at 100+ rows is several times the weight bytes, so a CTA takes 2 or 4 sub-tiles that
-//    share each activation tile (one TMEM accumulator each), and the split-K factor is chosen
-//    for whole waves of one CTA per SM.  Candidates are ranked by a cost model calibrated on
-//    measurements (K blocks per CTA times the cost of one, plus the epilogue, times waves).
-cs_status cs_gemm_shape(const cs_ctx* ctx, const GemmPlan* g, int rows, bool two_terms, GemmShape* out) {
-  GemmShape sh = {};
-  sh.n_tok = cs_ceil_div(rows, 16) * 16;
-  const int terms = two_terms ? 2 : 1;
-  const int xbytes = terms * sh.n_tok * 128;
-  const int tiles = cs_ceil_div(g->N, CS_GEMM_BM), kb = cs_ceil_div(g->K, CS_GEMM_BK);
-  // behind the ring: up to 2 * 8 + 1 barriers, the TMEM slot and flags, the ARGMAX scratch and 1/rms
-  const int fixed = 1024 /*alignment slack*/ + (2 * 8 + 1) * 8 + 16 + 9 * sh.n_tok * 4;
-  const size_t park = (size_t)sh.n_tok * (CS_GEMM_BM + 32) * 4;   // parked tile + sums of squares reuse the ring
-  const int sb1 = kTileABytes + xbytes;
-  // Two CTAs per SM wherever two stages fit into half an SM: the grids (224-240 CTAs) are
-  // sized for the 296 slots that gives.  Only blocks too tall for that take the whole SM.
-  int stages = (100 * 1024 - fixed) / sb1;
-  bool tall = false;
-  if (stages < 4) {
-    const int two = (113 * 1024 - fixed) / sb1;
-    if (two >= 2 && (size_t)two * sb1 >= park) stages = two;
-    else tall = true;
-  }
-  if (!tall) {
-    sh.mt = 1;
-    sh.stages = stages > 8 ? 8 : stages;
-    sh.splits = g->splits;
-    sh.kb_per_split = g->kb_per_split;
-    sh.stage_bytes = sb1;
-  } else {
-    long best = -1;
-    for (int mt = 1; mt <= 4; mt *= 2) {
-      if (mt * sh.n_tok > 512 || (mt > 1 && mt > tiles)) continue;
-      const int sb = mt * kTileABytes + xbytes;
-      int st = (220 * 1024 - fixed) / sb;
-      if (st > 8) st = 8;
-      if (st < 2 || (size_t)st * sb < park) continue;
-      const int ctas = cs_ceil_div(tiles, mt);
-      // Cycles of one K block, calibrated on 176-row blocks: the mt * terms * 4 MMAs take n_tok / 2
-      // cycles each; a stage comes back L cycles after it was handed to the producer (about 2,100
-      // for a 61 KB stage, 3,300 for a 77 KB one), and with `st` stages in flight a K block costs
-      // (L + mma) / st unless the tensor pipe is the slower.  The epilogue (accumulator read-out,
-      // split-K reduction over the cluster, stores) costs about 4,000 + 145 n_tok cycles per sub-tile.
-      const long mma = (long)mt * terms * 4 * (sh.n_tok / 2);
-      const long lat = 2120 + (long)((sb - 62464) * 0.072);
-      const long turn = ((lat > 1000 ? lat : 1000) + mma) / st;
-      const long per_kb = mma > turn ? mma : turn;
-      const long epi = (long)mt * (4000 + 145L * sh.n_tok);
-      const int smax = g->allow_split ? max(1, min(CS_MAX_SPLITS, kb / 4)) : 1;
-      for (int sp = 1; sp <= smax; ++sp) {
-        const int kps = cs_ceil_div(kb, sp), spl = cs_ceil_div(kb, kps);
-        const long waves = cs_ceil_div(ctas, tall_clusters_at_once(ctx, mt, spl, fixed + st * sb));
-        const long cost = waves * ((long)kps * per_kb + epi);
-        if (best < 0 || cost < best) {
-          best = cost;
-          sh.mt = mt; sh.stages = st; sh.splits = spl; sh.kb_per_split = kps; sh.stage_bytes = sb;
-        }
-      }
-    }
-    if (best < 0) return CS_ERR_UNSUPPORTED;
-  }
-  if (sh.stages < 2 || (size_t)sh.stages * sh.stage_bytes < park) return CS_ERR_UNSUPPORTED;
-  sh.smem = fixed + sh.stages * sh.stage_bytes;
-  *out = sh;
   return CS_OK;
 }
 
@@ -816,26 +614,18 @@ cs_status cs_make_act_map(cs_ctx* ctx, CUtensorMap* tm, const void* base, int ro
 cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode,
                          float* out, __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q,
                          const NormFuse* nf, cudaStream_t st) {
-  GemmShape sh;
-  if (cs_gemm_shape(ctx, g, rows, lo_row >= 0, &sh) != CS_OK) {
-    snprintf(ctx->err, sizeof(ctx->err), "no GEMM launch shape fits shared memory for %d rows", rows);
-    return CS_ERR_UNSUPPORTED;
-  }
-  const int tiles = cs_ceil_div(cs_ceil_div(g->N, CS_GEMM_BM), sh.mt);   // CTAs along the features
+  if (cs_gemm_on_pairs(mode, rows)) return cs_launch_gemm_pair(ctx, g, tmX, lo_row, rows, mode, out, act, act_lo, F, q, nf, st);
   GemmArgs a;
   a.rows = rows;
-  a.n_tok = sh.n_tok;
+  a.n_tok = cs_ceil_div(rows, 16) * 16;
   a.N = g->N;
   a.K = g->K;
   a.num_kb = cs_ceil_div(g->K, CS_GEMM_BK);
-  a.splits = sh.splits;
-  a.kb_per_split = sh.kb_per_split;
+  a.splits = g->splits;
+  a.kb_per_split = g->kb_per_split;
   a.mode = mode;
   a.out = out;
-  a.act = act;
-  a.act_lo = act_lo;
   a.lo_row = lo_row;
-  a.F = F;
   if (q != nullptr) a.q = *q;
   a.nf = NormFuse{};
   if (nf != nullptr) a.nf = *nf;
@@ -847,9 +637,12 @@ cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX,
   a.tile_idx = ctx->tile_idx;
   a.tile_stride = cs_ceil_div(g->N, CS_GEMM_BM);
   a.status = ctx->d_status;
-  a.stages = sh.stages;
-  const size_t smem = (size_t)sh.smem;
-  a.smem_bytes = sh.smem;
+  // 100 KB per CTA: two fit on an SM, and the grids (224-240 CTAs) are sized for the 296 slots that gives.
+  // The parked tile and the sums of squares reuse the ring (20 KB of at least 96 at 32 rows).
+  const int stage_bytes = kTileABytes + (lo_row >= 0 ? 2 : 1) * a.n_tok * 128, fixed = gemm_fixed_bytes(a.n_tok);
+  a.stages = min(8, (100 * 1024 - fixed) / stage_bytes);
+  a.smem_bytes = fixed + a.stages * stage_bytes;
+  const size_t smem = (size_t)a.smem_bytes;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, mode == CS_EPI_ARGMAX ? CS_FAM_LMHEAD : CS_FAM_GEMM);
   a.drop_kb = ctx->debug_drop_kb;
@@ -858,14 +651,12 @@ cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX,
     snprintf(ctx->err, sizeof(ctx->err), "the dropped-tile test hook is for launches without split-K");
     return CS_ERR_UNSUPPORTED;
   }
-  void (*kernel)(const CUtensorMap, const CUtensorMap, GemmArgs) =
-      sh.mt == 4 ? k_gemm_tc<4> : (sh.mt == 2 ? k_gemm_tc<2> : k_gemm_tc<1>);
   {
     const cs_status as = ensure_gemm_attrs(ctx);
     if (as != CS_OK) return as;
   }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(tiles, a.splits, 1);
+  lc.gridDim = dim3(cs_ceil_div(g->N, CS_GEMM_BM), a.splits, 1);
   lc.blockDim = dim3(kThreads, 1, 1);
   lc.dynamicSmemBytes = smem;
   lc.stream = st;
@@ -883,7 +674,7 @@ cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX,
   }
   lc.attrs = at;
   lc.numAttrs = na;
-  CS_CUDA_OK(ctx, cudaLaunchKernelEx(&lc, kernel, g->tmW, *tmX, a));
+  CS_CUDA_OK(ctx, cudaLaunchKernelEx(&lc, k_gemm_tc, g->tmW, *tmX, a));
   return CS_OK;
 }
 
@@ -917,7 +708,7 @@ cs_status static_scratch(void** out) {
   if (g_lm_scratch_dev[dev] == nullptr) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_lm_scratch) != cudaSuccess || p == nullptr) return CS_ERR_CUDA;
-    if (cudaFuncSetAttribute(k_gemm_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
       return CS_ERR_CUDA;
     g_lm_scratch_dev[dev] = p;
   }
@@ -990,17 +781,14 @@ extern "C" cs_status cs_lm_head_static(const void* X, const void* W, int rows, i
   a.splits = 1;
   a.mode = CS_EPI_ARGMAX;
   a.out = nullptr;
-  a.act = nullptr;
-  a.act_lo = nullptr;
   a.lo_row = -1;
-  a.F = 0;
   a.nf = NormFuse{};
   a.tile_max = tile_max;
   a.tile_idx = tile_idx;
   a.tile_stride = kStaticMaxTiles;
   a.status = status;
   const int stage_bytes = kTileABytes + a.n_tok * 128;
-  const int fixed = 1024 + (2 * 8 + 1) * 8 + 16 + 9 * a.n_tok * 4;
+  const int fixed = gemm_fixed_bytes(a.n_tok);
   int stages = (100 * 1024 - fixed) / stage_bytes;   // at least 4 for rows <= 64
   if (stages > 8) stages = 8;
   a.stages = stages;
@@ -1018,7 +806,7 @@ extern "C" cs_status cs_lm_head_static(const void* X, const void* W, int rows, i
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  if (cudaLaunchKernelEx(&lc, k_gemm_tc<1>, tmW, tmX, a) != cudaSuccess) return CS_ERR_CUDA;
+  if (cudaLaunchKernelEx(&lc, k_gemm_tc, tmW, tmX, a) != cudaSuccess) return CS_ERR_CUDA;
   if (cs_launch_pdl(k_tile_reduce_static, dim3(rows), dim3(128), 0, st, (const float*)tile_max,
                     (const int*)tile_idx, tiles, kStaticMaxTiles, (const int*)status, ids) != cudaSuccess)
     return CS_ERR_CUDA;
