@@ -53,8 +53,8 @@
  * when they are stored in the cache.
  *
  * Environment, read once by cs_create (measurement and test switches; not needed in use):
- *   CS_NO_GRAPH=1          steps are enqueued kernel by kernel instead of replayed from a
- *                          captured CUDA graph (cs_loop_*, cs_step_host, cs_decode_loop_drafted);
+ *   CS_NO_GRAPH=1          cs_loop_steps enqueues its steps kernel by kernel, as the other calls
+ *                          do, instead of replaying them from a captured CUDA graph;
  *   CS_ATTN_KERNEL=tc|tcw|mma  forces one attention kernel: tcgen05 with the query rows as the
  *                          M dimension (tc), tcgen05 with the keys and head dims as M (tcw), or
  *                          mma.sync (mma).  Default: by head size, and between the two tcgen05
@@ -242,9 +242,7 @@ cs_status cs_verify_step(cs_ctx* ctx, const int32_t* last_tok, const int32_t* dr
  * that call appended.  Anything else (other buffers, B, stride, a length the call did not
  * produce) uploads the rows in full.  A caller that rewrites tokens below hist_len_host[b] in
  * place without changing the length must call cs_step_host_reset first.
- * The kernels of the step are replayed as a CUDA graph that the context keeps while B, k, gamma,
- * the policy, the mode and the device buffers stay the same (first call and every change: one
- * capture).  The context's loop buffers serve as scratch: not to be mixed with an open
+ * The context's loop buffers serve as scratch: not to be mixed with an open
  * cs_loop_begin session.  Errors: CS_ERR_ARG / CS_ERR_CAPACITY on the host before any copy, CS_ERR_CUDA. */
 cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, int B, int stride,
                        int32_t* hist_dev, int32_t* hist_len_dev, void* kv_cache, int32_t* kv_len,

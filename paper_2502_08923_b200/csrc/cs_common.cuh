@@ -61,28 +61,13 @@ struct LoopState {
 };
 static constexpr int CS_LOOP_UNROLL = 4;   // steps per launch of graph_n
 
-// cs_step_host keeps the graph of its last launch shape: the kernels of one step between the
-// host -> device and device -> host copies
-struct HostStepGraph {
-  const void *hist_dev, *hist_len_dev, *kv_cache, *kv_len;
-  int B, stride, gamma, k, policy, scripted;
-  cudaGraph_t graph;
-  cudaGraphExec_t exec;
-  // what the device copy of the histories holds: rows [0, uploaded[b]) of up_host -> up_dev
-  const void *up_host, *up_dev;
-  int up_B, up_stride;
+// What cs_step_host has already uploaded: rows [0, uploaded[b]) of host -> dev
+struct HostStep {
+  const void *host, *dev;
+  int B, stride;
   int uploaded[CS_MAX_ROWS];    // tokens of row b on the device
   int host_len[CS_MAX_ROWS];    // hist_len_host[b] as the previous call left it
 };
-
-// cs_verify_step_cached keeps the graphs of its last few launch shapes
-struct VerifyGraph {
-  const void* key[9];   // last_tok, draft, draft_len, kv_cache, kv_len, script, accept_len, out_tokens, argmax_ids
-  int B, k;
-  cudaGraph_t graph;
-  cudaGraphExec_t exec;
-};
-static constexpr int CS_VERIFY_GRAPHS = 8;
 
 // Step timeline (cs_set_stamps): every stamped launch of a step owns one 64-bit slot of a
 // caller-provided device buffer, into which each of its CTAs leaves the time at which it
@@ -127,6 +112,7 @@ struct cs_ctx {
   int* row_lim;              // number of keys a row attends to (0 = dead row)
   int* row_write;            // 1 = this row's K/V go into the cache
   int* seq_ok;               // per sequence: 1 = takes part in this step
+  int* iota;                 // 0 .. CS_MAX_ROWS - 1 (device-side constants for host-ordered steps)
   float* pair_part;          // two-SM GEMM: sums of tiles cut between pairs [CS_MAX_PAIRS][2][CS_MAX_ROWS][128]
   int* pair_flag;            // and their "written" flags [CS_MAX_PAIRS][2], 0 between launches
   int* d_status;             // device status word
@@ -152,8 +138,8 @@ struct cs_ctx {
   const void* tmKV_base;
   int tmQ_R;
   // Cached lengths [max_batch] that stay as they are until the forward being enqueued has
-  // finished, and whose cache rows are complete: set only where the step opens with an
-  // ordinary stream-ordered launch (the generation loop); NULL elsewhere.  The attention
+  // finished, and whose cache rows are complete: set where the step opens with an
+  // ordinary stream-ordered launch (everywhere but in prefill); NULL elsewhere.  The attention
   // kernel may then fetch tiles of cached keys before it waits for the preceding kernel.
   const int* kv_len_early;
   // shared-memory opt-ins already made for this context's device (per context, not per
@@ -163,7 +149,7 @@ struct cs_ctx {
   unsigned attn_mma_attr_set;   // bit DH/32 per head size
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
-  bool no_graph;             // CS_NO_GRAPH=1 at creation: steps are enqueued kernel by kernel
+  bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
 
@@ -171,9 +157,11 @@ struct cs_ctx {
   int match_index_cap;
 
   LoopState loop;
-  HostStepGraph host_step;
-  VerifyGraph verify_graphs[CS_VERIFY_GRAPHS];
-  int verify_graph_next;
+  HostStep host_step;
+  // Pinned host word that cs_decode_loop's steps report to: (steps done << 32) | most tokens any
+  // sequence still has to emit; and the device's address of it.
+  unsigned long long *progress, *progress_dev;
+  int* host_ints;            // pinned host scratch behind it [CS_MAX_ROWS + 1]
   unsigned long long* stamp_buf;   // device, caller-owned; NULL = no stamps
   int stamp_cap, stamp_n;          // slots available / handed out for the step being enqueued
   unsigned char stamp_fam[CS_STAMP_MAX];
@@ -245,8 +233,8 @@ struct NormFuse {
   asm volatile("griddepcontrol.wait;" ::: "memory")
 
 template <typename... KArgs, typename... Args>
-static inline cudaError_t cs_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                        cudaStream_t st, Args&&... args) {
+static inline cudaError_t cs_launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                            cudaStream_t st, bool programmatic, Args&&... args) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = grid;
   lc.blockDim = block;
@@ -256,8 +244,13 @@ static inline cudaError_t cs_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
-  lc.numAttrs = 1;
+  lc.numAttrs = programmatic ? 1 : 0;
   return cudaLaunchKernelEx(&lc, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t cs_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                                        cudaStream_t st, Args&&... args) {
+  return cs_launch_chained(kernel, grid, block, smem, st, true, static_cast<Args&&>(args)...);
 }
 
 // split-K factor limit for a GEMM of `tiles` 128-row tiles and `kb` 64-wide K blocks
@@ -309,17 +302,10 @@ cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap*
 // cs_layers.cu
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip,
-                           int B, int k, cudaStream_t st);
+                           int B, int k, bool opens_step, cudaStream_t st);
 void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, int B,
                              int stride, int start, int R, cudaStream_t st);
 void cs_launch_embed_rmsnorm(cs_ctx* ctx, const __nv_bfloat16* gain, int rows, cudaStream_t st);
-// cs_verify_step replayed from a graph kept per launch shape (all pointers and B, k equal):
-// for host-ordered loops that call it with a few fixed sets of buffers.  The launch is one
-// stream-ordered unit, so the attention kernel may fetch cached tiles early.
-cs_status cs_verify_step_cached(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft, const int32_t* draft_len,
-                                int B, int k, void* kv_cache, int32_t* kv_len, const int32_t* target_script,
-                                int32_t* accept_len, int32_t* out_tokens, int32_t* argmax_ids, cudaStream_t st);
-
 void cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R,
                          cudaStream_t st);
 void cs_launch_attn_merge(cs_ctx* ctx, int nsplit, int rows, cudaStream_t st);
@@ -340,10 +326,13 @@ void cs_launch_accept(cs_ctx* ctx, int B, int k, const int32_t* draft, const int
 void cs_launch_tile_reduce(cs_ctx* ctx, int rows, int32_t* ids, cudaStream_t st);
 void cs_launch_truncate(cs_ctx* ctx, int32_t* kv_len, const int32_t* new_len, int B,
                         cudaStream_t st);
+void cs_launch_append(int32_t* hist, int32_t* hist_len, int n, const int32_t* tokens, int count, int32_t* kv_len,
+                      int32_t* kv_len_2, int new_len_2, cudaStream_t st);
 void cs_launch_prefill_finish(cs_ctx* ctx, const int32_t* hist_len, int32_t* kv_len, int B,
                               cudaStream_t st);
 void cs_launch_loop_init(cs_ctx* ctx, const int32_t* hist_len, const int32_t* kv_len, int B,
                          int stride, int max_new, int k, cudaStream_t st);
+// `progress` (device address of a pinned host word, or NULL) gets (step + 1) << 32 | tokens still wanted
 void cs_launch_loop_commit(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, int stride,
                            int32_t* kv_len, int k, int max_new, int eos_id, int scripted,
-                           cudaStream_t st);
+                           unsigned long long* progress, int step, cudaStream_t st);

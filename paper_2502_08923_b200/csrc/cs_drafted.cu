@@ -13,13 +13,13 @@
 //
 // The host reads the match position and the accepted block back every step, so this loop
 // synchronises once or twice per step; the device-resident loop without a draft model is
-// cs_decode_loop.  Every forward is replayed from a graph kept per launch shape (the target's
-// block, the draft model's catch-up block, its single-row steps).  Scratch: the loop buffers
+// cs_decode_loop.  Forwards read their tokens where they already are - the history, the script, the
+// target's draft row - and their draft lengths from a table of constants, so that a step's launches
+// follow one another without copies in between.  Scratch: the loop buffers
 // of the two contexts' workspaces (CS_MAX_ROWS ints each), so neither context may have a
 // cs_loop_begin session open.
 #include <algorithm>
 #include <cstring>
-#include <vector>
 
 #include "cs_common.cuh"
 
@@ -85,101 +85,67 @@ extern "C" cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int
   int32_t* t_out = target->loop_out;
   int32_t* t_argmax = target->loop_argmax;
   int32_t* t_script = target->loop_emitted;            // this step's slice of the script
-  int32_t* t_newlen = target->loop_last;
-  std::vector<int32_t> out_h((size_t)kt + 1);
+  int32_t* word_h = target->host_ints;                 // pinned: match position, later the accepted length
+  int32_t* out_h = target->host_ints + 1;              // pinned: the emitted tokens
   int emitted = 0;
   bool done = false;
 
   while (emitted < max_new && !done) {
     // ---- step 1: search; the host needs to know whether there was a match
     DR_OK(cs_find_match(hist, hist_len, 1, stride, gamma, k, policy, t_mpos, t_draft, t_dlen, st));
-    int mpos = -1;
-    DR_CUDA(cudaMemcpyAsync(&mpos, t_mpos, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DR_CUDA(cudaMemcpyAsync(word_h, t_mpos, sizeof(int), cudaMemcpyDeviceToHost, st));
     DR_CUDA(cudaStreamSynchronize(st));
+    const int mpos = *word_h;
     const bool drafted = mpos < 0 && delta > 0;
     if (drafted) {
       // ---- step 3(a): catch up on tokens hist[d_len .. n), forced through in blocks of kd + 1
       // rows (scripted acceptance against the tokens themselves); the last row's greedy token
       // is the first proposal
-      int32_t* d_draft = drafter->loop_draft;
-      int32_t* d_dlen = drafter->loop_dlen;
-      int32_t* d_script = drafter->loop_emitted;
       int32_t* d_accept = drafter->loop_accept;
       int32_t* d_out = drafter->loop_out;
       int32_t* d_argmax = drafter->loop_argmax;
-      // (fixed buffers and a fixed block height of kd + 1 rows, rows past the block's tokens dead,
-      //  so that every block replays the same graph)
-      int32_t* d_last = drafter->loop_last + 1;
       int r = 0;
       while (d_len < n) {
         r = std::min(n - d_len, kd + 1);
-        const int dl = r - 1;
-        DR_CUDA(cudaMemcpyAsync(d_last, hist + d_len, sizeof(int), cudaMemcpyDeviceToDevice, st));
-        // script row: the dl draft tokens, then values that are never looked at by this loop
-        DR_CUDA(cudaMemsetAsync(d_script, 0xFF, (size_t)(kd + 1) * 4, st));
-        if (dl > 0) {
-          DR_CUDA(cudaMemcpyAsync(d_draft, hist + d_len + 1, (size_t)dl * 4, cudaMemcpyDeviceToDevice, st));
-          DR_CUDA(cudaMemcpyAsync(d_script, hist + d_len + 1, (size_t)dl * 4, cudaMemcpyDeviceToDevice, st));
-        }
-        DR_CUDA(cudaMemcpyAsync(d_dlen, &dl, sizeof(int), cudaMemcpyHostToDevice, st));
-        DR_OK(cs_verify_step_cached(drafter, d_last, d_draft, d_dlen, 1, kd, kv_drafter, kv_len_drafter, d_script,
-                                    d_accept, d_out, d_argmax, st));
+        // (the script row's last entry, the token behind the block, is never accepted against)
+        DR_OK(cs_verify_step(drafter, hist + d_len, hist + d_len + 1, drafter->iota + (r - 1), 1, r - 1, kv_drafter,
+                             kv_len_drafter, hist + d_len + 1, d_accept, d_out, d_argmax, nullptr, st));
         d_len += r;
       }
       DR_CUDA(cudaMemcpyAsync(t_draft, d_argmax + (r - 1), sizeof(int), cudaMemcpyDeviceToDevice, st));
-      // the remaining delta - 1 proposals, one single-row greedy step each; the new token is
-      // copied into the target's draft row
-      // (through one fixed input slot and one fixed output slot, so that all of them replay the same graph)
-      int32_t* d_zero = drafter->loop_last + 2;
-      int32_t* d_in = drafter->loop_mpos;
-      int32_t* d_tok = drafter->loop_mpos + 1;
-      const int zero = 0;
-      DR_CUDA(cudaMemcpyAsync(d_zero, &zero, sizeof(int), cudaMemcpyHostToDevice, st));
+      // the remaining delta - 1 proposals, one single-row greedy step each, along the target's draft row
       for (int i = 1; i < delta; ++i) {
-        DR_CUDA(cudaMemcpyAsync(d_in, t_draft + (i - 1), sizeof(int), cudaMemcpyDeviceToDevice, st));
-        DR_OK(cs_verify_step_cached(drafter, d_in, nullptr, d_zero, 1, 0, kv_drafter, kv_len_drafter, nullptr,
-                                    d_accept, d_tok, d_argmax, st));
-        DR_CUDA(cudaMemcpyAsync(t_draft + i, d_tok, sizeof(int), cudaMemcpyDeviceToDevice, st));
+        DR_OK(cs_verify_step(drafter, t_draft + (i - 1), nullptr, drafter->iota, 1, 0, kv_drafter, kv_len_drafter, nullptr,
+                             d_accept, t_draft + i, d_argmax, nullptr, st));
         d_len += 1;
       }
-      DR_CUDA(cudaMemcpyAsync(t_dlen, &delta, sizeof(int), cudaMemcpyHostToDevice, st));
     }
     // ---- steps 2 / 3(b): one target block over [last token, draft]
-    const int32_t* script_row = nullptr;
-    if (script != nullptr) {
-      const int have = std::min(kt + 1, max_new - emitted);   // rows past the script's end cannot be accepted
+    const int32_t* script_row = script != nullptr ? script + emitted : nullptr;
+    const int have = max_new - emitted;
+    if (script != nullptr && have < kt + 1) {              // rows past the script's end cannot be accepted
       DR_CUDA(cudaMemsetAsync(t_script, 0xFF, (size_t)(kt + 1) * 4, st));
-      DR_CUDA(cudaMemcpyAsync(t_script, script + emitted, (size_t)have * 4, cudaMemcpyDeviceToDevice, st));
+      DR_CUDA(cudaMemcpyAsync(t_script, script_row, (size_t)have * 4, cudaMemcpyDeviceToDevice, st));
       script_row = t_script;
     }
-    int32_t* t_last = target->loop_last + 1;
-    DR_CUDA(cudaMemcpyAsync(t_last, hist + (n - 1), sizeof(int), cudaMemcpyDeviceToDevice, st));
-    DR_OK(cs_verify_step_cached(target, t_last, t_draft, t_dlen, 1, kt, kv_target, kv_len_target, script_row,
-                                t_accept, t_out, t_argmax, st));
-    int tau = -1;
-    DR_CUDA(cudaMemcpyAsync(&tau, t_accept, sizeof(int), cudaMemcpyDeviceToHost, st));
-    DR_CUDA(cudaMemcpyAsync(out_h.data(), t_out, (size_t)(kt + 1) * 4, cudaMemcpyDeviceToHost, st));
+    DR_OK(cs_verify_step(target, hist + (n - 1), t_draft, drafted ? target->iota + delta : t_dlen, 1, kt, kv_target,
+                         kv_len_target, script_row, t_accept, t_out, t_argmax, nullptr, st));
+    DR_CUDA(cudaMemcpyAsync(word_h, t_accept, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DR_CUDA(cudaMemcpyAsync(out_h, t_out, (size_t)(kt + 1) * 4, cudaMemcpyDeviceToHost, st));
     DR_CUDA(cudaStreamSynchronize(st));
+    const int tau = *word_h;
     if (tau < 0 || tau > kt) break;                    // the device refused the step; the status word says why
     int c = std::min(tau + 1, max_new - emitted);
     if (script == nullptr && eos_id >= 0) {
       for (int i = 0; i < c; ++i)
-        if (out_h[(size_t)i] == eos_id) { c = i + 1; done = true; break; }
+        if (out_h[i] == eos_id) { c = i + 1; done = true; break; }
     }
     // ---- step 4 and the roll-backs: append, then cut both caches to the accepted prefix
-    DR_CUDA(cudaMemcpyAsync(hist + n, t_out, (size_t)c * 4, cudaMemcpyDeviceToDevice, st));
     const int n_new = n + c;
-    DR_CUDA(cudaMemcpyAsync(hist_len, &n_new, sizeof(int), cudaMemcpyHostToDevice, st));
-    if (c - 1 < tau) {                                 // clipped by max_new or EOS: the step kept tau rows
-      const int nl = n_new - 1;
-      DR_CUDA(cudaMemcpyAsync(t_newlen, &nl, sizeof(int), cudaMemcpyHostToDevice, st));
-      DR_OK(cs_kv_truncate(target, kv_len_target, t_newlen, 1, st));
-    }
-    if (drafted && d_len > n + c - 1) {                // positions n .. n+c-2 hold accepted proposals
-      d_len = n + c - 1;
-      DR_CUDA(cudaMemcpyAsync(drafter->loop_last, &d_len, sizeof(int), cudaMemcpyHostToDevice, st));
-      DR_OK(cs_kv_truncate(drafter, kv_len_drafter, drafter->loop_last, 1, st));
-    }
+    const bool cut = drafted && d_len > n_new - 1;     // positions n .. n_new - 2 hold accepted proposals
+    if (cut) d_len = n_new - 1;
+    cs_launch_append(hist, hist_len, n, t_out, c, kv_len_target, cut ? kv_len_drafter : nullptr, d_len, st);
+    DR_CUDA(cudaGetLastError());
     n = n_new;
     emitted += c;
     stats.steps += 1;

@@ -317,6 +317,19 @@ __global__ void k_truncate(int* kv_len, const int* new_len, int B, int* status) 
   else kv_len[b] = nl;
 }
 
+// Host-ordered loop, end of a step: the emitted tokens go to the history, the lengths of history and
+// cache follow, and so does a second model's cache length when it has one to cut.
+__global__ void k_append(int* hist, int* hist_len, int n, const int* tokens, int count, int* kv_len, int* kv_len_2, int new_len_2) {
+  CS_PDL_PROLOGUE();
+  const int i = threadIdx.x;
+  if (i < count) hist[n + i] = tokens[i];
+  if (i == 0) {
+    *hist_len = n + count;
+    *kv_len = n + count - 1;
+    if (kv_len_2 != nullptr) *kv_len_2 = new_len_2;
+  }
+}
+
 __global__ void k_prefill_finish(const int* hist_len, const int* seq_ok, int* kv_len, int B) {
   CS_PDL_PROLOGUE();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -351,46 +364,61 @@ __global__ void k_loop_init(const int* hist_len, const int* kv_len, int B, int s
 
 // Append the step's tokens to the history (App. B.3 step 4), clip at max_new, stop at
 // EOS in real mode, advance the lengths (the KV truncation of App. B.2) and count.
-__global__ void k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, int max_new,
-                              int eos_id, int scripted, const int* accept, const int* out, const int* mpos,
-                              int* emitted, int* done, int max_batch, unsigned long long* stats,
-                              unsigned long long* stamp) {
+// One CTA (a batch has at most CS_MAX_ROWS sequences).  With `progress`, a word in pinned host memory, the
+// step also reports how many tokens the sequence furthest from its end still wants, so that the
+// host knows without a synchronisation whether another step is needed.
+__global__ void __launch_bounds__(CS_MAX_ROWS)
+k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, int max_new,
+              int eos_id, int scripted, const int* accept, const int* out, const int* mpos,
+              int* emitted, int* done, int max_batch, unsigned long long* stats,
+              const int* status, unsigned long long* progress, int step, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  const int b = threadIdx.x;
   if (b == 0) cs_stamp_end(stamp);   // (the kernel is a few dozen instructions: its start stands for its end)
-  if (b >= B || done[b]) return;
-  cs_stats* st = reinterpret_cast<cs_stats*>(stats);
-  const int tau = accept[b];
-  if (tau < 0) {            // the step skipped this sequence (capacity): it stops here
-    done[b] = 1;
-    atomicAdd(&done[max_batch], 1);
-    return;
+  int wanted = 0;
+  if (b < B && !done[b]) {
+    cs_stats* st = reinterpret_cast<cs_stats*>(stats);
+    const int tau = accept[b];
+    bool fin = tau < 0;     // the step skipped this sequence (capacity): it stops here
+    if (!fin) {
+      const int R = k + 1;
+      const int n = hist_len[b], e = emitted[b];
+      int c = min(tau + 1, max_new - e);
+      if (!scripted && eos_id >= 0) {
+        for (int i = 0; i < c; ++i)
+          if (out[(size_t)b * R + i] == eos_id) { c = i + 1; fin = true; break; }
+      }
+      for (int i = 0; i < c; ++i) hist[(size_t)b * stride + n + i] = out[(size_t)b * R + i];
+      hist_len[b] = n + c;
+      kv_len[b] = n + c - 1;
+      emitted[b] = e + c;
+      if (e + c >= max_new) fin = true;
+      atomicAdd((unsigned long long*)&st->steps, 1ull);
+      atomicAdd((unsigned long long*)&st->emitted, (unsigned long long)c);
+      if (mpos[b] >= 0) {
+        atomicAdd((unsigned long long*)&st->attempts, 1ull);
+        atomicAdd((unsigned long long*)&st->accepted, (unsigned long long)(c - 1));
+        atomicAdd((unsigned long long*)&st->tau_hist[min(c - 1, CS_TAU_HIST - 1)], 1ull);
+      } else {
+        atomicAdd((unsigned long long*)&st->no_match, 1ull);
+      }
+      if (!fin) wanted = max_new - e - c;
+    }
+    if (fin) {
+      done[b] = 1;
+      atomicAdd(&done[max_batch], 1);
+    }
   }
-  const int R = k + 1;
-  const int n = hist_len[b], e = emitted[b];
-  int c = min(tau + 1, max_new - e);
-  bool fin = false;
-  if (!scripted && eos_id >= 0) {
-    for (int i = 0; i < c; ++i)
-      if (out[(size_t)b * R + i] == eos_id) { c = i + 1; fin = true; break; }
-  }
-  for (int i = 0; i < c; ++i) hist[(size_t)b * stride + n + i] = out[(size_t)b * R + i];
-  hist_len[b] = n + c;
-  kv_len[b] = n + c - 1;
-  emitted[b] = e + c;
-  if (e + c >= max_new) fin = true;
-  atomicAdd((unsigned long long*)&st->steps, 1ull);
-  atomicAdd((unsigned long long*)&st->emitted, (unsigned long long)c);
-  if (mpos[b] >= 0) {
-    atomicAdd((unsigned long long*)&st->attempts, 1ull);
-    atomicAdd((unsigned long long*)&st->accepted, (unsigned long long)(c - 1));
-    atomicAdd((unsigned long long*)&st->tau_hist[min(c - 1, CS_TAU_HIST - 1)], 1ull);
-  } else {
-    atomicAdd((unsigned long long*)&st->no_match, 1ull);
-  }
-  if (fin) {
-    done[b] = 1;
-    atomicAdd(&done[max_batch], 1);
+  if (progress != nullptr) {
+    __shared__ int s_wanted;
+    if (b == 0) s_wanted = 0;
+    __syncthreads();
+    if (wanted > 0) atomicMax(&s_wanted, wanted);
+    __syncthreads();
+    if (b == 0) {
+      const unsigned rest = (*status & CS_DEV_TIMEOUT) ? 0u : (unsigned)s_wanted;   // (a wait that ran out ends the loop)
+      *reinterpret_cast<volatile unsigned long long*>(progress) = ((unsigned long long)(unsigned)(step + 1) << 32) | rest;
+    }
   }
 }
 
@@ -398,9 +426,11 @@ __global__ void k_loop_commit(int* hist, int* hist_len, int B, int stride, int* 
 
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip, int B,
-                           int k, cudaStream_t st) {
+                           int k, bool opens_step, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
-  cs_launch_pdl(k_block_setup, dim3(1), dim3(256), 0, st, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
+  // A step that opens here (no search in front of it) opens with an ordinary stream-ordered launch, so
+  // that kernels further down the chain may rely on everything enqueued earlier being complete.
+  cs_launch_chained(k_block_setup, dim3(1), dim3(256), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
                 c.vocab, c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write,
                 ctx->seq_ok, ctx->rope_cs, ctx->d_status, cs_next_stamp(ctx, CS_FAM_OTHER));
 }
@@ -447,6 +477,11 @@ void cs_launch_truncate(cs_ctx* ctx, int32_t* kv_len, const int32_t* new_len, in
   cs_launch_pdl(k_truncate, dim3(cs_ceil_div(B, 128)), dim3(128), 0, st, kv_len, new_len, B, ctx->d_status);
 }
 
+void cs_launch_append(int32_t* hist, int32_t* hist_len, int n, const int32_t* tokens, int count, int32_t* kv_len,
+                      int32_t* kv_len_2, int new_len_2, cudaStream_t st) {
+  cs_launch_pdl(k_append, dim3(1), dim3(CS_MAX_ROWS), 0, st, hist, hist_len, n, tokens, count, kv_len, kv_len_2, new_len_2);
+}
+
 void cs_launch_prefill_finish(cs_ctx* ctx, const int32_t* hist_len, int32_t* kv_len, int B, cudaStream_t st) {
   cs_launch_pdl(k_prefill_finish, dim3(cs_ceil_div(B, 128)), dim3(128), 0, st, hist_len, ctx->seq_ok, kv_len, B);
 }
@@ -458,8 +493,10 @@ void cs_launch_loop_init(cs_ctx* ctx, const int32_t* hist_len, const int32_t* kv
 }
 
 void cs_launch_loop_commit(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, int stride, int32_t* kv_len,
-                           int k, int max_new, int eos_id, int scripted, cudaStream_t st) {
-  cs_launch_pdl(k_loop_commit, dim3(cs_ceil_div(B, 128)), dim3(128), 0, st, hist, hist_len, B, stride, kv_len, k,
+                           int k, int max_new, int eos_id, int scripted, unsigned long long* progress, int step,
+                           cudaStream_t st) {
+  cs_launch_pdl(k_loop_commit, dim3(1), dim3(cs_ceil_div(B, 32) * 32), 0, st, hist, hist_len, B, stride, kv_len, k,
                 max_new, eos_id, scripted, ctx->loop_accept, ctx->loop_out, ctx->loop_mpos, ctx->loop_emitted,
-                ctx->loop_done, ctx->cfg.max_batch, ctx->loop_stats, cs_next_stamp(ctx, CS_FAM_OTHER));
+                ctx->loop_done, ctx->cfg.max_batch, ctx->loop_stats, ctx->d_status, progress, step,
+                cs_next_stamp(ctx, CS_FAM_OTHER));
 }
