@@ -139,7 +139,7 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     if (s != CS_OK) return s;
     take_norm = NormFuse{};
     take_norm.ssq_in = ctx->ssq;
-    take_norm.slots_in = cs_ceil_div(L.o.N, CS_GEMM_BM) * cs_gemm_splits(ctx, &L.o, CS_EPI_RESIDUAL, rows, true);
+    take_norm.slots_in = cs_norm_slots(&L.o, rows);
     take_norm.slot_stride = ctx->ssq_stride;
     take_norm.inv_d = 1.f / (float)c.d_model;
     take_norm.eps = c.rms_eps;
@@ -152,7 +152,7 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     s = cs_launch_gemm(ctx, &L.down, &ctx->tmAct, lo_row, rows, CS_EPI_RESIDUAL, ctx->x, nullptr, nullptr, 0, nullptr,
                        &give, st);
     if (s != CS_OK) return s;
-    take_norm.slots_in = cs_ceil_div(L.down.N, CS_GEMM_BM) * cs_gemm_splits(ctx, &L.down, CS_EPI_RESIDUAL, rows, true);
+    take_norm.slots_in = cs_norm_slots(&L.down, rows);
   }
   if (with_lm) {
     s = cs_launch_gemm(ctx, &ctx->lm, &ctx->tmXn, lo_row, rows, CS_EPI_ARGMAX, logits, nullptr, nullptr, 0, nullptr,

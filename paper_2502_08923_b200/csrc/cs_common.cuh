@@ -27,8 +27,8 @@ static constexpr int CS_GEMM_BK = 64;     // K elements per stage (one 128-byte 
 static constexpr int CS_MAX_GAMMA = 8;
 static constexpr int CS_MAX_SPLITS = 8;   // split-K factor limit (portable cluster size)
 static constexpr int CS_SPLIT_TILE_CAP = 640;  // tiles * splits never exceeds this (unless splits == 1)
-static constexpr int CS_PAIR_MAX_SPLITS = 4;   // split-K factor limit of the two-SM GEMM (its clusters hold 2 x splits CTAs)
-static constexpr int CS_MAX_PAIRS = 80;        // persistent SM pairs of its stream form, at most
+static constexpr int CS_PAIR_MAX_SPLITS = 8;   // split-K factor limit of the two-SM GEMM
+static constexpr int CS_MAX_PAIRS = 80;        // SM pairs whose sums meet in the workspace, at most
 
 struct GemmPlan {
   CUtensorMap tmW;      // weights [N][K], box 128 x 64, 128-byte swizzle
@@ -113,8 +113,8 @@ struct cs_ctx {
   int* row_write;            // 1 = this row's K/V go into the cache
   int* seq_ok;               // per sequence: 1 = takes part in this step
   int* iota;                 // 0 .. CS_MAX_ROWS - 1 (device-side constants for host-ordered steps)
-  float* pair_part;          // two-SM GEMM: sums of tiles cut between pairs [CS_MAX_PAIRS][2][CS_MAX_ROWS][128]
-  int* pair_flag;            // and their "written" flags [CS_MAX_PAIRS][2], 0 between launches
+  float* pair_part;          // two-SM GEMM: sums that pairs hand to one another [CS_MAX_PAIRS][2][CS_MAX_ROWS][128]
+  int* pair_flag;            // and the words that announce them [CS_MAX_PAIRS][2], 0 between launches
   int* d_status;             // device status word
   // loop state, all [max_batch] unless noted
   int* loop_last;
@@ -145,7 +145,7 @@ struct cs_ctx {
   // shared-memory opt-ins already made for this context's device (per context, not per
   // process: another context may live on another GPU)
   bool gemm_attr_set, pair_attr_set;
-  int pair_clusters[CS_PAIR_MAX_SPLITS + 1];   // clusters of 2 x S CTAs that can run at once, by S (0 = not asked yet)
+  int pairs_at_once;         // two-CTA clusters of the two-SM GEMM that can run at once (0 = not asked yet)
   unsigned attn_mma_attr_set;   // bit DH/32 per head size
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
@@ -295,7 +295,7 @@ static inline int cs_gemm_act_box(int mode, int rows, bool two_terms) {
   const int n_tok = cs_ceil_div(rows, 16) * 16;
   return !cs_gemm_on_pairs(mode, rows) || (two_terms && n_tok <= 128) ? n_tok : n_tok / 2;
 }
-int cs_gemm_splits(const cs_ctx* ctx, const GemmPlan* g, int mode, int rows, bool two_terms);   // split-K factor of a launch
+int cs_norm_slots(const GemmPlan* g, int rows);   // sums of squares per token that a residual GEMM leaves for the next norm
 cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode, float* out,
                               __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
                               cudaStream_t st);
