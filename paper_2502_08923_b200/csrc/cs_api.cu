@@ -3,6 +3,7 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <mutex>
 #include <new>
 
 #include <string.h>
@@ -82,6 +83,39 @@ WsLayout ws_layout(const cs_model_config* c) {
   L.loop_stats = take(&off, sizeof(cs_stats));
   L.total = off;
   return L;
+}
+
+// Pinned host memory of the contexts: one 64 KB block for the process, handed out in slots (pinning takes from
+// a tenth of a millisecond to tens of them, so it is not done per context).  Slots are given back by
+// cs_destroy; a context that finds none left pins its own.
+constexpr size_t kSlotBytes = 2048;
+constexpr int kSlots = 32;
+static_assert(64 + (CS_MAX_ROWS + 1) * sizeof(int) <= kSlotBytes, "progress word and host scratch fit a slot");
+std::mutex g_slot_lock;
+char* g_slots = nullptr;
+unsigned g_slots_taken = 0;
+
+cudaError_t take_slot(char** out) {
+  const unsigned flags = cudaHostAllocMapped | cudaHostAllocPortable;
+  std::lock_guard<std::mutex> hold(g_slot_lock);
+  if (g_slots == nullptr) {
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&g_slots), kSlotBytes * kSlots, flags);
+    if (e != cudaSuccess) { g_slots = nullptr; return e; }
+  }
+  for (int i = 0; i < kSlots; ++i)
+    if (!(g_slots_taken >> i & 1u)) {
+      g_slots_taken |= 1u << i;
+      *out = g_slots + i * kSlotBytes;
+      return cudaSuccess;
+    }
+  return cudaHostAlloc(reinterpret_cast<void**>(out), kSlotBytes, flags);
+}
+
+void give_slot(void* p) {
+  char* at = static_cast<char*>(p);
+  std::lock_guard<std::mutex> hold(g_slot_lock);
+  if (g_slots != nullptr && at >= g_slots && at < g_slots + kSlotBytes * kSlots) g_slots_taken &= ~(1u << ((at - g_slots) / kSlotBytes));
+  else cudaFreeHost(p);
 }
 
 // cs_create has no context to leave an error text in: the last failure of this thread is kept here
@@ -282,8 +316,7 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   ctx->qkv_elems = L.qkv_elems;
   ctx->layers = new (std::nothrow) LayerPlan[cfg->n_layers];
   cs_status s = CS_OK;
-  int dev = 0;
-  cudaDeviceProp prop;
+  int dev = 0, major = 0, minor = 0;
 #define CREATE_OK(call)                                                                        \
   do {                                                                                         \
     cudaError_t e__ = (call);                                                                  \
@@ -295,16 +328,18 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   } while (0)
   if (ctx->layers == nullptr) { cs_destroy(ctx); return create_fail(CS_ERR_ARG, "out of host memory"); }
   CREATE_OK(cudaGetDevice(&dev));
-  CREATE_OK(cudaGetDeviceProperties(&prop, dev));
-  if (prop.major != 10) {
+  // (single attributes: reading the whole property table takes milliseconds)
+  CREATE_OK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+  CREATE_OK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev));
+  CREATE_OK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev));
+  if (major != 10) {
     snprintf(g_create_err, sizeof(g_create_err), "cs_create: this library is built for sm_100a only (device is sm_%d%d)",
-             prop.major, prop.minor);
+             major, minor);
     cs_destroy(ctx);
     return CS_ERR_UNSUPPORTED;
   }
-  ctx->num_sms = prop.multiProcessorCount;
   CREATE_OK(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-  CREATE_OK(cudaHostAlloc(reinterpret_cast<void**>(&ctx->progress), 64 + (CS_MAX_ROWS + 1) * sizeof(int), cudaHostAllocMapped));
+  CREATE_OK(take_slot(reinterpret_cast<char**>(&ctx->progress)));
   CREATE_OK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->progress_dev), ctx->progress, 0));
   ctx->host_ints = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + 64);
   char* base = static_cast<char*>(workspace);
@@ -389,7 +424,7 @@ void cs_destroy(cs_ctx* ctx) {
   if (ctx == nullptr) return;
   cs_loop_end(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-  if (ctx->progress) cudaFreeHost(ctx->progress);
+  if (ctx->progress) give_slot(ctx->progress);
   delete[] ctx->layers;
   delete ctx;
 }
