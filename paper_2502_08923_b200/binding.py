@@ -125,18 +125,29 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.cs_step_host_reset.argtypes = [vp]
     lib.cs_debug_drop_tile.restype = i
     lib.cs_debug_drop_tile.argtypes = [vp, i]
+    lib.cs_gram_index_bytes.restype = C.c_size_t
+    lib.cs_gram_index_bytes.argtypes = [i, i]
+    lib.cs_gram_index_reset.restype = i
+    lib.cs_gram_index_reset.argtypes = [vp, i, i, vp]
+    lib.cs_gram_index_update.restype = i
+    lib.cs_gram_index_update.argtypes = [vp, i, i, ip, ip, i, i, vp]
+    lib.cs_find_match_indexed.restype = i
+    lib.cs_find_match_indexed.argtypes = [vp, i, i, ip, ip, i, i, i, i, ip, ip, ip, vp]
+    lib.cs_gram_index_status.restype = i
+    lib.cs_gram_index_status.argtypes = [vp, i, i, vp]
     lib.cs_linear.restype = i
     lib.cs_linear.argtypes = [vp, vp, vp, i, i, i, vp, vp]
     _lib = lib
     return lib
 
 
+# Addresses travel as plain integers: every pointer argument is declared c_void_p.
 def _ptr(t):
     if t is None:
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _host_i32(t, name):
@@ -144,35 +155,43 @@ def _host_i32(t, name):
         return None
     if t.is_cuda or not t.is_contiguous() or t.dtype != torch.int32:
         raise ValueError(f"{name} must be a contiguous int32 host tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _i32(t, name):
-    if t is not None and t.dtype != torch.int32:
+    if t is None:
+        return None
+    if t.dtype is not torch.int32:
         raise ValueError(f"{name} must be int32")
-    return _ptr(t)
+    if not t.is_cuda or not t.is_contiguous():
+        raise ValueError("expected a contiguous CUDA tensor")
+    return t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of the current stream.  The search takes about 5 us on the device, and building a
+    torch.cuda.Stream object for every call takes as long; the raw handle takes 0.2 us."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+def _match_outputs(hist, hist_len, k):
+    return torch.empty_like(hist_len), hist.new_empty((hist.shape[0], k)), torch.empty_like(hist_len)
 
 
 def cs_find_match(hist, hist_len, gamma, k, policy=LATEST, out=None):
     """Suffix-match search and draft gather.  hist [B][stride] int32, hist_len [B] int32 (CUDA).
     Returns (match_pos [B], draft [B][k], draft_len [B]); `out` may supply those tensors."""
-    lib = load()
     B, stride = hist.shape
     if out is None:
-        out = (torch.empty(B, dtype=torch.int32, device=hist.device),
-               torch.empty(B, max(k, 1), dtype=torch.int32, device=hist.device)[:, :k].contiguous(),
-               torch.empty(B, dtype=torch.int32, device=hist.device))
-    mp, dr, dl = out
-    rc = lib.cs_find_match(_i32(hist, "hist"), _i32(hist_len, "hist_len"), B, stride, gamma, k, policy,
-                           _i32(mp, "match_pos"), C.c_void_p(dr.data_ptr()) if k > 0 else None,
-                           _i32(dl, "draft_len"), _stream())
+        out = mp, dr, dl = _match_outputs(hist, hist_len, k)
+        mp, dl = mp.data_ptr(), dl.data_ptr()
+    else:
+        mp, dr, dl = _i32(out[0], "match_pos"), out[1], _i32(out[2], "draft_len")
+    rc = (_lib or load()).cs_find_match(_i32(hist, "hist"), _i32(hist_len, "hist_len"), B, stride, gamma, k, policy,
+                                        mp, dr.data_ptr() if k > 0 else None, dl, _stream())
     if rc != CS_OK:
         raise CsError(rc, "cs_find_match")
-    return mp, dr, dl
+    return out
 
 
 class GramIndex:
@@ -181,13 +200,12 @@ class GramIndex:
     def __init__(self, B, capacity_tokens, gamma, device="cuda"):
         self.lib = load()
         self.B, self.cap, self.gamma = B, capacity_tokens, gamma
-        self.lib.cs_gram_index_bytes.restype = C.c_size_t
         nbytes = self.lib.cs_gram_index_bytes(B, capacity_tokens)
         self.buf = torch.empty(nbytes, dtype=torch.uint8, device=device)
         self.cs_gram_index_reset()
 
     def _p(self):
-        return C.c_void_p(self.buf.data_ptr())
+        return self.buf.data_ptr()
 
     def cs_gram_index_reset(self):
         rc = self.lib.cs_gram_index_reset(self._p(), self.B, self.cap, _stream())
@@ -203,14 +221,10 @@ class GramIndex:
 
     def cs_find_match_indexed(self, hist, hist_len, k, policy=LATEST, out=None):
         B, stride = hist.shape
-        if out is None:
-            out = (torch.empty(B, dtype=torch.int32, device=hist.device),
-                   torch.empty(B, max(k, 1), dtype=torch.int32, device=hist.device)[:, :k].contiguous(),
-                   torch.empty(B, dtype=torch.int32, device=hist.device))
-        mp, dr, dl = out
+        mp, dr, dl = _match_outputs(hist, hist_len, k) if out is None else out
         rc = self.lib.cs_find_match_indexed(self._p(), B, self.cap, _i32(hist, "hist"), _i32(hist_len, "hist_len"), stride,
                                             self.gamma, k, policy, _i32(mp, "match_pos"),
-                                            C.c_void_p(dr.data_ptr()) if k > 0 else None, _i32(dl, "draft_len"), _stream())
+                                            dr.data_ptr() if k > 0 else None, _i32(dl, "draft_len"), _stream())
         if rc != CS_OK:
             raise CsError(rc, "cs_find_match_indexed")
         return mp, dr, dl
@@ -341,7 +355,7 @@ class Context:
                    torch.empty(B, k + 1, dtype=torch.int32, device=dev))
         al, ot, am = out
         rc = self.lib.cs_verify_step(self.handle, _i32(last_tok, "last_tok"),
-                                     C.c_void_p(draft.data_ptr()) if k > 0 else None,
+                                     draft.data_ptr() if k > 0 else None,
                                      _i32(draft_len, "draft_len"), B, k, _ptr(kv_cache), _i32(kv_len, "kv_len"),
                                      _i32(target_script, "target_script"), _i32(al, "accept_len"),
                                      _i32(ot, "out_tokens"), _i32(am, "argmax_ids"), _ptr(logits_dbg), _stream())
