@@ -2,7 +2,7 @@
 // (Sec. 3.2; App. B.2), for head_dim 128.
 //
 // One CTA = one (sequence, KV head), one slice of the key range and one group of block rows (the
-// (k+1) block rows of the G query heads sharing the KV head: at most 96 query rows per group).
+// (k+1) block rows of the G query heads sharing the KV head: at most 48 query rows per group).
 // The cached keys and the head dims are the M dimension of the two products and the query rows
 // the N dimension, so the operand traffic scales with the real number of query rows (44 for an
 // 11-row block of a 4:1 GQA model) instead of a padded 128:
@@ -13,8 +13,7 @@
 // K and V - which the cache stores in bf16 - are rounded.  The
 // two terms of the second operand are laid side by side along N - [Q_hi; Q_lo] as one operand of
 // 2 NQ rows, [P_hi^T | P_lo^T] as one of 2 NQ columns - and one instruction per 16 K-elements
-// does the work of two, reading the K or V tile once; the two halves of the accumulator are added where it is read (S^T keeps
-// one NQ-wide accumulator and two instructions when TMEM has no room for 2 NQ columns twice).
+// does the work of two, reading the K or V tile once; the two halves of the accumulator are added where it is read.
 // TMEM lane = key (S^T) or head dim (O^T), column = query row.  Softmax: twelve warps in three
 // column groups; thread t of a lane quarter owns key t of the tile and a third of the query
 // columns (warps w, w + 4 and w + 8 share the lanes).  Each column has a running reference point
@@ -29,11 +28,9 @@
 // Each thread keeps its own share of every column's sum;
 // the shares are added up once at the end.  P^T is written as one swizzled 16-byte chunk per 8
 // columns into the row of the thread's key, which is exactly the MN-major operand layout, so
-// nothing is transposed.  S^T is double-buffered in TMEM: the score product of tile i+1 runs
-// during the softmax of tile i.  Blocks of up to 48 query rows have room for four S^T buffers:
-// their softmax takes the key tiles two at a time (one wait, one vote, two sets of weights).
-// K tiles move through a two-stage TMA ring and V tiles through a one- or two-stage ring, each
-// fed by its own producer thread, so K runs a tile ahead.  Each CTA
+// nothing is transposed.  There are four S^T buffers in TMEM: the score products of the next tiles run during the
+// softmax, which takes the key tiles two at a time (one wait, one vote, two sets of weights).
+// K tiles and V tiles move through a two-stage TMA ring each, fed by its own producer thread, so K runs a tile ahead.  Each CTA
 // writes its un-normalised (O, m, sum); k_attn_merge combines the key slices.  When the caller
 // vouches for the cached lengths (kv_len_early), tiles that lie wholly below the cached length
 // are requested before the wait for the preceding kernel: those rows were written by earlier
@@ -43,8 +40,8 @@
 //
 // Bound by the softmax warps' issue slots and, at batch 16, by HBM.  Measured per layer (8B shape, issue
 // by an elected lane with uniform operands, before that from one lane): 176 rows over 16 x 8,192 keys
-// 120.6 -> 93.6 us (0.54 GB: 5.8 TB/s), 16 rows over the same 114.2 -> 83.2 us, 168 rows over
-// 8 x 16,384 keys 159.8 -> 136.7 us, 11 rows over 30,720 keys 33.8 -> 29.2 us.
+// 120.6 -> 93.6 us (0.54 GB: 5.8 TB/s), 16 rows over the same 114.2 -> 83.2 us.  (Taller groups and shorter
+// walks are the business of the kernel with the query rows as M; its file has both sides' figures.)
 #include <stdlib.h>
 
 #include "cs_common.cuh"
@@ -59,14 +56,15 @@ constexpr int kProdWarp = 12, kMmaWarp = 13, kVProdWarp = 14;   // (a warp of it
 constexpr int kTileKeys = 128;
 constexpr int kDh = 128;
 constexpr int kHalfBytes = kTileKeys * 128;          // one [128 keys x 64 dims] half tile (also one P^T atom)
-constexpr int kNQMax = 96;                           // query rows per CTA
+constexpr int kNQMax = 48;                           // query rows per CTA
 constexpr int kCols = kNQMax / 3;                    // query columns per softmax thread, at most
+constexpr int kSBufs = 4, kPBufs = 2, kStages = 2;   // S^T buffers in TMEM, P^T buffers, K and V stages
 constexpr int kCtlBytes = 192;                       // 16 mbarriers + TMEM slot + flags
 
 struct AttnArgs {
   const int* row_lim;
   const int* kv_len_early;   // cached lengths that no kernel in flight changes, or NULL
-  int layer, R, Rg, G, H, Hkv, max_batch, max_seq, nsplit, NQ, rows, vstages, pbufs, qstack;   // Rg = block rows per row group; pbufs = P^T buffers (1 or 2)
+  int layer, R, Rg, G, H, Hkv, max_batch, max_seq, nsplit, NQ, rows;   // Rg = block rows per row group
   int smem_bytes;            // dynamic shared memory of the launch
   float scale_log2e;
   float* out_o;
@@ -162,26 +160,23 @@ __device__ __forceinline__ bool group_any(int id, bool pred) {
   return out != 0;
 }
 
-// KC = query columns per softmax thread at most (register arrays), NSB = S^T buffers in TMEM: 2, or 4
-// for blocks of up to 48 query rows, whose softmax then takes the key tiles two at a time.
-template <int KC, int NSB>
 __global__ void __launch_bounds__(kThreads, 1)
 k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmQ, AttnArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
-  // blockIdx.z picks a group of Rg consecutive block rows (blocks taller than 96 / G rows)
+  // blockIdx.z picks a group of Rg consecutive block rows (blocks taller than 48 / G rows)
   const int NQ = a.NQ, G = a.G, R = a.R, r0 = blockIdx.z * a.Rg, Rcur = min(a.Rg, R - r0);
-  const int nq = G * Rcur, nq_box = G * a.Rg, vstages = a.vstages;
+  const int nq = G * Rcur, nq_box = G * a.Rg;
   const int natoms = (2 * NQ + 63) >> 6;               // 64-column atoms of P^T (both terms side by side)
   const uint32_t qhalf = (uint32_t)NQ * 128u;          // [NQ rows x 64 dims] of one term
   const uint32_t pbuf = (uint32_t)natoms * kHalfBytes; // [atom][128 keys][128 B]
   uint8_t* sQ = smem;                                  // [half][term][NQ][128 B]: per dim half, the 2 NQ rows of both terms in a row
   uint8_t* sP = sQ + 4 * qhalf;                        // [buffer][atom][128 keys][128 B]: columns q (leading terms) and NQ + q
-  uint8_t* sK = sP + (size_t)a.pbufs * pbuf;                        // [2 stages][half][128 keys][128 B]
-  uint8_t* sV = sK + 2 * 2 * kHalfBytes;               // [vstages][half][128 keys][128 B]
-  uint8_t* ctl = sV + (size_t)vstages * 2 * kHalfBytes;
+  uint8_t* sK = sP + (size_t)kPBufs * pbuf;                        // [2 stages][half][128 keys][128 B]
+  uint8_t* sV = sK + 2 * 2 * kHalfBytes;               // [2 stages][half][128 keys][128 B]
+  uint8_t* ctl = sV + 2 * 2 * kHalfBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(ctl);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 20);
   volatile int* s_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -201,19 +196,19 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
 
   const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int b = blockIdx.x / a.Hkv, kvh = blockIdx.x % a.Hkv, split = blockIdx.y;
-  // TMEM columns: S^T of even tiles, S^T of odd tiles (each NQ wide, or 2 NQ when the two query terms
-  // are kept apart), then O^T, 2 NQ wide: the leading and the trailing weight terms' shares
-  const uint32_t cstride = (uint32_t)(((a.qstack ? 2 * NQ : NQ) + 31) & ~31);
-  const uint32_t ocol = NSB * cstride;
+  // TMEM columns: four S^T buffers, 2 NQ wide (the two query terms' shares), then O^T, 2 NQ wide: the
+  // leading and the trailing weight terms' shares (480 columns at 48 query rows)
+  const uint32_t cstride = (uint32_t)((2 * NQ + 31) & ~31);
+  const uint32_t ocol = kSBufs * cstride;
   uint32_t tmem_cols = 32;
-  while (tmem_cols < ocol + (uint32_t)((2 * NQ + 31) & ~31)) tmem_cols <<= 1;
+  while (tmem_cols < ocol + cstride) tmem_cols <<= 1;
 
   if (tid == kProdWarp * 32) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(b_kfull + 8 * s, 1); mbar_init(b_kfree + 8 * s, 1);
       mbar_init(b_vfull + 8 * s, 1); mbar_init(b_vfree + 8 * s, 1);
     }
-    for (int s = 0; s < NSB; ++s) mbar_init(b_sready + 8 * s, 1);
+    for (int s = 0; s < kSBufs; ++s) mbar_init(b_sready + 8 * s, 1);
     mbar_init(b_qfull, 1);
     mbar_init(b_pready, kSoftThreads); mbar_init(b_pready + 8, kSoftThreads);
     mbar_init(b_odone, 1); mbar_init(b_odone + 8, 1);
@@ -243,7 +238,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
   };
   // one producer warp feeds K, one feeds V
   const bool is_k = warp == kProdWarp, is_prod = is_k || warp == kVProdWarp;
-  const int st = is_k ? 2 : vstages;
+  constexpr int st = kStages;
   const uint32_t ring = smem_u32(is_k ? sK : sV), bfree = is_k ? b_kfree : b_vfree, bfull = is_k ? b_kfull : b_vfull;
   const long long first_row = is_k ? krow : vrow;
   // tiles of cached keys only: nothing in flight writes them, so they need not wait for the
@@ -311,38 +306,26 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issuer
     if (ntl > 0) {
-      // bf16 x bf16 -> fp32, M = 128.  The two bf16 terms of the second operand sit side by side along N
-      // wherever TMEM has the columns: one instruction then does the work of two, and the two halves
-      // of the result are added when they are read.
+      // bf16 x bf16 -> fp32, M = 128.  The two bf16 terms of the second operand sit side by side along N:
+      // one instruction does the work of two, and the two halves of the result are added when they are read.
       auto idesc = [](int n) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24); };
-      const uint32_t idesc_s = idesc(a.qstack ? 2 * NQ : NQ);
+      const uint32_t idesc_s = idesc(2 * NQ);
       const uint32_t idesc_o = idesc(2 * NQ) | (1u << 15) | (1u << 16);   // A (= V) and B (= P^T) are MN-major
       const uint64_t dq = desc_kmajor(smem_u32(sQ)), dp0 = desc_mnmajor(smem_u32(sP), kHalfBytes);
       const uint64_t dk0 = desc_kmajor(smem_u32(sK)), dv0 = desc_mnmajor(smem_u32(sV), kHalfBytes);
       auto issue_scores = [&](int i) -> bool {
-        const int s = i & 1, sb = i & (NSB - 1);           // K stage, S^T buffer
+        const int s = i & 1, sb = i & (kSBufs - 1);           // K stage, S^T buffer
         if (!mbar_wait_warp(b_kfull + 8 * s, (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns)) return false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (elect_one()) {
           const uint64_t dk = dk0 + (uint64_t)(uint32_t)(s * (2 * kHalfBytes >> 4));
           const uint32_t acc = tmem_base + (uint32_t)sb * cstride;
-          if (a.qstack) {
 #pragma unroll
-            for (int dh = 0; dh < 2; ++dh)
+          for (int dh = 0; dh < 2; ++dh)
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                umma_bf16(acc, dk + dh * (kHalfBytes >> 4) + 2 * kk, dq + (uint64_t)((dh * 2 * qhalf) >> 4) + 2 * kk, idesc_s,
-                          (dh | kk) ? 1u : 0u);
-          } else {
-#pragma unroll
-            for (int term = 0; term < 2; ++term)
-#pragma unroll
-              for (int dh = 0; dh < 2; ++dh)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  umma_bf16(acc, dk + dh * (kHalfBytes >> 4) + 2 * kk, dq + (uint64_t)(((2 * dh + term) * qhalf) >> 4) + 2 * kk,
-                            idesc_s, (term | dh | kk) ? 1u : 0u);
-          }
+            for (int kk = 0; kk < 4; ++kk)
+              umma_bf16(acc, dk + dh * (kHalfBytes >> 4) + 2 * kk, dq + (uint64_t)((dh * 2 * qhalf) >> 4) + 2 * kk, idesc_s,
+                        (dh | kk) ? 1u : 0u);
           umma_commit(b_kfree + 8 * s);
           umma_commit(b_sready + 8 * sb);
         }
@@ -354,13 +337,13 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
       uint32_t ph = 0;
       for (int i = 0; i < ntl && ok; ++i) {
         // The scores of the next tiles go first: they run during this tile's softmax.  The S^T buffer
-        // of tile t was last read by the softmax of tile t - NSB, which had finished before P^T of
+        // of tile t was last read by the softmax of tile t - kSBufs, which had finished before P^T of
         // that tile was signalled - and this warp has waited for the P^T of every tile before i.
         // A column group whose tiles are quick - all its rows masked - can therefore be a tile ahead
         // of the others, which is why "P^T written" has a barrier per tile parity: it cannot be two
         // ahead, because the scores of tile i + 2 are only issued after P^T of tile i (with four
         // buffers the softmax hands tiles over in pairs, odd after even, so parity still tells them apart).
-        while (qk < ntl && qk < i + NSB && ok) { ok = issue_scores(qk); ++qk; }
+        while (qk < ntl && qk < i + kSBufs && ok) { ok = issue_scores(qk); ++qk; }
         if (!ok) break;
         ok = mbar_wait_warp(b_pready + 8 * (i & 1), (uint32_t)(i >> 1) & 1u, s_abort, a.wait_ns) &&
              mbar_wait_warp(b_vfull + 8 * s, ph, s_abort, a.wait_ns);
@@ -374,8 +357,8 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
           umma_commit(b_vfree + 8 * s);
           umma_commit(b_odone + 8 * (i & 1));
         }
-        if (++s == vstages) { s = 0; ph ^= 1u; }
-        if (++pb == a.pbufs) pb = 0;
+        if (++s == kStages) { s = 0; ph ^= 1u; }
+        pb ^= 1;
       }
       if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
     }
@@ -384,13 +367,13 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     // thread = one TMEM lane (a key of the tile for S^T, a head dim for O^T) and half of the columns
     const int wq = warp & 3, grp = warp >> 2;
     const int row = wq * 32 + lane;                    // TMEM lane of this thread
-    const int ncol = NQ / 3, nch = ncol >> 3;          // this thread's columns (8, 16, 24 or 32), in chunks of 8
+    const int ncol = NQ / 3, nch = ncol >> 3;          // this thread's columns (8 or 16), in chunks of 8
     const int q0 = grp * ncol;
     const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16);
     const float sc = a.scale_log2e;
-    f32x2 lsum[KC / 2];                             // this key lane's share of every column's sum, two columns per register pair
+    f32x2 lsum[kCols / 2];                             // this key lane's share of every column's sum, two columns per register pair
 #pragma unroll
-    for (int j = 0; j < KC / 2; ++j) lsum[j] = pack2(0.f, 0.f);
+    for (int j = 0; j < kCols / 2; ++j) lsum[j] = pack2(0.f, 0.f);
     const f32x2 sc2 = pack2(sc, sc);
     // This warp's own copy of its columns' running reference points (every warp of the group works
     // out the same values): the reference m (log2 domain), the raw score above which it has to
@@ -410,37 +393,31 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     const int limmin = *s_limmin;
     // ---- the pieces of one tile's softmax
     // this key's scores of this thread's columns (masked keys count as -inf)
-    auto load_scores = [&](int t, float (&v)[KC]) -> bool {
-      const int sb = t & (NSB - 1);
+    auto load_scores = [&](int t, float (&v)[kCols]) -> bool {
+      const int sb = t & (kSBufs - 1);
       const int tile0 = (split + t * a.nsplit) * kTileKeys;
-      const bool ok = mbar_wait(b_sready + 8 * sb, (uint32_t)(t / NSB) & 1u, s_abort, a.wait_ns);
+      const bool ok = mbar_wait(b_sready + 8 * sb, (uint32_t)(t / kSBufs) & 1u, s_abort, a.wait_ns);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t s_addr = lane_base + (uint32_t)sb * cstride + (uint32_t)q0;
 #pragma unroll
-      for (int c = 0; c < KC / 8; ++c)
+      for (int c = 0; c < kCols / 8; ++c)
         if (c < nch) tmem_ld8_nowait(s_addr + 8 * c, v + 8 * c);
-      if (a.qstack) {                                    // the trailing query terms' share, NQ columns further
+      // the trailing query terms' share, NQ columns further
 #pragma unroll
-        for (int c = 0; c < KC / 8; ++c)
-          if (c < nch) {
-            float w[8];
-            tmem_ld8_nowait(s_addr + (uint32_t)NQ + 8 * c, w);
-            tmem_ld_wait();
-            tmem_landed8(w);
-            tmem_landed8(v + 8 * c);                     // (requested before w: landed as well)
+      for (int c = 0; c < kCols / 8; ++c)
+        if (c < nch) {
+          float w[8];
+          tmem_ld8_nowait(s_addr + (uint32_t)NQ + 8 * c, w);
+          tmem_ld_wait();
+          tmem_landed8(w);
+          tmem_landed8(v + 8 * c);                       // (requested before w: landed as well)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[8 * c + j] += w[j];
-          }
-      } else {
-        tmem_ld_wait();
-#pragma unroll
-        for (int c = 0; c < KC / 8; ++c)
-          if (c < nch) tmem_landed8(v + 8 * c);
-      }
+          for (int j = 0; j < 8; ++j) v[8 * c + j] += w[j];
+        }
       if (tile0 + kTileKeys > limmin) {                  // some live query row masks a key of this tile
         const int key = tile0 + row;                     // the key of this lane
 #pragma unroll
-        for (int c = 0; c < KC / 8; ++c)
+        for (int c = 0; c < kCols / 8; ++c)
           if (c < nch) {
 #pragma unroll
             for (int j = 0; j < 8; ++j)
@@ -453,10 +430,10 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     // none)?  Softmax does not depend on the reference point, and weights up to 2^8 are as exact in
     // two bf16 terms as weights up to 1, so the reference only has to follow the true maximum from
     // afar: on most tiles nothing moves, no maximum is worked out and O^T is left alone.
-    auto exceeds = [&](const float (&v)[KC]) -> bool {
+    auto exceeds = [&](const float (&v)[kCols]) -> bool {
       bool exceed = false;
 #pragma unroll
-      for (int c = 0; c < KC / 8; ++c)
+      for (int c = 0; c < kCols / 8; ++c)
         if (c < nch) {
           const float4 ta = *reinterpret_cast<const float4*>(w_thr + 8 * c), tb = *reinterpret_cast<const float4*>(w_thr + 8 * c + 4);
           exceed = exceed || v[8 * c] > ta.x || v[8 * c + 1] > ta.y || v[8 * c + 2] > ta.z || v[8 * c + 3] > ta.w ||
@@ -466,14 +443,14 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     };
     // tile t's P^T buffer was last read by the P V product of tile t - pbufs
     auto pbuf_free = [&](int t) -> bool {
-      return t < a.pbufs || mbar_wait(b_odone + 8 * ((t - a.pbufs) & 1), (uint32_t)((t - a.pbufs) >> 1) & 1u, s_abort, a.wait_ns);
+      return t < kPBufs || mbar_wait(b_odone + 8 * ((t - kPBufs) & 1), (uint32_t)((t - kPBufs) >> 1) & 1u, s_abort, a.wait_ns);
     };
     // weights 2^(score * scale - m), this lane's share of the column sums, P^T, and the hand-over of tile t
-    auto emit = [&](int t, float (&v)[KC]) {
+    auto emit = [&](int t, float (&v)[kCols]) {
       const int tile0 = (split + t * a.nsplit) * kTileKeys;
-      uint8_t* prow = sP + (size_t)(t % a.pbufs) * pbuf + (size_t)row * 128;
+      uint8_t* prow = sP + (size_t)(t % kPBufs) * pbuf + (size_t)row * 128;
 #pragma unroll
-      for (int c = 0; c < KC / 8; ++c)
+      for (int c = 0; c < kCols / 8; ++c)
         if (c < nch) {
           const float4 na = *reinterpret_cast<const float4*>(w_nme + 8 * c), nb = *reinterpret_cast<const float4*>(w_nme + 8 * c + 4);
           const float nm[8] = {na.x, na.y, na.z, na.w, nb.x, nb.y, nb.z, nb.w};
@@ -501,8 +478,8 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       // keys past the longest row of this sequence hold whatever the cache held: zero their V rows
       if (tile0 + kTileKeys > lmax) {
-        const int s = t % vstages;
-        if (!mbar_wait(b_vfull + 8 * s, (uint32_t)(t / vstages) & 1u, s_abort, a.wait_ns)) *s_abort = 1;
+        const int s = t % kStages;
+        if (!mbar_wait(b_vfull + 8 * s, (uint32_t)(t / kStages) & 1u, s_abort, a.wait_ns)) *s_abort = 1;
         uint8_t* vs = sV + (size_t)s * 2 * kHalfBytes;
         for (int rr = max(lmax - tile0, 0) + (warp * 32 + lane); rr < kTileKeys; rr += kSoftThreads) {
 #pragma unroll
@@ -516,21 +493,19 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive(b_pready + 8 * (t & 1));
     };
-    // With four S^T buffers the tiles are taken two at a time: one wait for both score products, one
+    // The tiles are taken two at a time: one wait for both score products, one
     // vote, then the two sets of weights back to back - half the hand-overs per key.  When the vote
     // says that a reference point has to move, the tile is finished on its own and the next turn
     // starts with its neighbour.
     for (int i = 0; i < ntl;) {
       const int sp = i & 1;
-      const bool pair = NSB == 4 && i + 1 < ntl;
-      float v[KC], v_next[NSB == 4 ? KC : 1];
+      const bool pair = i + 1 < ntl;
+      float v[kCols], v_next[kCols];
       bool ok = load_scores(i, v);
       bool exceed = exceeds(v);
-      if constexpr (NSB == 4) {
-        if (pair) {
-          ok = load_scores(i + 1, v_next) && ok;
-          exceed = exceed || exceeds(v_next);
-        }
+      if (pair) {
+        ok = load_scores(i + 1, v_next) && ok;
+        exceed = exceed || exceeds(v_next);
       }
       ok = pbuf_free(i) && ok;
       const bool bad = !ok || *s_abort != 0;
@@ -543,7 +518,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
         {
           float x[32];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) x[j] = (j < KC && j < ncol) ? v[j < KC ? j : 0] : -INFINITY;
+          for (int j = 0; j < 32; ++j) x[j] = (j < kCols && j < ncol) ? v[j < kCols ? j : 0] : -INFINITY;
           const float r = warp_max32(x, lane);
           if (lane < ncol) red_w[lane] = r;
         }
@@ -560,9 +535,9 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
           crA = mvA ? ((mo == -INFINITY) ? 0.f : ex2(mo - t)) : 1.f;
         }
         const unsigned grewA = __ballot_sync(0xffffffffu, mvA);
-        bool prev_done = a.pbufs == 1;                   // is the P V product of tile i - 1 known to have retired?
+        bool prev_done = false;                          // is the P V product of tile i - 1 known to have retired?
 #pragma unroll
-        for (int c = 0; c < KC / 8; ++c) {
+        for (int c = 0; c < kCols / 8; ++c) {
           if (c < nch) {
             const bool grew = ((grewA >> (8 * c)) & 0xffu) != 0;   // the same in every thread of the group
             if (grew) {
@@ -603,16 +578,14 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
           w_nme[lane] = (mnA == -INFINITY) ? -INFINITY : -mnA;
         }
         __syncwarp();
-              emit(i, v);
+        emit(i, v);
         i += 1;
         continue;
       }
       emit(i, v);
-      if constexpr (NSB == 4) {
-        if (pair) {
-          if (!pbuf_free(i + 1)) *s_abort = 1;
-          emit(i + 1, v_next);
-        }
+      if (pair) {
+        if (!pbuf_free(i + 1)) *s_abort = 1;
+        emit(i + 1, v_next);
       }
       i += pair ? 2 : 1;
     }
@@ -625,7 +598,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // O^T: this thread holds head dim `row` of its columns; one 512-byte row of the partial output per column
 #pragma unroll
-    for (int c = 0; c < KC / 8; ++c) {
+    for (int c = 0; c < kCols / 8; ++c) {
       if (c < nch) {
         float o[8];
         if (have) {
@@ -654,7 +627,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
     // the column sums: add the 128 key lanes' shares up (warp shuffle, then the four warps of the group)
     float* sum_w = s_red + warp * kCols;
 #pragma unroll
-    for (int c = 0; c < KC / 8; ++c) {
+    for (int c = 0; c < kCols / 8; ++c) {
       if (c < nch) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -701,7 +674,7 @@ int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B,
   const cs_model_config& c = ctx->cfg;
   const int G = c.n_heads / c.n_kv_heads;
   if (c.head_dim != kDh || G > kNQMax || R < 1 || R > 256) return 0;
-  // blocks with more than 96 query rows per KV head are cut into groups of block rows
+  // blocks with more than 48 query rows per KV head are cut into groups of block rows
   const int ngroups = cs_ceil_div(G * R, kNQMax), Rg = cs_ceil_div(R, ngroups);
   if (G * Rg > kNQMax) return 0;
   const int nq = G * Rg;
@@ -721,28 +694,16 @@ int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B,
     if (cs_encode_tiled(ctx, &ctx->tmQ, ctx->qbuf, 3, dims, strides, box) != CS_OK) return -1;
     ctx->tmQ_R = Rg;
   }
-  // one CTA per SM: Q (two terms), P^T (two terms, 64-column atoms), two K stages, one or two V stages,
-  // then barriers, flags and the softmax scratch; 1 KB of slack for the 1024-byte alignment
+  // one CTA per SM: 1 KB of slack for the 1024-byte alignment, Q (two terms), two P^T buffers (two terms,
+  // 64-column atoms), two K and two V stages, then barriers, flags and the softmax scratch
   const size_t natoms = (size_t)(2 * NQ + 63) / 64;
-  const size_t base = 1024 + (size_t)4 * NQ * 128 + (size_t)2 * 2 * kHalfBytes;
-  const size_t pbuf = natoms * kHalfBytes, vstage = (size_t)2 * kHalfBytes;
-  const size_t ctl = (size_t)kCtlBytes + kNQMax * 4 + kSoftWarps * 3 * kCols * 4 + 2 * kSoftWarps * kCols * 4;
-  const size_t limit = 227 * 1024;
-  // in order of what it buys: a second P^T buffer (the softmax no longer waits for the previous
-  // tile's P V product), then a second V stage
-  const int pbufs = (base + 2 * pbuf + vstage + ctl <= limit) ? 2 : 1;
-  const int vstages = (base + pbufs * pbuf + 2 * vstage + ctl <= limit) ? 2 : 1;
-  const size_t smem = base + pbufs * pbuf + vstages * vstage + ctl;
-  if (smem > limit) return 0;
+  const size_t smem = 1024 + (size_t)4 * NQ * 128 + kPBufs * natoms * kHalfBytes + (size_t)2 * kStages * 2 * kHalfBytes +
+                      kCtlBytes + kNQMax * 4 + kSoftWarps * 3 * kCols * 4 + 2 * kSoftWarps * kCols * 4;
   int nsplit = ctx->num_sms / (B * c.n_kv_heads * ngroups);
   if (nsplit > ctx->attn_splits) nsplit = ctx->attn_splits;
   if (nsplit < 1) nsplit = 1;
-  // up to 48 query rows (16 columns per softmax thread) with two P^T buffers: four S^T buffers, tiles in pairs
-  const bool dual = NQ <= 48 && pbufs == 2;
-  auto kernel = dual ? k_attn_tcw<16, 4> : k_attn_tcw<kCols, 2>;
-  if (smem > ctx->attn_tcw_smem_set) {                 // (both instantiations are raised together: one high-water mark)
-    if (cudaFuncSetAttribute(k_attn_tcw<16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(k_attn_tcw<kCols, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  if (smem > ctx->attn_tcw_smem_set) {
+    if (cudaFuncSetAttribute(k_attn_tcw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       snprintf(ctx->err, sizeof(ctx->err), "attention needs %zu bytes of shared memory", smem);
       return -1;
     }
@@ -752,15 +713,13 @@ int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B,
   a.row_lim = ctx->row_lim;
   a.kv_len_early = ctx->kv_len_early;
   a.layer = layer; a.R = R; a.Rg = Rg; a.G = G; a.H = c.n_heads; a.Hkv = c.n_kv_heads;
-  a.max_batch = c.max_batch; a.max_seq = c.max_seq; a.nsplit = nsplit; a.NQ = NQ; a.rows = B * R; a.vstages = vstages; a.pbufs = pbufs;
-  a.qstack = (3 * ((2 * NQ + 31) / 32 * 32) <= 512) ? 1 : 0;   // TMEM columns: two score buffers and the output, 2 NQ wide each
-  if (dual && 5 * ((2 * NQ + 31) / 32 * 32) > 512) return 0;   // (four score buffers and the output: 480 columns at 48 query rows)
+  a.max_batch = c.max_batch; a.max_seq = c.max_seq; a.nsplit = nsplit; a.NQ = NQ; a.rows = B * R;
   a.smem_bytes = (int)smem;
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)kDh);
   a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.status = ctx->d_status;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, CS_FAM_ATTENTION);
-  if (cs_launch_pdl(kernel, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
+  if (cs_launch_pdl(k_attn_tcw, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
     snprintf(ctx->err, sizeof(ctx->err), "attention launch failed");
     return -1;
   }
