@@ -213,24 +213,24 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  if (warp < kSoftWarps) {
-    int lm = 0;
-    for (int r = tid; r < Rcur; r += kSoftWarps * 32) lm = max(lm, a.row_lim[b * R + r0 + r]);
-    lm = __reduce_max_sync(0xffffffffu, lm);
-    if (lane == 0 && lm > 0) atomicMax(s_lmax, lm);
-  }
   const int quarter = warp & 3, part = warp >> 2, q = quarter * 32 + lane;   // of a softmax thread: query row = TMEM lane, quarter of the columns
   const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-  if (warp < kSoftWarps && quarter < nact) {
-    // queries into tensor memory: this thread one half (64 dims) of one term of its row
+  const bool softmax = warp < kSoftWarps && quarter < nact, valid = softmax && q < nq;
+  int lim = 0;                                         // keys this row attends to
+  if (softmax) {
+    // queries into tensor memory: this thread one half (64 dims) of one term of its row, asked for together with
+    // the row's limit
     uint32_t w[32];
     const __nv_bfloat16* src = a.qbuf + (((size_t)(part >> 1) * CS_MAX_ROWS + (b * R + r0 + q / G)) * a.H + kvh * G + q % G) * kDh + (part & 1) * 64;
 #pragma unroll
     for (int j = 0; j < 32; ++j) w[j] = 0u;
-    if (q < nq) {
+    if (valid) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) load8(src + 16 * j, w + 8 * j);   // (whole 32-byte sectors)
+      lim = a.row_lim[b * R + r0 + q / G];
     }
+    const int lm = __reduce_max_sync(0xffffffffu, lim);
+    if (lane == 0 && part == 0 && lm > 0) atomicMax(s_lmax, lm);
     tmem_st16(lane_base + kQCol + 32u * (uint32_t)part, w);
     tmem_st16(lane_base + kQCol + 32u * (uint32_t)part + 16u, w + 16);
     tmem_st_wait();
@@ -322,10 +322,8 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
       }
       if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
     }
-  } else if ((warp & 3) < nact) {
+  } else if (softmax) {
     // ------------------------------------------------------------------ softmax + epilogue (four threads per query row)
-    const bool valid = q < nq;
-    const int lim = valid ? a.row_lim[b * R + r0 + q / G] : 0;
     const float sc = a.scale_log2e;
     const f32x2 sc2 = pack2(sc, sc);
     float m = -INFINITY, thr = valid ? -INFINITY : INFINITY;   // reference point (log2 domain); raw score above which it moves

@@ -31,7 +31,8 @@
 // Copies and MMAs are issued by an elected lane with uniform operands (cs_tcgen.cuh): a stage goes
 // back to the producer some 800 clocks sooner than when one lane issued the eight MMAs of a K block.
 // Measured on an 11-row block of the 8B shape, before and after: QKV 12.4 -> 12.1 us, attention output
-// 11.0 -> 9.8, down 23.7 -> 22.2.
+// 11.0 -> 9.8, down 23.7 -> 22.2; with what the epilogue needs besides the sums asked for ahead of the MMAs'
+// end: attention output 9.7 -> 9.2, down 22.6 -> 22.3 (QKV stays at 12).
 //
 // Every wait is bounded: when it runs out the CTA records CS_DEV_TIMEOUT, drains its
 // copies, still takes part in the cluster barriers, frees its TMEM and returns.
@@ -175,6 +176,17 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = uniform(*tmem_slot);
   bool ok = true;
+  // What an epilogue thread's first item needs besides the sums - residual row and gain, or rotation factors and
+  // the row's place in the cache - is asked for while the MMAs run
+  const int e = threadIdx.x;
+  const int r_fs = ((CS_GEMM_BM + a.splits - 1) / a.splits + 3) & ~3, r_flo = split * r_fs;   // STORE, RESIDUAL: this rank's features
+  const int r_per_tok = max(0, min(CS_GEMM_BM, r_flo + r_fs) - r_flo) >> 2;
+  const int q_js = ((64 + a.splits - 1) / a.splits + 3) & ~3, q_jlo = split * q_js;           // QKV: this rank's rotation pairs
+  const int q_per_tok = max(0, min(64, q_jlo + q_js) - q_jlo) >> 2;
+  const bool feeds_norm = a.mode == CS_EPI_RESIDUAL && a.nf.gain_out != nullptr;
+  float4 pre_a = make_float4(0.f, 0.f, 0.f, 0.f), pre_b = pre_a;
+  uint2 pre_g = make_uint2(0u, 0u);
+  int pre_w = 0, pre_p = 0;
 
   if (warp == 4) {
     // ------------------------------------------------------------- TMA producer
@@ -246,6 +258,20 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   } else {
     // ------------------------------------------------------------- epilogue warps 0-3: wait for the accumulators
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (a.mode == CS_EPI_RESIDUAL && (a.N & 3) == 0 && e < r_per_tok * a.rows) {
+      const int f = r_flo + 4 * (e % r_per_tok), tok = e / r_per_tok;
+      if (n0 + f + 3 < a.N) {
+        pre_a = *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
+        if (feeds_norm) pre_g = *reinterpret_cast<const uint2*>(a.nf.gain_out + n0 + f);
+      }
+    } else if (a.mode == CS_EPI_QKV && e < q_per_tok * a.rows) {
+      const int half = a.q.Dh >> 1, i = (q_jlo + 4 * (e % q_per_tok)) % half, tok = e / q_per_tok;
+      const float4* csp = reinterpret_cast<const float4*>(a.q.rope_cs + 2 * ((size_t)tok * half + i));
+      pre_a = csp[0];
+      pre_b = csp[1];
+      pre_w = a.q.row_write[tok];
+      pre_p = a.q.row_pos[tok];
+    }
     if (a.nf.ssq_in != nullptr) {
       // 1/rms of every token row while the main loop runs: slots summed in a fixed order.  Eight
       // rows at a time, so that a tall block's loads overlap instead of queueing row after row.
@@ -339,16 +365,6 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
     // still reads its tile) is split: a warp arrives as soon as the last remote reads of its lanes
     // have returned and only waits after its global stores, which hides the barrier behind them.
     if (a.splits > 1) cluster_arrive();
-    const int e = threadIdx.x;
-    // residual update: the first item's x (and gain) can be on their way during the barrier
-    const int r_fs = ((CS_GEMM_BM + a.splits - 1) / a.splits + 3) & ~3;
-    const int r_flo = split * r_fs, r_per_tok = max(0, min(CS_GEMM_BM, r_flo + r_fs) - r_flo) >> 2;
-    const bool r_vec = (a.N & 3) == 0;
-    float4 x_pre = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (warp < 4 && a.mode == CS_EPI_RESIDUAL && r_vec && e < r_per_tok * a.rows) {
-      const int f = r_flo + 4 * (e % r_per_tok), tok = e / r_per_tok;
-      if (n0 + f + 3 < a.N) x_pre = *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
-    }
     if (a.splits > 1) cluster_wait();
     bool arrived = a.splits <= 1;                  // this thread's half of barrier 2
     if (warp < 4) {
@@ -358,9 +374,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
         // the first halves of the tile's heads; each rank finishes a slice of j, four at a time.
         const QkvEpi& Q = a.q;
         const int half = Q.Dh >> 1;
-        const int js = ((64 + a.splits - 1) / a.splits + 3) & ~3;
-        const int j_lo = split * js, j_n = max(0, min(64, j_lo + js) - j_lo);
-        const int per_tok = j_n >> 2;
+        const int j_lo = q_jlo, per_tok = q_per_tok;
         const int total = per_tok * a.rows, iters = (total + 127) >> 7;   // same trip count for every thread
         for (int it = 0; it < iters; ++it) {
           const int idx = e + (it << 7);
@@ -372,8 +386,9 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
           // the rotation factors and the row's place in the cache do not depend on the sums: they are
           // requested first, so that their latency runs under the remote reads
           const float4* csp = reinterpret_cast<const float4*>(Q.rope_cs + 2 * ((size_t)tok * half + i));
-          const float4 cs01 = csp[0], cs23 = csp[1];      // (cos, sin) of dims i .. i + 3
-          const int row_w = Q.row_write[tok], row_p = Q.row_pos[tok];
+          const bool first = it == 0;
+          const float4 cs01 = first ? pre_a : csp[0], cs23 = first ? pre_b : csp[1];      // (cos, sin) of dims i .. i + 3
+          const int row_w = first ? pre_w : Q.row_write[tok], row_p = first ? pre_p : Q.row_pos[tok];
           float4 av = make_float4(0.f, 0.f, 0.f, 0.f), bv = av;
           if (a.splits > 1) {
             if (act) {
@@ -422,10 +437,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
           }
         }
       } else {
-        const int fs = ((CS_GEMM_BM + a.splits - 1) / a.splits + 3) & ~3;
-        const int f_lo = split * fs, f_n = max(0, min(CS_GEMM_BM, f_lo + fs) - f_lo);
-        const int per_tok = f_n >> 2;
-        const bool feeds_norm = a.mode == CS_EPI_RESIDUAL && a.nf.gain_out != nullptr;
+        const int f_lo = r_flo, per_tok = r_per_tok;
         float* part = dump + a.n_tok * CS_GEMM_BM;   // [rows][32] sums of squares, behind the parked tile
         const int total = per_tok * a.rows, iters = (total + 127) >> 7;
         const bool vec_n = (a.N & 3) == 0;
@@ -440,7 +452,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
             if (a.splits > 1) y = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok * CS_GEMM_BM + f), a.splits);
             else y = *reinterpret_cast<const float4*>(dump + tok * CS_GEMM_BM + f);
             if (a.mode == CS_EPI_RESIDUAL && vec)
-              x = (it == 0) ? x_pre : *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
+              x = (it == 0) ? pre_a : *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
           }
           if (a.splits > 1 && it == iters - 1) { keep_alive(y, y); cluster_arrive(); arrived = true; }
           if (!act) continue;
@@ -450,7 +462,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
             const float4 o = make_float4(y.x + x.x, y.y + x.y, y.z + x.z, y.w + x.w);   // (x stays 0 unless this is a residual update)
             *reinterpret_cast<float4*>(dst) = o;
             if (feeds_norm) {
-              const uint2 gw = *reinterpret_cast<const uint2*>(a.nf.gain_out + n0 + f);
+              const uint2 gw = it == 0 ? pre_g : *reinterpret_cast<const uint2*>(a.nf.gain_out + n0 + f);
               const float2 g01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.x));
               const float2 g23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gw.y));
               const float w0 = o.x * g01.x, w1 = o.y * g01.y, w2 = o.z * g23.x, w3 = o.w * g23.y;
