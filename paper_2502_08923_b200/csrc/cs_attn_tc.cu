@@ -8,7 +8,9 @@
 //     O [128 x 128 dims] += P_hi V_tile   + P_lo V_tile     (A = P in tensor memory, B = V tile, MN-major
 //                                                            straight from the cache layout)
 // Queries and softmax weights enter as two bf16 terms each, so they are fp32-equivalent and only K and V -
-// which the cache stores in bf16 - are rounded.  Both A operands live in TMEM: queries are put there once,
+// which the cache stores in bf16 - are rounded.  Both A operands live in TMEM: queries are put there once
+// (they arrive by TMA in the ring's last slots; fetched by the softmax threads themselves, lane = row, they took up
+// to 2 us at 11 rows and the layer 0.3 - 1 us longer),
 // and a tile's weights overwrite its scores (128 fp32 columns = 64 columns of leading and 64 of second bf16
 // terms), so shared memory holds nothing but the K and V tiles and the tensor cores read only those from it.
 // Two S buffers: the scores of tile i + 1 are ready or under way while the softmax of tile i runs, and the MMA
@@ -34,7 +36,8 @@
 //   256 rows over 3,840+ keys 98.6 -> 51.0 us (117.2), 168 rows over 8 x 16,384 keys 234 -> 114 us (142),
 //   11 rows over 4,096 keys 15.9 -> 14.6 us (17.7), 44 over 4 x 8,192 46.3 -> 36.1 us (37.2),
 //   1 row over 2,048 keys 10.7 -> 11.1 us, 256 rows over one tile 13.6 -> 14.2 us.
-// Queries in TMEM instead of shared memory: 122 -> 112 us at 168 rows over 8 x 16,384 keys, six slots for all.
+// Taken back: handing O over through shared memory to store whole rows per warp, 9.4 -> 10.5 us at 11 rows over
+// 4,096 keys.  Queries in TMEM instead of shared memory: 122 -> 112 us at 168 rows over 8 x 16,384 keys, six slots for all.
 //
 // Every wait is bounded (2 s by default): on expiry the CTA flags CS_DEV_TIMEOUT, drains its copies, frees
 // its TMEM and returns; the softmax threads of a lane quarter decide together.
@@ -52,7 +55,6 @@ constexpr uint32_t kOCol = 256, kQCol = 384, kTmemCols = 512;   // two S / P buf
 constexpr int kCtlBytes = 256;                   // mbarriers, TMEM slot, flags
 
 struct AttnArgs {
-  const __nv_bfloat16* qbuf;
   const int* row_lim;
   const int* kv_len_early;   // cached lengths that no kernel in flight changes, or NULL
   int layer, R, Rg, G, H, Hkv, max_batch, max_seq, nsplit, rows;   // Rg = block rows per row group
@@ -125,10 +127,6 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-__device__ __forceinline__ void load8(const void* src, uint32_t* v) {
-  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "l"(src) : "memory");
-}
 __device__ __forceinline__ void store8(float* dst, const float* v) {
   asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                ::"l"(dst), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]) : "memory");
@@ -143,7 +141,7 @@ __device__ __forceinline__ bool quarter_any(int quarter, bool pred) {
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
+k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmQ, AttnArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -151,6 +149,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
   // blockIdx.z picks a group of Rg consecutive block rows (blocks taller than 128 / G rows)
   const int G = a.G, R = a.R, r0 = blockIdx.z * a.Rg, Rcur = min(a.Rg, R - r0), nq = G * Rcur;
   uint8_t* ring = smem;                                // [slot][half][128 keys][128 B], K and V tiles in the order of use
+  // the queries pass through the last slots on their way to tensor memory: [term][half][NQ rows][128 B]
+  const uint32_t qpart = (uint32_t)((G * a.Rg + 7) & ~7) * 128u;
+  const int qslot = kSlots - (int)((4 * qpart + kSlotBytes - 1) / kSlotBytes);
+  uint8_t* sQ = ring + (size_t)qslot * kSlotBytes;
   uint8_t* ctl = ring + (size_t)kSlots * kSlotBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(ctl);    // full, free per slot; 2 S, 2 P, 4 O, Q
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 24);
@@ -165,7 +167,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
   }
   const uint32_t b_full = smem_u32(bars), b_free = smem_u32(bars + kSlots), b_sready = smem_u32(bars + 2 * kSlots),
                  b_pready = smem_u32(bars + 2 * kSlots + 2), b_odone = smem_u32(bars + 2 * kSlots + 4),
-                 b_qfull = smem_u32(bars + 2 * kSlots + 8);
+                 b_qfull = smem_u32(bars + 2 * kSlots + 8), b_qland = smem_u32(bars + 2 * kSlots + 9);
 
   const int tid = threadIdx.x, warp = (int)uniform(tid >> 5), lane = tid & 31;
   const int b = blockIdx.x / a.Hkv, kvh = blockIdx.x % a.Hkv, split = blockIdx.y;
@@ -176,6 +178,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
     for (int s = 0; s < 2; ++s) { mbar_init(b_sready + 8 * s, 1); mbar_init(b_pready + 8 * s, (uint32_t)nact * 4u); }
     for (int s = 0; s < 4; ++s) mbar_init(b_odone + 8 * s, 1);
     mbar_init(b_qfull, (uint32_t)nact * 4u);
+    mbar_init(b_qland, 1);
     *s_abort = 0; *s_never = 0; *s_lmax = 0; *s_asked = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmKV) : "memory");
@@ -213,24 +216,32 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
+  if (warp == kProdWarp && elect_one()) {
+    mbar_expect_tx(b_qland, (uint32_t)(4 * G * a.Rg * 128));
+    for (int term = 0; term < 2; ++term)
+      for (int dh = 0; dh < 2; ++dh)
+        tma_load_3d(smem_u32(sQ) + (uint32_t)(2 * term + dh) * qpart, &tmQ, b_qland, dh * 64, kvh * G,
+                    term * CS_MAX_ROWS + b * R + r0);   // the box is always Rg rows tall; rows past the group are never used
+  }
   const int quarter = warp & 3, part = warp >> 2, q = quarter * 32 + lane;   // of a softmax thread: query row = TMEM lane, quarter of the columns
   const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
   const bool softmax = warp < kSoftWarps && quarter < nact, valid = softmax && q < nq;
   int lim = 0;                                         // keys this row attends to
   if (softmax) {
-    // queries into tensor memory: this thread one half (64 dims) of one term of its row, asked for together with
-    // the row's limit
-    uint32_t w[32];
-    const __nv_bfloat16* src = a.qbuf + (((size_t)(part >> 1) * CS_MAX_ROWS + (b * R + r0 + q / G)) * a.H + kvh * G + q % G) * kDh + (part & 1) * 64;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) w[j] = 0u;
-    if (valid) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) load8(src + 16 * j, w + 8 * j);   // (whole 32-byte sectors)
-      lim = a.row_lim[b * R + r0 + q / G];
-    }
+    // queries into tensor memory: this thread one half (64 dims) of one term of its row (swizzled rows: eight lanes
+    // read eight different 16-byte columns)
+    if (valid) lim = a.row_lim[b * R + r0 + q / G];
     const int lm = __reduce_max_sync(0xffffffffu, lim);
     if (lane == 0 && part == 0 && lm > 0) atomicMax(s_lmax, lm);
+    if (!mbar_wait(b_qland, 0, s_abort, a.wait_ns)) *s_abort = 1;
+    __syncwarp();
+    uint32_t w[32];
+    const uint8_t* src = sQ + (uint32_t)part * qpart + (uint32_t)q * 128u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const uint4 t = valid ? *reinterpret_cast<const uint4*>(src + ((j ^ (q & 7)) << 4)) : make_uint4(0u, 0u, 0u, 0u);
+      w[4 * j] = t.x; w[4 * j + 1] = t.y; w[4 * j + 2] = t.z; w[4 * j + 3] = t.w;
+    }
     tmem_st16(lane_base + kQCol + 32u * (uint32_t)part, w);
     tmem_st16(lane_base + kQCol + 32u * (uint32_t)part + 16u, w + 16);
     tmem_st_wait();
@@ -253,6 +264,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
     for (; j < items; ++j) {
       const bool is_k = tk < 2 ? (tk == 0 || (tk < ntl && tv == 0)) : (tk < ntl && tk < tv + 2);
       if (j >= kSlots) ok = mbar_wait_warp(b_free + 8 * s, ph, s_abort, a.wait_ns);
+      if (j >= qslot && j < kSlots && ok) ok = mbar_wait_warp(b_qfull, 0, s_abort, a.wait_ns);   // (the queries have left the slot)
       if (!ok) break;
       if (j >= asked && elect_one()) load_tile(s, is_k ? krow : vrow, is_k ? tk : tv);
       if (is_k) ++tk; else ++tv;
@@ -262,6 +274,7 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, AttnArgs a) {
     __syncwarp();
     // copies that nobody will consume must land before the shared memory goes away
     if ((*s_abort || ntl == 0) && lane == 0) {
+      mbar_wait(b_qland, 0, s_never, a.wait_ns);
       for (int i = max(0, j - kSlots); i < j; ++i) mbar_wait(b_full + 8 * (i % kSlots), (uint32_t)(i / kSlots) & 1u, s_never, a.wait_ns);
     }
   } else if (warp == kMmaWarp) {
@@ -484,6 +497,13 @@ int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, 
     if (cs_encode_tiled(ctx, &ctx->tmKV, kv_cache, 2, dims, strides, box) != CS_OK) return -1;
     ctx->tmKV_base = kv_cache;
   }
+  if (ctx->tmQ_R != Rg) {
+    const unsigned long long dims[3] = {(unsigned long long)kDh, (unsigned long long)c.n_heads, 2ull * CS_MAX_ROWS};
+    const unsigned long long strides[2] = {kDh * 2, (unsigned long long)c.n_heads * kDh * 2};
+    const unsigned box[3] = {64, (unsigned)G, (unsigned)Rg};
+    if (cs_encode_tiled(ctx, &ctx->tmQ, ctx->qbuf, 3, dims, strides, box) != CS_OK) return -1;
+    ctx->tmQ_R = Rg;
+  }
   // one CTA per SM; 1 KB of slack for the 1024-byte alignment, then the ring, and barriers, flags and the exchange
   // rows of the softmax
   const size_t smem = 1024 + (size_t)kSlots * kSlotBytes + kCtlBytes + 4 * 128 * 4;
@@ -498,7 +518,6 @@ int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, 
     ctx->attn_tc_smem_set = smem;
   }
   AttnArgs a;
-  a.qbuf = ctx->qbuf;
   a.row_lim = ctx->row_lim;
   a.kv_len_early = ctx->kv_len_early;
   a.layer = layer; a.R = R; a.Rg = Rg; a.G = G; a.H = c.n_heads; a.Hkv = c.n_kv_heads;
@@ -508,7 +527,7 @@ int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, 
   a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.status = ctx->d_status;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, CS_FAM_ATTENTION);
-  if (cs_launch_pdl(k_attn_tc, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, a) != cudaSuccess) {
+  if (cs_launch_pdl(k_attn_tc, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
     snprintf(ctx->err, sizeof(ctx->err), "attention launch failed");
     return -1;
   }
