@@ -44,7 +44,7 @@ WsLayout ws_layout(const cs_model_config* c) {
   const size_t d = c->d_model, qd = (size_t)c->n_heads * c->head_dim, F = c->d_ffn;
   const size_t qkv = qd + 2 * (size_t)c->n_kv_heads * c->head_dim;
   L.qkv_elems = rows * (qkv > 4096 ? qkv : 4096);
-  int as = cs_ceil_div(c->max_seq, 128);
+  int as = cs_ceil_div(c->max_seq, c->head_dim == 128 ? 128 : 64);   // key tiles of the attention kernels
   L.attn_splits = as < 1 ? 1 : (as > 64 ? 64 : as);
   const size_t lm_tiles = cs_ceil_div(c->vocab, CS_GEMM_BM);
   size_t off = 0;

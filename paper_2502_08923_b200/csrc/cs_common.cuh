@@ -146,7 +146,7 @@ struct cs_ctx {
   // process: another context may live on another GPU)
   bool gemm_attr_set, pair_attr_set;
   int pairs_at_once;         // two-CTA clusters of the two-SM GEMM that can run at once (0 = not asked yet)
-  unsigned attn_mma_attr_set;   // bit DH/32 per head size
+  unsigned attn_mma_attr_set;   // a bit per head size and key grouping
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
