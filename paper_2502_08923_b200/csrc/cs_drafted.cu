@@ -57,7 +57,7 @@ extern "C" cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int
     return fail2(target, CS_ERR_ARG, "bad argument");
   if (delta > 0 && (drafter == nullptr || kv_drafter == nullptr || kv_len_drafter == nullptr || drafter == target))
     return fail2(target, CS_ERR_ARG, "delta > 0 needs a draft model context of its own, its cache and its length");
-  const int kt = std::max(k, delta);                   // rows of a target block beyond the first
+  const int kt = std::max(k, delta);                   // rows of a target block beyond the first, at most
   if (kt > target->cfg.k_max) return fail2(target, CS_ERR_ARG, "k or delta above the target context's k_max");
   if (delta > 0 && drafter->cfg.vocab != target->cfg.vocab)
     return fail2(target, CS_ERR_ARG, "draft model and target must share the vocabulary");
@@ -97,6 +97,9 @@ extern "C" cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int
     DR_CUDA(cudaStreamSynchronize(st));
     const int mpos = *word_h;
     const bool drafted = mpos < 0 && delta > 0;
+    // this step's: the proposals, or what the history holds behind the match (blocks of max(k, delta) + 1 rows
+    // every time took 84.0 instead of 83.1 ms for a call with three proposals and k = 10)
+    const int ks = drafted ? delta : (mpos >= 0 ? std::min(k, n - (mpos + gamma)) : 0);
     if (drafted) {
       // ---- step 3(a): catch up on tokens hist[d_len .. n), forced through in blocks of kd + 1
       // rows (scripted acceptance against the tokens themselves); the last row's greedy token
@@ -123,18 +126,18 @@ extern "C" cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int
     // ---- steps 2 / 3(b): one target block over [last token, draft]
     const int32_t* script_row = script != nullptr ? script + emitted : nullptr;
     const int have = max_new - emitted;
-    if (script != nullptr && have < kt + 1) {              // rows past the script's end cannot be accepted
-      DR_CUDA(cudaMemsetAsync(t_script, 0xFF, (size_t)(kt + 1) * 4, st));
+    if (script != nullptr && have < ks + 1) {              // rows past the script's end cannot be accepted
+      DR_CUDA(cudaMemsetAsync(t_script, 0xFF, (size_t)(ks + 1) * 4, st));
       DR_CUDA(cudaMemcpyAsync(t_script, script_row, (size_t)have * 4, cudaMemcpyDeviceToDevice, st));
       script_row = t_script;
     }
-    DR_OK(cs_verify_step(target, hist + (n - 1), t_draft, drafted ? target->iota + delta : t_dlen, 1, kt, kv_target,
+    DR_OK(cs_verify_step(target, hist + (n - 1), t_draft, drafted ? target->iota + delta : t_dlen, 1, ks, kv_target,
                          kv_len_target, script_row, t_accept, t_out, t_argmax, nullptr, st));
     DR_CUDA(cudaMemcpyAsync(word_h, t_accept, sizeof(int), cudaMemcpyDeviceToHost, st));
-    DR_CUDA(cudaMemcpyAsync(out_h, t_out, (size_t)(kt + 1) * 4, cudaMemcpyDeviceToHost, st));
+    DR_CUDA(cudaMemcpyAsync(out_h, t_out, (size_t)(ks + 1) * 4, cudaMemcpyDeviceToHost, st));
     DR_CUDA(cudaStreamSynchronize(st));
     const int tau = *word_h;
-    if (tau < 0 || tau > kt) break;                    // the device refused the step; the status word says why
+    if (tau < 0 || tau > ks) break;                    // the device refused the step; the status word says why
     int c = std::min(tau + 1, max_new - emitted);
     if (script == nullptr && eos_id >= 0) {
       for (int i = 0; i < c; ++i)
