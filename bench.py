@@ -48,7 +48,7 @@ SAMPLE_LAYERS = 4          # decoder layers of the CPU oracle's bounded sample
 
 # DRAM counters of the dominant kernel, written beside its ncu summary: `key = value` lines
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_gemm_tc_verify8b_2layer_ncu_traffic.txt")
-KERNEL_SOURCES = [os.path.join(ROOT, "paper_2502_08923_b200", "csrc", f) for f in ("cs_gemm.cu", "cs_common.cuh")]
+KERNEL_SOURCES = [os.path.join(ROOT, "paper_2502_08923_b200", "csrc", f) for f in ("cs_gemm.cu", "cs_gemm_pair.cu", "cs_tcgen.cuh", "cs_common.cuh")]
 
 
 def _kernel_hash():
