@@ -85,12 +85,13 @@ WsLayout ws_layout(const cs_model_config* c) {
   return L;
 }
 
-// Pinned host memory of the contexts: one 64 KB block for the process, handed out in slots (pinning takes from
+// Pinned host memory of the contexts: one block for the process, handed out in slots (pinning takes from
 // a tenth of a millisecond to tens of them, so it is not done per context).  Slots are given back by
 // cs_destroy; a context that finds none left pins its own.
-constexpr size_t kSlotBytes = 2048;
+constexpr size_t kStepInAt = 2048, kStepOutAt = kStepInAt + CS_STEP_IN_MAX * sizeof(int);
+constexpr size_t kSlotBytes = kStepOutAt + 2 * CS_MAX_ROWS * sizeof(int) + 1024;
 constexpr int kSlots = 32;
-static_assert(64 + (CS_MAX_ROWS + 1) * sizeof(int) <= kSlotBytes, "progress word and host scratch fit a slot");
+static_assert(64 + (CS_MAX_ROWS + 1) * sizeof(int) <= kStepInAt && kSlotBytes % 1024 == 0, "progress word and host scratch");
 std::mutex g_slot_lock;
 char* g_slots = nullptr;
 unsigned g_slots_taken = 0;
@@ -212,7 +213,7 @@ cs_status enqueue_loop_step(cs_ctx* ctx, cudaStream_t st, int step = -1) {
                                            cs_next_stamp(ctx, CS_FAM_OTHER));
   if (r != CS_OK) return fail(ctx, r, "match kernel launch failed");
   cs_launch_block_setup(ctx, ctx->loop_last, ctx->loop_draft, ctx->loop_dlen, L.kv_len, ctx->loop_done, L.B, L.k, false, st);
-  // the step opened with a stream-ordered launch and nothing before k_loop_commit changes kv_len
+  // k_block_setup lets nothing pass that was enqueued before the step, and nothing before k_loop_commit changes kv_len
   ctx->kv_len_early = L.kv_len;
   r = enqueue_forward(ctx, L.B, L.k + 1, L.kv_cache, true, nullptr, st);
   ctx->kv_len_early = nullptr;
@@ -342,6 +343,10 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   CREATE_OK(take_slot(reinterpret_cast<char**>(&ctx->progress)));
   CREATE_OK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->progress_dev), ctx->progress, 0));
   ctx->host_ints = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + 64);
+  ctx->step_in = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + kStepInAt);
+  ctx->step_in_dev = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress_dev) + kStepInAt);
+  ctx->step_out = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + kStepOutAt);
+  ctx->step_out_dev = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress_dev) + kStepOutAt);
   char* base = static_cast<char*>(workspace);
   ctx->ws = base;
   ctx->ws_bytes = L.total;
@@ -495,41 +500,59 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   // script rows
   HostStep& G = ctx->host_step;
   const bool known = G.host == hist_host && G.dev == hist_dev && G.B == B && G.stride == stride;
+  int* in = ctx->step_in;                              // (every earlier step of this context has been waited for)
+  int tokens = 0;
   for (int b = 0; b < B; ++b) {
     const int n = hist_len_host[b];
-    const int have = (known && G.host_len[b] == n && G.uploaded[b] <= n) ? G.uploaded[b] : 0;
-    if (n > have)
+    int have = (known && G.host_len[b] == n && G.uploaded[b] <= n) ? G.uploaded[b] : 0;
+    if (n - have > k + 1) {
       CS_CUDA_OK(ctx, cudaMemcpyAsync(hist_dev + (size_t)b * stride + have, hist_host + (size_t)b * stride + have,
                                       (size_t)(n - have) * 4, cudaMemcpyHostToDevice, st));
+      have = n;
+    }
+    in[b] = n;
+    in[B + b] = have;
+    in[2 * B + b] = tokens;
+    if (n > have) memcpy(in + 3 * B + tokens, hist_host + (size_t)b * stride + have, (size_t)(n - have) * 4);
+    tokens += n - have;
     G.uploaded[b] = n;
   }
   G.host = hist_host; G.dev = hist_dev; G.B = B; G.stride = stride;
-  CS_CUDA_OK(ctx, cudaMemcpyAsync(hist_len_dev, hist_len_host, (size_t)B * 4, cudaMemcpyHostToDevice, st));
-  const int32_t* script_dev = nullptr;
-  if (script_host != nullptr) {
-    CS_CUDA_OK(ctx, cudaMemcpyAsync(ctx->loop_emitted, script_host, (size_t)B * (k + 1) * 4, cudaMemcpyHostToDevice, st));
-    script_dev = ctx->loop_emitted;
-  }
+  const int script_ints = script_host != nullptr ? B * (k + 1) : 0;
+  const int32_t* script_dev = script_host != nullptr ? ctx->loop_emitted : nullptr;
+  if (script_host != nullptr) memcpy(in + 3 * B + tokens, script_host, (size_t)script_ints * 4);
+  *ctx->progress = 0ull;
+  cs_launch_host_in(ctx->step_in_dev, B, tokens, script_ints, stride, hist_dev, hist_len_dev, ctx->loop_emitted, st);
   // ---- App. B.3 step 1 (search, gather), step 2 (verify, accept, truncate).  Enqueued launch by launch:
   // the device starts on the first kernel while the rest is enqueued (0.45 ms of host time beside 3.4 ms
   // on the device at the 8B shape; a graph replay took 0.16 ms before the first kernel began).
   ctx->stamp_n = 0;
   cs_status s = cs_launch_find_match(hist_dev, hist_len_dev, B, stride, gamma, k, (int)policy, ctx->loop_mpos,
                                      ctx->loop_draft, ctx->loop_dlen, ctx->loop_last, nullptr, st);
-  if (s != CS_OK) return fail(ctx, s, "match kernel launch failed");
+  if (s != CS_OK) {
+    (void)cudaStreamSynchronize(st);                   // (the input kernel reads the pinned words)
+    return fail(ctx, s, "match kernel launch failed");
+  }
   cs_launch_block_setup(ctx, ctx->loop_last, ctx->loop_draft, ctx->loop_dlen, kv_len, nullptr, B, k, false, st);
-  // the search opens the step stream-ordered and every call ends synchronised, so the cached
-  // rows and kv_len are settled while the forward runs
+  // every call ends when its last kernel has reported, and k_block_setup lets nothing pass that was enqueued
+  // earlier, so the cached rows and kv_len are settled while the forward runs
   ctx->kv_len_early = kv_len;
   s = enqueue_forward(ctx, B, k + 1, kv_cache, true, nullptr, st);
   ctx->kv_len_early = nullptr;
-  if (s != CS_OK) return s;
+  if (s != CS_OK) {
+    (void)cudaStreamSynchronize(st);
+    return s;
+  }
   cs_launch_accept(ctx, B, k, ctx->loop_draft, ctx->loop_dlen, script_dev, k + 1, nullptr, k + 1, ctx->loop_accept,
                    ctx->loop_out, ctx->loop_argmax, kv_len, 1, st);
   // ---- device -> host, then step 4 on the host: append what was emitted
-  CS_CUDA_OK(ctx, cudaMemcpyAsync(accept_len_host, ctx->loop_accept, (size_t)B * 4, cudaMemcpyDeviceToHost, st));
-  CS_CUDA_OK(ctx, cudaMemcpyAsync(out_tokens_host, ctx->loop_out, (size_t)B * (k + 1) * 4, cudaMemcpyDeviceToHost, st));
-  CS_CUDA_OK(ctx, cudaStreamSynchronize(st));
+  cs_launch_host_out(ctx->loop_accept, ctx->loop_out, B, k, ctx->step_out_dev, ctx->progress_dev, st);
+  CS_CUDA_OK(ctx, cudaGetLastError());
+  int done;
+  s = wait_progress(ctx, 0, &done, st);
+  if (s != CS_OK) return s;
+  memcpy(accept_len_host, ctx->step_out, (size_t)B * 4);
+  memcpy(out_tokens_host, ctx->step_out + CS_MAX_ROWS, (size_t)B * (k + 1) * 4);
   for (int b = 0; b < B; ++b) {
     const int tau = accept_len_host[b];
     if (tau < 0 || tau > k) continue;                  // the device skipped this sequence (status word)

@@ -162,6 +162,7 @@ struct cs_ctx {
   // sequence still has to emit; and the device's address of it.
   unsigned long long *progress, *progress_dev;
   int* host_ints;            // pinned host scratch behind it [CS_MAX_ROWS + 1]
+  int *step_in, *step_in_dev, *step_out, *step_out_dev;   // and cs_step_host's inputs [CS_STEP_IN_MAX] and results [2 * CS_MAX_ROWS]
   unsigned long long* stamp_buf;   // device, caller-owned; NULL = no stamps
   int stamp_cap, stamp_n;          // slots available / handed out for the step being enqueued
   unsigned char stamp_fam[CS_STAMP_MAX];
@@ -332,6 +333,13 @@ void cs_launch_prefill_finish(cs_ctx* ctx, const int32_t* hist_len, int32_t* kv_
                               cudaStream_t st);
 void cs_launch_loop_init(cs_ctx* ctx, const int32_t* hist_len, const int32_t* kv_len, int B,
                          int stride, int max_new, int k, cudaStream_t st);
+// cs_step_host: inputs from, and results to, pinned host memory.  `in` holds per sequence the history length, the
+// first token to copy and where its tokens begin, then the tokens, then the script rows.
+constexpr int CS_STEP_IN_MAX = 5 * CS_MAX_ROWS;
+void cs_launch_host_in(const int* in, int B, int tokens, int script_ints, int stride, int32_t* hist, int32_t* hist_len,
+                       int32_t* script, cudaStream_t st);
+void cs_launch_host_out(const int32_t* accept_len, const int32_t* out_tokens, int B, int k, int* out,
+                        unsigned long long* progress, cudaStream_t st);
 // `progress` (device address of a pinned host word, or NULL) gets (step + 1) << 32 | tokens still wanted
 void cs_launch_loop_commit(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, int stride,
                            int32_t* kv_len, int k, int max_new, int eos_id, int scripted,

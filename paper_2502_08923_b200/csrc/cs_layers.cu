@@ -474,6 +474,41 @@ k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, i
   }
 }
 
+// The two ends of a step that a client drives from host memory.  Its few words travel in one kernel each way
+// instead of three copies in and two out, and the host waits for a word that the last kernel writes instead of
+// for the stream: every copy hands the stream from the SMs to a copy engine and back.  HOSTFIG
+__global__ void __launch_bounds__(CS_MAX_ROWS)
+k_host_in(const int* in, int B, int tokens, int script_ints, int stride, int* hist, int* hist_len, int* script) {
+  __shared__ int s_in[CS_STEP_IN_MAX];
+  const int n = 3 * B + tokens + script_ints, tid = threadIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int v[CS_STEP_IN_MAX / CS_MAX_ROWS];                 // (one trip over the bus, and ahead of the wait)
+#pragma unroll
+  for (int q = 0; q < CS_STEP_IN_MAX / CS_MAX_ROWS; ++q)
+    v[q] = q * CS_MAX_ROWS + tid < n ? *reinterpret_cast<const volatile int*>(in + q * CS_MAX_ROWS + tid) : 0;
+#pragma unroll
+  for (int q = 0; q < CS_STEP_IN_MAX / CS_MAX_ROWS; ++q) s_in[q * CS_MAX_ROWS + tid] = v[q];
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid < B) {
+    const int len = s_in[tid], from = s_in[B + tid], at = 3 * B + s_in[2 * B + tid];
+    for (int i = from; i < len; ++i) hist[(size_t)tid * stride + i] = s_in[at + i - from];
+    hist_len[tid] = len;
+  }
+  if (tid < script_ints) script[tid] = s_in[3 * B + tokens + tid];
+}
+
+__global__ void __launch_bounds__(CS_MAX_ROWS)
+k_host_out(const int* accept_len, const int* out_tokens, int B, int n_out, int* out, unsigned long long* progress) {
+  CS_PDL_PROLOGUE();
+  const int tid = threadIdx.x;
+  if (tid < B) out[tid] = __ldcg(accept_len + tid);
+  if (tid < n_out) out[CS_MAX_ROWS + tid] = __ldcg(out_tokens + tid);
+  __threadfence_system();
+  __syncthreads();
+  if (tid == 0) *reinterpret_cast<volatile unsigned long long*>(progress) = 1ull << 32;
+}
+
 }  // namespace
 
 // one angle per thread up to a quarter of the chip
@@ -536,6 +571,16 @@ void cs_launch_truncate(cs_ctx* ctx, int32_t* kv_len, const int32_t* new_len, in
 void cs_launch_append(int32_t* hist, int32_t* hist_len, int n, const int32_t* tokens, int count, int32_t* kv_len,
                       int32_t* kv_len_2, int new_len_2, cudaStream_t st) {
   cs_launch_pdl(k_append, dim3(1), dim3(CS_MAX_ROWS), 0, st, hist, hist_len, n, tokens, count, kv_len, kv_len_2, new_len_2);
+}
+
+void cs_launch_host_in(const int* in, int B, int tokens, int script_ints, int stride, int32_t* hist, int32_t* hist_len,
+                       int32_t* script, cudaStream_t st) {
+  cs_launch_pdl(k_host_in, dim3(1), dim3(CS_MAX_ROWS), 0, st, in, B, tokens, script_ints, stride, hist, hist_len, script);
+}
+
+void cs_launch_host_out(const int32_t* accept_len, const int32_t* out_tokens, int B, int k, int* out,
+                        unsigned long long* progress, cudaStream_t st) {
+  cs_launch_pdl(k_host_out, dim3(1), dim3(CS_MAX_ROWS), 0, st, accept_len, out_tokens, B, B * (k + 1), out, progress);
 }
 
 void cs_launch_prefill_finish(cs_ctx* ctx, const int32_t* hist_len, int32_t* kv_len, int B, cudaStream_t st) {
