@@ -53,7 +53,7 @@
  * when they are stored in the cache.
  *
  * Environment, read once by cs_create (measurement and test switches; not needed in use):
- *   CS_NO_GRAPH=1          cs_loop_steps enqueues its steps kernel by kernel, as the other calls
+ *   CS_NO_GRAPH=1          cs_loop_steps and cs_decode_loop enqueue their steps kernel by kernel, as the other calls
  *                          do, instead of replaying them from a captured CUDA graph;
  *   CS_ATTN_KERNEL=tc|tcw|mma  forces one attention kernel: tcgen05 with the query rows as the
  *                          M dimension (tc), tcgen05 with the keys and head dims as M (tcw), or

@@ -158,6 +158,9 @@ struct cs_ctx {
 
   LoopState loop;
   HostStep host_step;
+  // the graph of the last cs_decode_loop, destroyed when the next one is built
+  cudaGraph_t old_graph;
+  cudaGraphExec_t old_exec;
   // Pinned host word that cs_decode_loop's steps report to: (steps done << 32) | most tokens any
   // sequence still has to emit; and the device's address of it.
   unsigned long long *progress, *progress_dev;
@@ -340,7 +343,7 @@ void cs_launch_host_in(const int* in, int B, int tokens, int script_ints, int st
                        int32_t* script, cudaStream_t st);
 void cs_launch_host_out(const int32_t* accept_len, const int32_t* out_tokens, int B, int k, int* out,
                         unsigned long long* progress, cudaStream_t st);
-// `progress` (device address of a pinned host word, or NULL) gets (step + 1) << 32 | tokens still wanted
+// `progress` (device address of a pinned host word, or NULL) gets steps done << 32 | tokens still wanted
 void cs_launch_loop_commit(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, int stride,
                            int32_t* kv_len, int k, int max_new, int eos_id, int scripted,
-                           unsigned long long* progress, int step, cudaStream_t st);
+                           unsigned long long* progress, cudaStream_t st);

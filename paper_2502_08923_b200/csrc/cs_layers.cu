@@ -411,7 +411,7 @@ __global__ void k_loop_init(const int* hist_len, const int* kv_len, int B, int s
     if (d) atomicAdd(&s_done, 1);
   }
   __syncthreads();
-  if (t == 0) done[max_batch] = s_done;
+  if (t == 0) { done[max_batch] = s_done; done[max_batch + 1] = 0; }
 }
 
 // Append the step's tokens to the history (App. B.3 step 4), clip at max_new, stop at
@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(CS_MAX_ROWS)
 k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, int max_new,
               int eos_id, int scripted, const int* accept, const int* out, const int* mpos,
               int* emitted, int* done, int max_batch, unsigned long long* stats,
-              const int* status, unsigned long long* progress, int step, unsigned long long* stamp) {
+              const int* status, unsigned long long* progress, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
   const int b = threadIdx.x;
   if (b == 0) cs_stamp_end(stamp);   // (the kernel is a few dozen instructions: its start stands for its end)
@@ -468,8 +468,9 @@ k_loop_commit(int* hist, int* hist_len, int B, int stride, int* kv_len, int k, i
     if (wanted > 0) atomicMax(&s_wanted, wanted);
     __syncthreads();
     if (b == 0) {
+      const int step = ++done[max_batch + 1];            // steps of this loop
       const unsigned rest = (*status & CS_DEV_TIMEOUT) ? 0u : (unsigned)s_wanted;   // (a wait that ran out ends the loop)
-      *reinterpret_cast<volatile unsigned long long*>(progress) = ((unsigned long long)(unsigned)(step + 1) << 32) | rest;
+      *reinterpret_cast<volatile unsigned long long*>(progress) = ((unsigned long long)(unsigned)step << 32) | rest;
     }
   }
 }
@@ -595,10 +596,10 @@ void cs_launch_loop_init(cs_ctx* ctx, const int32_t* hist_len, const int32_t* kv
 }
 
 void cs_launch_loop_commit(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, int stride, int32_t* kv_len,
-                           int k, int max_new, int eos_id, int scripted, unsigned long long* progress, int step,
+                           int k, int max_new, int eos_id, int scripted, unsigned long long* progress,
                            cudaStream_t st) {
   cs_launch_pdl(k_loop_commit, dim3(1), dim3(cs_ceil_div(B, 32) * 32), 0, st, hist, hist_len, B, stride, kv_len, k,
                 max_new, eos_id, scripted, ctx->loop_accept, ctx->loop_out, ctx->loop_mpos, ctx->loop_emitted,
-                ctx->loop_done, ctx->cfg.max_batch, ctx->loop_stats, ctx->d_status, progress, step,
+                ctx->loop_done, ctx->cfg.max_batch, ctx->loop_stats, ctx->d_status, progress,
                 cs_next_stamp(ctx, CS_FAM_OTHER));
 }
