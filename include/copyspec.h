@@ -380,6 +380,13 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
  * non-clustered launches (a GEMM small enough to run without split-K).  k_block < 0 clears it. */
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block);
 
+/* Test hook for the hand-over of work between SM pairs (no counterpart in the paper): where the K
+ * ranges of a projection above 32 rows are split between pairs, the pairs whose K range is in the
+ * bit mask `mask` (0 <= mask < 256) leave their share of the tokens to the others, as pairs do that
+ * finish before all of their tile have started, and the others wait.  The last K range is never left
+ * out, so every share is finished; results are the same bit for bit.  Stays set until changed; 0 clears it. */
+cs_status cs_debug_leave_shares(cs_ctx* ctx, int mask);
+
 /* The LM-head stage of the verification forward on its own (Sec. 3.2; App. B.2: greedy
  * token at temperature 0): ids[r] = the lowest token id with the largest logit of
  * X[r] . lm_head^T, for rows already normalised and rounded to bf16.  X bf16 [rows][d_model],

@@ -600,6 +600,12 @@ cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block) {
   return CS_OK;
 }
 
+cs_status cs_debug_leave_shares(cs_ctx* ctx, int mask) {
+  if (ctx == nullptr || mask < 0 || mask >= 1 << CS_PAIR_MAX_SPLITS) return CS_ERR_ARG;
+  ctx->debug_leave = mask;
+  return CS_OK;
+}
+
 cs_status cs_kv_truncate(cs_ctx* ctx, int32_t* kv_len, const int32_t* new_len, int B, void* stream) {
   if (ctx == nullptr) return CS_ERR_ARG;
   if (B < 0 || kv_len == nullptr || new_len == nullptr) return fail(ctx, CS_ERR_ARG, "bad argument");

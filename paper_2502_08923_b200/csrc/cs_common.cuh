@@ -152,6 +152,7 @@ struct cs_ctx {
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
+  int debug_leave;           // test hook: K ranges whose SM pairs leave their shares to others (0 = none)
 
   void* match_index;         // cs_set_match_index: the loop searches through this gamma-gram index (NULL = scan)
   int match_index_cap;

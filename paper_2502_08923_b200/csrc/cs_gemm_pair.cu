@@ -67,6 +67,7 @@ struct PairArgs {
   int tile_stride;
   float* part;                // sums handed to other pairs, [pair][half][256 tokens][128 features]
   int* part_flag;             // stream form: "written", [pair][half]; split form: who is where, [tile][half]; 0 between launches
+  int leave;                  // test hook, split form: K ranges whose pairs leave their shares to others (bit mask; 0 = as they come)
   int* status;
   unsigned long long wait_ns;
   unsigned long long* stamp;
@@ -521,6 +522,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         if (S > 1) {
           __threadfence();
           all_started = all_started || started(word) == S;
+          if (a.leave != 0) all_started = !(a.leave >> split & 1);
           atomicAdd(word, all_started ? 1 : 1 + (1 << (8 + split)));
           mine = 0;
           if (all_started) {
@@ -552,7 +554,9 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         return y;
       };
       const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int r = 0; r < S; ++r) {
+      // The own share first: x_pre holds its residual rows, and other shares load theirs over them
+      for (int turn = 0; turn < S; ++turn) {
+        const int r = split + turn < S ? split + turn : split + turn - S;
         if (!(shares >> r & 1)) continue;
         const int lo = r * share, hi = min(a.rows, lo + share);
         if (a.mode == CS_EPI_QKV) {
@@ -778,6 +782,7 @@ cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap*
     lc.gridDim = dim3(2 * pairs, 1, 1);
   } else {
     pair_splits(ctx, g, rows, lo_row >= 0, &a.splits, &a.kb_per_split);
+    a.leave = ctx->debug_leave & ((1 << (a.splits - 1)) - 1);   // (the last K range's pair always waits for the others)
     lc.gridDim = dim3(2 * tiles2 * a.splits, 1, 1);
   }
   lc.blockDim = dim3(pair_threads(groups), 1, 1);
