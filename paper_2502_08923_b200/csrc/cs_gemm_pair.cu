@@ -58,6 +58,7 @@ struct PairArgs {
   int stages, terms, stacked, mode;
   int lo_row;                 // row coordinate of the activations' second term
   float* out;
+  bool vec_out;               // four values of a row of `out` lie on a 16-byte boundary (the caller's logits may start anywhere)
   __nv_bfloat16 *act, *act_lo;
   int F;
   QkvEpi q;
@@ -197,7 +198,7 @@ __device__ __forceinline__ void finish_argmax(const PairArgs& a, const float* pa
       if (n0 + f + e < a.N && v[e] > best) { best = v[e]; idx = n0 + f + e; }
     if (a.out != nullptr && tok < a.rows) {
       float* dst = a.out + (size_t)tok * a.N + n0 + f;
-      if ((a.N & 3) == 0 && n0 + f < a.N) {
+      if (a.vec_out && n0 + f < a.N) {
         *reinterpret_cast<float4*>(dst) = y;
       } else {
 #pragma unroll
@@ -758,7 +759,9 @@ cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap*
   a.stacked = (a.terms == 2 && a.n_tok <= 128) ? 1 : 0;
   a.lo_row = lo_row;
   a.mode = mode;
-  a.out = out; a.act = act; a.act_lo = act_lo; a.F = F;
+  a.out = out;
+  a.vec_out = (g->N & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  a.act = act; a.act_lo = act_lo; a.F = F;
   if (q != nullptr) a.q = *q;
   if (nf != nullptr) a.nf = *nf;
   a.tile_max = ctx->tile_max; a.tile_idx = ctx->tile_idx; a.tile_stride = cs_ceil_div(g->N, CS_GEMM_BM);
