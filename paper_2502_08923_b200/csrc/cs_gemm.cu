@@ -56,6 +56,7 @@ struct GemmArgs {
   int rows, n_tok, N, K;
   int num_kb, kb_per_split, splits, stages, mode;
   float* out;            // STORE / RESIDUAL: [rows][N] fp32; ARGMAX: optional logits [rows][N]
+  bool vec_out;          // four values of a row of `out` lie on a 16-byte boundary (a caller's buffer may start anywhere)
   int lo_row;            // row coordinate of the activation operand's second bf16 term, -1 = none
   QkvEpi q;              // QKV: where the rotated queries and the new K/V rows go
   NormFuse nf;           // RMSNorm folded into this GEMM's read-out (consumer) or residual update (producer)
@@ -258,7 +259,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
   } else {
     // ------------------------------------------------------------- epilogue warps 0-3: wait for the accumulators
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (a.mode == CS_EPI_RESIDUAL && (a.N & 3) == 0 && e < r_per_tok * a.rows) {
+    if (a.mode == CS_EPI_RESIDUAL && a.vec_out && e < r_per_tok * a.rows) {
       const int f = r_flo + 4 * (e % r_per_tok), tok = e / r_per_tok;
       if (n0 + f + 3 < a.N) {
         pre_a = *reinterpret_cast<const float4*>(a.out + (size_t)tok * a.N + n0 + f);
@@ -440,13 +441,12 @@ k_gemm_tc(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUten
         const int f_lo = r_flo, per_tok = r_per_tok;
         float* part = dump + a.n_tok * CS_GEMM_BM;   // [rows][32] sums of squares, behind the parked tile
         const int total = per_tok * a.rows, iters = (total + 127) >> 7;
-        const bool vec_n = (a.N & 3) == 0;
         for (int it = 0; it < iters; ++it) {
           const int idx = e + (it << 7);
           const bool act = idx < total;
           const int idc = act ? idx : 0;
           const int f = f_lo + 4 * (idc % per_tok), tok = idc / per_tok;
-          const bool vec = vec_n && n0 + f + 3 < a.N;
+          const bool vec = a.vec_out && n0 + f + 3 < a.N;
           float4 y = make_float4(0.f, 0.f, 0.f, 0.f), x = y;
           if (act) {
             if (a.splits > 1) y = sum_over_ranks(dump_addr + 4u * (uint32_t)(tok * CS_GEMM_BM + f), a.splits);
@@ -637,6 +637,7 @@ cs_status cs_launch_gemm(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX,
   a.kb_per_split = g->kb_per_split;
   a.mode = mode;
   a.out = out;
+  a.vec_out = (g->N & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   a.lo_row = lo_row;
   if (q != nullptr) a.q = *q;
   a.nf = NormFuse{};
@@ -793,6 +794,7 @@ extern "C" cs_status cs_lm_head_static(const void* X, const void* W, int rows, i
   a.splits = 1;
   a.mode = CS_EPI_ARGMAX;
   a.out = nullptr;
+  a.vec_out = false;
   a.lo_row = -1;
   a.nf = NormFuse{};
   a.tile_max = tile_max;

@@ -58,7 +58,7 @@ struct PairArgs {
   int stages, terms, stacked, mode;
   int lo_row;                 // row coordinate of the activations' second term
   float* out;
-  bool vec_out;               // four values of a row of `out` lie on a 16-byte boundary (the caller's logits may start anywhere)
+  bool vec_out;               // four values of a row of `out` lie on a 16-byte boundary (a caller's buffer may start anywhere)
   __nv_bfloat16 *act, *act_lo;
   int F;
   QkvEpi q;
@@ -484,7 +484,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       const int share = (a.rows + S - 1) / S;                    // tokens a pair finishes
       const int f = 4 * lane;                                    // STORE, RESIDUAL: a warp per token, four features per lane
       const bool resid = a.mode == CS_EPI_RESIDUAL, feeds = a.nf.gain_out != nullptr;
-      const bool vec = (a.N & 3) == 0 && n0 + f + 3 < a.N;
+      const bool vec = a.vec_out && n0 + f + 3 < a.N;
       // the residual rows and the next norm's gain are asked for while the MMAs still run
       float4 x_pre[kBatch];
       uint2 gain = make_uint2(0u, 0u);

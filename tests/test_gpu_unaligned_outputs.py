@@ -44,3 +44,18 @@ def test_logits_anywhere(vocab, B, k):
     for pair in got[1:]:
         assert torch.equal(pair[0], got[0][0]) and torch.equal(pair[1], got[0][1])
     ctx.close()
+
+
+@pytest.mark.parametrize("N", [264, 265])
+@pytest.mark.parametrize("rows", [5, 32, 33, 200])     # one-SM tiles up to 32 rows, SM pairs above
+def test_linear_output_anywhere(N, rows):
+    cfg = inputs.ModelConfig(n_layers=1, d_model=256, n_heads=2, n_kv_heads=2, head_dim=128, d_ffn=512, vocab=512)
+    ctx, _ = make_pair(cfg, 64, 1, 10)
+    X = torch.randn((rows + 15) // 16 * 16, 2048, device="cuda").to(torch.bfloat16)
+    W = torch.randn(N, 2048, device="cuda").to(torch.bfloat16)
+    want = ctx.cs_linear(X, W, rows=rows)
+    for off in (1, 2, 3):
+        buf, Y = _view(off, rows, N)
+        ctx._check(ctx.lib.cs_linear(ctx.handle, X.data_ptr(), W.data_ptr(), rows, N, 2048, Y.data_ptr(), torch.cuda.current_stream().cuda_stream), "cs_linear")
+        assert ctx.cs_sync_status() == 0 and torch.equal(Y, want) and _intact(buf, off, rows * N)
+    ctx.close()
