@@ -731,15 +731,15 @@ cs_status static_scratch(void** out) {
 
 // greedy token per row from the per-tile pairs; -2 marks a row whose GEMM gave up on a wait
 __global__ void __launch_bounds__(128)
-k_tile_reduce_static(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, int tiles,
-                     int tile_stride, const int* __restrict__ status, int* __restrict__ ids) {
+k_tile_reduce_static(const float* tile_max, const int* tile_idx, int tiles,
+                     int tile_stride, const int* status, int* __restrict__ ids) {
   CS_PDL_PROLOGUE();
   const int row = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float val = -INFINITY;
   int idx = INT32_MAX;
   for (int t = threadIdx.x; t < tiles; t += 128) {
-    const float v = tile_max[(size_t)row * tile_stride + t];
-    const int id = tile_idx[(size_t)row * tile_stride + t];
+    const float v = __ldcg(tile_max + (size_t)row * tile_stride + t);
+    const int id = __ldcg(tile_idx + (size_t)row * tile_stride + t);
     if (v > val || (v == val && id < idx)) { val = v; idx = id; }
   }
   __shared__ float sv[4];
@@ -754,7 +754,7 @@ k_tile_reduce_static(const float* __restrict__ tile_max, const int* __restrict__
   if (threadIdx.x == 0) {
     for (int w = 1; w < 4; ++w)
       if (sv[w] > val || (sv[w] == val && si[w] < idx)) { val = sv[w]; idx = si[w]; }
-    ids[row] = (*status != 0) ? -2 : ((idx == INT32_MAX) ? -1 : idx);
+    ids[row] = (__ldcg(status) != 0) ? -2 : ((idx == INT32_MAX) ? -1 : idx);
   }
 }
 

@@ -20,11 +20,13 @@ namespace {
 // 17.8 -> 3.4 us at 168 rows, 22.0 -> 2.6 at 256).  Dependents are let go behind the wait and not ahead of it: the search in front of this
 // kernel is launched early itself, and kernels further down the chain read cached rows and lengths
 // ahead of their own waits, relying on the step before being complete.
+// Words that other kernels of the chain write (the search's results, lengths, rows, tile maxima) are read through L2, here
+// and in every kernel of the library that starts early: it may be resident while they still change, and the read-only
+// path, which a const __restrict__ pointer allows the compiler, is not coherent across that.
 constexpr int kSetupThreads = 256;
 __global__ void __launch_bounds__(kSetupThreads)
-k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
-                              const int* __restrict__ draft_len, const int* __restrict__ kv_len,
-                              const int* __restrict__ skip, int B, int k, int max_seq, int vocab,
+k_block_setup(const int* last_tok, const int* draft, const int* draft_len, const int* kv_len,
+                              const int* skip, int B, int k, int max_seq, int vocab,
                               int half, const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                               int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status,
                               unsigned long long* stamp) {
@@ -33,10 +35,10 @@ k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
   const int R = k + 1, rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
-    int dl = draft_len[b];
+    int dl = __ldcg(draft_len + b);
     dl = dl < 0 ? 0 : (dl > k ? k : dl);
-    const int kv = kv_len[b];
-    const bool skipped = (skip != nullptr && skip[b] != 0);
+    const int kv = __ldcg(kv_len + b);
+    const bool skipped = (skip != nullptr && __ldcg(skip + b) != 0);
     const bool fits = (kv >= 0 && kv + dl + 1 <= max_seq);
     const bool ok = fits && !skipped;
     if (r == 0) {
@@ -44,7 +46,7 @@ k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
       if (!fits && !skipped) atomicOr(status, CS_DEV_CAPACITY);
     }
     const bool valid = ok && r <= dl;
-    int tok = (r == 0 || !valid) ? last_tok[b] : draft[(size_t)b * k + r - 1];
+    int tok = __ldcg((r == 0 || !valid) ? last_tok + b : draft + (size_t)b * k + r - 1);
     tok = tok < 0 ? 0 : (tok >= vocab ? vocab - 1 : tok);
     row_tok[row] = tok;
     row_pos[row] = (kv < 0 ? 0 : kv) + r;
@@ -54,7 +56,7 @@ k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
   for (int i = blockIdx.x * kSetupThreads + threadIdx.x; i < rows * half; i += gridDim.x * kSetupThreads) {
     const int row = i / half, j = i % half;
     const int b = row / R, r = row % R;
-    const int kv = kv_len[b];
+    const int kv = __ldcg(kv_len + b);
     const double ang = (double)((kv < 0 ? 0 : kv) + r) * inv_freq[j];
     double s, c;
     sincos(ang, &s, &c);
@@ -70,7 +72,7 @@ k_block_setup(const int* __restrict__ last_tok, const int* __restrict__ draft,
 // Forced rows for filling the cache from a history: row r of sequence b is token
 // hist[b][start + r]; only positions below hist_len[b] - 1 are computed.
 __global__ void __launch_bounds__(kSetupThreads)
-k_prefill_setup(const int* __restrict__ hist, const int* __restrict__ hist_len, int B,
+k_prefill_setup(const int* hist, const int* hist_len, int B,
                                 int stride, int start, int R, int max_seq, int vocab, int half,
                                 const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                                 int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status) {
@@ -79,14 +81,14 @@ k_prefill_setup(const int* __restrict__ hist, const int* __restrict__ hist_len, 
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
     const int p = start + r;
-    const int n = hist_len[b];
+    const int n = __ldcg(hist_len + b);
     const bool fits = (n - 1 <= max_seq && n <= stride);
     if (r == 0) {
       seq_ok[b] = fits ? 1 : 0;
       if (!fits) atomicOr(status, CS_DEV_CAPACITY);
     }
     const bool valid = fits && p < n - 1;
-    int tok = valid ? hist[(size_t)b * stride + p] : 0;
+    int tok = valid ? __ldcg(hist + (size_t)b * stride + p) : 0;
     tok = tok < 0 ? 0 : (tok >= vocab ? vocab - 1 : tok);
     row_tok[row] = tok;
     row_pos[row] = p;
@@ -109,12 +111,12 @@ k_prefill_setup(const int* __restrict__ hist, const int* __restrict__ hist_len, 
 // into the GEMMs around it.
 constexpr int kNormThreads = 1024;
 __global__ void __launch_bounds__(kNormThreads)
-k_embed_rmsnorm(const __nv_bfloat16* __restrict__ E, const int* __restrict__ row_tok, float* __restrict__ x, int d,
+k_embed_rmsnorm(const __nv_bfloat16* __restrict__ E, const int* row_tok, float* __restrict__ x, int d,
                 const __nv_bfloat16* __restrict__ gain, float eps, __nv_bfloat16* __restrict__ xn,
                 __nv_bfloat16* __restrict__ xn_lo, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
   const int row = blockIdx.x;
-  const __nv_bfloat16* er = E + (size_t)row_tok[row] * d;
+  const __nv_bfloat16* er = E + (size_t)__ldcg(row_tok + row) * d;
   float* xr = x + (size_t)row * d;
   auto fetch = [&](int i) {
     const uint2 w = *reinterpret_cast<const uint2*>(er + i);          // four bf16
@@ -251,10 +253,9 @@ k_attn_merge(const float* __restrict__ in_o, const float* __restrict__ in_ml, in
 // vocabulary of 128,256: 11 rows 12.4 -> 6.9, 16 x 11 rows 17.4 -> 8.4, 8 x 21 rows 36 -> 11.5).
 constexpr int kAcceptThreads = 1024;
 __global__ void __launch_bounds__(kAcceptThreads)
-k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, int tiles, int tile_stride,
-         int k, const int* __restrict__ draft, const int* __restrict__ draft_len,
-         const int* __restrict__ seq_ok, const int* __restrict__ script, int script_stride,
-         const int* __restrict__ script_off, int script_limit, int* __restrict__ accept_len,
+k_accept(const float* tile_max, const int* tile_idx, int tiles, int tile_stride,
+         int k, const int* draft, const int* draft_len, const int* seq_ok, const int* script, int script_stride,
+         const int* script_off, int script_limit, int* __restrict__ accept_len,
          int* __restrict__ out_tokens, int* __restrict__ argmax_ids, int* __restrict__ kv_len,
          int update_kv, unsigned long long* stamp) {
   CS_PDL_PROLOGUE();
@@ -263,9 +264,9 @@ k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, i
   const int warp = tid >> 5, lane = tid & 31;
   __shared__ unsigned long long s_key[CS_MAX_ROWS];   // (largest logit, lowest id) as one ordered number; 0 = none
   __shared__ int s_tau;
-  int dl = draft_len[b];
+  int dl = __ldcg(draft_len + b);
   dl = dl < 0 ? 0 : (dl > k ? k : dl);
-  const bool ok = seq_ok[b] != 0;
+  const bool ok = __ldcg(seq_ok + b) != 0;
   if (tid < R) s_key[tid] = 0ull;
   if (tid == 0) s_tau = dl;
   __syncthreads();
@@ -312,10 +313,10 @@ k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, i
     if (tid < live) {
       tgt = arg;
       if (script != nullptr) {
-        const int at = (script_off != nullptr ? script_off[b] : 0) + tid;
-        tgt = at < script_limit ? script[(size_t)b * script_stride + at] : -1;
+        const int at = (script_off != nullptr ? __ldcg(script_off + b) : 0) + tid;
+        tgt = at < script_limit ? __ldcg(script + (size_t)b * script_stride + at) : -1;
       }
-      if (tid < dl && draft[(size_t)b * k + tid] != tgt) atomicMin(&s_tau, tid);
+      if (tid < dl && __ldcg(draft + (size_t)b * k + tid) != tgt) atomicMin(&s_tau, tid);
     }
   }
   __syncthreads();
@@ -333,15 +334,15 @@ k_accept(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, i
 
 // Greedy token of each row from the LM head's per-tile (max, id) pairs (lowest id on ties).
 __global__ void __launch_bounds__(128)
-k_tile_reduce(const float* __restrict__ tile_max, const int* __restrict__ tile_idx, int tiles, int tile_stride,
+k_tile_reduce(const float* tile_max, const int* tile_idx, int tiles, int tile_stride,
               int* __restrict__ ids) {
   CS_PDL_PROLOGUE();
   const int row = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float val = -INFINITY;
   int idx = INT32_MAX;
   for (int t = threadIdx.x; t < tiles; t += 128) {
-    const float v = tile_max[(size_t)row * tile_stride + t];
-    const int id = tile_idx[(size_t)row * tile_stride + t];
+    const float v = __ldcg(tile_max + (size_t)row * tile_stride + t);
+    const int id = __ldcg(tile_idx + (size_t)row * tile_stride + t);
     if (v > val || (v == val && id < idx)) { val = v; idx = id; }
   }
   __shared__ float sv[4];
