@@ -536,7 +536,6 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
         *s_shares = mine;
       }
       epi_barrier<kEpiThreads>();
-      const int shares = *s_shares;
       const float* sums = a.part + (size_t)(2 * t_lo * S + half) * CS_GEMM_BM * CS_MAX_ROWS;
       // four features of one token from four pairs (requests only; S is rarely above 4), and their sum in
       // the order of the K ranges
@@ -556,9 +555,7 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       };
       const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
       // The own share first: x_pre holds its residual rows, and other shares load theirs over them
-      for (int turn = 0; turn < S; ++turn) {
-        const int r = split + turn < S ? split + turn : split + turn - S;
-        if (!(shares >> r & 1)) continue;
+      for (int todo = *s_shares, r = split; todo != 0; todo &= ~(1 << r), r = __ffs(todo) - 1) {
         const int lo = r * share, hi = min(a.rows, lo + share);
         if (a.mode == CS_EPI_QKV) {
           // RoPE pairs feature i of a head with i + Dh/2: both lie in this tile; j in [0, 64) walks the first
