@@ -376,8 +376,10 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
  * launch of this context leaves out the loads of 64-wide K block `k_block` of every CTA, so the
  * consumer's wait for that block runs out after the context's wait limit (CS_WAIT_LIMIT_US),
  * the CTA drains its other copies, frees its tensor memory and returns, and cs_sync_status
- * reports CS_ERR_TIMEOUT.  Nothing faults and the context stays usable.  Meant for
- * non-clustered launches (a GEMM small enough to run without split-K).  k_block < 0 clears it. */
+ * reports CS_ERR_TIMEOUT.  Nothing faults and the context stays usable.  The streamed projections
+ * (gate/up and LM head) leave the block out on every second pair of SMs, so that the others wait for
+ * sums that never come.  Launches of at most 32 rows that split K over a cluster refuse the hook
+ * (CS_ERR_UNSUPPORTED; the cluster barrier has no time limit).  k_block < 0 clears it. */
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block);
 
 /* Test hook for the hand-over of work between SM pairs (no counterpart in the paper): where the K

@@ -68,6 +68,7 @@ struct PairArgs {
   int tile_stride;
   float* part;                // sums handed to other pairs, [pair][half][256 tokens][128 features]
   int* part_flag;             // stream form: "written", [pair][half]; split form: who is where, [tile][half]; 0 between launches
+  int drop_kb;                // test hook: K block of a run whose loads are left out, by every pair (split form) or every second one (stream form); -1 = none
   int leave;                  // test hook, split form: K ranges whose pairs leave their shares to others (bit mask; 0 = as they come)
   int* status;
   unsigned long long wait_ns;
@@ -121,6 +122,11 @@ __device__ __forceinline__ void cluster_sync() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the peer's abort flag; seen by whoever sees an arrival that follows
+__device__ __forceinline__ void abort_peer(uint32_t flag) {
+  asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(flag) : "memory");
+  asm volatile("fence.acq_rel.cluster;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   uint32_t r;
@@ -291,15 +297,16 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     const int xrow = a.stacked ? half * a.lo_row : half * (n_tok >> 1);
     const bool second = a.terms == 2 && !a.stacked;
     int tw = t_lo, kw = u0 - tw * a.num_kb, kx = kw;             // next weight tile and its K block; next K block of the activations
-    auto load_w = [&](int s) {
-      if (elect_one()) {
+    const int drop = STREAM && !(pair & 1) ? -1 : a.drop_kb;
+    auto load_w = [&](int i, int s) {
+      if (i != drop && elect_one()) {
         if (half == 0) mbar_expect_tx(b_full + 8 * s, 2u * (uint32_t)stage_bytes);   // both CTAs' copies of the stage
         tma_load_pair(ring + (uint32_t)(s * stage_bytes), &tmW, full_even + 8 * s, kw * CS_GEMM_BK, (2 * tw + half) * CS_GEMM_BM);
       }
       if (++kw == a.num_kb) { kw = 0; ++tw; }
     };
-    auto load_x = [&](int s) {
-      if (elect_one()) {
+    auto load_x = [&](int i, int s) {
+      if (i != drop && elect_one()) {
         const uint32_t sx = ring + (uint32_t)(s * stage_bytes) + kABytes;
         tma_load_pair(sx, &tmX, full_even + 8 * s, kx * CS_GEMM_BK, xrow);
         if (second) tma_load_pair(sx + (uint32_t)n_tok * 64u, &tmX, full_even + 8 * s, kx * CS_GEMM_BK, a.lo_row + xrow);
@@ -310,14 +317,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     bool ok = true;
     int i = 0, s = 0;
     uint32_t ph = 0;
-    for (; i < npre; ++i) load_w(i);                             // weights depend on nothing
+    for (; i < npre; ++i) load_w(i, i);                             // weights depend on nothing
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (i = 0; i < npre; ++i) load_x(i);
+    for (i = 0; i < npre; ++i) load_x(i, i);
     for (; i < n; ++i) {
       ok = mbar_wait_warp(b_empty + 8 * s, ph, s_abort, a.wait_ns);
       if (!ok) break;
-      load_w(s);
-      load_x(s);
+      load_w(i, s);
+      load_x(i, s);
       if (++s == stages) { s = 0; ph ^= 1u; }
     }
     if (!ok && lane == 0) { *s_abort = 1; atomicOr(a.status, CS_DEV_TIMEOUT); }
@@ -326,7 +333,8 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
       // copies in flight land before this CTA's shared memory goes away: the even CTA sees them on its
       // barriers, the odd one gives them a thousand times their latency
       if (half == 0) {
-        for (int j = max(0, i - stages); j < i; ++j) mbar_wait(b_full + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, 1000000ull);
+        for (int j = max(0, i - stages); j < i; ++j)
+          if (j != drop) mbar_wait(b_full + 8 * (j % stages), (uint32_t)(j / stages) & 1u, s_never, 1000000ull);
       } else {
         const unsigned long long t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 1000000ull) {}
@@ -367,12 +375,14 @@ k_gemm_pair(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
           acc_on = 1u;
           if (++s == stages) { s = 0; ph ^= 1u; }
         }
+        if (!ok && lane == 0) {                                  // (both CTAs know before the accumulator looks finished)
+          *s_abort = 1;
+          abort_peer(map_rank(smem_u32(const_cast<int*>(s_abort)), 1));
+          atomicOr(a.status, CS_DEV_TIMEOUT);
+        }
+        __syncwarp();
         if (elect_one()) umma_commit_pair(b_accf + 8 * buf, mask);
         if (!ok) {
-          if (lane == 0) {
-            *s_abort = 1;
-            atomicOr(a.status, CS_DEV_TIMEOUT);
-          }
           mbar_wait(b_accf + 8 * buf, (uint32_t)(j >> 1) & 1u, s_never, a.wait_ns);   // what was issued has retired
         }
       }
@@ -738,11 +748,6 @@ cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap*
                               __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
                               cudaStream_t st) {
   const bool stream = mode == CS_EPI_SWIGLU || mode == CS_EPI_ARGMAX;
-  if (ctx->debug_drop_kb >= 0) {
-    ctx->debug_drop_kb = -1;
-    snprintf(ctx->err, sizeof(ctx->err), "the dropped-tile test hook is for blocks of at most 32 rows");
-    return CS_ERR_UNSUPPORTED;
-  }
   if (nf != nullptr && nf->gain_out != nullptr && (mode != CS_EPI_RESIDUAL || (g->N & 3) != 0)) {
     snprintf(ctx->err, sizeof(ctx->err), "a norm can only be folded into a residual GEMM whose width is a multiple of 4");
     return CS_ERR_UNSUPPORTED;
@@ -763,6 +768,8 @@ cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap*
   if (nf != nullptr) a.nf = *nf;
   a.tile_max = ctx->tile_max; a.tile_idx = ctx->tile_idx; a.tile_stride = cs_ceil_div(g->N, CS_GEMM_BM);
   a.part = ctx->pair_part; a.part_flag = ctx->pair_flag;
+  a.drop_kb = ctx->debug_drop_kb;
+  ctx->debug_drop_kb = -1;            // the hook covers one launch
   a.status = ctx->d_status;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, mode == CS_EPI_ARGMAX ? CS_FAM_LMHEAD : CS_FAM_GEMM);
