@@ -141,7 +141,9 @@ void cs_destroy(cs_ctx* ctx);
 const char* cs_last_error(const cs_ctx* ctx);
 
 /* Waits for `stream`, then returns and clears the device status word of the context:
- * CS_OK, CS_ERR_CAPACITY, CS_ERR_ARG (cs_kv_truncate asked to grow) or CS_ERR_TIMEOUT. */
+ * CS_OK, CS_ERR_CAPACITY, CS_ERR_ARG (cs_kv_truncate asked to grow) or CS_ERR_TIMEOUT.  After
+ * CS_ERR_TIMEOUT the call in which the wait ran out has no valid results; calls that run a forward are right
+ * again from the next one on, cs_linear and cs_lm_head from the next one after this status was taken. */
 cs_status cs_sync_status(cs_ctx* ctx, void* stream);
 
 /* Suffix-match search and draft gather (Sec. 3.1; Sec. 3.2; App. B.3 step 1).  Async.

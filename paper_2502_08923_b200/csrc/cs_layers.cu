@@ -12,6 +12,13 @@
 
 namespace {
 
+// A wait that ran out may have left words raised by which the two-SM GEMM's pairs hand sums over, and the
+// next forward would take sums of the one before.  Everything enqueued earlier is complete where this is called.
+__device__ __forceinline__ void lower_pair_flags(const int* status, int* pair_flag) {
+  if (blockIdx.x == 0 && (__ldcg(status) & CS_DEV_TIMEOUT) != 0)
+    for (int i = threadIdx.x; i < 2 * CS_MAX_PAIRS; i += blockDim.x) pair_flag[i] = 0;
+}
+
 // ----------------------------------------------------------------- block assembly
 // Rows of sequence b: r = 0 is the last accepted token, r = 1..draft_len[b] the draft
 // (Sec. 3.2: the speculative tokens are appended to the context).  Rows past the draft
@@ -29,9 +36,10 @@ k_block_setup(const int* last_tok, const int* draft, const int* draft_len, const
                               const int* skip, int B, int k, int max_seq, int vocab,
                               int half, const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                               int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status,
-                              unsigned long long* stamp) {
+                              int* pair_flag, unsigned long long* stamp) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  lower_pair_flags(status, pair_flag);
   const int R = k + 1, rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
@@ -75,8 +83,9 @@ __global__ void __launch_bounds__(kSetupThreads)
 k_prefill_setup(const int* hist, const int* hist_len, int B,
                                 int stride, int start, int R, int max_seq, int vocab, int half,
                                 const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
-                                int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status) {
+                                int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status, int* pair_flag) {
   CS_PDL_PROLOGUE();
+  lower_pair_flags(status, pair_flag);
   const int rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
     const int b = row / R, r = row % R;
@@ -525,7 +534,7 @@ void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* 
   // that kernels further down the chain may rely on everything enqueued earlier being complete.
   cs_launch_chained(k_block_setup, setup_grid(B * (k + 1), c.head_dim / 2), dim3(kSetupThreads), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
                 c.vocab, c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write,
-                ctx->seq_ok, ctx->rope_cs, ctx->d_status, cs_next_stamp(ctx, CS_FAM_OTHER));
+                ctx->seq_ok, ctx->rope_cs, ctx->d_status, ctx->pair_flag, cs_next_stamp(ctx, CS_FAM_OTHER));
 }
 
 void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, int B, int stride,
@@ -533,7 +542,7 @@ void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hi
   const cs_model_config& c = ctx->cfg;
   cs_launch_pdl(k_prefill_setup, setup_grid(B * R, c.head_dim / 2), dim3(kSetupThreads), 0, st, hist, hist_len, B, stride, start, R, c.max_seq, c.vocab,
                 c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write, ctx->seq_ok,
-                ctx->rope_cs, ctx->d_status);
+                ctx->rope_cs, ctx->d_status, ctx->pair_flag);
 }
 
 void cs_launch_embed_rmsnorm(cs_ctx* ctx, const __nv_bfloat16* gain, int rows, cudaStream_t st) {

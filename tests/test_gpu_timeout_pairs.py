@@ -73,3 +73,41 @@ def test_split_projection(monkeypatch, rows, K):
         assert torch.equal(ctx.cs_linear(X, W, rows=rows), want) and ctx.cs_sync_status() == cs.CS_OK
     assert ctx.workspace_guards_intact()
     ctx.close()
+
+
+def test_forward_after_a_timeout_nobody_asked_about(monkeypatch):
+    """Clients that never take a status: the forward after the one that timed out is right."""
+    monkeypatch.setenv("CS_WAIT_LIMIT_US", "2000")
+    ctx, _ = make_pair(CFG, 96, 2, 4)
+    kv0 = inputs.synthetic_kv(CFG, 2, 96, 40, seed=3, device="cuda")
+    rng = np.random.default_rng(4)
+    hist = torch.from_numpy(rng.integers(0, CFG.vocab, size=(2, 40)).astype(np.int32)).cuda()
+    len40 = torch.full((2,), 40, dtype=torch.int32, device="cuda")
+
+    def step():
+        kv, logits = kv0.clone(), torch.zeros(2, 5, CFG.vocab, dtype=torch.float32, device="cuda")
+        out = ctx.cs_verify_step(hist[:, 0].contiguous(), hist[:, 1:5].contiguous(), torch.full_like(len40, 4), kv, len40.clone(), logits_dbg=logits)
+        return [kv, logits, *out]
+
+    def prefill():
+        kv = torch.zeros_like(kv0)
+        ctx.cs_prefill(hist, len40, 40, kv, torch.zeros_like(len40))
+        return [kv]
+
+    X = torch.randn(256, CFG.d_model, device="cuda").to(torch.bfloat16)
+    want = step(), prefill()
+    assert ctx.cs_sync_status() == cs.CS_OK
+    words = ctx._raw[ctx._ws_off:ctx._ws_off + ctx.workspace_bytes].view(torch.int32)
+    for call, expect in zip((step, prefill), want):
+        for rows in (16, 256):
+            ctx.cs_lm_head(X, rows=rows)
+            rest = words.clone()
+            ctx.cs_debug_drop_tile(0)
+            ctx.cs_lm_head(X, rows=rows)                 # every second pair gives up and does not take its neighbours' sums
+            raised = (rest == 0) & (words == 1)          # (few other words of the workspace go from 0 to 1 here)
+            assert int(raised.sum()) >= 20
+            got = call()
+            assert not bool(words[raised].any())
+            assert ctx.cs_sync_status() == cs.CS_ERR_TIMEOUT
+            assert all(torch.equal(a, b) for a, b in zip(got, expect))
+    ctx.close()
