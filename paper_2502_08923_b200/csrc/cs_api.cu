@@ -10,6 +10,7 @@
 #include <string.h>
 
 #include "cs_common.cuh"
+#include "cs_loop_host.h"
 
 namespace {
 
@@ -275,13 +276,12 @@ void capture_step(cs_ctx* ctx) {
   (void)cudaGetLastError();
 }
 
-// Waits until the step with index `step` of cs_decode_loop has reported; *wanted = the most tokens any
-// sequence still has to emit.  Ends with an error when the stream failed, or ran dry without a report.
-cs_status wait_progress(cs_ctx* ctx, int step, int* wanted, cudaStream_t st) {
+// Waits until the progress word tells of more steps than *at, and takes it over.  Ends with an error when the
+// stream failed, or ran dry without a report.
+cs_status wait_progress(cs_ctx* ctx, LoopProgress* at, cudaStream_t st) {
   cudaError_t state = cudaErrorNotReady;
   for (unsigned spin = 0;; ++spin) {
-    const unsigned long long w = __atomic_load_n(ctx->progress, __ATOMIC_ACQUIRE);
-    if ((int)(w >> 32) > step) { *wanted = (int)(w & 0xffffffffu); return CS_OK; }
+    if (newer_report([ctx] { return __atomic_load_n(ctx->progress, __ATOMIC_ACQUIRE); }, at)) return CS_OK;
     if (state != cudaErrorNotReady) break;      // (looked once more after the stream had ended)
     if ((spin & 1023u) == 1023u) state = cudaStreamQuery(st);
 #if defined(__x86_64__)
@@ -574,8 +574,8 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   // ---- device -> host, then step 4 on the host: append what was emitted
   cs_launch_host_out(ctx->loop_accept, ctx->loop_out, B, k, ctx->step_out_dev, ctx->progress_dev, st);
   CS_CUDA_OK(ctx, cudaGetLastError());
-  int done;
-  s = wait_progress(ctx, 0, &done, st);
+  LoopProgress done = {0, 0};
+  s = wait_progress(ctx, &done, st);
   if (s != CS_OK) return s;
   memcpy(accept_len_host, ctx->step_out, (size_t)B * 4);
   memcpy(out_tokens_host, ctx->step_out + CS_MAX_ROWS, (size_t)B * (k + 1) * 4);
@@ -786,22 +786,19 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->loop.active = true;
   *ctx->progress = 0ull;               // (every earlier loop of this context has been waited for)
-  int sent = 0, seen = 0, wanted = max_new;
-  while (s == CS_OK && wanted > 0 && seen < max_new) {
-    if (sent < max_new && sent - seen < 2 && wanted > (long)(sent - seen) * (k + 1)) {
-      if (ctx->loop.exec != nullptr) {
-        const cudaError_t e = cudaGraphLaunch(ctx->loop.exec, st);
-        if (e != cudaSuccess) s = fail(ctx, CS_ERR_CUDA, cudaGetErrorString(e));
-      } else {
-        s = enqueue_loop_step(ctx, st, true);
-      }
-      if (++sent == 2 && s == CS_OK && wanted > (long)4 * (k + 1) && !ctx->no_graph && layer_bytes(ctx->cfg) >= (32ll << 20))
-        capture_step(ctx);
+  auto send = [&](int sent, int wanted) {
+    cs_status r;
+    if (ctx->loop.exec != nullptr) {
+      const cudaError_t e = cudaGraphLaunch(ctx->loop.exec, st);
+      r = e == cudaSuccess ? CS_OK : fail(ctx, CS_ERR_CUDA, cudaGetErrorString(e));
     } else {
-      s = wait_progress(ctx, seen, &wanted, st);
-      seen = (int)(__atomic_load_n(ctx->progress, __ATOMIC_ACQUIRE) >> 32);
+      r = enqueue_loop_step(ctx, st, true);
     }
-  }
+    if (sent == 2 && r == CS_OK && wanted > (long)4 * (k + 1) && !ctx->no_graph && layer_bytes(ctx->cfg) >= (32ll << 20))
+      capture_step(ctx);
+    return r;
+  };
+  s = (cs_status)drive_loop(max_new, k, send, [&](LoopProgress* at) { return wait_progress(ctx, at, st); });
   // A status that concerns single sequences (no room, inconsistent lengths: those were marked
   // finished and left alone while the others ran to their end) is returned here as well.
   if (s == CS_OK) s = cs_loop_poll(ctx, stats_out, nullptr, stream);
