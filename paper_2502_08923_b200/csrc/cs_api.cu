@@ -4,7 +4,6 @@
 #include <stdlib.h>
 
 #include <mutex>
-#include <utility>
 #include <new>
 
 #include <string.h>
@@ -257,22 +256,16 @@ long long layer_bytes(const cs_model_config& c) {
   return 2 * d * (2 * qd + 2 * kvd + 3ll * c.d_ffn);
 }
 
-void drop_old_graph(cs_ctx* ctx) {
-  if (ctx->old_exec) cudaGraphExecDestroy(ctx->old_exec);
-  if (ctx->old_graph) cudaGraphDestroy(ctx->old_graph);
-  ctx->old_exec = nullptr;
-  ctx->old_graph = nullptr;
-}
-
 // One reporting step of the loop as a graph (captured on the context's own stream: the legacy default stream
 // cannot).  Without it the loop goes on enqueueing, so a failure here is not one of the call.
 void capture_step(cs_ctx* ctx) {
   LoopState& L = ctx->loop;
-  drop_old_graph(ctx);
   if (cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) { (void)cudaGetLastError(); return; }
   const cs_status s = enqueue_loop_step(ctx, ctx->cap_stream, true);
   const cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &L.graph);
   if (s != CS_OK || e != cudaSuccess || cudaGraphInstantiate(&L.exec, L.graph, 0) != cudaSuccess) L.exec = nullptr;
+  if (L.graph) cudaGraphDestroy(L.graph);    // (while the first steps run; what replays is a copy)
+  L.graph = nullptr;
   (void)cudaGetLastError();
 }
 
@@ -454,7 +447,6 @@ void cs_destroy(cs_ctx* ctx) {
   if (ctx == nullptr) return;
   cs_loop_end(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-  drop_old_graph(ctx);
   if (ctx->progress) give_slot(ctx->progress);
   delete[] ctx->layers;
   delete ctx;
@@ -803,9 +795,6 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   // finished and left alone while the others ran to their end) is returned here as well.
   if (s == CS_OK) s = cs_loop_poll(ctx, stats_out, nullptr, stream);
   else (void)cudaStreamSynchronize(st);
-  // (destroying the graph takes a moment too: the next loop does it while its first steps run)
-  std::swap(ctx->old_graph, ctx->loop.graph);
-  std::swap(ctx->old_exec, ctx->loop.exec);
   cs_loop_end(ctx);
   return s;
 }

@@ -159,9 +159,6 @@ struct cs_ctx {
 
   LoopState loop;
   HostStep host_step;
-  // the graph of the last cs_decode_loop, destroyed when the next one is built
-  cudaGraph_t old_graph;
-  cudaGraphExec_t old_exec;
   // Pinned host word that cs_decode_loop's steps report to: (steps done << 32) | most tokens any
   // sequence still has to emit; and the device's address of it.
   unsigned long long *progress, *progress_dev;
