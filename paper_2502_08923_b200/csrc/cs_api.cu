@@ -86,38 +86,66 @@ WsLayout ws_layout(const cs_model_config* c) {
   return L;
 }
 
-// Pinned host memory of the contexts: one block for the process, handed out in slots (pinning takes from
-// a tenth of a millisecond to tens of them, so it is not done per context).  Slots are given back by
-// cs_destroy; a context that finds none left pins its own.
+// Pinned host memory of the contexts, in slots of one block per device: cs_create takes a slot and cs_destroy gives it
+// back; a context that finds none left pins its own.  A block stays (0.3 MB, one per device) because pinning is slow:
+// with memory of its own for every context, creating one takes 2.8 ms instead of 0.25 and destroying it 0.5 instead
+// of 0.06, each up to 0.9 s now and then.  A block belongs to the CUDA context it was pinned in and goes with it when
+// the process resets the device, so a block is known by that context's id.
 constexpr size_t kStepInAt = 2048, kStepOutAt = kStepInAt + CS_STEP_IN_MAX * sizeof(int);
 constexpr size_t kSlotBytes = kStepOutAt + 2 * CS_MAX_ROWS * sizeof(int) + 1024;
-constexpr int kSlots = 32;
+constexpr int kSlots = 32, kBlocks = 64;
 static_assert(64 + (CS_MAX_ROWS + 1) * sizeof(int) <= kStepInAt && kSlotBytes % 1024 == 0, "progress word and host scratch");
-std::mutex g_slot_lock;
-char* g_slots = nullptr;
-unsigned g_slots_taken = 0;
+struct PinnedBlock {
+  char* at;
+  unsigned taken;
+  unsigned long long owner;
+};
+std::mutex g_pinned_lock;
+PinnedBlock g_pinned[kBlocks] = {};
 
-cudaError_t take_slot(char** out) {
-  const unsigned flags = cudaHostAllocMapped | cudaHostAllocPortable;
-  std::lock_guard<std::mutex> hold(g_slot_lock);
-  if (g_slots == nullptr) {
-    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&g_slots), kSlotBytes * kSlots, flags);
-    if (e != cudaSuccess) { g_slots = nullptr; return e; }
+// id of the current CUDA context, never given twice in a process; 0 = the driver does not say
+unsigned long long cuda_context_id() {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  unsigned long long id = 0;
+  if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+    (void)cudaGetLastError();
+    return 0;
   }
-  for (int i = 0; i < kSlots; ++i)
-    if (!(g_slots_taken >> i & 1u)) {
-      g_slots_taken |= 1u << i;
-      *out = g_slots + i * kSlotBytes;
-      return cudaSuccess;
-    }
-  return cudaHostAlloc(reinterpret_cast<void**>(out), kSlotBytes, flags);
+  return reinterpret_cast<CUresult (*)(CUcontext, unsigned long long*)>(p)(nullptr, &id) == CUDA_SUCCESS ? id : 0;
 }
 
-void give_slot(void* p) {
-  char* at = static_cast<char*>(p);
-  std::lock_guard<std::mutex> hold(g_slot_lock);
-  if (g_slots != nullptr && at >= g_slots && at < g_slots + kSlotBytes * kSlots) g_slots_taken &= ~(1u << ((at - g_slots) / kSlotBytes));
-  else cudaFreeHost(p);
+cudaError_t take_pinned(PinnedSlot* out, int dev) {
+  const unsigned flags = cudaHostAllocMapped | cudaHostAllocPortable;
+  const unsigned long long id = dev < kBlocks ? cuda_context_id() : 0;
+  std::lock_guard<std::mutex> hold(g_pinned_lock);
+  if (id != 0) {
+    PinnedBlock& k = g_pinned[dev];
+    if (k.owner != id) k = PinnedBlock{};              // (there is none yet, or it went with the context before this one)
+    if (k.at == nullptr) {
+      const cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&k.at), kSlotBytes * kSlots, flags);
+      if (e != cudaSuccess) { k = PinnedBlock{}; return e; }
+      k.owner = id;
+    }
+    for (int i = 0; i < kSlots; ++i)
+      if (!(k.taken >> i & 1u)) {
+        k.taken |= 1u << i;
+        *out = PinnedSlot{k.at + i * kSlotBytes, id, dev, i};
+        return cudaSuccess;
+      }
+  }
+  void* own = nullptr;
+  const cudaError_t e = cudaHostAlloc(&own, kSlotBytes, flags);
+  if (e == cudaSuccess) *out = PinnedSlot{static_cast<char*>(own), 0, dev, -1};
+  return e;
+}
+
+void give_pinned(const PinnedSlot& s) {
+  if (s.at == nullptr) return;
+  if (s.index < 0) { cudaFreeHost(s.at); return; }
+  std::lock_guard<std::mutex> hold(g_pinned_lock);
+  PinnedBlock& k = g_pinned[s.block];
+  if (k.owner == s.owner) k.taken &= ~(1u << s.index);   // (or else the block is gone already)
 }
 
 // cs_create has no context to leave an error text in: the last failure of this thread is kept here
@@ -358,7 +386,8 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
     return CS_ERR_UNSUPPORTED;
   }
   CREATE_OK(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-  CREATE_OK(take_slot(reinterpret_cast<char**>(&ctx->progress)));
+  CREATE_OK(take_pinned(&ctx->pinned, dev));
+  ctx->progress = reinterpret_cast<unsigned long long*>(ctx->pinned.at);
   CREATE_OK(cudaHostGetDevicePointer(reinterpret_cast<void**>(&ctx->progress_dev), ctx->progress, 0));
   ctx->host_ints = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + 64);
   ctx->step_in = reinterpret_cast<int*>(reinterpret_cast<char*>(ctx->progress) + kStepInAt);
@@ -447,7 +476,7 @@ void cs_destroy(cs_ctx* ctx) {
   if (ctx == nullptr) return;
   cs_loop_end(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
-  if (ctx->progress) give_slot(ctx->progress);
+  give_pinned(ctx->pinned);
   delete[] ctx->layers;
   delete ctx;
 }

@@ -69,6 +69,14 @@ struct HostStep {
   int host_len[CS_MAX_ROWS];    // hist_len_host[b] as the previous call left it
 };
 
+// A context's share of pinned host memory: slot `index` of a device's block that belongs to CUDA context `owner`,
+// or memory of its own (index -1)
+struct PinnedSlot {
+  char* at;
+  unsigned long long owner;
+  int block, index;
+};
+
 // Step timeline (cs_set_stamps): every stamped launch of a step owns one 64-bit slot of a
 // caller-provided device buffer, into which each of its CTAs leaves the time at which it
 // finished (largest wins).  Kernel i's share of the pipelined step is then
@@ -159,6 +167,7 @@ struct cs_ctx {
 
   LoopState loop;
   HostStep host_step;
+  PinnedSlot pinned;
   // Pinned host word that cs_decode_loop's steps report to: (steps done << 32) | most tokens any
   // sequence still has to emit; and the device's address of it.
   unsigned long long *progress, *progress_dev;
