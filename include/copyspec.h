@@ -29,7 +29,7 @@
  *   history    int32 [B][stride]; sequence b holds hist_len[b] accepted tokens: prompt,
  *              earlier turns and everything generated so far (Sec. 3.1).
  *   KV cache   bf16 [n_layers][2 (K then V)][max_batch][n_kv_heads][max_seq][head_dim],
- *              contiguous; K is stored rotated (RoPE applied).  Only positions
+ *              contiguous, 16-byte aligned; K is stored rotated (RoPE applied).  Only positions
  *              [0, kv_len[b]) of sequence b are meaningful (App. B.2).
  *   weights    bf16 row-major [out][in]:  embed [V][d], lm_head [V][d], final_norm [d];
  *              per layer attn_norm [d], wqkv [(H + 2 Hkv) Dh][d] (q rows, k rows, v

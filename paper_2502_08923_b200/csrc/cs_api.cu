@@ -156,6 +156,8 @@ cs_status fail(cs_ctx* ctx, cs_status s, const char* msg) {
   return s;
 }
 
+bool aligned(const void* p, unsigned bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
+
 cs_status ensure_act_maps(cs_ctx* ctx, int rows) {
   const int box = cs_gemm_act_box(CS_EPI_RESIDUAL, rows, true);
   if (ctx->act_box == box) return CS_OK;
@@ -338,6 +340,10 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
       w->wqkv == nullptr || w->wo == nullptr || w->ffn_norm == nullptr || w->w_gate_up == nullptr ||
       w->w_down == nullptr)
     return create_fail(CS_ERR_ARG, "NULL weight pointer");
+  // what the kernels' loads of these need (the matrices' 16 bytes are checked where their operand maps are made)
+  bool rows_ok = aligned(w->embed, 8) && aligned(w->final_norm, 8);
+  for (int l = 0; l < cfg->n_layers; ++l) rows_ok = rows_ok && aligned(w->attn_norm[l], l == 0 ? 4 : 8) && aligned(w->ffn_norm[l], 8);
+  if (!rows_ok) return create_fail(CS_ERR_ARG, "embedding or norm gain not aligned (16 bytes)");
   const WsLayout L = ws_layout(cfg);
   if (workspace_bytes < L.total) return create_fail(CS_ERR_CAPACITY, "workspace smaller than cs_workspace_bytes");
   if (reinterpret_cast<uintptr_t>(workspace) & 1023) return create_fail(CS_ERR_ARG, "workspace not 1024-byte aligned");
@@ -514,6 +520,7 @@ cs_status cs_verify_step(cs_ctx* ctx, const int32_t* last_tok, const int32_t* dr
   if (last_tok == nullptr || draft_len == nullptr || (draft == nullptr && k > 0) || kv_cache == nullptr ||
       kv_len == nullptr || accept_len == nullptr || out_tokens == nullptr || argmax_ids == nullptr)
     return fail(ctx, CS_ERR_ARG, "NULL argument");
+  if (!aligned(kv_cache, 16)) return fail(ctx, CS_ERR_ARG, "KV cache not 16-byte aligned");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->stamp_n = 0;
   cs_launch_block_setup(ctx, last_tok, draft, draft_len, kv_len, nullptr, B, k, true, st);
@@ -538,6 +545,7 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   if (hist_host == nullptr || hist_len_host == nullptr || hist_dev == nullptr || hist_len_dev == nullptr ||
       kv_cache == nullptr || kv_len == nullptr || accept_len_host == nullptr || out_tokens_host == nullptr)
     return fail(ctx, CS_ERR_ARG, "NULL argument");
+  if (!aligned(kv_cache, 16)) return fail(ctx, CS_ERR_ARG, "KV cache not 16-byte aligned");
   for (int b = 0; b < B; ++b)
     if (hist_len_host[b] < 1 || hist_len_host[b] + k + 1 > stride)
       return fail(ctx, CS_ERR_CAPACITY, "history row too short for one more block");
@@ -642,6 +650,7 @@ cs_status cs_prefill(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, 
   if (B < 1 || B > ctx->cfg.max_batch || hist == nullptr || hist_len == nullptr || kv_cache == nullptr ||
       kv_len == nullptr || max_len < 0 || stride < max_len)
     return fail(ctx, CS_ERR_ARG, "bad argument");
+  if (!aligned(kv_cache, 16)) return fail(ctx, CS_ERR_ARG, "KV cache not 16-byte aligned");
   if (max_len - 1 > ctx->cfg.max_seq) return fail(ctx, CS_ERR_CAPACITY, "history longer than the KV cache");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int R = CS_MAX_ROWS / B;
@@ -670,6 +679,7 @@ static cs_status loop_prepare(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int
   if (policy != CS_MATCH_LATEST && policy != CS_MATCH_FIRST) return fail(ctx, CS_ERR_ARG, "bad policy");
   if (hist == nullptr || hist_len == nullptr || kv_cache == nullptr || kv_len == nullptr)
     return fail(ctx, CS_ERR_ARG, "NULL argument");
+  if (!aligned(kv_cache, 16)) return fail(ctx, CS_ERR_ARG, "KV cache not 16-byte aligned");
   cs_loop_end(ctx);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   LoopState& L = ctx->loop;

@@ -57,6 +57,8 @@ extern "C" cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int
     return fail2(target, CS_ERR_ARG, "bad argument");
   if (delta > 0 && (drafter == nullptr || kv_drafter == nullptr || kv_len_drafter == nullptr || drafter == target))
     return fail2(target, CS_ERR_ARG, "delta > 0 needs a draft model context of its own, its cache and its length");
+  if (((reinterpret_cast<uintptr_t>(kv_target) | (delta > 0 ? reinterpret_cast<uintptr_t>(kv_drafter) : 0)) & 15) != 0)
+    return fail2(target, CS_ERR_ARG, "KV cache not 16-byte aligned");
   const int kt = std::max(k, delta);                   // rows of a target block beyond the first, at most
   if (kt > target->cfg.k_max) return fail2(target, CS_ERR_ARG, "k or delta above the target context's k_max");
   if (delta > 0 && drafter->cfg.vocab != target->cfg.vocab)
