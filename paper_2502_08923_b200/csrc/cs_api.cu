@@ -555,14 +555,18 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   // script rows
   HostStep& G = ctx->host_step;
   const bool known = G.host == hist_host && G.dev == hist_dev && G.B == B && G.stride == stride;
+  G.host = nullptr;                                    // (a call that fails on its way leaves nothing to rely on)
+  // ends the call with an error; the input kernel may still be reading the pinned words
+  auto give_up = [&](cs_status e) { (void)cudaStreamSynchronize(st); (void)cudaGetLastError(); return e; };
   int* in = ctx->step_in;                              // (every earlier step of this context has been waited for)
   int tokens = 0;
   for (int b = 0; b < B; ++b) {
     const int n = hist_len_host[b];
     int have = (known && G.host_len[b] == n && G.uploaded[b] <= n) ? G.uploaded[b] : 0;
     if (n - have > k + 1) {
-      CS_CUDA_OK(ctx, cudaMemcpyAsync(hist_dev + (size_t)b * stride + have, hist_host + (size_t)b * stride + have,
-                                      (size_t)(n - have) * 4, cudaMemcpyHostToDevice, st));
+      const cudaError_t e = cudaMemcpyAsync(hist_dev + (size_t)b * stride + have, hist_host + (size_t)b * stride + have,
+                                            (size_t)(n - have) * 4, cudaMemcpyHostToDevice, st);
+      if (e != cudaSuccess) return give_up(fail(ctx, CS_ERR_CUDA, cudaGetErrorString(e)));
       have = n;
     }
     in[b] = n;
@@ -572,7 +576,6 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
     tokens += n - have;
     G.uploaded[b] = n;
   }
-  G.host = hist_host; G.dev = hist_dev; G.B = B; G.stride = stride;
   const int script_ints = script_host != nullptr ? B * (k + 1) : 0;
   const int32_t* script_dev = script_host != nullptr ? ctx->loop_emitted : nullptr;
   if (script_host != nullptr) memcpy(in + 3 * B + tokens, script_host, (size_t)script_ints * 4);
@@ -584,28 +587,23 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   ctx->stamp_n = 0;
   cs_status s = cs_launch_find_match(hist_dev, hist_len_dev, B, stride, gamma, k, (int)policy, ctx->loop_mpos,
                                      ctx->loop_draft, ctx->loop_dlen, ctx->loop_last, nullptr, st);
-  if (s != CS_OK) {
-    (void)cudaStreamSynchronize(st);                   // (the input kernel reads the pinned words)
-    return fail(ctx, s, "match kernel launch failed");
-  }
+  if (s != CS_OK) return give_up(fail(ctx, s, "match kernel launch failed"));
   cs_launch_block_setup(ctx, ctx->loop_last, ctx->loop_draft, ctx->loop_dlen, kv_len, nullptr, B, k, false, st);
   // every call ends when its last kernel has reported, and k_block_setup lets nothing pass that was enqueued
   // earlier, so the cached rows and kv_len are settled while the forward runs
   ctx->kv_len_early = kv_len;
   s = enqueue_forward(ctx, B, k + 1, kv_cache, true, nullptr, st);
   ctx->kv_len_early = nullptr;
-  if (s != CS_OK) {
-    (void)cudaStreamSynchronize(st);
-    return s;
-  }
+  if (s != CS_OK) return give_up(s);
   cs_launch_accept(ctx, B, k, ctx->loop_draft, ctx->loop_dlen, script_dev, k + 1, nullptr, k + 1, ctx->loop_accept,
                    ctx->loop_out, ctx->loop_argmax, kv_len, 1, st);
   // ---- device -> host, then step 4 on the host: append what was emitted
   cs_launch_host_out(ctx->loop_accept, ctx->loop_out, B, k, ctx->step_out_dev, ctx->progress_dev, st);
-  CS_CUDA_OK(ctx, cudaGetLastError());
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return give_up(fail(ctx, CS_ERR_CUDA, cudaGetErrorString(e)));
   LoopProgress done = {0, 0};
   s = wait_progress(ctx, &done, st);
-  if (s != CS_OK) return s;
+  if (s != CS_OK) return give_up(s);
   memcpy(accept_len_host, ctx->step_out, (size_t)B * 4);
   memcpy(out_tokens_host, ctx->step_out + CS_MAX_ROWS, (size_t)B * (k + 1) * 4);
   for (int b = 0; b < B; ++b) {
@@ -616,6 +614,7 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
     hist_len_host[b] = n + tau + 1;
   }
   for (int b = 0; b < B; ++b) G.host_len[b] = hist_len_host[b];
+  G.host = hist_host; G.dev = hist_dev; G.B = B; G.stride = stride;
   return CS_OK;
 }
 
