@@ -813,6 +813,8 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   // While those two run the host captures the step and replays it from then on: the projections of a step
   // enqueued directly take 3.44 instead of 3.35 ms.  Building the graph takes 1 - 2 ms, so it is only done where
   // two steps last longer (32 MB of weights a layer; at 2 MB they last 0.15 ms) and at least three more are certain.
+  // Calls of 8 steps with a graph and without, us a step: 24 layers of 34 MB 957 / 1,006, 28 of 93 MB 1,393 / 1,442, 16 of
+  // 122 MB 935 / 965.  The graph is destroyed at the end of the call (0.1 ms).
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->loop.active = true;
   *ctx->progress = 0ull;               // (every earlier loop of this context has been waited for)

@@ -358,8 +358,10 @@ void cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, in
   // only that of the real rows, and takes blocks of up to 48 rows per KV head whose CTAs walk many tiles.
   // Measured per layer, rows as M / keys as M, attention and merge, 44 rows: 13 tiles 32.4 / 33.2 us,
   // 16 tiles 36.1 / 37.2 (and its successor starts 2 us sooner), 27 tiles 52.1 / 49.6, 32 tiles 59.1 / 54.8,
-  // 64 tiles 118 / 102.5; 84 rows, 64 tiles: 114 / 142.  The register-resident mma.sync kernel takes the
-  // other head sizes.
+  // 64 tiles 118 / 102.5; 84 rows, 64 tiles: 114 / 142.  Blocks of few rows would gain from the other kernel
+  // much sooner than this line: 4 rows, 2 tiles 12.8 / 13.8, 4 tiles 16.5 / 16.2, 8 tiles 23.0 / 20.3, 16 tiles 33.4 / 29.4,
+  // 32 tiles 54.1 / 47.3; 16 rows, 4 tiles 16.5 / 16.6, 8 tiles 22.7 / 20.9, 14 tiles 31.2 / 28.8; 28 rows, 8 tiles
+  // 22.5 / 23.6, 14 tiles 31.5 / 31.3.  The register-resident mma.sync kernel takes the other head sizes.
   // CS_ATTN_KERNEL=tc|tcw|mma, read when the context is created, forces one of them (tests run
   // them on the same inputs).
   int nsplit = 0;

@@ -146,9 +146,9 @@ struct cs_ctx {
   const void* tmKV_base;
   int tmQ_R;
   // Cached lengths [max_batch] that stay as they are until the forward being enqueued has
-  // finished, and whose cache rows are complete: set where the step opens with an
-  // ordinary stream-ordered launch (everywhere but in prefill); NULL elsewhere.  The attention
-  // kernel may then fetch tiles of cached keys before it waits for the preceding kernel.
+  // finished, and whose cache rows are complete; NULL in prefill.  The step's set-up kernel sees to that: it
+  // lets its dependents go only behind its own wait, with everything enqueued earlier complete.  The
+  // attention kernel may then fetch tiles of cached keys before it waits for the preceding kernel.
   const int* kv_len_early;
   // shared-memory opt-ins already made for this context's device (per context, not per
   // process: another context may live on another GPU)

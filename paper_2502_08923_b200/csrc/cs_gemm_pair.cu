@@ -28,9 +28,10 @@
 //
 // Measured on the 8B shape (us per launch: QKV / attention output / gate/up / down / LM head), one-SM
 // tiles with launch shapes by a cost model -> this kernel:
-//    88 rows  23.5 19.9 54.9 36.5 272 -> 17.0 17.5 49.3 28.1 183
-//   176 rows  31.8 26.7 90.7 49.1 509 -> 21.5 20.4 59.8 35.2 241   (two-term tensor floor 10.6 7.1 49 25 222)
-//   256 rows  42.2 36.4 114 70.7 791  -> 24.2 24.7 73.2 44.3 269 with 256 keys cached
+//    88 rows  23.5 19.9 54.9 36.5 272 -> 17.4 16.5 49.3 28.2 184
+//   176 rows  31.8 26.7 90.7 49.1 509 -> 24.2 20.6 66.6 38.5 257   (two-term tensor floor 10.6 7.1 49 25 222)
+//   256 rows  42.2 36.4 114 70.7 791  -> 25.7 23.7 75.0 45.4 287 with 2,048 keys cached
+// (the power cap's share differs from GPU to GPU: 21.7 18.9 61.0 36.1 250 at 176 rows on another one)
 // and the stream form at 11 rows: gate/up 42.2 -> 41.1, LM head 168 -> 157 us (6.7 TB/s).  Clusters that
 // add up over distributed shared memory instead of the split form's exchange: 24.2, 25.6, 45.5 us at
 // 176 rows, 29.5, 32.7, 60.4 at 256 (QKV, output, down).

@@ -3,7 +3,7 @@
 // the first RMSNorm, the merge of the attention's key slices, the reduction of the LM-head
 // tile maxima with prefix acceptance, KV truncation, and the loop's init and commit steps.
 // RoPE, the K/V append, SwiGLU, the residual adds and every later RMSNorm live in the GEMM
-// epilogues (cs_gemm.cu); attention is in cs_attn_tc.cu and cs_attn.cu.
+// epilogues (cs_gemm.cu, cs_gemm_pair.cu); attention is in cs_attn_tc.cu, cs_attn_tcw.cu and cs_attn.cu.
 #include <math.h>
 
 #include <algorithm>
@@ -187,9 +187,9 @@ k_embed_rmsnorm(const __nv_bfloat16* __restrict__ E, const int* row_tok, float* 
 // Combine the key slices: o = sum_s o_s e^(m_s - M) / sum_s l_s e^(m_s - M).  W warps per (row, head), each
 // taking every W-th slice, at most NS of them; a lane holds four dims.  All of a thread's partial outputs
 // are requested at once, so their latencies overlap each other and the weight computation.  Bound by
-// that latency.  Measured at 11 rows x 32 heads x 33 slices (one thread per dim and all slices before):
-// 5.8 -> 5.5 us; at 176 rows and one slice 5.6 -> 3.1, at 256 rows and four slices 8.5 -> 3.6 (and the next
-// kernel starts 2 us earlier: a quarter of the CTAs hold thread slots).
+// that latency.  Measured (one thread per dim and all slices before): at 11 rows x 32 heads x 33 slices 5.8 -> 5.5 us (4.6
+// with the 18 slices that the tcgen05 kernels leave of one sequence now); at 176 rows and one slice 5.6 -> 3.1, at 256 rows and
+// four slices 8.5 -> 3.6 (and the next kernel starts 2 us earlier: a quarter of the CTAs hold thread slots).
 constexpr int kMergeThreads = 128;
 template <int W, int NS>
 __global__ void __launch_bounds__(kMergeThreads)
