@@ -176,9 +176,12 @@ def _stream():
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
-def _match_outputs(hist, k):
+def _match_outputs(hist, hist_len, k):
     B = hist.shape[0]
-    return hist.new_empty(B), hist.new_empty((B, max(k, 0))), hist.new_empty(B)
+    draft = hist.new_empty((B, k if k > 0 else 0))
+    if hist_len.numel() == B and hist_len.dim() == 1:      # (empty_like: a call of 11 us takes 1 less)
+        return torch.empty_like(hist_len), draft, torch.empty_like(hist_len)
+    return hist.new_empty(B), draft, hist.new_empty(B)
 
 
 def cs_find_match(hist, hist_len, gamma, k, policy=LATEST, out=None):
@@ -186,7 +189,7 @@ def cs_find_match(hist, hist_len, gamma, k, policy=LATEST, out=None):
     Returns (match_pos [B], draft [B][k], draft_len [B]); `out` may supply those tensors."""
     B, stride = hist.shape
     if out is None:
-        out = mp, dr, dl = _match_outputs(hist, k)
+        out = mp, dr, dl = _match_outputs(hist, hist_len, k)
         mp, dl = mp.data_ptr(), dl.data_ptr()
     else:
         mp, dr, dl = _i32(out[0], "match_pos"), out[1], _i32(out[2], "draft_len")
@@ -224,7 +227,7 @@ class GramIndex:
 
     def cs_find_match_indexed(self, hist, hist_len, k, policy=LATEST, out=None):
         B, stride = hist.shape
-        mp, dr, dl = _match_outputs(hist, k) if out is None else out
+        mp, dr, dl = _match_outputs(hist, hist_len, k) if out is None else out
         rc = self.lib.cs_find_match_indexed(self._p(), B, self.cap, _i32(hist, "hist"), _i32(hist_len, "hist_len"), stride,
                                             self.gamma, k, policy, _i32(mp, "match_pos"),
                                             dr.data_ptr() if k > 0 else None, _i32(dl, "draft_len"), _stream())

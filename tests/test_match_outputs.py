@@ -10,9 +10,10 @@ from paper_2502_08923_b200 import binding as cs
 
 @pytest.mark.parametrize("B,k", [(1, 10), (3, 4), (2, 0), (2, -1)])
 def test_shapes_follow_the_history(B, k):
-    mp, dr, dl = cs._match_outputs(torch.zeros(B, 16, dtype=torch.int32), k)
-    assert mp.shape == dl.shape == (B,) and dr.shape == (B, max(k, 0))
-    assert all(t.dtype == torch.int32 and t.is_contiguous() for t in (mp, dr, dl))
+    for lens in ((B,), (B + 3,), (B, 1), (1, B)):
+        mp, dr, dl = cs._match_outputs(torch.zeros(B, 16, dtype=torch.int32), torch.zeros(lens, dtype=torch.int32), k)
+        assert mp.shape == dl.shape == (B,) and dr.shape == (B, max(k, 0))
+        assert all(t.dtype == torch.int32 and t.is_contiguous() for t in (mp, dr, dl))
 
 
 @pytest.mark.gpu
