@@ -814,7 +814,8 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   // enqueued directly take 3.44 instead of 3.35 ms.  Building the graph takes 1 - 2 ms, so it is only done where
   // two steps last longer (32 MB of weights a layer; at 2 MB they last 0.15 ms) and at least three more are certain.
   // Calls of 8 steps with a graph and without, us a step: 24 layers of 34 MB 957 / 1,006, 28 of 93 MB 1,393 / 1,442, 16 of
-  // 122 MB 935 / 965.  The graph is destroyed at the end of the call (0.1 ms).
+  // 122 MB 935 / 965.  Destroying the graph takes 0.1 - 0.6 ms, so that is done while what will likely be the last steps
+  // run (it may be in flight then: the driver frees it when they are done); steps still needed after that are enqueued.
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->loop.active = true;
   *ctx->progress = 0ull;               // (every earlier loop of this context has been waited for)
@@ -830,7 +831,14 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
       capture_step(ctx);
     return r;
   };
-  s = (cs_status)drive_loop(max_new, k, send, [&](LoopProgress* at) { return wait_progress(ctx, at, st); });
+  auto wait = [&](LoopProgress* at, int sent) {
+    if (ctx->loop.exec != nullptr && likely_last(*at, sent, max_new)) {
+      cudaGraphExecDestroy(ctx->loop.exec);
+      ctx->loop.exec = nullptr;
+    }
+    return wait_progress(ctx, at, st);
+  };
+  s = (cs_status)drive_loop(max_new, k, send, wait);
   // A status that concerns single sequences (no room, inconsistent lengths: those were marked
   // finished and left alone while the others ran to their end) is returned here as well.
   if (s == CS_OK) s = cs_loop_poll(ctx, stats_out, nullptr, stream);

@@ -19,9 +19,15 @@ static inline bool newer_report(Word word, LoopProgress* at) {
   return true;
 }
 
+// Whether the steps in flight will likely be the last: going by the tokens a step has brought so far, they bring all that
+// are wanted.  (Certain where a step brings one token.)
+static inline bool likely_last(const LoopProgress& at, int sent, int max_new) {
+  return at.steps > 0 && (long)at.wanted * at.steps <= (long)(sent - at.steps) * (max_new - at.wanted);
+}
+
 // Runs the loop until no sequence wants a token.  At most two steps are ahead of the reports, and a step is sent
 // ahead of a report only where it is needed whatever the steps in flight accept (at most k + 1 tokens each).
-// `send(n, wanted)` sends step number n (from 1); `wait(&at)` returns with a newer report.  Both return a
+// `send(n, wanted)` sends step number n (from 1); `wait(&at, sent)` returns with a newer report.  Both return a
 // status; the first that is not 0 ends the loop.
 template <typename Send, typename Wait>
 static inline int drive_loop(int max_new, int k, Send send, Wait wait) {
@@ -32,7 +38,7 @@ static inline int drive_loop(int max_new, int k, Send send, Wait wait) {
       ++sent;
       status = send(sent, at.wanted);
     } else {
-      status = wait(&at);
+      status = wait(&at, sent);
     }
   }
   return status;

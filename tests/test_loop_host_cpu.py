@@ -41,7 +41,9 @@ int main(int argc, char** argv) {
     if (sent - done > ahead) ahead = sent - done;
     return 0;
   };
-  auto wait = [&](LoopProgress* at) {
+  auto wait = [&](LoopProgress* at, int n) {
+    if (n != sent) return 4;
+    if (k == 0 && likely_last(*at, n, max_new) != (at->wanted <= n - at->steps && at->steps > 0)) return 5;   // certain where a step brings one token
     for (int i = 0; i < 64; ++i)
       if (newer_report(word, at)) return 0;
     return 3;                                          // waited for a report that cannot come
