@@ -55,6 +55,8 @@
  * Environment, read once by cs_create (measurement and test switches; not needed in use):
  *   CS_NO_GRAPH=1          cs_loop_steps and cs_decode_loop enqueue their steps kernel by kernel, as the other calls
  *                          do, instead of replaying them from a captured CUDA graph;
+ *   CS_NO_CHAIN=1          blocks of at most 32 rows run as a launch per projection too, instead of one launch per
+ *                          layer for everything between two attentions;
  *   CS_ATTN_KERNEL=tc|tcw|mma  forces one attention kernel: tcgen05 with the query rows as the
  *                          M dimension (tc), tcgen05 with the keys and head dims as M (tcw), or
  *                          mma.sync (mma).  Default: by head size, and between the two tcgen05
@@ -383,6 +385,10 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
  * sums that never come.  Launches of at most 32 rows that split K over a cluster refuse the hook
  * (CS_ERR_UNSUPPORTED; the cluster barrier has no time limit).  k_block < 0 clears it. */
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block);
+
+/* The same for the chained projections of blocks of at most 32 rows: the next such launch leaves out the
+ * weights of the unit-th K block of every run it hands to an SM.  unit < 0 clears it. */
+cs_status cs_debug_drop_chain_tile(cs_ctx* ctx, int unit);
 
 /* Test hook for the hand-over of work between SM pairs (no counterpart in the paper): where the K
  * ranges of a projection above 32 rows are split between pairs, the pairs whose K range is in the

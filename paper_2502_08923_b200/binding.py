@@ -51,7 +51,7 @@ class CsStats(C.Structure):
 WORKSPACE_GUARD, GUARD_BYTE = 4096, 0xA5   # guard bands around a Context's workspace
 EXPORTS = ("cs_workspace_bytes", "cs_create", "cs_destroy", "cs_last_error", "cs_sync_status",
            "cs_find_match", "cs_verify_step", "cs_kv_truncate", "cs_decode_loop", "cs_decode_loop_drafted", "cs_step_host",
-           "cs_prefill", "cs_linear", "cs_step_host_reset", "cs_debug_drop_tile", "cs_debug_leave_shares",
+           "cs_prefill", "cs_linear", "cs_step_host_reset", "cs_debug_drop_tile", "cs_debug_drop_chain_tile", "cs_debug_leave_shares",
            "cs_loop_begin", "cs_loop_steps", "cs_loop_poll", "cs_loop_end", "cs_loop_last_step", "cs_set_stamps", "cs_stamp_layout", "cs_set_match_index",
            "cs_loop_launches_per_step", "cs_lm_head", "cs_lm_head_static", "cs_gram_index_bytes",
            "cs_gram_index_reset", "cs_gram_index_update", "cs_find_match_indexed", "cs_gram_index_status")
@@ -125,6 +125,8 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.cs_step_host_reset.argtypes = [vp]
     lib.cs_debug_drop_tile.restype = i
     lib.cs_debug_drop_tile.argtypes = [vp, i]
+    lib.cs_debug_drop_chain_tile.restype = i
+    lib.cs_debug_drop_chain_tile.argtypes = [vp, i]
     lib.cs_debug_leave_shares.restype = i
     lib.cs_debug_leave_shares.argtypes = [vp, i]
     lib.cs_gram_index_bytes.restype = C.c_size_t
@@ -385,6 +387,9 @@ class Context:
 
     def cs_debug_drop_tile(self, k_block):
         self._check(self.lib.cs_debug_drop_tile(self.handle, k_block), "cs_debug_drop_tile")
+
+    def cs_debug_drop_chain_tile(self, unit):
+        self._check(self.lib.cs_debug_drop_chain_tile(self.handle, unit), "cs_debug_drop_chain_tile")
 
     def cs_debug_leave_shares(self, mask):
         self._check(self.lib.cs_debug_leave_shares(self.handle, mask), "cs_debug_leave_shares")

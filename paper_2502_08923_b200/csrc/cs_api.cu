@@ -15,7 +15,7 @@ namespace {
 
 struct WsLayout {
   size_t x, xn, attn_out, act, qbuf, partial, attn_o, attn_ml, ssq, rope_cs, inv_freq, tile_max, tile_idx,
-      row_tok, row_pos, row_lim, row_write, seq_ok, iota, pair_part, pair_flag, status, loop_last, loop_draft, loop_dlen, loop_mpos,
+      row_tok, row_pos, row_lim, row_write, seq_ok, iota, pair_part, pair_flag, chain_part, chain_epoch, chain_ctl, status, loop_last, loop_draft, loop_dlen, loop_mpos,
       loop_emitted, loop_done, loop_accept, loop_out, loop_argmax, loop_stats, total;
   size_t qkv_elems;
   int attn_splits;
@@ -71,6 +71,9 @@ WsLayout ws_layout(const cs_model_config* c) {
   L.iota = take(&off, rows * 4);
   L.pair_part = take(&off, (size_t)CS_MAX_PAIRS * 2 * CS_MAX_ROWS * CS_GEMM_BM * 4);
   L.pair_flag = take(&off, CS_MAX_PAIRS * 2 * 4);
+  L.chain_part = take(&off, (size_t)4 * CS_CHAIN_MAX_RUNS * CS_CHAIN_MAX_ROWS / 2 * CS_GEMM_BM * sizeof(uint4));
+  L.chain_epoch = take(&off, 256);
+  L.chain_ctl = take(&off, (size_t)c->n_layers * cs_chain_words(c) * 4);
   L.status = take(&off, 256);
   L.loop_last = take(&off, rows * 4);
   L.loop_draft = take(&off, rows * 4);
@@ -184,17 +187,39 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
   // it: the residual GEMM before it writes gain * x (two bf16 terms) and sums of squares, the
   // GEMM after it scales its accumulators by 1/rms.
   NormFuse take_norm = {};           // how the next norm-consuming GEMM finds its 1/rms
+  auto qkv_epi = [&](int l) {
+    return QkvEpi{ctx->rope_cs, ctx->row_pos, ctx->row_write, ctx->qbuf, static_cast<__nv_bfloat16*>(kv_cache),
+                  R, l, c.n_heads, c.n_kv_heads, c.head_dim, c.max_batch, c.max_seq};
+  };
+  if (cs_chain_takes(ctx, rows)) {
+    // short blocks: two launches per layer, the attention and everything up to the next one
+    cs_launch_embed_rmsnorm(ctx, ctx->layers[0].attn_norm, rows, st);
+    const QkvEpi q0 = qkv_epi(0);
+    s = cs_launch_gemm(ctx, &ctx->layers[0].qkv, &ctx->tmXn, lo_row, rows, CS_EPI_QKV, nullptr, nullptr, nullptr, 0, &q0, &take_norm, st);
+    for (int l = 0; l < c.n_layers && s == CS_OK; ++l) {
+      const int nsplit = cs_launch_attention(ctx, kv_cache, l, B, R, false, st);
+      const bool last = l + 1 == c.n_layers;
+      const QkvEpi qn = qkv_epi(l + 1);
+      s = cs_launch_chain(ctx, l, nsplit, rows, last ? nullptr : &qn,
+                          !last ? ctx->layers[l + 1].attn_norm : (with_lm ? ctx->final_norm : nullptr), st);
+    }
+    if (s != CS_OK) return s;
+    take_norm.ssq_in = ctx->ssq;
+    take_norm.slots_in = cs_ceil_div(c.d_model, CS_GEMM_BM);
+    take_norm.slot_stride = ctx->ssq_stride;
+    take_norm.inv_d = 1.f / (float)c.d_model;
+    take_norm.eps = c.rms_eps;
+  } else
   for (int l = 0; l < c.n_layers; ++l) {
     const LayerPlan& L = ctx->layers[l];
     if (l == 0) {
       cs_launch_embed_rmsnorm(ctx, L.attn_norm, rows, st);
     }
-    const QkvEpi qe = {ctx->rope_cs, ctx->row_pos, ctx->row_write, ctx->qbuf, static_cast<__nv_bfloat16*>(kv_cache),
-                       R, l, c.n_heads, c.n_kv_heads, c.head_dim, c.max_batch, c.max_seq};
+    const QkvEpi qe = qkv_epi(l);
     s = cs_launch_gemm(ctx, &L.qkv, &ctx->tmXn, lo_row, rows, CS_EPI_QKV, nullptr, nullptr, nullptr, 0, &qe,
                        &take_norm, st);
     if (s != CS_OK) return s;
-    cs_launch_attention(ctx, kv_cache, l, B, R, st);
+    cs_launch_attention(ctx, kv_cache, l, B, R, true, st);
     NormFuse give = {};
     give.gain_out = L.ffn_norm;
     give.xn_out = ctx->xn;
@@ -361,10 +386,13 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
     ctx->attn_force = (k == nullptr) ? 0 : (strcmp(k, "mma") == 0 ? 1 : (strcmp(k, "tc") == 0 ? 2 : (strcmp(k, "tcw") == 0 ? 3 : 0)));
     const char* ng = getenv("CS_NO_GRAPH");
     ctx->no_graph = ng != nullptr && ng[0] == '1';
+    const char* nc = getenv("CS_NO_CHAIN");
+    ctx->no_chain = nc != nullptr && nc[0] == '1';
     const char* wl = getenv("CS_WAIT_LIMIT_US");
     const long long us = (wl != nullptr) ? atoll(wl) : 0;
     ctx->wait_limit_ns = (us > 0) ? (unsigned long long)us * 1000ull : 2000000000ull;
     ctx->debug_drop_kb = -1;
+    ctx->debug_drop_chain = -1;
   }
   ctx->qkv_elems = L.qkv_elems;
   ctx->layers = new (std::nothrow) LayerPlan[cfg->n_layers];
@@ -426,6 +454,9 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   ctx->iota = reinterpret_cast<int*>(base + L.iota);
   ctx->pair_part = reinterpret_cast<float*>(base + L.pair_part);
   ctx->pair_flag = reinterpret_cast<int*>(base + L.pair_flag);
+  ctx->chain_part = reinterpret_cast<uint4*>(base + L.chain_part);
+  ctx->chain_epoch = reinterpret_cast<int*>(base + L.chain_epoch);
+  ctx->chain_ctl = reinterpret_cast<int*>(base + L.chain_ctl);
   ctx->d_status = reinterpret_cast<int*>(base + L.status);
   ctx->loop_last = reinterpret_cast<int*>(base + L.loop_last);
   ctx->loop_draft = reinterpret_cast<int*>(base + L.loop_draft);
@@ -625,6 +656,12 @@ void cs_step_host_reset(cs_ctx* ctx) {
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block) {
   if (ctx == nullptr) return CS_ERR_ARG;
   ctx->debug_drop_kb = k_block < 0 ? -1 : k_block;
+  return CS_OK;
+}
+
+cs_status cs_debug_drop_chain_tile(cs_ctx* ctx, int unit) {
+  if (ctx == nullptr) return CS_ERR_ARG;
+  ctx->debug_drop_chain = unit < 0 ? -1 : unit;
   return CS_OK;
 }
 

@@ -352,7 +352,7 @@ int launch(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, cudaStrea
 
 }  // namespace
 
-void cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, cudaStream_t st) {
+int cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, bool merge, cudaStream_t st) {
   // head_dim 128 runs on the tcgen05 kernels.  The one with the query rows as M does a tile's work of
   // 128 rows whatever the block holds, but has the shorter chain; the one with keys and head dims as M does
   // only that of the real rows, and takes blocks of up to 48 rows per KV head whose CTAs walk many tiles.
@@ -371,14 +371,12 @@ void cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, in
     if (wide) nsplit = cs_launch_attention_tcw(ctx, kv_cache, layer, B, R, st);
     if (nsplit == 0) nsplit = cs_launch_attention_tc(ctx, kv_cache, layer, B, R, st);
   }
-  if (nsplit > 0) {
-    cs_launch_attn_merge(ctx, nsplit, B * R, st);
-    return;
-  }
-  switch (ctx->cfg.head_dim) {
-    case 32: nsplit = launch<32>(ctx, kv_cache, layer, B, R, st); break;
-    case 64: nsplit = launch<64>(ctx, kv_cache, layer, B, R, st); break;
-    default: nsplit = launch<128>(ctx, kv_cache, layer, B, R, st); break;
-  }
-  cs_launch_attn_merge(ctx, nsplit, B * R, st);
+  if (nsplit <= 0)
+    switch (ctx->cfg.head_dim) {
+      case 32: nsplit = launch<32>(ctx, kv_cache, layer, B, R, st); break;
+      case 64: nsplit = launch<64>(ctx, kv_cache, layer, B, R, st); break;
+      default: nsplit = launch<128>(ctx, kv_cache, layer, B, R, st); break;
+    }
+  if (merge) cs_launch_attn_merge(ctx, nsplit, B * R, st);
+  return nsplit;
 }

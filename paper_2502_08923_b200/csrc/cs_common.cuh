@@ -29,6 +29,8 @@ static constexpr int CS_MAX_SPLITS = 8;   // split-K factor limit (portable clus
 static constexpr int CS_SPLIT_TILE_CAP = 640;  // tiles * splits never exceeds this (unless splits == 1)
 static constexpr int CS_PAIR_MAX_SPLITS = 8;   // split-K factor limit of the two-SM GEMM
 static constexpr int CS_MAX_PAIRS = 80;        // SM pairs whose sums meet in the workspace, at most
+static constexpr int CS_CHAIN_MAX_ROWS = 32;   // rows of a block whose layers run as one chained launch each, at most
+static constexpr int CS_CHAIN_MAX_RUNS = 160;  // runs of one projection in it, at most
 
 struct GemmPlan {
   CUtensorMap tmW;      // weights [N][K], box 128 x 64, 128-byte swizzle
@@ -123,6 +125,9 @@ struct cs_ctx {
   int* iota;                 // 0 .. CS_MAX_ROWS - 1 (device-side constants for host-ordered steps)
   float* pair_part;          // two-SM GEMM: sums that pairs hand to one another [CS_MAX_PAIRS][2][CS_MAX_ROWS][128]
   int* pair_flag;            // and the words that announce them [CS_MAX_PAIRS][2], 0 between launches
+  uint4* chain_part;         // chained projections: sums that runs hand to one another [4][CS_CHAIN_MAX_RUNS][CS_CHAIN_MAX_ROWS / 2][128]
+  int* chain_epoch;          // and how many forwards there have been
+  int* chain_ctl;            // counters and "done" words of the chained projections, a set per layer; cleared by a forward's set-up kernel
   int* d_status;             // device status word
   // loop state, all [max_batch] unless noted
   int* loop_last;
@@ -139,6 +144,8 @@ struct cs_ctx {
   // activation operand maps, rebuilt when the block height changes
   int act_box;               // token rows per copy
   CUtensorMap tmXn, tmAttn, tmAct;
+  int chain_box;             // the same for the chained projections: token rows, and both terms in one copy
+  CUtensorMap tmChainXn, tmChainAttn, tmChainAct;
 
   // tensor-core attention: maps over the whole KV cache (rebuilt when the cache pointer
   // changes) and over the rotated queries (rebuilt when the block height changes)
@@ -152,14 +159,16 @@ struct cs_ctx {
   const int* kv_len_early;
   // shared-memory opt-ins already made for this context's device (per context, not per
   // process: another context may live on another GPU)
-  bool gemm_attr_set, pair_attr_set;
+  bool gemm_attr_set, pair_attr_set, chain_attr_set;
   int pairs_at_once;         // two-CTA clusters of the two-SM GEMM that can run at once (0 = not asked yet)
   unsigned attn_mma_attr_set;   // a bit per head size and key grouping
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
+  bool no_chain;             // CS_NO_CHAIN=1 at creation: a launch per projection whatever the block's height
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
+  int debug_drop_chain;      // test hook: the next chained launch leaves out this unit of every run (-1 = none)
   int debug_leave;           // test hook: K ranges whose SM pairs leave their shares to others (0 = none)
 
   void* match_index;         // cs_set_match_index: the loop searches through this gamma-gram index (NULL = scan)
@@ -310,6 +319,11 @@ int cs_norm_slots(const GemmPlan* g, int rows);   // sums of squares per token t
 cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode, float* out,
                               __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
                               cudaStream_t st);
+// cs_chain.cu: merge of the attention's slices, attention output, gate/up, down and the next layer's QKV in one launch
+size_t cs_chain_words(const cs_model_config* c);   // control words of a layer
+bool cs_chain_takes(const cs_ctx* ctx, int rows);
+// next_q = where the next layer's QKV projection puts its results (NULL behind the last layer), next_gain = gain of the norm behind this layer
+cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const QkvEpi* next_q, const __nv_bfloat16* next_gain, cudaStream_t st);
 // cs_layers.cu
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip,
@@ -317,8 +331,9 @@ void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* 
 void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, int B,
                              int stride, int start, int R, cudaStream_t st);
 void cs_launch_embed_rmsnorm(cs_ctx* ctx, const __nv_bfloat16* gain, int rows, cudaStream_t st);
-void cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R,
-                         cudaStream_t st);
+// returns the number of key slices; `merge` = 0 leaves their merge to the caller
+int cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, bool merge,
+                        cudaStream_t st);
 void cs_launch_attn_merge(cs_ctx* ctx, int nsplit, int rows, cudaStream_t st);
 // tcgen05 path (head_dim 128, at most 128 query heads per KV head); returns the number of key
 // slices written, 0 when the shape is not covered, -1 on a host error (ctx->err set)

@@ -19,6 +19,16 @@ __device__ __forceinline__ void lower_pair_flags(const int* status, int* pair_fl
     for (int i = threadIdx.x; i < 2 * CS_MAX_PAIRS; i += blockDim.x) pair_flag[i] = 0;
 }
 
+// Counters and "done" words of the forward's chained projections (cs_chain.cu) start at zero.  Their kernels may take runs
+// ahead of their own wait, so a set-up kernel clears the words before it lets its dependents go.
+__device__ __forceinline__ void clear_chain_words(int4* words, int quads, int* epoch) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *epoch = __ldcg(epoch) + 1;   // (marks the sums of this forward)
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += gridDim.x * blockDim.x) words[i] = make_int4(0, 0, 0, 0);
+  __threadfence();
+  __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ----------------------------------------------------------------- block assembly
 // Rows of sequence b: r = 0 is the last accepted token, r = 1..draft_len[b] the draft
 // (Sec. 3.2: the speculative tokens are appended to the context).  Rows past the draft
@@ -36,9 +46,9 @@ k_block_setup(const int* last_tok, const int* draft, const int* draft_len, const
                               const int* skip, int B, int k, int max_seq, int vocab,
                               int half, const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                               int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status,
-                              int* pair_flag, unsigned long long* stamp) {
+                              int* pair_flag, int4* chain_words, int chain_quads, int* chain_epoch, unsigned long long* stamp) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  clear_chain_words(chain_words, chain_quads, chain_epoch);
   lower_pair_flags(status, pair_flag);
   const int R = k + 1, rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
@@ -83,8 +93,10 @@ __global__ void __launch_bounds__(kSetupThreads)
 k_prefill_setup(const int* hist, const int* hist_len, int B,
                                 int stride, int start, int R, int max_seq, int vocab, int half,
                                 const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
-                                int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status, int* pair_flag) {
-  CS_PDL_PROLOGUE();
+                                int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status, int* pair_flag,
+                                int4* chain_words, int chain_quads, int* chain_epoch) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  clear_chain_words(chain_words, chain_quads, chain_epoch);
   lower_pair_flags(status, pair_flag);
   const int rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
@@ -523,26 +535,33 @@ k_host_out(const int* accept_len, const int* out_tokens, int B, int n_out, int* 
 
 }  // namespace
 
-// one angle per thread up to a quarter of the chip
-static dim3 setup_grid(int rows, int half) { return dim3(std::min(cs_ceil_div(rows * half, kSetupThreads), 37)); }
+// one angle, or four words to clear, per thread up to a quarter of the chip
+static dim3 setup_grid(int rows, int half, int quads) { return dim3(std::min(cs_ceil_div(std::max(rows * half, quads), kSetupThreads), 37)); }
+// chained projections' words that a forward over so many rows needs cleared, in fours
+static int chain_quads(const cs_ctx* ctx, int rows) {
+  return cs_chain_takes(ctx, rows) ? (int)(ctx->cfg.n_layers * cs_chain_words(&ctx->cfg) / 4) : 0;
+}
 
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip, int B,
                            int k, bool opens_step, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
+  const int quads = chain_quads(ctx, B * (k + 1));
   // A step that opens here (no search in front of it) opens with an ordinary stream-ordered launch, so
   // that kernels further down the chain may rely on everything enqueued earlier being complete.
-  cs_launch_chained(k_block_setup, setup_grid(B * (k + 1), c.head_dim / 2), dim3(kSetupThreads), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
+  cs_launch_chained(k_block_setup, setup_grid(B * (k + 1), c.head_dim / 2, quads), dim3(kSetupThreads), 0, st, !opens_step, last_tok, draft, draft_len, kv_len, skip, B, k, c.max_seq,
                 c.vocab, c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write,
-                ctx->seq_ok, ctx->rope_cs, ctx->d_status, ctx->pair_flag, cs_next_stamp(ctx, CS_FAM_OTHER));
+                ctx->seq_ok, ctx->rope_cs, ctx->d_status, ctx->pair_flag, reinterpret_cast<int4*>(ctx->chain_ctl), quads, ctx->chain_epoch,
+                cs_next_stamp(ctx, CS_FAM_OTHER));
 }
 
 void cs_launch_prefill_setup(cs_ctx* ctx, const int32_t* hist, const int32_t* hist_len, int B, int stride,
                              int start, int R, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
-  cs_launch_pdl(k_prefill_setup, setup_grid(B * R, c.head_dim / 2), dim3(kSetupThreads), 0, st, hist, hist_len, B, stride, start, R, c.max_seq, c.vocab,
+  const int quads = chain_quads(ctx, B * R);
+  cs_launch_pdl(k_prefill_setup, setup_grid(B * R, c.head_dim / 2, quads), dim3(kSetupThreads), 0, st, hist, hist_len, B, stride, start, R, c.max_seq, c.vocab,
                 c.head_dim / 2, ctx->inv_freq, ctx->row_tok, ctx->row_pos, ctx->row_lim, ctx->row_write, ctx->seq_ok,
-                ctx->rope_cs, ctx->d_status, ctx->pair_flag);
+                ctx->rope_cs, ctx->d_status, ctx->pair_flag, reinterpret_cast<int4*>(ctx->chain_ctl), quads, ctx->chain_epoch);
 }
 
 void cs_launch_embed_rmsnorm(cs_ctx* ctx, const __nv_bfloat16* gain, int rows, cudaStream_t st) {

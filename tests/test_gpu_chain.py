@@ -1,0 +1,98 @@
+"""The chained projections of short blocks (one launch for everything between two attentions) at the sizes where
+they can go wrong: rows at the edges of their three paddings, widths that are no multiple of the 128-feature tiles or
+of the 64-wide K blocks, every head size, tiles shared by many runs and runs that hold several tiles.  Against a
+launch per projection (CS_NO_CHAIN=1) on the same inputs.
+
+Tolerance: both carry activations as two bf16 terms and sum in fp32, in another order, so the first layer agrees to
+about 2^-15; a K or V element of the next layers that this moves across a rounding boundary of bf16 differs by 2^-8 of
+itself and is one of many keys, so no logit can move by more than 2^-8 of the largest, no cached value by more
+than one bf16 step of the largest."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2502_08923_b200 import binding as cs, inputs
+from helpers import i32, make_pair
+
+pytestmark = pytest.mark.gpu
+
+
+def _cfg(d, heads, kv_heads, dh, ffn, layers=3):
+    return inputs.ModelConfig(n_layers=layers, d_model=d, n_heads=heads, n_kv_heads=kv_heads, head_dim=dh, d_ffn=ffn, vocab=777)
+
+
+CONFIGS = {
+    "ragged": _cfg(520, 5, 5, 32, 328),             # 4.06 tiles, 8.1 K blocks, a head group of 32 features at the end
+    "tiny": _cfg(256, 8, 8, 32, 1024, layers=2),    # fewer runs than SMs
+    "shared": _cfg(256, 16, 2, 128, 9000),          # tiles of down shared by 35 runs
+    "wide": _cfg(2048, 16, 4, 64, 2048),            # gate/up: runs inside a tile; many key slices to merge
+    "long": _cfg(256, 2, 1, 128, 20000),            # runs that hold several whole tiles
+}
+
+
+def _step(cfg, w, B, k, kv_len, max_seq, alone, monkeypatch):
+    monkeypatch.setenv("CS_NO_CHAIN", "1" if alone else "0")
+    ctx = cs.Context(cfg, w, max_seq=max_seq, max_batch=B, k_max=max(k, 1))
+    rng = np.random.default_rng(k + kv_len)
+    last, draft = i32(rng.integers(0, cfg.vocab, size=B)), i32(rng.integers(0, cfg.vocab, size=(B, k)))
+    dlen = i32([max(0, k - 2 * b) for b in range(B)])
+    kv = inputs.synthetic_kv(cfg, B, max_seq, kv_len, seed=3, device="cuda")
+    lens = i32([kv_len - 5 * b for b in range(B)])
+    outs = []
+    for _ in range(2):                              # (the second forward finds the counters of the first)
+        l, logits = lens.clone(), torch.zeros(B, k + 1, cfg.vocab, dtype=torch.float32, device="cuda")
+        ctx.cs_verify_step(last, draft, dlen, kv, l, logits_dbg=logits)
+        assert ctx.cs_sync_status() == cs.CS_OK
+        outs.append(logits)
+    assert torch.equal(outs[0], outs[1]) and ctx.workspace_guards_intact()
+    ctx.close()
+    return outs[0], kv.float(), [int(n) for n in dlen]
+
+
+@pytest.mark.parametrize("B,k", [(1, 0), (1, 7), (1, 8), (2, 7), (1, 16), (4, 7)])
+@pytest.mark.parametrize("name", list(CONFIGS))
+def test_agrees_with_a_launch_per_projection(name, B, k, monkeypatch):
+    cfg = CONFIGS[name]
+    w = inputs.weights_to(inputs.make_weights(cfg, seed=4, gain_jitter=0.05), "cuda")
+    kv_len = 900 if name == "wide" else 150
+    want, kv_want, dlen = _step(cfg, w, B, k, kv_len, kv_len + 40, True, monkeypatch)
+    got, kv_got, _ = _step(cfg, w, B, k, kv_len, kv_len + 40, False, monkeypatch)
+    for b in range(B):                              # rows behind the draft attend to nothing
+        a, c = want[b, :dlen[b] + 1], got[b, :dlen[b] + 1]
+        assert float((a - c).abs().max()) <= float(a.abs().max()) / 256
+    assert float((kv_want - kv_got).abs().max()) <= float(kv_want.abs().max()) / 128
+
+
+def test_wait_runs_out_and_the_context_stays_usable(monkeypatch):
+    """One K block of every run is left out: the MMA warps' waits run out, then those for the tiles that were never
+    finished; nothing hangs, and the next forward is right without anybody asking for the status in between."""
+    monkeypatch.setenv("CS_WAIT_LIMIT_US", "2000")
+    monkeypatch.setenv("CS_NO_CHAIN", "0")
+    cfg = CONFIGS["wide"]
+    ctx, _ = make_pair(cfg, 128, 1, 10)
+    kv0 = inputs.synthetic_kv(cfg, 1, 128, 100, seed=3, device="cuda")
+    tok = i32(np.random.default_rng(0).integers(0, cfg.vocab, size=(1, 11)))
+
+    def step():
+        kv, logits = kv0.clone(), torch.zeros(1, 11, cfg.vocab, dtype=torch.float32, device="cuda")
+        ctx.cs_verify_step(tok[:, 0].contiguous(), tok[:, 1:].contiguous(), i32([10]), kv, i32([100]), logits_dbg=logits)
+        return kv, logits
+
+    want = step()
+    assert ctx.cs_sync_status() == cs.CS_OK
+    for unit in (0, 2):
+        for ask in (True, False):
+            ctx.cs_debug_drop_chain_tile(unit)
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            step()
+            ev[1].record()
+            torch.cuda.synchronize()
+            assert 1.0 <= ev[0].elapsed_time(ev[1]) <= 500.0
+            if ask:
+                assert ctx.cs_sync_status() == cs.CS_ERR_TIMEOUT
+            got = step()
+            assert ctx.cs_sync_status() == (cs.CS_OK if ask else cs.CS_ERR_TIMEOUT)
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert ctx.workspace_guards_intact()
+    ctx.close()
