@@ -386,8 +386,8 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
     ctx->attn_force = (k == nullptr) ? 0 : (strcmp(k, "mma") == 0 ? 1 : (strcmp(k, "tc") == 0 ? 2 : (strcmp(k, "tcw") == 0 ? 3 : 0)));
     const char* ng = getenv("CS_NO_GRAPH");
     ctx->no_graph = ng != nullptr && ng[0] == '1';
-    const char* nc = getenv("CS_NO_CHAIN");
-    ctx->no_chain = nc != nullptr && nc[0] == '1';
+    const char* ch = getenv("CS_CHAIN");
+    ctx->chain_force = ch == nullptr ? 0 : (ch[0] == '0' ? -1 : (ch[0] == '1' ? 1 : 0));
     const char* wl = getenv("CS_WAIT_LIMIT_US");
     const long long us = (wl != nullptr) ? atoll(wl) : 0;
     ctx->wait_limit_ns = (us > 0) ? (unsigned long long)us * 1000ull : 2000000000ull;

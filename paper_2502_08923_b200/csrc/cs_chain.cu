@@ -174,13 +174,18 @@ __device__ __forceinline__ bool take_sums(const uint4* from, size_t step, int n,
 #pragma unroll 1
   for (int c0 = 0; c0 < n; c0 += kB) {
     uint4 w[kB][kP];
+#pragma unroll
+    for (int c = 0; c < kB; ++c)
+#pragma unroll
+      for (int q = 0; q < kP; ++q) w[c][q] = make_uint4(0u, mark, 0u, c0 + c < n && q < pairs ? ~mark : mark);
     for (uint32_t it = 0;; ++it) {
-      bool there = true;
+      // (asks again only for what was not there: the others' sums come at different times)
 #pragma unroll
       for (int c = 0; c < kB; ++c)
 #pragma unroll
         for (int q = 0; q < kP; ++q)
-          w[c][q] = c0 + c < n && q < pairs ? peek_pair(from + (size_t)(c0 + c) * step + q * CS_GEMM_BM) : make_uint4(0u, mark, 0u, mark);
+          if (w[c][q].w != mark || w[c][q].y != mark) w[c][q] = peek_pair(from + (size_t)(c0 + c) * step + q * CS_GEMM_BM);
+      bool there = true;
 #pragma unroll
       for (int c = 0; c < kB; ++c)
 #pragma unroll
@@ -206,16 +211,6 @@ __device__ __forceinline__ bool take_sums(const uint4* from, size_t step, int n,
 __device__ __forceinline__ int uni(int v) { return (int)uniform((uint32_t)v); }
 // Weights are read once per forward: they leave L2 first, so that what the layers pass to one another (and the norms' gains
 // and rotation factors) is still there when it is wanted, instead of waiting in the queue that the weights keep full.
-__device__ __forceinline__ uint64_t evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void load_weights(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "l"(policy) : "memory");
-}
 struct Run {
   int p, i, u0, u1, num_kb, t0, kb0;
 };
@@ -237,7 +232,7 @@ __device__ __forceinline__ Run decode(const ChainArgs& a, int run) {
 
 // The merge of one share of (row, 128 features) items: o = sum_s o_s e^(m_s - M) / sum_s l_s e^(m_s - M).  Several warps per
 // item where a share leaves warps over, each with its share of the slices; a lane holds four features.
-__device__ __forceinline__ void merge_share(const ChainArgs& a, int share, uint8_t* scratch, int warp, int lane) {
+__device__ __forceinline__ void merge_share(const ChainArgs& a, int share, bool first, uint8_t* scratch, int warp, int lane) {
   const int W = a.warps_per_item, part = warp % W, total = a.rows * a.merge_groups;
   float4* s_acc = reinterpret_cast<float4*>(scratch);
   float2* s_ml = reinterpret_cast<float2*>(scratch + kEpiWarps * 32 * 16);
@@ -247,6 +242,9 @@ __device__ __forceinline__ void merge_share(const ChainArgs& a, int share, uint8
     const int row = item / a.merge_groups, g = item - row * a.merge_groups, f = 128 * g + 4 * lane;
     const bool live = item < hi, has = live && f < a.qd;
     const int head = has ? f / a.Dh : 0;
+    const float* from_o = a.attn_o + (size_t)row * a.qd + f;
+    const float2* from_ml = reinterpret_cast<const float2*>(a.attn_ml) + (size_t)row * a.H + head;
+    if (first) asm volatile("griddepcontrol.wait;" ::: "memory");
     float M = -INFINITY, L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s0 = part; s0 < a.nsplit; s0 += W * kSlices) {
@@ -256,9 +254,9 @@ __device__ __forceinline__ void merge_share(const ChainArgs& a, int share, uint8
       for (int q = 0; q < kSlices; ++q) {
         const int s = s0 + q * W;
         const bool in = has && s < a.nsplit;
-        const size_t at = (size_t)s * a.rows + row;
-        v[q] = in ? __ldcg(reinterpret_cast<const float4*>(a.attn_o + at * a.qd + f)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        ml[q] = in ? __ldcg(reinterpret_cast<const float2*>(a.attn_ml) + at * a.H + head) : make_float2(-INFINITY, 0.f);
+        const size_t at = (size_t)s * a.rows;
+        v[q] = in ? __ldcg(reinterpret_cast<const float4*>(from_o + at * a.qd)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        ml[q] = in ? __ldcg(from_ml + at * a.H) : make_float2(-INFINITY, 0.f);
       }
       float m = M;
 #pragma unroll
@@ -494,7 +492,7 @@ k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArg
 
   if (warp == kWWarp) {
     // ------------------------------------------------------------- weights: take runs, stream their tiles
-    const uint64_t policy = evict_first();
+    const uint64_t policy = l2_evict_first();
     auto take = [&]() -> int { return lane == 0 ? atomicAdd(a.ctl + kTicket, 1) : 0; };
     int s = 0, issued = 0, landed = 0, sl = 0;         // slots filled, slots known to have landed, the next one to
     uint32_t ph = 1, eph = 1, lph = 0;                 // (the rings start empty)
@@ -525,8 +523,8 @@ k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArg
         if ((a.drop < u - r.u0 || a.drop >= u - r.u0 + nk) && elect_one()) {
           const uint32_t dst = smem_u32(smem) + (uint32_t)(s * kStep * kWBytes);
           mbar_expect_tx(b_wf + 8 * s, (uint32_t)(nk * kWBytes));
-          load_weights(dst, tm, b_wf + 8 * s, kb * CS_GEMM_BK, t * CS_GEMM_BM, policy);
-          if (nk > 1) load_weights(dst + kWBytes, tm, b_wf + 8 * s, (kb + 1) * CS_GEMM_BK, t * CS_GEMM_BM, policy);
+          tma_load_2d_hint(dst, tm, b_wf + 8 * s, kb * CS_GEMM_BK, t * CS_GEMM_BM, policy);
+          if (nk > 1) tma_load_2d_hint(dst + kWBytes, tm, b_wf + 8 * s, (kb + 1) * CS_GEMM_BK, t * CS_GEMM_BM, policy);
         }
         ++issued;
         kb += nk;
@@ -661,16 +659,16 @@ k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArg
       for (int p = 0; p < 4; ++p) asm volatile("" ::"r"(a.ph[p].first), "r"(a.ph[p].units), "r"(a.ph[p].done), "r"(a.ph[p].mode));
       asm volatile("" ::"r"(a.nsplit), "l"(a.attn_o), "l"(a.attn_ml), "l"(a.attn_out), "r"(a.merge_word), "l"(a.part), "l"(a.epoch), "l"(a.merge_stamp));
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (;;) {                                         // the merge, until nobody has a share left to take
+    for (bool first = true;; first = false) {          // the merge, until nobody has a share left to take
       if (tid == 0) *s_word = share;
       epi_sync();
       const int m = *s_word;
       if (m >= a.merge_shares) break;
+      merge_share(a, m, first, parkb, warp, lane);
       if (tid == 0) share = atomicAdd(a.ctl + kMergeTicket, 1);
-      merge_share(a, m, parkb, warp, lane);
       epi_sync();
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int wq = warp & 3, cg = warp >> 2, feat = wq * 32 + lane;
     const uint32_t lane_base = tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(cg * 2 * NT);
     const uint32_t mark = (uint32_t)__ldcg(a.epoch) * (uint32_t)a.n_layers + (uint32_t)a.layer + 1u;
@@ -812,7 +810,18 @@ size_t cs_chain_words(const cs_model_config* c) {
   return (size_t)chain_words(c->d_model, c->n_heads * c->head_dim, c->d_ffn).total;
 }
 
-bool cs_chain_takes(const cs_ctx* ctx, int rows) { return rows <= CS_CHAIN_MAX_ROWS && !ctx->no_chain; }
+// Short phases do not pay: a hand-over between two projections takes 5 - 6 us whatever they hold, a launch boundary 4 - 5, and
+// only the weights streamed meanwhile make up for it.  Verify steps of 8 layers, launch per projection / chained, us:
+//   436 MB a layer  1 row 793 / 704, 11 rows 830 / 740, 22 rows 873 / 801, 32 rows 1,062 / 1,000
+//   122 MB          1 row 397 / 349, 11 rows 454 / 442, 22 rows 503 / 527, 32 rows 516 / 517
+//    33 MB          1 row 278 / 292, 11 rows 318 / 361;  19 MB 260 / 251, 300 / 307
+bool cs_chain_takes(const cs_ctx* ctx, int rows) {
+  const cs_model_config& c = ctx->cfg;
+  const long long qd = (long long)c.n_heads * c.head_dim, kvd = (long long)c.n_kv_heads * c.head_dim;
+  const long long mb = (2ll * c.d_model * (2 * qd + 2 * kvd + 3ll * c.d_ffn)) >> 20;   // weights of a layer
+  if (rows > CS_CHAIN_MAX_ROWS || ctx->chain_force < 0) return false;
+  return ctx->chain_force > 0 || mb >= 192 || (mb >= 96 && rows <= 12);
+}
 
 cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const QkvEpi* next_q, const __nv_bfloat16* next_gain, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;

@@ -164,7 +164,7 @@ struct cs_ctx {
   unsigned attn_mma_attr_set;   // a bit per head size and key grouping
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
-  bool no_chain;             // CS_NO_CHAIN=1 at creation: a launch per projection whatever the block's height
+  int chain_force;           // 0 = chained projections by block height and layer size, -1 = never, 1 = for layers of any size (CS_CHAIN at creation)
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)

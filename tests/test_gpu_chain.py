@@ -1,7 +1,7 @@
 """The chained projections of short blocks (one launch for everything between two attentions) at the sizes where
 they can go wrong: rows at the edges of their three paddings, widths that are no multiple of the 128-feature tiles or
 of the 64-wide K blocks, every head size, tiles shared by many runs and runs that hold several tiles.  Against a
-launch per projection (CS_NO_CHAIN=1) on the same inputs.
+launch per projection (CS_CHAIN=0) on the same inputs.
 
 Tolerance: both carry activations as two bf16 terms and sum in fp32, in another order, so the first layer agrees to
 about 2^-15; a K or V element of the next layers that this moves across a rounding boundary of bf16 differs by 2^-8 of
@@ -31,7 +31,7 @@ CONFIGS = {
 
 
 def _step(cfg, w, B, k, kv_len, max_seq, alone, monkeypatch):
-    monkeypatch.setenv("CS_NO_CHAIN", "1" if alone else "0")
+    monkeypatch.setenv("CS_CHAIN", "0" if alone else "1")
     ctx = cs.Context(cfg, w, max_seq=max_seq, max_batch=B, k_max=max(k, 1))
     rng = np.random.default_rng(k + kv_len)
     last, draft = i32(rng.integers(0, cfg.vocab, size=B)), i32(rng.integers(0, cfg.vocab, size=(B, k)))
@@ -67,7 +67,7 @@ def test_wait_runs_out_and_the_context_stays_usable(monkeypatch):
     """One K block of every run is left out: the MMA warps' waits run out, then those for the tiles that were never
     finished; nothing hangs, and the next forward is right without anybody asking for the status in between."""
     monkeypatch.setenv("CS_WAIT_LIMIT_US", "2000")
-    monkeypatch.setenv("CS_NO_CHAIN", "0")
+    monkeypatch.setenv("CS_CHAIN", "1")
     cfg = CONFIGS["wide"]
     ctx, _ = make_pair(cfg, 128, 1, 10)
     kv0 = inputs.synthetic_kv(cfg, 1, 128, 100, seed=3, device="cuda")
