@@ -195,12 +195,15 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
   // Slice `split` works on key tiles split, split + nsplit, ...  Items of the ring: K0 K1 V0 K2 V1 ... (one tile: K0 V0)
   const long long krow = ((((long long)a.layer * 2 + 0) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
   const long long vrow = ((((long long)a.layer * 2 + 1) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
+  // (K and V are read once a forward and leave L2 first: us a layer 118.4 -> 117.0 at 4 x 11 rows over 4,096 keys, a prefill
+  // of 4,096 tokens 126.9 -> 126.5 ms)
+  const uint64_t policy = l2_evict_first();
   auto load_tile = [&](int s, long long first, int t) {          // tile t of this slice into slot s (by the elected lane)
     const uint32_t dst = smem_u32(ring) + (uint32_t)(s * kSlotBytes), bar = b_full + 8 * s;
     const int key0 = (split + t * a.nsplit) * kTileKeys;
     mbar_expect_tx(bar, (uint32_t)kSlotBytes);
-    tma_load_2d(dst, &tmKV, bar, 0, (int)(first + key0));
-    tma_load_2d(dst + kHalfBytes, &tmKV, bar, 64, (int)(first + key0));
+    tma_load_2d_hint(dst, &tmKV, bar, 0, (int)(first + key0), policy);
+    tma_load_2d_hint(dst + kHalfBytes, &tmKV, bar, 64, (int)(first + key0), policy);
   };
   // the first items are asked for before the preceding kernel is done while their tiles hold cached keys only
   int asked = 0;
