@@ -472,7 +472,7 @@ def run_ours(args):
     achieved = layer_bytes / gemm_launches / (fam_ms["gemm"] / gemm_launches * 1e-3) / 1e9
     step_bytes = cfg.streamed_params() * 2 + (n0 - 1 + 0.5 * emitted) * cfg.kv_bytes_per_token()
     step_gbs = step_bytes / (ms / K * 1e-3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "k_gemm_tc, k_gemm_pair (layer projections)", "achieved": achieved, "peak": peak,
+    roofline = {"bound": "hbm", "kernel": "k_chain (layer projections; the first layer's QKV: k_gemm_tc)", "achieved": achieved, "peak": peak,
                 "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
                 "traffic": _ncu_traffic(),
                 "bytes_per_launch": layer_bytes / gemm_launches, "launches_per_step": gemm_launches,
