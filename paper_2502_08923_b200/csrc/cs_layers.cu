@@ -26,7 +26,6 @@ __device__ __forceinline__ void clear_chain_words(int4* words, int quads, int* e
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < quads; i += gridDim.x * blockDim.x) words[i] = make_int4(0, 0, 0, 0);
   __threadfence();
   __syncthreads();
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ----------------------------------------------------------------- block assembly
@@ -48,7 +47,8 @@ k_block_setup(const int* last_tok, const int* draft, const int* draft_len, const
                               int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status,
                               int* pair_flag, int4* chain_words, int chain_quads, int* chain_epoch, unsigned long long* stamp) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  clear_chain_words(chain_words, chain_quads, chain_epoch);
+  if (chain_quads > 0) clear_chain_words(chain_words, chain_quads, chain_epoch);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   lower_pair_flags(status, pair_flag);
   const int R = k + 1, rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
@@ -95,8 +95,12 @@ k_prefill_setup(const int* hist, const int* hist_len, int B,
                                 const double* __restrict__ inv_freq, int* row_tok, int* row_pos,
                                 int* row_lim, int* row_write, int* seq_ok, float* rope_cs, int* status, int* pair_flag,
                                 int4* chain_words, int chain_quads, int* chain_epoch) {
+  if (chain_quads == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  clear_chain_words(chain_words, chain_quads, chain_epoch);
+  if (chain_quads > 0) {
+    clear_chain_words(chain_words, chain_quads, chain_epoch);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   lower_pair_flags(status, pair_flag);
   const int rows = B * R;
   for (int row = threadIdx.x; row < rows && blockIdx.x == 0; row += kSetupThreads) {
