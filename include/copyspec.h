@@ -354,7 +354,8 @@ cs_status cs_decode_loop_drafted(cs_ctx* target, cs_ctx* drafter, int32_t* hist,
  * embedding + first norm, the projection GEMMs, the attention and merge kernels, the LM-head
  * GEMM, acceptance, commit - has each of its CTAs leave the nanosecond time (%globaltimer) at
  * which it finished in stamps[i], largest wins, so stamps[i] - stamps[i-1] is what kernel i added
- * to the pipelined step (the index kernels of cs_set_match_index are not stamped: they count
+ * to the pipelined step.  A launch that chains the merge and several projections leaves a stamp for each of them, when the
+ * last part of that phase was finished (the index kernels of cs_set_match_index are not stamped: they count
  * towards the slot that follows).  Set it before cs_loop_begin / the first cs_step_host; it cannot change while a loop
  * is in progress.  cs_stamp_layout returns the number of slots one step uses and writes the
  * kernel family of each slot to the HOST array `family` (0 = layer projection GEMM,

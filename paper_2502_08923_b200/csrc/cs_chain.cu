@@ -8,10 +8,10 @@
 // tiles of all four projections in order, held back by nothing but its ring (192 KB of 16 KB tiles on
 // each of 148 SMs: 4 us of HBM), and only the activations wait for what they depend on.
 // Measured, us a layer with its attention, launch per projection -> this kernel (4,096 keys): 1 row 94.9 -> 82.9, 8 rows
-// 97.3 -> 86.1, 11 rows 99.2 -> 89.2, 16 rows 100.5 -> 91.5, 32 rows 108.9 -> 103.6.  What made it pay, in the order found
+// 97.3 -> 86.1, 11 rows 99.2 -> 88.1, 16 rows 100.5 -> 91.5, 32 rows 108.9 -> 103.0.  What made it pay, in the order found
 // (11 rows): runs taken one at a time behind the wait and not ahead of it (150 -> 109), sums handed over without fences and
 // what finishing needs asked for early (98), two K blocks per ring slot and activations without padding rows (93.5), weights
-// that leave L2 first (89.2).
+// that leave L2 first (89.2), sums asked for again only where they were missing (88.1).
 //
 // Work: each projection's (128-feature tile, 64-wide K block) units are dealt out in equal contiguous runs, one
 // per SM, so a tile is shared by the runs that cover it.  The run that holds the tile's head collects the others' sums
