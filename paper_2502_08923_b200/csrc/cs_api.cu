@@ -191,7 +191,8 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     return QkvEpi{ctx->rope_cs, ctx->row_pos, ctx->row_write, ctx->qbuf, static_cast<__nv_bfloat16*>(kv_cache),
                   R, l, c.n_heads, c.n_kv_heads, c.head_dim, c.max_batch, c.max_seq};
   };
-  if (cs_chain_takes(ctx, rows)) {
+  const bool chained = cs_chain_takes(ctx, rows);
+  if (chained) {
     // short blocks: two launches per layer, the attention and everything up to the next one
     cs_launch_embed_rmsnorm(ctx, ctx->layers[0].attn_norm, rows, st);
     const QkvEpi q0 = qkv_epi(0);
@@ -209,8 +210,8 @@ cs_status enqueue_forward(cs_ctx* ctx, int B, int R, void* kv_cache, bool with_l
     take_norm.slot_stride = ctx->ssq_stride;
     take_norm.inv_d = 1.f / (float)c.d_model;
     take_norm.eps = c.rms_eps;
-  } else
-  for (int l = 0; l < c.n_layers; ++l) {
+  }
+  for (int l = 0; l < c.n_layers && !chained; ++l) {
     const LayerPlan& L = ctx->layers[l];
     if (l == 0) {
       cs_launch_embed_rmsnorm(ctx, L.attn_norm, rows, st);
