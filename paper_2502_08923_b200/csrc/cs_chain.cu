@@ -154,14 +154,16 @@ __device__ __forceinline__ void split4(const float (&v)[4], uint2& hi, uint2& lo
   lo = make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
 }
 // Sums that one run hands to another: every value travels with a word that is different in every launch, so that the
-// reader polls the values themselves and neither side needs a fence (8 aligned bytes are written and read as one).
+// reader polls the values themselves and neither side needs a fence.  A value and its word are one 64-bit element of the
+// access: the elements of a vector access are accesses of their own, in no stated order, but each is written and read whole.
 __device__ __forceinline__ void put_pair(uint4* p, float v0, float v1, uint32_t mark) {
-  asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};"
+  asm volatile("{\n.reg .b64 a, b;\nmov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\nst.volatile.global.v2.b64 [%0], {a, b};\n}"
                ::"l"(p), "r"(__float_as_uint(v0)), "r"(mark), "r"(__float_as_uint(v1)), "r"(mark) : "memory");
 }
 __device__ __forceinline__ uint4 peek_pair(const uint4* p) {
   uint4 v;
-  asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  asm volatile("{\n.reg .b64 a, b;\nld.volatile.global.v2.b64 {a, b}, [%4];\nmov.b64 {%0, %1}, a;\nmov.b64 {%2, %3}, b;\n}"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
   return v;
 }
 // Adds the sums of the runs behind this one that cover the tile, in the order of K: `n` of them, `step` apart, NT tokens of
