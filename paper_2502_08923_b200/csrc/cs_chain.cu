@@ -119,7 +119,10 @@ __device__ __noinline__ uint32_t poll_words(const int* base, int n, int target, 
   for (uint32_t it = 0;; ++it) {
     const int v = lane < n ? ld_acquire(base + lane) : target - 1;
     const uint32_t got = __ballot_sync(0xffffffffu, v >= target);
-    if ((got & want) == want) return got;
+    if ((got & want) == want) {
+      __syncwarp();                                    // what one lane has acquired, all of them may read now (a vote orders no memory)
+      return got;
+    }
     if ((it & 63u) == 63u) {
       bool stop = *abort_flag != 0;
       const unsigned long long now = globaltimer_ns();

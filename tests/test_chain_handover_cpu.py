@@ -23,3 +23,9 @@ def test_a_sum_and_its_mark_are_one_element_of_the_access():
         accesses = re.findall(r"\b(ld|st)\.[\w.]*global[\w.]*", _function(name))
         assert accesses == [kind], name
         assert re.search(rf"\b{kind}\.[\w.]*global\.v2\.b64\b", _function(name)), name
+
+
+def test_a_poll_by_a_warp_orders_memory_for_all_its_lanes():
+    # the lane whose word it was has acquired it; a vote says so to the others but orders nothing for them
+    body = _function("poll_words")
+    assert "ld_acquire" in body and re.search(r"__ballot_sync.*__syncwarp\(\);\s*return got;", body, flags=re.S)
