@@ -230,11 +230,15 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
   // range only has to let them land).
   const long long krow = ((((long long)a.layer * 2 + 0) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
   const long long vrow = ((((long long)a.layer * 2 + 1) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
+  // (K and V leave L2 first, as the weights do that follow them: left at normal priority they keep all of L2 and what the layers
+  // pass to one another goes to HBM.  us a layer of the 8B shape, 8 x 4 rows over 8,000 keys 141.7 -> 130.0, 2 x 11 rows over
+  // 30,000 139.0 -> 127.4; above 32 rows, 4 x 11 over 16,384 148.4 -> 143.4)
+  const uint64_t policy = l2_evict_first();
   auto load_tile = [&](uint32_t buf, uint32_t bar, long long first, int i) {   // tile i of this slice (by the elected lane)
     const int key0 = (split + i * a.nsplit) * kTileKeys;
     mbar_expect_tx(bar, 2u * kHalfBytes);
-    tma_load_2d(buf, &tmKV, bar, 0, (int)(first + key0));
-    tma_load_2d(buf + kHalfBytes, &tmKV, bar, 64, (int)(first + key0));
+    tma_load_2d_hint(buf, &tmKV, bar, 0, (int)(first + key0), policy);
+    tma_load_2d_hint(buf + kHalfBytes, &tmKV, bar, 64, (int)(first + key0), policy);
   };
   // one producer warp feeds K, one feeds V
   const bool is_k = warp == kProdWarp, is_prod = is_k || warp == kVProdWarp;
