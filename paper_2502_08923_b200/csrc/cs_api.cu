@@ -307,11 +307,6 @@ cs_status take_status(cs_ctx* ctx, int* bits, cudaStream_t st) {
   return CS_OK;
 }
 
-long long layer_bytes(const cs_model_config& c) {
-  const long long d = c.d_model, qd = (long long)c.n_heads * c.head_dim, kvd = (long long)c.n_kv_heads * c.head_dim;
-  return 2 * d * (2 * qd + 2 * kvd + 3ll * c.d_ffn);
-}
-
 // One reporting step of the loop as a graph (captured on the context's own stream: the legacy default stream
 // cannot).  Without it the loop goes on enqueueing, so a failure here is not one of the call.
 void capture_step(cs_ctx* ctx) {
@@ -865,7 +860,7 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
     } else {
       r = enqueue_loop_step(ctx, st, true);
     }
-    if (sent == 2 && r == CS_OK && wanted > (long)4 * (k + 1) && !ctx->no_graph && layer_bytes(ctx->cfg) >= (32ll << 20))
+    if (sent == 2 && r == CS_OK && wanted > (long)4 * (k + 1) && !ctx->no_graph && cs_layer_bytes(ctx->cfg) >= (32ll << 20))
       capture_step(ctx);
     return r;
   };

@@ -815,18 +815,37 @@ size_t cs_chain_words(const cs_model_config* c) {
   return (size_t)chain_words(c->d_model, c->n_heads * c->head_dim, c->d_ffn).total;
 }
 
-// Short phases do not pay: a hand-over between two projections takes 5 - 6 us whatever they hold, a launch boundary 4 - 5, and
-// only the weights streamed meanwhile make up for it.  Verify steps of 8 layers, launch per projection / chained, us:
-//   436 MB a layer  1 row 793 / 704, 11 rows 830 / 740, 22 rows 873 / 801, 32 rows 1,062 / 1,000
-//   122 MB          1 row 397 / 349, 11 rows 454 / 442, 22 rows 503 / 527, 32 rows 516 / 517
-//    33 MB          1 row 278 / 292, 11 rows 318 / 361;  19 MB 260 / 251, 300 / 307
-bool cs_chain_takes(const cs_ctx* ctx, int rows) {
-  const cs_model_config& c = ctx->cfg;
-  const long long qd = (long long)c.n_heads * c.head_dim, kvd = (long long)c.n_kv_heads * c.head_dim;
-  const long long mb = (2ll * c.d_model * (2 * qd + 2 * kvd + 3ll * c.d_ffn)) >> 20;   // weights of a layer
-  if (rows > CS_CHAIN_MAX_ROWS || ctx->chain_force < 0) return false;
-  return ctx->chain_force > 0 || mb >= 192 || (mb >= 96 && rows <= 12);
+// Highest block that is chained.  A hand-over between two projections takes 5 - 6 us whatever they hold, a launch boundary
+// 4 - 5, and only the weights streamed meanwhile make up for it; the taller the block, the more sums it has to hand over,
+// and heads of 64 come in more key slices, whose merge is part of the launch.  Verify steps of 8 layers over 500 to 30,000 keys,
+// 1 to 32 sequences, launch per projection / chained, us at 2,000 keys (rows of one sequence; S = one row each of so many):
+//   MiB a layer              1        8       11      12 S     16       24       32       32 S
+//   416                   779/685  807/703  817/721  963/885  827/731  868/780  897/809  1293/1230
+//   288, heads of 64      602/530  660/571  681/604  710/651  696/626  754/696  794/736   908/886
+//   245, narrow (d 2,048) 597/528  624/548  633/584  690/655  642/593  664/652  678/680   834/876
+//   245, heads of 64      559/507  613/545  643/602  669/644  650/615  706/689  718/719   848/881
+//   192                   502/441  532/461  540/490  683/657  549/500  573/534  592/560   940/940
+//   195, heads of 64      487/442  537/483  561/539  586/582  568/554  625/630  636/654   770/822
+//   154                   449/418  478/442  482/468  545/540  494/479  520/535  536/549   682/743
+//   135                   429/398  454/420  458/446  524/514  472/458  496/514  514/528   662/722
+//   122                   416/370  438/387  436/415  505/498  443/428  471/474  486/506   639/726
+//   116, heads of 64      395/365  426/400  436/442  494/479  451/461  491/494  504/539   672/727
+//   112, QKV of 3 d       409/394  434/418  440/447  594/624  447/463  482/518  493/558   843/939
+//   108, heads of 64      386/389  416/430  424/480  483/492  434/505  482/489  495/546   662/727
+//    98                   390/346  404/366  411/393  474/483  420/406  443/458  462/483   617/689
+//    92, heads of 64      367/363  400/399  404/455  466/461  417/476  462/489  477/593   645/728
+// The lines lie where the worst of the lengths and batches is no loss (at most 1 %: 154 MiB, heads of 64, 12 sequences).  Below
+// them some layers gain (92 MiB with heads of 128 at 1 row 381/334) and others lose a quarter (32 MiB at 22 rows 360/485).
+int cs_chain_max_rows(const cs_model_config& c, int force) {
+  if (force != 0) return force > 0 ? CS_CHAIN_MAX_ROWS : 0;
+  const long long mib = cs_layer_bytes(c) >> 20;
+  const bool wide = c.head_dim == 128;
+  if (mib >= 280) return CS_CHAIN_MAX_ROWS;
+  if (mib >= 192 && wide) return 24;
+  if (mib >= 128) return 12;
+  return mib >= (wide ? 96 : 112) && (c.n_heads + 2 * c.n_kv_heads) * c.head_dim <= 2 * c.d_model ? 8 : 0;
 }
+bool cs_chain_takes(const cs_ctx* ctx, int rows) { return rows <= cs_chain_max_rows(ctx->cfg, ctx->chain_force); }
 
 cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const QkvEpi* next_q, const __nv_bfloat16* next_gain, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;

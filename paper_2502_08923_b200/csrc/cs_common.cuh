@@ -164,7 +164,7 @@ struct cs_ctx {
   unsigned attn_mma_attr_set;   // a bit per head size and key grouping
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
-  int chain_force;           // 0 = chained projections by block height and layer size, -1 = never, 1 = for layers of any size (CS_CHAIN at creation)
+  int chain_force;           // 0 = chained projections by block height and shape of the layer, -1 = never, 1 = for layers of any size (CS_CHAIN at creation)
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
@@ -319,8 +319,14 @@ int cs_norm_slots(const GemmPlan* g, int rows);   // sums of squares per token t
 cs_status cs_launch_gemm_pair(cs_ctx* ctx, const GemmPlan* g, const CUtensorMap* tmX, int lo_row, int rows, int mode, float* out,
                               __nv_bfloat16* act, __nv_bfloat16* act_lo, int F, const QkvEpi* q, const NormFuse* nf,
                               cudaStream_t st);
+// weights of a layer
+static inline long long cs_layer_bytes(const cs_model_config& c) {
+  const long long d = c.d_model, qd = (long long)c.n_heads * c.head_dim, kvd = (long long)c.n_kv_heads * c.head_dim;
+  return 2 * d * (2 * qd + 2 * kvd + 3ll * c.d_ffn);
+}
 // cs_chain.cu: merge of the attention's slices, attention output, gate/up, down and the next layer's QKV in one launch
 size_t cs_chain_words(const cs_model_config* c);   // control words of a layer
+int cs_chain_max_rows(const cs_model_config& c, int force);
 bool cs_chain_takes(const cs_ctx* ctx, int rows);
 // next_q = where the next layer's QKV projection puts its results (NULL behind the last layer), next_gain = gain of the norm behind this layer
 cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const QkvEpi* next_q, const __nv_bfloat16* next_gain, cudaStream_t st);

@@ -96,3 +96,29 @@ def test_wait_runs_out_and_the_context_stays_usable(monkeypatch):
             assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert ctx.workspace_guards_intact()
     ctx.close()
+
+
+# what decides whether a block is chained: MiB of a layer's weights, head size, QKV features against model features
+RULE = {"89": (_cfg(2048, 16, 4, 128, 5888, layers=1), 0), "98": (_cfg(2048, 16, 4, 128, 6656, layers=1), 8),
+        "98, QKV of 3 d": (_cfg(2048, 16, 16, 128, 5632, layers=1), 0), "108, heads of 64": (_cfg(2048, 32, 8, 64, 7488, layers=1), 0),
+        "116, heads of 64": (_cfg(2048, 32, 8, 64, 8192, layers=1), 8), "135": (_cfg(2560, 20, 4, 128, 7168, layers=1), 12),
+        "192": (_cfg(3072, 24, 8, 128, 8192, layers=1), 24), "195, heads of 64": (_cfg(3072, 48, 8, 64, 8704, layers=1), 12),
+        "245": (_cfg(2048, 16, 4, 128, 19200, layers=1), 24), "287": (_cfg(3584, 28, 4, 128, 11264, layers=1), 32)}
+
+
+@pytest.mark.parametrize("name", list(RULE))
+def test_blocks_are_chained_where_that_was_measured_to_gain(name, monkeypatch):
+    """Three launches a layer where the block is chained, six where it is not."""
+    monkeypatch.delenv("CS_CHAIN", raising=False)
+    cfg, most = RULE[name]
+    ctx = cs.Context(cfg, inputs.make_weights(cfg, seed=4, device="cuda"), max_seq=64, max_batch=1, k_max=32)
+    launches = []
+    for rows in (1, 8, 9, 12, 13, 24, 25, 32, 33):
+        hd, ld, kvl = i32(np.zeros((1, 64))), i32([8]), i32([7])
+        ctx.cs_loop_begin(hd, ld, ctx.alloc_kv(), kvl, 3, rows - 1, 4)
+        launches.append((rows, ctx.cs_loop_launches_per_step()))
+        ctx.cs_loop_end()
+    ctx.close()
+    most_launches = max(n for _, n in launches)
+    assert [rows for rows, n in launches if n == most_launches - 3] == [r for r in (1, 8, 9, 12, 13, 24, 25, 32, 33) if r <= most]
+    assert {n for _, n in launches} <= {most_launches, most_launches - 3}
