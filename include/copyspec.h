@@ -52,7 +52,7 @@
  * stream, norms, RoPE and softmax are fp32.  Only K/V rows are rounded (to nearest-even bf16)
  * when they are stored in the cache.
  *
- * Environment, read once by cs_create (measurement and test switches; not needed in use):
+ * Environment, read once by cs_create, CS_CHAIN by cs_workspace_bytes too (measurement and test switches; not needed in use):
  *   CS_NO_GRAPH=1          cs_loop_steps and cs_decode_loop enqueue their steps kernel by kernel, as the other calls
  *                          do, instead of replaying them from a captured CUDA graph;
  *   CS_CHAIN=0|1           blocks of at most 32 rows: a launch per projection (0), or one launch per layer for everything

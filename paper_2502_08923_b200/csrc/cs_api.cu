@@ -39,6 +39,12 @@ size_t take(size_t* off, size_t bytes) {
   return at;
 }
 
+// CS_CHAIN: chained projections 0 = by the shape of the layer, -1 = never, 1 = always
+int chain_switch() {
+  const char* v = getenv("CS_CHAIN");
+  return v == nullptr ? 0 : (v[0] == '0' ? -1 : (v[0] == '1' ? 1 : 0));
+}
+
 WsLayout ws_layout(const cs_model_config* c) {
   WsLayout L;
   const size_t rows = CS_MAX_ROWS;
@@ -71,9 +77,10 @@ WsLayout ws_layout(const cs_model_config* c) {
   L.iota = take(&off, rows * 4);
   L.pair_part = take(&off, (size_t)CS_MAX_PAIRS * 2 * CS_MAX_ROWS * CS_GEMM_BM * 4);
   L.pair_flag = take(&off, CS_MAX_PAIRS * 2 * 4);
-  L.chain_part = take(&off, (size_t)4 * CS_CHAIN_MAX_RUNS * CS_CHAIN_MAX_ROWS / 2 * CS_GEMM_BM * sizeof(uint4));
-  L.chain_epoch = take(&off, 256);
-  L.chain_ctl = take(&off, (size_t)c->n_layers * cs_chain_words(c) * 4);
+  const size_t chained = cs_chain_max_rows(*c, chain_switch()) > 0 ? 1 : 0;   // (21 MB that other models need not hold)
+  L.chain_part = take(&off, chained * 4 * CS_CHAIN_MAX_RUNS * CS_CHAIN_MAX_ROWS / 2 * CS_GEMM_BM * sizeof(uint4));
+  L.chain_epoch = take(&off, chained * 256);
+  L.chain_ctl = take(&off, chained * c->n_layers * cs_chain_words(c) * 4);
   L.status = take(&off, 256);
   L.loop_last = take(&off, rows * 4);
   L.loop_draft = take(&off, rows * 4);
@@ -377,13 +384,12 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
   ctx->rows_pad = CS_MAX_ROWS;
   ctx->attn_splits = L.attn_splits;
   {
-    // the environment switches of the library, all read here and nowhere else
+    // the environment switches of the library, all read here (CS_CHAIN for the size of the workspace too) and nowhere else
     const char* k = getenv("CS_ATTN_KERNEL");
     ctx->attn_force = (k == nullptr) ? 0 : (strcmp(k, "mma") == 0 ? 1 : (strcmp(k, "tc") == 0 ? 2 : (strcmp(k, "tcw") == 0 ? 3 : 0)));
     const char* ng = getenv("CS_NO_GRAPH");
     ctx->no_graph = ng != nullptr && ng[0] == '1';
-    const char* ch = getenv("CS_CHAIN");
-    ctx->chain_force = ch == nullptr ? 0 : (ch[0] == '0' ? -1 : (ch[0] == '1' ? 1 : 0));
+    ctx->chain_force = chain_switch();
     const char* wl = getenv("CS_WAIT_LIMIT_US");
     const long long us = (wl != nullptr) ? atoll(wl) : 0;
     ctx->wait_limit_ns = (us > 0) ? (unsigned long long)us * 1000ull : 2000000000ull;

@@ -45,6 +45,21 @@ def test_workspace_bytes_is_host_arithmetic():
     assert lib.cs_workspace_bytes(C.byref(bad)) == 0
 
 
+def test_only_contexts_that_chain_hold_its_workspace(monkeypatch):
+    """The sums that the chained projections hand over take 21 MB; models whose layers are never chained do without."""
+    lib = cs.load()
+
+    def size(cfg, switch):
+        monkeypatch.delenv("CS_CHAIN", raising=False)
+        if switch is not None:
+            monkeypatch.setenv("CS_CHAIN", switch)
+        return lib.cs_workspace_bytes(C.byref(_cfg(cfg)))
+
+    part = 4 * 160 * 16 * 128 * 16
+    assert size(inputs.TINY, None) == size(inputs.TINY, "0") <= size(inputs.TINY, "1") - part
+    assert size(inputs.LLAMA8B, None) == size(inputs.LLAMA8B, "1") >= size(inputs.LLAMA8B, "0") + part
+
+
 def test_find_match_argument_errors_need_no_device():
     lib = cs.load()
     assert lib.cs_find_match(None, None, 0, 0, 3, 10, 0, None, None, None, None) == cs.CS_OK       # B == 0
