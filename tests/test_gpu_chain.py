@@ -11,8 +11,9 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import copyspec_oracle as O
 from paper_2502_08923_b200 import binding as cs, inputs
-from helpers import i32, make_pair
+from helpers import LOGIT_TOL, i32, make_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -27,7 +28,10 @@ CONFIGS = {
     "shared": _cfg(256, 16, 2, 128, 9000),          # tiles of down shared by 35 runs
     "wide": _cfg(2048, 16, 4, 64, 2048),            # gate/up: runs inside a tile; many key slices to merge
     "long": _cfg(256, 2, 1, 128, 20000),            # runs that hold several whole tiles
+    "deep": _cfg(4104, 2, 1, 128, 328),             # norms of 33 tiles: their words, and the projections', beyond one window of 32
 }
+# at 32 rows the merge has more slices than a warp's first pass takes: 29 for one warp an item, 49 for two (keys)
+SLICES = {"one warp": (_cfg(256, 20, 5, 128, 1024, layers=2), 4000), "two warps": (_cfg(256, 12, 3, 128, 1024, layers=2), 6500)}
 
 
 def _step(cfg, w, B, k, kv_len, max_seq, alone, monkeypatch):
@@ -63,8 +67,68 @@ def test_agrees_with_a_launch_per_projection(name, B, k, monkeypatch):
     assert float((kv_want - kv_got).abs().max()) <= float(kv_want.abs().max()) / 128
 
 
+@pytest.mark.parametrize("name", list(SLICES))
+def test_merge_takes_its_slices_in_several_passes(name, monkeypatch):
+    cfg, kv_len = SLICES[name]
+    w = inputs.weights_to(inputs.make_weights(cfg, seed=4, gain_jitter=0.05), "cuda")
+    want, kv_want, _ = _step(cfg, w, 1, 31, kv_len, kv_len + 40, True, monkeypatch)
+    got, kv_got, _ = _step(cfg, w, 1, 31, kv_len, kv_len + 40, False, monkeypatch)
+    assert float((want - got).abs().max()) <= float(want.abs().max()) / 256
+    assert float((kv_want - kv_got).abs().max()) <= float(kv_want.abs().max()) / 128
+
+
+@pytest.mark.parametrize("rows", [1, 11, 32])
+@pytest.mark.parametrize("name", ["ragged", "shared", "long", "deep"])
+def test_agrees_with_the_oracle(name, rows, monkeypatch):
+    """Logits and appended keys and values against the 64-bit oracle; tolerances as for a launch per projection."""
+    monkeypatch.setenv("CS_CHAIN", "1")
+    cfg = inputs.ModelConfig(**{**CONFIGS[name].__dict__, "n_layers": 2})
+    ctx, model = make_pair(cfg, 200, 1, 31, gain_jitter=0.05)
+    kv_len = 70
+    kv = inputs.synthetic_kv(cfg, 1, 200, kv_len, seed=3, device="cuda")
+    cache = O.KVCache(cfg, 1, 200)
+    cache.a[:, :, :, :, :kv_len] = kv[:, :, :, :, :kv_len].float().cpu().numpy()
+    tok = np.random.default_rng(rows).integers(0, cfg.vocab, size=rows).astype(np.int32)
+    logits = torch.zeros(1, rows, cfg.vocab, dtype=torch.float32, device="cuda")
+    ctx.cs_verify_step(i32(tok[:1]), i32(tok[None, 1:]), i32([rows - 1]), kv, i32([kv_len]), logits_dbg=logits)
+    assert ctx.cs_sync_status() == cs.CS_OK
+    want = model.forward_block(tok.tolist(), kv_len, cache, 0)
+    assert float(np.abs(logits[0].cpu().numpy() - want).max()) <= LOGIT_TOL
+    new = slice(kv_len, kv_len + rows)
+    assert float(np.abs(kv[:, :, 0, :, new].float().cpu().numpy() - cache.a[:, :, 0, :, new]).max()) <= 2e-2
+    ctx.close()
+
+
+@pytest.mark.parametrize("B,rows", [(1, 1), (1, 17), (1, 32), (3, 10), (2, 1)])
+@pytest.mark.parametrize("name", ["ragged", "wide"])
+def test_prefill_ends_in_a_short_chunk(name, B, rows, monkeypatch):
+    """A chunk of full height (on SM pairs), then one that is chained: its last layer has neither a QKV projection nor
+    a norm behind it.  A verify step over the cache follows."""
+    cfg = CONFIGS[name]
+    w = inputs.weights_to(inputs.make_weights(cfg, seed=4, gain_jitter=0.05), "cuda")
+    n = 256 // B + rows + 1
+    rng = np.random.default_rng(rows)
+    hist, last, draft = rng.integers(0, cfg.vocab, size=(B, n + 7)), rng.integers(0, cfg.vocab, size=B), rng.integers(0, cfg.vocab, size=(B, 4))
+    outs = []
+    for switch in "01":
+        monkeypatch.setenv("CS_CHAIN", switch)
+        ctx = cs.Context(cfg, w, max_seq=n + 40, max_batch=B, k_max=4)
+        kv, kvl, lens = ctx.alloc_kv(), i32(np.zeros(B)), i32([n] + [n - 1] * (B - 1))
+        for _ in range(2):
+            kv.zero_()
+            ctx.cs_prefill(i32(hist), lens, n, kv, kvl)
+        assert kvl.cpu().tolist() == [n - 1] + [n - 2] * (B - 1)
+        logits = torch.zeros(B, 5, cfg.vocab, dtype=torch.float32, device="cuda")
+        ctx.cs_verify_step(i32(last), i32(draft), i32([4] * B), kv, kvl, logits_dbg=logits)
+        assert ctx.cs_sync_status() == cs.CS_OK and ctx.workspace_guards_intact()
+        outs.append((logits, kv.float()))
+        ctx.close()
+    for a, c, share in zip(outs[0], outs[1], (256, 128)):
+        assert float((a - c).abs().max()) <= float(a.abs().max()) / share
+
+
 def test_wait_runs_out_and_the_context_stays_usable(monkeypatch):
-    """One K block of every run is left out: the MMA warps' waits run out, then those for the tiles that were never
+    """One ring slot of every run is left out: the MMA warps' waits run out, then those for the tiles that were never
     finished; nothing hangs, and the next forward is right without anybody asking for the status in between."""
     monkeypatch.setenv("CS_WAIT_LIMIT_US", "2000")
     monkeypatch.setenv("CS_CHAIN", "1")
