@@ -47,8 +47,8 @@ WORKLOAD = "verify_8b_b1_kv4096_k10_scripted_tau_uniform"
 SAMPLE_LAYERS = 4          # decoder layers of the CPU oracle's bounded sample
 
 # DRAM counters of the dominant kernel, written beside its ncu summary: `key = value` lines
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_gemm_tc_verify8b_2layer_ncu_traffic.txt")
-KERNEL_SOURCES = [os.path.join(ROOT, "paper_2502_08923_b200", "csrc", f) for f in ("cs_gemm.cu", "cs_gemm_pair.cu", "cs_tcgen.cuh", "cs_common.cuh")]
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_chain_verify8b_2layer_ncu_traffic.txt")
+KERNEL_SOURCES = [os.path.join(ROOT, "paper_2502_08923_b200", "csrc", f) for f in ("cs_chain.cu", "cs_tcgen.cuh", "cs_common.cuh")]
 
 
 def _kernel_hash():
@@ -59,9 +59,10 @@ def _kernel_hash():
     return h.hexdigest()[:16]
 
 
-def _ncu_traffic():
+def _ncu_traffic(layers):
     """dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel from the
-    committed capture, or None when there is none or the kernel's source changed since."""
+    committed capture (mean over the launches of a step; the last one holds no QKV projection), or
+    None when there is none or the kernel's source changed since."""
     try:
         kv = {}
         for line in open(TRAFFIC_FILE):
@@ -70,7 +71,7 @@ def _ncu_traffic():
                 kv[k.strip()] = v.strip()
         if kv.get("kernel_source_sha256_16") != _kernel_hash():
             return None
-        return float(kv["dram_bytes_per_projection_launch"])
+        return ((layers - 1) * float(kv["dram_bytes_per_launch"]) + float(kv["dram_bytes_last_launch"])) / layers
     except Exception:
         return None
 
@@ -466,20 +467,29 @@ def run_ours(args):
             fam_ms[f] += (ends[i, j] - (ends[i, j - 1] if j else prev)) * 1e-6 / S
             fam_n[f] += 1 if i == 1 else 0
     timeline_step = float(np.mean(step_ms))
+    # Blocks of this height run as two launches per layer: the attention, and everything up to the next one (k_chain: the merge,
+    # O, gate/up, down and the next QKV), which leaves a stamp for each of its phases.  Its time is all of them, its weights are
+    # all but the first layer's QKV, a launch of its own (the first "gemm" stamp).  With CS_CHAIN=0 every stamp is a launch.
+    chained = launches_per_step < nst
     layer_bytes = cfg.n_layers * cfg.params_per_layer() * 2
-    gemm_launches = max(1, fam_n["gemm"])
+    first_gemm = fams.index("gemm")
+    first_ms = float(np.mean(ends[1:, first_gemm] - ends[1:, first_gemm - 1])) * 1e-6
+    kernel_ms = fam_ms["gemm"] + (fam_ms["merge"] - first_ms if chained else 0.0)
+    kernel_bytes = layer_bytes - (cfg.qkv_dim * cfg.d_model * 2 if chained else 0)
+    kernel_launches = cfg.n_layers if chained else max(1, fam_n["gemm"])
     peak, peak_kind = _peaks()
-    achieved = layer_bytes / gemm_launches / (fam_ms["gemm"] / gemm_launches * 1e-3) / 1e9
+    achieved = kernel_bytes / (kernel_ms * 1e-3) / 1e9
     step_bytes = cfg.streamed_params() * 2 + (n0 - 1 + 0.5 * emitted) * cfg.kv_bytes_per_token()
     step_gbs = step_bytes / (ms / K * 1e-3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "k_chain (layer projections; the first layer's QKV: k_gemm_tc)", "achieved": achieved, "peak": peak,
-                "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
-                "traffic": _ncu_traffic(),
-                "bytes_per_launch": layer_bytes / gemm_launches, "launches_per_step": gemm_launches,
-                "how": ("kernel time = end of its last CTA minus end of the preceding kernel's last CTA (%globaltimer stamps inside "
-                        f"the pipelined step graph, mean of {S} consecutive steps); the families add up to the step"),
-                "timeline_ms_per_step": fam_ms, "timeline_launches_per_step": fam_n, "timeline_step_ms": timeline_step,
-                "dominant_kernel_share_of_step": fam_ms["gemm"] / timeline_step,
+    roofline = {"bound": "hbm", "kernel": "k_chain (merge, layer projections)" if chained else "k_gemm_tc, k_gemm_pair (layer projections)",
+                "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
+                "traffic": _ncu_traffic(cfg.n_layers) if chained else None,
+                "bytes_per_launch": kernel_bytes / kernel_launches, "launches_per_step": kernel_launches, "ms_per_step": kernel_ms,
+                "how": ("%globaltimer stamps inside the pipelined step graph, one when the last CTA of a launch, or of a phase of k_chain, was "
+                        f"done; a share = its stamp minus the one before it, mean of {S} consecutive steps, so the families add up to the step; "
+                        "achieved = weights of the launches named / all their shares, the merge that k_chain holds among them"),
+                "timeline_ms_per_step": fam_ms, "timeline_stamps_per_step": fam_n, "timeline_step_ms": timeline_step,
+                "dominant_kernel_share_of_step": kernel_ms / timeline_step,
                 "step": {"algorithmic_gb": step_bytes / 1e9, "achieved_gbs": step_gbs, "frac_of_measured_copy": step_gbs / peak,
                          "frac_of_8tbs": step_gbs / 8000.0}}
 

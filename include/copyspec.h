@@ -390,7 +390,8 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block);
 
 /* The same for the chained projections of blocks of at most 32 rows: the next such launch leaves out the
- * weights of the unit-th K block of every run it hands to an SM.  unit < 0 clears it. */
+ * weights that travel with the unit-th K block of every run it hands to an SM (a ring slot: up to two blocks).
+ * unit < 0 clears it. */
 cs_status cs_debug_drop_chain_tile(cs_ctx* ctx, int unit);
 
 /* Test hook for the hand-over of work between SM pairs (no counterpart in the paper): where the K

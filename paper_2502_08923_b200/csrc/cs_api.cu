@@ -615,8 +615,8 @@ cs_status cs_step_host(cs_ctx* ctx, int32_t* hist_host, int32_t* hist_len_host, 
   *ctx->progress = 0ull;
   cs_launch_host_in(ctx->step_in_dev, B, tokens, script_ints, stride, hist_dev, hist_len_dev, ctx->loop_emitted, st);
   // ---- App. B.3 step 1 (search, gather), step 2 (verify, accept, truncate).  Enqueued launch by launch:
-  // the device starts on the first kernel while the rest is enqueued (0.45 ms of host time beside 3.4 ms
-  // on the device at the 8B shape; a graph replay took 0.16 ms before the first kernel began).
+  // the device starts on the first kernel while the rest is enqueued (0.16 ms of host time beside 3.0 ms
+  // on the device at the 8B shape, 0.45 beside 3.4 with a launch per projection; a graph replay took 0.16 ms before the first kernel began).
   ctx->stamp_n = 0;
   cs_status s = cs_launch_find_match(hist_dev, hist_len_dev, B, stride, gamma, k, (int)policy, ctx->loop_mpos,
                                      ctx->loop_draft, ctx->loop_dlen, ctx->loop_last, nullptr, st);
@@ -844,13 +844,14 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   cs_status s = loop_prepare(ctx, hist, hist_len, B, stride, kv_cache, kv_len, gamma, k, policy, max_new, eos_id,
                              script, stream);
   if (s != CS_OK) return s;
-  // The first two steps are enqueued launch by launch (0.45 ms of host time each against 3.4 ms on the device at
-  // the 8B shape, 42 against 72 us for two small layers), at most two ahead of the device.  The device
+  // The first two steps are enqueued launch by launch (0.16 ms of host time each against 3.0 ms on the device at
+  // the 8B shape, 0.45 against 3.4 with a launch per projection, 42 against 72 us for two small layers), at most two ahead of the device.  The device
   // reports after every step how many tokens are still wanted, and a step is enqueued ahead of that report
   // only where it is needed whatever the steps in flight accept: the loop used to look every four
   // steps and ran up to three whole forwards for nothing.
-  // While those two run the host captures the step and replays it from then on: the projections of a step
-  // enqueued directly take 3.44 instead of 3.35 ms.  Building the graph takes 1 - 2 ms, so it is only done where
+  // While those two run the host captures the step and replays it from then on: with a launch per projection a step
+  // enqueued directly takes 3.44 instead of 3.35 ms.  (Chained layers do not need it: calls of 4, 8, 11 and 24 steps at the 8B shape
+  // take 2.97, 2.97, 2.95 and 2.96 ms a step with a graph, 2.97, 2.96, 2.96 and 2.96 without.)  Building the graph takes 1 - 2 ms, so it is only done where
   // two steps last longer (32 MB of weights a layer; at 2 MB they last 0.15 ms) and at least three more are certain.
   // Calls of 8 steps with a graph and without, us a step: 24 layers of 34 MB 957 / 1,006, 28 of 93 MB 1,393 / 1,442, 16 of
   // 122 MB 935 / 965.  Destroying the graph takes 0.1 - 0.6 ms, so that is done while what will likely be the last steps

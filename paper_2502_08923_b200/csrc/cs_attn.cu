@@ -356,12 +356,12 @@ int cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int
   // head_dim 128 runs on the tcgen05 kernels.  The one with the query rows as M does a tile's work of
   // 128 rows whatever the block holds, but has the shorter chain; the one with keys and head dims as M does
   // only that of the real rows, and takes blocks of up to 48 rows per KV head whose CTAs walk many tiles.
-  // Measured per layer, rows as M / keys as M, attention and merge, 44 rows: 13 tiles 32.4 / 33.2 us,
-  // 16 tiles 36.1 / 37.2 (and its successor starts 2 us sooner), 27 tiles 52.1 / 49.6, 32 tiles 59.1 / 54.8,
-  // 64 tiles 118 / 102.5; 84 rows, 64 tiles: 114 / 142.  Blocks of few rows would gain from the other kernel
-  // much sooner than this line: 4 rows, 2 tiles 12.8 / 13.8, 4 tiles 16.5 / 16.2, 8 tiles 23.0 / 20.3, 16 tiles 33.4 / 29.4,
-  // 32 tiles 54.1 / 47.3; 16 rows, 4 tiles 16.5 / 16.6, 8 tiles 22.7 / 20.9, 14 tiles 31.2 / 28.8; 28 rows, 8 tiles
-  // 22.5 / 23.6, 14 tiles 31.5 / 31.3.  The register-resident mma.sync kernel takes the other head sizes.
+  // Measured per layer, rows as M / keys as M, attention and merge, 44 rows: 14 tiles 30.3 / 28.6 us, 17 tiles
+  // 34.5 / 31.9, 20 tiles 39.8 / 35.7, 28 tiles 50.7 / 44.3, 33 tiles 58.0 / 49.7, 65 tiles 113.8 / 89.8; 84 rows,
+  // 65 tiles: 120.2 / 173.9.  The line is older than these figures (K and V of the other kernel did not leave L2 first,
+  // 13 tiles were 32.4 / 33.2 and 16 tiles 36.1 / 37.2), and blocks of few rows would gain from that kernel sooner still: 4 rows, 5 tiles
+  // 18.0 / 18.1, 9 tiles 23.8 / 21.4, 17 tiles 35.0 / 30.8, 32 tiles 56.4 / 48.5; 16 rows, 5 tiles 20.2 / 18.7, 9 tiles
+  // 24.9 / 22.1, 14 tiles 32.4 / 29.1, 32 tiles 56.5 / 49.6; 28 rows, 9 tiles 25.0 / 25.1, 15 tiles 32.7 / 31.2.  The register-resident mma.sync kernel takes the other head sizes.
   // CS_ATTN_KERNEL=tc|tcw|mma, read when the context is created, forces one of them (tests run
   // them on the same inputs).
   int nsplit = 0;

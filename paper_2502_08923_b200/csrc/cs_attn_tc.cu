@@ -195,8 +195,10 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
   // Slice `split` works on key tiles split, split + nsplit, ...  Items of the ring: K0 K1 V0 K2 V1 ... (one tile: K0 V0)
   const long long krow = ((((long long)a.layer * 2 + 0) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
   const long long vrow = ((((long long)a.layer * 2 + 1) * a.max_batch + b) * a.Hkv + kvh) * (long long)a.max_seq;
-  // (K and V are read once a forward and leave L2 first: us a layer 118.4 -> 117.0 at 4 x 11 rows over 4,096 keys, a prefill
-  // of 4,096 tokens 126.9 -> 126.5 ms)
+  // K and V leave L2 first, so that queries, sums and residual rows stay.  Blocks of at most 128 query rows per KV head read them
+  // once; the row groups of taller ones run close enough together that the later ones still find them.  8 layers of the 8B shape
+  // in turn, without / with, us: 11 rows over 30,000 keys 1,056 / 1,026, 8 x 21 over 4,096 1,699 / 1,685, over 16,384 2,364 / 2,356,
+  // 256 rows (eight groups) behind 2,048 keys 2,063 / 2,059, behind 3,840 2,157 / 2,147
   const uint64_t policy = l2_evict_first();
   auto load_tile = [&](int s, long long first, int t) {          // tile t of this slice into slot s (by the elected lane)
     const uint32_t dst = smem_u32(ring) + (uint32_t)(s * kSlotBytes), bar = b_full + 8 * s;

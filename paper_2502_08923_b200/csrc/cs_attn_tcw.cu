@@ -40,7 +40,8 @@
 //
 // Bound by the softmax warps' issue slots and, at batch 16, by HBM.  Measured per layer (8B shape, issue
 // by an elected lane with uniform operands, before that from one lane): 176 rows over 16 x 8,192 keys
-// 120.6 -> 93.6 us (0.54 GB: 5.8 TB/s), 16 rows over the same 114.2 -> 83.2 us.  (Taller groups and shorter
+// 120.6 -> 93.6 us, 16 rows over the same 114.2 -> 83.2 us; since K and V leave L2 first 90.2 us at 176 rows
+// (0.54 GB: 6.0 TB/s).  (Taller groups and shorter
 // walks are the business of the kernel with the query rows as M; its file has both sides' figures.)
 #include <stdlib.h>
 

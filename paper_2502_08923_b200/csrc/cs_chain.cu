@@ -7,8 +7,8 @@
 // 29 of 98 us a layer.  Here the weight stream does not stop: a producer warp per SM walks the weight
 // tiles of all four projections in order, held back by nothing but its ring (192 KB of 16 KB tiles on
 // each of 148 SMs: 4 us of HBM), and only the activations wait for what they depend on.
-// Measured, us a layer with its attention, launch per projection -> this kernel (4,096 keys): 1 row 94.9 -> 82.9, 8 rows
-// 97.3 -> 86.1, 11 rows 99.2 -> 88.1, 16 rows 100.5 -> 91.5, 32 rows 108.9 -> 103.0.  What made it pay, in the order found
+// Measured, us a layer with its attention, launch per projection -> this kernel (4,096 keys): 1 row 93.6 -> 82.9, 8 rows
+// 95.7 -> 85.0, 11 rows 97.9 -> 87.4, 16 rows 99.2 -> 88.6, 32 rows 108.0 -> 100.3.  What made it pay, in the order found
 // (11 rows): runs taken one at a time behind the wait and not ahead of it (150 -> 109), sums handed over without fences and
 // what finishing needs asked for early (98), two K blocks per ring slot and activations without padding rows (93.5), weights
 // that leave L2 first (89.2), sums asked for again only where they were missing (88.1).
@@ -57,7 +57,7 @@ constexpr int kMergeBytes = kEpiWarps * 32 * 24;       // and what its warps han
 constexpr int kTicket = 0, kMergeTicket = 32, kWords = 64;   // control words of a layer: the counters, then the rest
 
 struct ChainPhase {
-  int mode, N, num_kb, tiles, units, items, first;     // first = number of this projection's first run
+  int mode, num_kb, units, items, first;               // first = number of this projection's first run
   int dep, dep_shift, dep_target, dep_n;               // words of the input's groups: K block kb needs word[dep + (kb >> dep_shift)] >= dep_target
   int done;                                            // words per tile: finished (-1 = nobody asks)
   int norm_tiles;                                      // > 0: scaled by 1/rms over so many tiles of the input
@@ -214,8 +214,6 @@ __device__ __forceinline__ bool take_sums(const uint4* from, size_t step, int n,
 // a run: its projection and its units, from K block kb0 of tile t0 on.  (Behind a division the compiler no longer
 // knows that a value is uniform, and instructions that want it in a uniform register loop over the lanes.)
 __device__ __forceinline__ int uni(int v) { return (int)uniform((uint32_t)v); }
-// Weights are read once per forward: they leave L2 first, so that what the layers pass to one another (and the norms' gains
-// and rotation factors) is still there when it is wanted, instead of waiting in the queue that the weights keep full.
 struct Run {
   int p, i, u0, u1, num_kb, t0, kb0;
 };
@@ -497,6 +495,8 @@ k_chain(const __grid_constant__ ChainMaps maps, const __grid_constant__ ChainArg
 
   if (warp == kWWarp) {
     // ------------------------------------------------------------- weights: take runs, stream their tiles
+    // Weights are read once per forward: they leave L2 first, so that what the layers pass to one another (and the norms' gains
+    // and rotation factors) is still there when it is wanted, instead of waiting in the queue that the weights keep full.
     const uint64_t policy = l2_evict_first();
     auto take = [&]() -> int { return lane == 0 ? atomicAdd(a.ctl + kTicket, 1) : 0; };
     int s = 0, issued = 0, landed = 0, sl = 0;         // slots filled, slots known to have landed, the next one to
@@ -877,10 +877,8 @@ cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const Qk
     ChainPhase& P = a.ph[p];
     m.w[p] = plans[p]->tmW;
     m.x[p] = *xs[p];
-    P.N = plans[p]->N;
     P.num_kb = cs_ceil_div(plans[p]->K, CS_GEMM_BK);
-    P.tiles = cs_ceil_div(P.N, CS_GEMM_BM);
-    P.units = P.tiles * P.num_kb;
+    P.units = cs_ceil_div(plans[p]->N, CS_GEMM_BM) * P.num_kb;
     P.items = max(1, min(fit, P.units / kMinRun));
     P.first = a.runs;
     a.runs += P.items;

@@ -36,8 +36,9 @@
 // add up over distributed shared memory instead of the split form's exchange: 24.2, 25.6, 45.5 us at
 // 176 rows, 29.5, 32.7, 60.4 at 256 (QKV, output, down).
 //
-// Weights leave L2 first, so that activations and sums stay: us a layer 121.9 -> 118.4 at 44 rows, 305 -> 295 at 168 rows over
-// 8 x 16,384 keys; a prefill of 4,096 tokens 128.6 -> 126.9 ms.
+// Weights leave L2 first, so that activations and sums stay, and so do K and V in the attention between (us a layer, both at
+// normal priority / both first): 44 rows over 4 x 4,096 keys 121.7 / 116.2, over 4 x 16,384 152.6 / 144.0, 176 rows over
+// 16 x 8,192 241.5 / 235.6, 256 rows behind 2,048 202.7 / 200.5, 168 rows over 8 x 16,384 no difference (267.5 / 268.7, +-3).
 //
 // Every wait is bounded as in cs_gemm.cu; waits for other pairs' sums are polls with the same limit.
 #include <algorithm>
