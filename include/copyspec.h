@@ -57,8 +57,8 @@
  *                          do, instead of replaying them from a captured CUDA graph;
  *   CS_CHAIN=0|1           blocks of at most 32 rows: a launch per projection (0), or one launch per layer for everything
  *                          between two attentions whatever the model's size (1).  Default: the latter up to 32 rows from
- *                          280 MiB of weights a layer on, up to 24 from 192 on (heads of 128), 12 from 128 on,
- *                          8 from 96 on (smaller heads: 112; QKV of at most twice the model's width);
+ *                          280 MiB of weights a layer on (192 with heads of 128; less for narrow models), up to 12
+ *                          from 128 on, 8 from 96 on (smaller heads: 112; QKV below twice the model's width);
  *   CS_ATTN_KERNEL=tc|tcw|mma  forces one attention kernel: tcgen05 with the query rows as the
  *                          M dimension (tc), tcgen05 with the keys and head dims as M (tcw), or
  *                          mma.sync (mma).  Default: by head size, and between the two tcgen05

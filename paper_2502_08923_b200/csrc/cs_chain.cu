@@ -834,16 +834,19 @@ size_t cs_chain_words(const cs_model_config* c) {
 //   108, heads of 64      386/389  416/430  424/480  483/492  434/505  482/489  495/546   662/727
 //    98                   390/346  404/366  411/393  474/483  420/406  443/458  462/483   617/689
 //    92, heads of 64      367/363  400/399  404/455  466/461  417/476  462/489  477/593   645/728
-// The lines lie where the worst of the lengths and batches is no loss (at most 1 %: 154 MiB, heads of 64, 12 sequences).  Below
-// them some layers gain (92 MiB with heads of 128 at 1 row 381/334) and others lose a quarter (32 MiB at 22 rows 360/485).
+// The lines lie where the worst of the lengths and batches of 42 shapes is no loss (at most 1 %: 154 MiB, heads of 64, 12
+// sequences; 192 MiB, 8 x 4 rows; 222 MiB with a QKV of 2 d, 4 x 6 rows).  A narrow model's tiles of O and down are few, so more runs share each
+// (232 MiB, d 2,560, 4 x 6 rows 0.98x, 16 rows 1.02x); a QKV of 2 d and more has more slices to merge (198 MiB, 3 d, 4 x 8
+// rows 0.97x).  Below the lines some layers gain (92 MiB with heads of 128 at 1 row 381/334, 98 MiB at 11 rows 411/393) and others lose
+// up to a quarter (103 MiB, d 2,304, 10 sequences 0.91x; 32 MiB at 22 rows 360/485).
 int cs_chain_max_rows(const cs_model_config& c, int force) {
   if (force != 0) return force > 0 ? CS_CHAIN_MAX_ROWS : 0;
   const long long mib = cs_layer_bytes(c) >> 20;
-  const bool wide = c.head_dim == 128;
-  if (mib >= 280) return CS_CHAIN_MAX_ROWS;
-  if (mib >= 192 && wide) return 24;
+  const bool wide = c.head_dim == 128, lean = (c.n_heads + 2 * c.n_kv_heads) * c.head_dim < 2 * c.d_model;
+  if (mib >= 280 && c.d_model >= 3072) return CS_CHAIN_MAX_ROWS;
+  if (mib >= 192 && wide) return c.d_model < 3072 ? 16 : lean ? CS_CHAIN_MAX_ROWS : 24;
   if (mib >= 128) return 12;
-  return mib >= (wide ? 96 : 112) && (c.n_heads + 2 * c.n_kv_heads) * c.head_dim <= 2 * c.d_model ? 8 : 0;
+  return lean && mib >= (wide ? 96 : 112) ? 8 : 0;
 }
 bool cs_chain_takes(const cs_ctx* ctx, int rows) { return rows <= cs_chain_max_rows(ctx->cfg, ctx->chain_force); }
 

@@ -166,8 +166,12 @@ def test_wait_runs_out_and_the_context_stays_usable(monkeypatch):
 RULE = {"89": (_cfg(2048, 16, 4, 128, 5888, layers=1), 0), "98": (_cfg(2048, 16, 4, 128, 6656, layers=1), 8),
         "98, QKV of 3 d": (_cfg(2048, 16, 16, 128, 5632, layers=1), 0), "108, heads of 64": (_cfg(2048, 32, 8, 64, 7488, layers=1), 0),
         "116, heads of 64": (_cfg(2048, 32, 8, 64, 8192, layers=1), 8), "135": (_cfg(2560, 20, 4, 128, 7168, layers=1), 12),
-        "192": (_cfg(3072, 24, 8, 128, 8192, layers=1), 24), "195, heads of 64": (_cfg(3072, 48, 8, 64, 8704, layers=1), 12),
-        "245": (_cfg(2048, 16, 4, 128, 19200, layers=1), 24), "287": (_cfg(3584, 28, 4, 128, 11264, layers=1), 32)}
+        "191": (_cfg(3072, 24, 8, 128, 8128, layers=1), 12), "192": (_cfg(3072, 24, 8, 128, 8192, layers=1), 32),
+        "198, QKV of 3 d": (_cfg(3072, 24, 24, 128, 7168, layers=1), 24), "195, heads of 64": (_cfg(3072, 48, 8, 64, 8704, layers=1), 12),
+        "245, narrow": (_cfg(2048, 16, 4, 128, 19200, layers=1), 16), "288, heads of 64": (_cfg(4096, 64, 8, 64, 9216, layers=1), 32)}
+
+
+ROWS = (1, 8, 9, 12, 13, 16, 17, 24, 25, 32, 33)
 
 
 @pytest.mark.parametrize("name", list(RULE))
@@ -177,12 +181,12 @@ def test_blocks_are_chained_where_that_was_measured_to_gain(name, monkeypatch):
     cfg, most = RULE[name]
     ctx = cs.Context(cfg, inputs.make_weights(cfg, seed=4, device="cuda"), max_seq=64, max_batch=1, k_max=32)
     launches = []
-    for rows in (1, 8, 9, 12, 13, 24, 25, 32, 33):
+    for rows in ROWS:
         hd, ld, kvl = i32(np.zeros((1, 64))), i32([8]), i32([7])
         ctx.cs_loop_begin(hd, ld, ctx.alloc_kv(), kvl, 3, rows - 1, 4)
         launches.append((rows, ctx.cs_loop_launches_per_step()))
         ctx.cs_loop_end()
     ctx.close()
     most_launches = max(n for _, n in launches)
-    assert [rows for rows, n in launches if n == most_launches - 3] == [r for r in (1, 8, 9, 12, 13, 24, 25, 32, 33) if r <= most]
+    assert [rows for rows, n in launches if n == most_launches - 3] == [r for r in ROWS if r <= most]
     assert {n for _, n in launches} <= {most_launches, most_launches - 3}
