@@ -59,6 +59,11 @@
  *                          between two attentions whatever the model's size (1).  Default: the latter up to 32 rows from
  *                          280 MiB of weights a layer on (192 with heads of 128; less for narrow models), up to 12
  *                          from 128 on, 8 from 96 on (smaller heads: 112; QKV below twice the model's width);
+ *   CS_SMALL=0|1           cs_decode_loop on small models: a launch per kernel of a step (0), or the whole loop in one launch for any
+ *                          model that fits it (1).  Default: the latter where a layer's weights take up to 3 MiB and the LM head
+ *                          up to 16, for blocks of up to 16 rows, history rows of up to 8,192 tokens (heads of 64: 4,096)
+ *                          and batches whose clusters run at once (7 sequences of sixteen SMs, or about 16 of eight);
+ *                          never while CS_ATTN_KERNEL, stamps or a match index are set;
  *   CS_ATTN_KERNEL=tc|tcw|mma  forces one attention kernel: tcgen05 with the query rows as the
  *                          M dimension (tc), tcgen05 with the keys and head dims as M (tcw), or
  *                          mma.sync (mma).  Default: by head size, and between the two tcgen05
@@ -390,7 +395,8 @@ cs_status cs_linear(cs_ctx* ctx, const void* X, const void* W, int rows, int N, 
 cs_status cs_debug_drop_tile(cs_ctx* ctx, int k_block);
 
 /* The same for the chained projections of blocks of at most 32 rows: the next such launch leaves out the
- * weights that travel with the unit-th K block of every run it hands to an SM (a ring slot: up to two blocks).
+ * weights that travel with the unit-th K block of every run it hands to an SM (a ring slot: up to two blocks).  Where a whole
+ * loop runs in one launch (CS_SMALL) the next one's first CTA never sends the unit-th kind of what CTAs hand to one another (0 - 6).
  * unit < 0 clears it. */
 cs_status cs_debug_drop_chain_tile(cs_ctx* ctx, int unit);
 

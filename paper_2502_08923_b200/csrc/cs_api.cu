@@ -104,6 +104,7 @@ WsLayout ws_layout(const cs_model_config* c) {
 constexpr size_t kStepInAt = 2048, kStepOutAt = kStepInAt + CS_STEP_IN_MAX * sizeof(int);
 constexpr size_t kSlotBytes = kStepOutAt + 2 * CS_MAX_ROWS * sizeof(int) + 1024;
 constexpr int kSlots = 32, kBlocks = 64;
+static_assert(sizeof(cs_stats) + 8 <= 2 * CS_MAX_ROWS * sizeof(int), "report of a whole loop");
 static_assert(64 + (CS_MAX_ROWS + 1) * sizeof(int) <= kStepInAt && kSlotBytes % 1024 == 0, "progress word and host scratch");
 struct PinnedBlock {
   char* at;
@@ -390,6 +391,8 @@ cs_status cs_create(cs_ctx** out, const cs_model_config* cfg, const cs_weights* 
     const char* ng = getenv("CS_NO_GRAPH");
     ctx->no_graph = ng != nullptr && ng[0] == '1';
     ctx->chain_force = chain_switch();
+    const char* sm = getenv("CS_SMALL");
+    ctx->small_force = sm == nullptr ? 0 : (sm[0] == '0' ? -1 : (sm[0] == '1' ? 1 : 0));
     const char* wl = getenv("CS_WAIT_LIMIT_US");
     const long long us = (wl != nullptr) ? atoll(wl) : 0;
     ctx->wait_limit_ns = (us > 0) ? (unsigned long long)us * 1000ull : 2000000000ull;
@@ -516,6 +519,7 @@ void cs_destroy(cs_ctx* ctx) {
   cs_loop_end(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   give_pinned(ctx->pinned);
+  cs_small_free(ctx);
   delete[] ctx->layers;
   delete ctx;
 }
@@ -859,6 +863,27 @@ cs_status cs_decode_loop(cs_ctx* ctx, int32_t* hist, int32_t* hist_len, int B, i
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->loop.active = true;
   *ctx->progress = 0ull;               // (every earlier loop of this context has been waited for)
+  bool whole = false;
+  s = cs_launch_small_loop(ctx, &whole, st);
+  if (whole) {
+    // a small model: all steps are in one launch, which reports once
+    LoopProgress at = {0, max_new};
+    s = wait_progress(ctx, &at, st);
+    if (s == CS_OK) {
+      const unsigned long long* report = reinterpret_cast<const unsigned long long*>(ctx->step_out);
+      if (stats_out != nullptr) memcpy(stats_out, report + 1, sizeof(cs_stats));
+      const int bits = (int)report[0];
+      // (as in take_status: the bit may be an earlier forward's)
+      if ((bits & CS_DEV_TIMEOUT) && (cudaMemsetAsync(ctx->pair_flag, 0, CS_MAX_PAIRS * 2 * sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess))
+        (void)cudaGetLastError();
+      s = status_from_bits(ctx, bits);
+    } else {
+      (void)cudaStreamSynchronize(st);
+    }
+    cs_loop_end(ctx);
+    return s;
+  }
+  if (s != CS_OK) { cs_loop_end(ctx); return s; }
   auto send = [&](int sent, int wanted) {
     cs_status r;
     if (ctx->loop.exec != nullptr) {

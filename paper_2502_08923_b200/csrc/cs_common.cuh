@@ -165,6 +165,9 @@ struct cs_ctx {
   size_t attn_tc_smem_set, attn_tcw_smem_set;
   int attn_force;            // 0 = choose by shape, 1 = mma.sync kernel, 2 = tcgen05 kernel (query rows as M), 3 = tcgen05 kernel (keys as M)
   int chain_force;           // 0 = chained projections by block height and shape of the layer, -1 = never, 1 = for layers of any size (CS_CHAIN at creation)
+  int small_force;           // 0 = one launch per generation loop by size of the model, -1 = never, 1 = for any model that fits (CS_SMALL at creation)
+  void* small_maps;          // operand maps of the one-launch loop (host), made when it is first taken
+  short small_fit[2][4];     // and how many of its clusters run at once, + 1, by cluster size and block height (0 = not asked yet)
   bool no_graph;             // CS_NO_GRAPH=1 at creation: cs_loop_steps enqueues kernel by kernel
   unsigned long long wait_limit_ns;   // limit of the kernels' bounded waits (CS_WAIT_LIMIT_US at creation; 2 s)
   int debug_drop_kb;         // test hook: the next GEMM launch leaves out this K block's loads (-1 = none)
@@ -330,6 +333,10 @@ int cs_chain_max_rows(const cs_model_config& c, int force);
 bool cs_chain_takes(const cs_ctx* ctx, int rows);
 // next_q = where the next layer's QKV projection puts its results (NULL behind the last layer), next_gain = gain of the norm behind this layer
 cs_status cs_launch_chain(cs_ctx* ctx, int layer, int nsplit, int rows, const QkvEpi* next_q, const __nv_bfloat16* next_gain, cudaStream_t st);
+// cs_small.cu: the whole loop that ctx->loop describes in one launch, for small models; `taken` = it was launched.  Its end is told as
+// the first step of the progress word, with status bits and the statistics in the words at ctx->step_out.
+cs_status cs_launch_small_loop(cs_ctx* ctx, bool* taken, cudaStream_t st);
+void cs_small_free(cs_ctx* ctx);
 // cs_layers.cu
 void cs_launch_block_setup(cs_ctx* ctx, const int32_t* last_tok, const int32_t* draft,
                            const int32_t* draft_len, const int32_t* kv_len, const int32_t* skip,
