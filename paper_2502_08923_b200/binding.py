@@ -57,6 +57,7 @@ EXPORTS = ("cs_workspace_bytes", "cs_create", "cs_destroy", "cs_last_error", "cs
            "cs_gram_index_reset", "cs_gram_index_update", "cs_find_match_indexed", "cs_gram_index_status")
 
 _lib = None
+_search = None      # cs_find_match in native code, for plain arguments
 
 
 def lib_path() -> str:
@@ -65,7 +66,7 @@ def lib_path() -> str:
 
 def load(build_if_missing: bool = True) -> C.CDLL:
     """Load libcopyspec.so (building it with nvcc first when it is missing or stale)."""
-    global _lib
+    global _lib, _search
     if _lib is not None:
         return _lib
     if build_if_missing:
@@ -141,6 +142,8 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.cs_gram_index_status.argtypes = [vp, i, i, vp]
     lib.cs_linear.restype = i
     lib.cs_linear.argtypes = [vp, vp, vp, i, i, i, vp, vp]
+    from . import _native
+    _search = _native.find_match
     _lib = lib
     return lib
 
@@ -189,6 +192,13 @@ def _match_outputs(hist, hist_len, k):
 def cs_find_match(hist, hist_len, gamma, k, policy=LATEST, out=None):
     """Suffix-match search and draft gather.  hist [B][stride] int32, hist_len [B] int32 (CUDA).
     Returns (match_pos [B], draft [B][k], draft_len [B]); `out` may supply those tensors."""
+    if out is None:
+        # (a call for one short history: 10.7 us through the lines below, 5.0 here)
+        got = (_search or (load() and _search))(hist, hist_len, gamma, k, policy)
+        if got.__class__ is tuple:
+            return got
+        if got is not None:
+            raise CsError(got, "cs_find_match")
     B, stride = hist.shape
     if out is None:
         out = mp, dr, dl = _match_outputs(hist, hist_len, k)
