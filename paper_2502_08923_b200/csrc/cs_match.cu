@@ -2,38 +2,51 @@
 //
 // One thread-block cluster per sequence.  The CTAs of a cluster split the candidate
 // start positions [0, n - 2*gamma] between them; each thread tests four consecutive
-// candidates from two 128-bit loads of the history, the best position is reduced by
-// warp vote / shared-memory atomics inside the CTA and through distributed shared
-// memory across the cluster, and the first CTA of the cluster then copies the draft.
+// candidates at a time, four such groups from loads that are in flight together, the best position is reduced by
+// warp vote / shared-memory atomics inside the CTA and sent to the first CTA of the cluster, which
+// copies the draft.
 // No global scratch memory, no global atomics, one launch, deterministic.
-#include <cooperative_groups.h>
+//
+// Bound by a chain of latencies: length, tokens (through L2), cluster barrier, draft.  Launched back to back, us a search, with a load waited
+// for per group of candidates and two barriers of the whole cluster behind them / now: 1 x 4,097 tokens 3.02 / 2.89, 1 x 32,768
+// 3.77 / 3.03, 8 x 8,192 3.97 / 3.24, 64 x 4,096 3.97 / 3.52, 64 x 32,768 7.53 / 5.39, 64 x 131,072 18.3 / 11.9.  (The second four
+// tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and 13.5 for the last two.)
 #include <limits.h>
 
 #include "cs_common.cuh"
 
-namespace cg = cooperative_groups;
-
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256, kMaxCluster = 8;
 
 // The history is read through L2 only: this kernel may be resident while the step before still appends to
 // it, and neither the read-only path nor L1 is coherent across that.
 __device__ __forceinline__ int4 ld_int4(const int* p) { return __ldcg(reinterpret_cast<const int4*>(p)); }
+// The cluster's barrier (warps arrive whole): a first phase, which everyone passes before anyone writes to another CTA's shared memory, says
+// that all of them run; a second, at which only the first CTA waits, that the best positions are there.
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+constexpr int kGroups = 4;             // groups of candidates whose tokens a thread has in flight
 
 __global__ void __launch_bounds__(kThreads)
 k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
              int k, int policy, int* __restrict__ match_pos, int* __restrict__ draft,
              int* __restrict__ draft_len, int* __restrict__ last_tok,
              const int* skip, unsigned long long* stamp) {
+  cluster_arrive();
   CS_PDL_PROLOGUE();
-  cg::cluster_group cluster = cg::this_cluster();
-  const int b = blockIdx.y;
-  const int rank = (int)cluster.block_rank();
-  const int nblk = (int)cluster.num_blocks();
-  const int tid = threadIdx.x;
+  uint32_t rank_u, nblk_u;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_u));
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(nblk_u));
+  const int b = blockIdx.y, rank = (int)rank_u, nblk = (int)nblk_u, tid = threadIdx.x, lane = tid & 31;
   __shared__ int s_best;
-  __shared__ int s_final;
+  __shared__ int s_all[kMaxCluster];   // first CTA: the best position of every CTA
 
   const int* h = hist + (size_t)b * stride;
   int n = __ldcg(hist_len + b);
@@ -58,49 +71,62 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
     const int lo = rank * per;
     const int hi = min(n_cand, lo + per);
     const bool vec_ok = ((reinterpret_cast<uintptr_t>(h) & 15) == 0) && gamma <= 5;
-    for (int p = lo + tid * 4; p < hi; p += kThreads * 4) {
-      if (vec_ok && p + 8 <= stride) {
-        // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies past the
-        // accepted length only feeds candidates that `hi` masks off
-        const int4 a = ld_int4(h + p);
-        const int4 c = ld_int4(h + p + 4);
-        const int t[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
+    auto test = [&](const int4& u, const int4& v, int p) {
+      // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies past the
+      // accepted length only feeds candidates that `hi` masks off
+      const int t[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          bool eq = (p + i < hi);
+      for (int i = 0; i < 4; ++i) {
+        bool eq = (p + i < hi);
 #pragma unroll
-          for (int j = 0; j < 5; ++j)
-            if (j < gamma) eq = eq && (t[i + j] == key[j]);
-          if (eq) best = latest ? max(best, p + i) : min(best, p + i);
+        for (int j = 0; j < 5; ++j)
+          if (j < gamma) eq = eq && (t[i + j] == key[j]);
+        if (eq) best = latest ? max(best, p + i) : min(best, p + i);
+      }
+    };
+    auto scan = [&](int p) {
+      for (int i = 0; i < 4 && p + i < hi; ++i) {
+        bool eq = true;
+        for (int j = 0; j < gamma; ++j) eq = eq && (__ldcg(h + p + i + j) == key[j]);
+        if (eq) best = latest ? max(best, p + i) : min(best, p + i);
+      }
+    };
+    for (int base = lo; base < hi; base += kGroups * kThreads * 4) {
+      int4 u[kGroups], v[kGroups];
+#pragma unroll
+      for (int q = 0; q < kGroups; ++q) {
+        const int p = base + (q * kThreads + tid) * 4;
+        if (vec_ok && p < hi && p + 8 <= stride) {
+          u[q] = ld_int4(h + p);
+          v[q] = ld_int4(h + p + 4);
         }
-      } else {
-        for (int i = 0; i < 4 && p + i < hi; ++i) {
-          bool eq = true;
-          for (int j = 0; j < gamma; ++j) eq = eq && (__ldcg(h + p + i + j) == key[j]);
-          if (eq) best = latest ? max(best, p + i) : min(best, p + i);
-        }
+      }
+#pragma unroll
+      for (int q = 0; q < kGroups; ++q) {
+        const int p = base + (q * kThreads + tid) * 4;
+        if (vec_ok && p + 8 <= stride) test(u[q], v[q], p);
+        else scan(p);
       }
     }
   }
   // warp vote, then one shared-memory atomic per warp
   best = latest ? __reduce_max_sync(0xffffffffu, best) : __reduce_min_sync(0xffffffffu, best);
-  if ((tid & 31) == 0 && best != none) {
+  if (lane == 0 && best != none) {
     if (latest) atomicMax(&s_best, best); else atomicMin(&s_best, best);
   }
   __syncthreads();
-  cluster.sync();
-  if (rank == 0 && tid == 0) {
-    int v = none;
-    for (int r = 0; r < nblk; ++r) {
-      const int o = *cluster.map_shared_rank(&s_best, r);
-      v = latest ? max(v, o) : min(v, o);
-    }
-    s_final = (v == INT_MAX) ? -1 : v;
+  cluster_wait();
+  if (tid == 0) {
+    uint32_t to;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(s_all + rank)));
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(to), "r"(s_best) : "memory");
   }
-  cluster.sync();   // remote shared memory stays alive until the first CTA has read it
+  cluster_arrive();
   if (rank != 0) return;
-
-  const int p0 = s_final;
+  cluster_wait();
+  int p0 = none;
+  for (int r = 0; r < nblk; ++r) p0 = latest ? max(p0, s_all[r]) : min(p0, s_all[r]);
+  if (p0 == INT_MAX) p0 = -1;
   const int start = p0 + gamma;
   const int len = (p0 < 0) ? 0 : min(k, n - start);
   if (tid == 0) {
@@ -128,7 +154,7 @@ cs_status cs_launch_find_match(const int32_t* hist, const int32_t* hist_len, int
   // 4096 candidates per CTA keep every thread at >= 4 vector iterations on long
   // histories; short ones use a single CTA per sequence
   int cl = 1;
-  while (cl < 8 && stride > cl * 4096) cl *= 2;
+  while (cl < kMaxCluster && stride > cl * 4096) cl *= 2;
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(cl, B, 1);
   lc.blockDim = dim3(kThreads, 1, 1);
