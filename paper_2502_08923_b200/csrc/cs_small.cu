@@ -26,7 +26,8 @@
 // model, one sequence, 11 rows, us a call of 11 steps: launch by launch 876; with divisions in the index arithmetic, stores to sixteen CTAs one by one and
 // cluster barriers 980 (11,400 instructions a warp and step); with hand-overs counted on mbarriers and K split over the warps 555; with the SwiGLU output
 // multiplied where it was made, one turn of code for all projections and weights out of the registers 500; with weights by TMA and the
-// statistics kept by a warp that nobody waits for 475.  What is left of 41 us a step: 17 turns or hand-overs of 1.5 - 2.5 us.
+// statistics kept by a warp that nobody waits for 475; with what a warp does for a tile worked out once and fragment loads that meet every bank once
+// 433.  What is left of 38 us a step: 17 turns or hand-overs of 1.5 - 2 us.
 //
 // Arithmetic as in the other kernels: activations, queries and softmax weights enter products as two bf16 terms, sums, norms,
 // rotation and softmax are fp32; every RMSNorm is folded into the projection behind it (1/rms scales the sums).
@@ -63,9 +64,16 @@ __host__ __device__ constexpr int tile_bytes(int Rp) { return (68 * Rp + 63) / 1
 struct SmallMaps {
   CUtensorMap w[4 * kMaxLayers + 1];
 };
+// What a warp does for a tile of a projection, worked out once for its first tile of each: the divisions and choices in it were 1,200 clocks a turn.
+struct __align__(16) Job {
+  int col, row, block, chunks;        // weights: coordinates of the first copy, how many (0 = the warp has no such job)
+  int jobs, tile, quarter, rows;      // jobs of the CTA; this one's tile, the first of its tokens' quarters and its tokens
+  int at, first, last, pieces;        // results: where they go in the CTAs first .. last - 1, and how many 16-byte pieces
+  int op, kb, one, whole;             // operand, blocks of 32 K elements, whether the job has one quarter of the tokens only, whether both terms travel
+};
 // where things lie in shared memory (bytes); the same in every CTA
 struct SmallSmem {
-  int xn, at, act, po, sums, stage, norm, red, q, kv, xres, gain, gain0, rope, turn, owner, kinds, ring, hist, misc, total;
+  int xn, at, act, sums, stage, norm, red, q, kv, xres, gain, gain0, rope, turn, jobs, ring, hist, misc, total;
 };
 struct SmallArgs {
   const __nv_bfloat16* norm[2 * kMaxLayers + 1];   // gains, in their order
@@ -87,6 +95,8 @@ struct SmallArgs {
   SmallSmem at;
 };
 
+// (what branches and copies go by: see uniform())
+__device__ __forceinline__ int uni(int v) { return (int)uniform((uint32_t)v); }
 __device__ __forceinline__ uint32_t peer(uint32_t addr, int rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -243,8 +253,8 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* s_xn = smem + a.at.xn;                                               // gain * x, in tiles
   uint8_t* s_at = smem + a.at.at;                                               // this CTA's KV head's attention output, in tiles
-  uint8_t* s_act = smem + a.at.act;                                             // this CTA's SwiGLU output, in tiles
-  uint8_t* s_po = smem + a.at.po;                                               // attention of the KV head's slices, each [rows][DH] and (max, sum) [rows]
+  uint8_t* s_act = smem + a.at.act;                                             // this CTA's SwiGLU output, in tiles; shares its place with the
+  uint8_t* s_po = s_act;                                                        // attention of the KV head's slices, each [rows][DH] and (max, sum) [rows]
   float* s_sums = reinterpret_cast<float*>(smem + a.at.sums);                   // sums of the residual stream by CTA that sent them, [sender][own tile][R][16]
   uint8_t* s_stage = smem + a.at.stage;                                         // results on their way to the others
   uint8_t* s_norm = smem + a.at.norm;                                           // the residual stream's next operand on its way to the others
@@ -252,7 +262,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
   float* s_red = reinterpret_cast<float*>(smem + a.at.ring + kRing * 1024);
   constexpr int kRed = kRing * 512;                                             // from one warp's to the next
   static_assert(16 * DH <= kRing * 256, "half a ring");
-  auto red_at = [](int row, int col) { return row * DH + ((col + 4 * row) & (DH - 1)); };
+  auto red_at = [](int r, int col) { return r * DH + ((col + 4 * r) & (DH - 1)); };
   float2* s_redml = reinterpret_cast<float2*>(smem + a.at.red);                 // and their (max, sum), [warp][16]
   uint8_t* s_q = smem + a.at.q;                                                 // this CTA's queries, in tiles (dims 8p .. and the partners half a head on)
   uint8_t* s_kn = smem + a.at.kv;                                               // the block's K rows of its KV head, [part][token][16], and V rows behind
@@ -261,12 +271,11 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
   __nv_bfloat16* s_gain0 = reinterpret_cast<__nv_bfloat16*>(smem + a.at.gain0); // gain of the first norm
   float2* s_rope = reinterpret_cast<float2*>(smem + a.at.rope);                 // rotation of the block's rows, [Rp][DH / 2]
   double2* s_turn = reinterpret_cast<double2*>(smem + a.at.turn);               // (cos, sin) of 0 .. R positions, [R + 1][DH / 2], then of the block's first row
-  int* s_owner = reinterpret_cast<int*>(smem + a.at.owner);                     // by tile of the residual stream: the CTA that holds it << 16 | how many it holds << 8 | which of them it is
-  int4* s_kind = reinterpret_cast<int4*>(smem + a.at.kinds);                    // by projection: tiles of this CTA, blocks of 32 K elements, the first of them, operand
+  Job* s_job = reinterpret_cast<Job*>(smem + a.at.jobs) + (threadIdx.x >> 5) * 6;   // this warp's first job of every projection, and its present one behind
   int* s_hist = reinterpret_cast<int*>(smem + a.at.hist);                       // the history, [stride]
-  uint2* s_max = reinterpret_cast<uint2*>(smem + a.at.misc);                    // largest logits and their ids by CTA, [kMaxCluster][Rp]; by warp:
-  uint2* s_wmax = s_max + kMaxCluster * Rp;                                     // [kWarps][Rp]
-  uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_wmax + kWarps * Rp);          // [kExchanges]
+  uint2* s_max = reinterpret_cast<uint2*>(smem + a.at.misc);                    // largest logits and their ids by CTA, [kMaxCluster][Rp]
+  uint2* s_wmax = reinterpret_cast<uint2*>(s_stage) + Rp;                       // by warp, [kWarps][Rp], behind this CTA's on their way to the others, [Rp]
+  uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_max + kMaxCluster * Rp);      // [kExchanges]
   uint64_t* s_wbar = s_bar + kExchanges;                                        // a warp's weights, [kWarps]
   int* s_script = reinterpret_cast<int*>(s_wbar + kWarps);                      // [Rp]
   int* s_tgt = s_script + Rp;                                                   // [Rp]
@@ -300,7 +309,10 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
   const uint32_t base = smem_u32(smem), bars = smem_u32(s_bar) - base;
   const uint32_t to = peer(base, warp & (NC - 1));             // the CTA that this warp sends to
   const uint32_t ring = base + (uint32_t)(a.at.ring + warp * (kRing * 2048)), ring_bar = smem_u32(s_wbar + warp);
-  const uint8_t* ring_at = smem + (ring - base) + g * 128;     // this thread's row of its warp's tiles
+  // This thread's rows of its warp's tiles are row and row + 8, not g and g + 8: rows 4 apart lie in the two halves of the copies' swizzle, and a fragment load
+  // of neighbouring lanes meets every bank once (with g, twice: the loads were what a projection took longest for).
+  const int row = g >> 1 | (g & 1) << 2;
+  const uint8_t* ring_at = smem + (ring - base) + row * 128;
   uint32_t ring_parity = 0;
   uint8_t* mine = s_stage + warp * (64 * Rp);                  // this warp's part of the stage
 
@@ -324,11 +336,6 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
   }
 #pragma unroll 1
   for (int i = tid; i < d; i += kThreads) s_gain0[i] = a.norm[0][i];
-#pragma unroll 1
-  for (int i = tid; i < dt; i += kThreads) {
-    const int p = ((i + 1) * NC - 1) / dt;
-    s_owner[i] = p << 16 | ((p + 1) * dt / NC - p * dt / NC) << 8 | (i - p * dt / NC);
-  }
   // Rotation factors in double, as everywhere: those of a block's first row times those of the distance.  (sincos in the loop over the steps costs 2,000
   // clocks a step and room in the instruction cache; a product is right to 2e-16, and the steps' errors add up to 1e-13 over a thousand of them.)
 #pragma unroll 1
@@ -339,13 +346,43 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     s_turn[i] = make_double2(co, sn);
   }
   double2* s_first = s_turn + (R + 1) * kHalf;
-  if (tid == 0) {
-    s_kind[kQkv] = make_int4(qn, d / 32, 0, a.at.xn);
-    s_kind[kOut] = make_int4(on, G * kParts / 2, kvh * G * DH, a.at.at);
-    s_kind[kGateUp] = make_int4(4 * fn, d / 32, 0, a.at.xn);
-    s_kind[kDown] = make_int4(dt, fn, 32 * f0, a.at.act);
-    s_kind[kLm] = make_int4(l1 - l0, d / 32, 0, a.at.xn);
-  }
+  // Few tiles: a warp for every quarter of the tokens.  Rows of a tile, of QKV: dims 8p .. and, half a head on, their partners in the rotation; of gate/up:
+  // gate rows and, 64 on, their up rows; else 16 neighbours.  Results of QKV go to every CTA of their KV head (of keys and values the leading terms: what the
+  // cache holds), of the attention output and down to the CTA that holds the tile.
+  auto describe = [&](Job* j, int kind, int job) {
+    const int tiles = kind == kQkv ? qn : kind == kOut ? on : kind == kGateUp ? 4 * fn : kind == kDown ? dt : l1 - l0;
+    const bool one = NT > 1 && kind != kLm && tiles * NT <= kWarps;
+    const int jobs = one ? tiles * NT : tiles, local = one ? job / NT : job, quarter = one ? job % NT : 0;
+    const int tile = local + (kind == kQkv ? q0 : kind == kOut ? o0 : kind == kGateUp ? 4 * f0 : kind == kLm ? l0 : 0);
+    const int kb = kind == kOut ? G * kParts / 2 : kind == kDown ? fn : d / 32;
+    j->col = kind == kOut ? kvh * G * DH : kind == kDown ? 32 * f0 : 0;
+    j->row = kind == kQkv ? tile % kParts * 8 : kind == kGateUp ? tile % 8 * 8 : 16 * tile;
+    j->block = kind == kQkv ? tile / kParts : kind == kGateUp ? tile / 8 : 0;
+    j->chunks = job < jobs ? (kb + 1) / 2 : 0;
+    j->jobs = jobs;
+    j->tile = kind == kGateUp ? local : tile;
+    j->quarter = quarter;
+    j->rows = min(R - 4 * quarter, one ? 4 : Rp);
+    j->op = kind == kOut ? a.at.at : kind == kDown ? a.at.act : a.at.xn;
+    j->kb = kb;
+    j->one = one;
+    const int head = tile / kParts, part = tile % kParts;
+    const bool is_q = head < H;
+    j->whole = kind != kQkv || is_q;
+    j->pieces = (j->whole ? 4 : 2) * j->rows;
+    if (kind == kQkv) {
+      const int kh = is_q ? head / G : (head - H) % Hkv;
+      j->first = kh * S;
+      j->last = j->first + S;
+      j->at = is_q ? a.at.q + kRows + ((head - kh * G) * kParts + part) * TB + quarter * 256 : a.at.kv + ((head - H) / Hkv * kParts + part) * 32 * Rp + quarter * 128;
+    } else if (kind == kOut || kind == kDown) {
+      const int p = ((tile + 1) * NC - 1) / dt, held = ((p + 1) * dt >> log_nc) - (p * dt >> log_nc);
+      j->first = p;
+      j->last = p + 1;
+      j->at = a.at.sums + ((kind == kOut ? kvh : c) * held + tile - (p * dt >> log_nc)) * 64 * R + quarter * 256;
+    }
+  };
+  if (lane <= kLm) describe(s_job + lane, lane, warp);
   // what a hand-over brings, in bytes
   auto arm = [&](int x) {
     expect(base + bars + 8 * x, (uint32_t)(x == kXQkv ? (G + 1) * kParts * 64 * R : x == kXAttn ? S * a.slice_bytes : x == kXOut ? Hkv * dn * 64 * R
@@ -383,23 +420,17 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     if (lane < Rp) s_rstd[lane] = rsqrtf(ss * a.inv_d + a.eps);
   };
 
-  // Asks for a tile's weights (by a whole warp), from K block `first` on; false = it has none.  Its rows, of QKV: dims 8p .. and, half a head on, their partners in the rotation; of gate/up: gate rows
-  // and, 64 on, their up rows; else 16 neighbours.
-  auto ask_more = [&](int turn, int job, int first) {
-    const int kind = turn == 4 * a.n_layers ? kLm : turn & 3;
-    const int4 par = s_kind[kind];
-    const bool one = NT > 1 && kind != kLm && par.x * NT <= kWarps;
-    if (job >= (one ? par.x * NT : par.x)) return false;
-    const int tile = one ? job / NT : job;
-    const int row = kind == kQkv ? (q0 + tile) % kParts * 8 : kind == kGateUp ? (4 * f0 + tile) % 8 * 8 : 16 * (tile + (kind == kOut ? o0 : kind == kLm ? l0 : 0));
-    const int block = kind == kQkv ? (q0 + tile) / kParts : kind == kGateUp ? (4 * f0 + tile) / 8 : 0;
-    ask(ring, ring_bar, &maps.w[turn], first, (par.y + 1) / 2, par.z, row, block);
-    return true;
+  // asks for a job's weights (by a whole warp), from copy `first` on
+  auto ask_for = [&](int turn, const Job* j, int first) {
+    const int4 w = *reinterpret_cast<const int4*>(j);
+    const int chunks = uni(w.w);
+    if (chunks > 0) ask(ring, ring_bar, &maps.w[turn], first, chunks, uni(w.x), uni(w.y), uni(w.z));
+    return chunks > 0;
   };
-  auto ask_tile = [&](int turn, int job) { return ask_more(turn, job, 0); };
+  auto ask_turn = [&](int turn) { return ask_for(turn, s_job + (turn == 4 * a.n_layers ? kLm : turn & 3), 0); };
 
   cluster_meet();                                              // every CTA of the cluster has its barriers set up
-  bool asked = !fin && ask_tile(0, warp);                      // the first weights of a step are asked for at the end of the one before
+  bool asked = !fin && ask_turn(0);                      // the first weights of a step are asked for at the end of the one before
   while (!fin) {
     // ---------------------------------------------------------------- search (Sec. 3.1; App. B.3 step 1); half of the warps: rotation factors
     const int nn = max(0, min(n, a.stride)), n_cand = nn - 2 * a.gamma + 1;
@@ -440,8 +471,8 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     // ---------------------------------------------------------------- embedding and first norm, all rows in every CTA.  Row r: the last accepted
     // token, then the draft (rows past it are dead: nothing of theirs is accepted or cached)
 #pragma unroll 1
-    for (int row = warp; row < R; row += kWarps) {
-      int tok = row == 0 || row > dl ? s_hist[nn - 1] : s_hist[from + row - 1];
+    for (int r = warp; r < R; r += kWarps) {
+      int tok = r == 0 || r > dl ? s_hist[nn - 1] : s_hist[from + r - 1];
       tok = tok < 0 ? 0 : (tok >= a.vocab ? a.vocab - 1 : tok);
       const __nv_bfloat16* er = a.embed + (size_t)tok * d;
       float ss = 0.f;
@@ -460,12 +491,12 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
           ss += v.x * v.x + v.y * v.y;
           split2(v.x * gv.x, v.y * gv.y, hi[q], lo[q]);
         }
-        uint8_t* dst = s_xn + (f >> 4) * TB + kRows + row * 64 + 2 * (f & 15);
+        uint8_t* dst = s_xn + (f >> 4) * TB + kRows + r * 64 + 2 * (f & 15);
         *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
         *reinterpret_cast<uint4*>(dst + 32) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         const int own = (f >> 4) - d0;
         if (own >= 0 && own < dn) {
-          float* xd = s_x + (own * Rp + row) * 16 + (f & 15);
+          float* xd = s_x + (own * Rp + r) * 16 + (f & 15);
           *reinterpret_cast<float4*>(xd) = make_float4(x[0], x[1], x[2], x[3]);
           *reinterpret_cast<float4*>(xd + 4) = make_float4(x[4], x[5], x[6], x[7]);
         }
@@ -473,7 +504,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
 #pragma unroll 1
-      for (int i = lane; i < dt; i += 32) *reinterpret_cast<float*>(s_xn + i * TB + 4 * row) = i == 0 ? ss : 0.f;
+      for (int i = lane; i < dt; i += 32) *reinterpret_cast<float*>(s_xn + i * TB + 4 * r) = i == 0 ? ss : 0.f;
     }
     __syncthreads();
     if (tid == 0) *s_best = none;
@@ -488,13 +519,9 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
 #pragma unroll 1
     for (int turn = 0; turn <= 4 * a.n_layers; ++turn) {
       const int l = min(turn >> 2, a.n_layers - 1), kind = turn == 4 * a.n_layers ? kLm : turn & 3;
-      const int4 par = s_kind[kind];
-      const int tiles = par.x, kb = par.y;
-      const uint8_t* op = smem + par.w + op_at;
+      const Job* job = s_job + kind;
       const uint32_t parity = (uint32_t)(layers_done + l) & 1u;
-      // few tiles: a warp for every quarter of the tokens
-      const bool one = NT > 1 && kind != kLm && tiles * NT <= kWarps;
-      const int qb = one ? warp % NT : 0, jobs = one ? tiles * NT : tiles, rows = min(R - 4 * qb, one ? 4 : 4 * NT);
+      const int jobs = uni(job->jobs);
       int tl = warp;                                           // job
 #pragma unroll 1
       do {
@@ -594,7 +621,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
             s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 1);
             s_lo += __shfl_xor_sync(0xffffffffu, s_lo, 2);
             s_hi += __shfl_xor_sync(0xffffffffu, s_hi, 2);
-            ask_tile(turn, warp);                              // this projection's weights, beside the reduction (lower half of the ring)
+            ask_turn(turn);                                    // this projection's weights, beside the reduction (lower half of the ring)
             // a thread holds dims kDims * 2t .. and kDims * (2t + 1) .. of its two rows
             float* so = s_red + warp * kRed;
 #pragma unroll
@@ -647,14 +674,14 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
             if (!silent(kXAttn))
 #pragma unroll 1
               for (int s = 0; s < S; ++s) {
-                const uint32_t dst = peer(base, kvh * S + s), at = dst + (uint32_t)(a.at.po + slice * a.slice_bytes);
+                const uint32_t dst = peer(base, kvh * S + s), at = dst + (uint32_t)(a.at.act + slice * a.slice_bytes);
 #pragma unroll 1
                 for (int i = 16 * tid; i < a.slice_bytes; i += 16 * kThreads) send16(at + i, *reinterpret_cast<const uint4*>(s_stage + i), dst + bars + 8 * kXAttn);
               }
             // the block's K/V rows into the cache, by the CTA that will read them
 #pragma unroll 1
-            for (int row = warp; row < 2 * (dl + 1); row += kWarps) {
-              const int tok = row >> 1, is_v = row & 1;
+            for (int r = warp; r < 2 * (dl + 1); r += kWarps) {
+              const int tok = r >> 1, is_v = r & 1;
               if ((((kv + tok) >> 4) & (S - 1)) == slice && lane < DH / 8)
                 *reinterpret_cast<uint4*>((is_v ? Vg : Kg) + (uint32_t)((kv + tok) * DH + 8 * lane)) =
                     *reinterpret_cast<const uint4*>(s_kn + ((is_v * kParts + lane % kParts) * Rp + tok) * 32 + lane / kParts * 16);
@@ -705,7 +732,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
                   const float* p = s_sums + (i * R + tok) * 16 + f;
                   float* x = s_x + (i * Rp + tok) * 16 + f;
                   v = *x;
-#pragma unroll 4
+#pragma unroll 8
                   for (int q = 0; q < senders; ++q) v += p[q * dn * R * 16];
                   *x = v;
                   __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(s_norm + i * TB + kRows + tok * 64) + f;
@@ -731,20 +758,23 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
         }
         float acc[NT][2];
         if (tl < jobs) {
-          // sums of this warp's tile: rows g and g + 8, tokens 4q + t; a thread's piece of a row of 128 bytes lies where the copy's swizzle put it
+          // sums of this warp's tile: rows row and row + 8, tokens 4q + t; a thread's piece of a row of 128 bytes lies where the copy's swizzle put it
           float sum[2][NT][4];
 #pragma unroll
           for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int q = 0; q < NT; ++q) { sum[h][q][0] = 0.f; sum[h][q][1] = 0.f; sum[h][q][2] = 0.f; sum[h][q][3] = 0.f; }
-          const uint8_t* opq = op + qb * 256;
+          const int4 what = *reinterpret_cast<const int4*>(&job->op);
+          const int kb = uni(what.y);
+          const bool one = uniform((uint32_t)what.z) != 0;
+          const uint8_t* opq = smem + what.x + op_at + job->quarter * 256;
 #pragma unroll 1
           for (int i0 = 0; i0 < kb; i0 += 2 * kRing) {
             if (!try_wait(ring_bar, ring_parity)) wait_long(ring_bar, ring_parity, s_abort, a.wait_ns, a.status);
             __syncwarp();
             ring_parity ^= 1u;
             const int here = min(2 * kRing, kb - i0);
-            const int at0 = 16 * (t ^ g), at1 = 16 * ((t + 4) ^ g);
+            const int at0 = 16 * (t ^ row), at1 = 16 * ((t + 4) ^ row);
             int i = 0;
 #pragma unroll 1
             for (; i + 4 <= here; i += 4)
@@ -754,7 +784,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
             for (; i < here; ++i) multiply_block<NT>(sum, ring_at + 2048 * (i >> 1) + (i & 1 ? at1 : at0), opq + 2 * TB * i, one);
             opq += 4 * TB * kRing;
             __syncwarp();                                      // (the ring is filled again)
-            if (i0 + 2 * kRing < kb) ask_more(turn, tl, i0 / 2 + kRing);
+            if (i0 + 2 * kRing < kb) ask_for(turn, job, i0 / 2 + kRing);
           }
 #pragma unroll
           for (int q = 0; q < NT; ++q) {
@@ -764,10 +794,11 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
         }
         if (tl == warp && (kind == kQkv || kind == kGateUp)) __syncthreads();   // (1/rms is there)
         if (tl < jobs) {
-          const int tile = one ? warp / NT : tl;
+          const int tile = job->tile, qb = job->quarter;
+          const bool one = uniform((uint32_t)job->one) != 0;
           if (kind == kLm) {
             // a tile of 16 ids: the largest sum of each token, and of the warp's tiles (1/rms scales all of a token's sums alike)
-            const int r0 = 16 * (l0 + tile) + g;
+            const int r0 = 16 * tile + row;
 #pragma unroll
             for (int q = 0; q < NT; ++q) {
               float v = r0 < a.vocab ? acc[q][0] : -INFINITY;
@@ -783,7 +814,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
               if (g == 0 && (tl == warp || v > __uint_as_float(best->x))) *best = make_uint2(__float_as_uint(v), (uint32_t)id);
             }
           } else if (kind == kGateUp) {
-            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(s_act + (tile >> 1) * TB + kRows) + (4 * qb + t) * 32 + (tile & 1) * 8 + g;
+            __nv_bfloat16* st = reinterpret_cast<__nv_bfloat16*>(s_act + (tile >> 1) * TB + kRows) + (4 * qb + t) * 32 + (tile & 1) * 8 + row;
 #pragma unroll
             for (int q = 0; q < NT; ++q)
               if (q == 0 || !one) {
@@ -791,10 +822,8 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
                 split1(__fdividef(gate, 1.f + __expf(-gate)) * up, st + q * 128, st + q * 128 + 16);
               }
           } else {
-            // queries, keys or values to every CTA of their KV head (of keys and values the leading terms: what the cache holds), or a tile's share
-            // of the residual stream's sums to the CTA that holds the tile
             const bool qkv = kind == kQkv;
-            const int head = (q0 + tile) / kParts, part = (q0 + tile) % kParts, own = s_owner[qkv ? 0 : kind == kOut ? o0 + tile : tile];
+            const int head = tile / kParts, part = tile % kParts;
             uint8_t* st = mine + (4 * qb + t) * 64;
             __syncwarp();
 #pragma unroll
@@ -804,14 +833,14 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
                 if (qkv) {
                   const int tok = min(4 * (qb + q) + t, R - 1);
                   const float rt = s_rstd[tok];
-                  const float2 r = head < H + Hkv ? s_rope[tok * kHalf + 8 * part + g] : make_float2(1.f, 0.f);
+                  const float2 r = head < H + Hkv ? s_rope[tok * kHalf + 8 * part + row] : make_float2(1.f, 0.f);
                   x *= rt;
                   y *= rt;
-                  __nv_bfloat16* sb = reinterpret_cast<__nv_bfloat16*>(st + q * 256) + g;
+                  __nv_bfloat16* sb = reinterpret_cast<__nv_bfloat16*>(st + q * 256) + row;
                   split1(x * r.x - y * r.y, sb, sb + 16);
                   split1(y * r.x + x * r.y, sb + 8, sb + 24);
                 } else {
-                  float* sf = reinterpret_cast<float*>(st + q * 256) + g;
+                  float* sf = reinterpret_cast<float*>(st + q * 256) + row;
                   sf[0] = x;
                   sf[8] = y;
                 }
@@ -819,27 +848,28 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
             __syncwarp();
             const int x = qkv ? kXQkv : kind == kOut ? kXOut : kXDown;
             if (!silent(x)) {
-              const bool is_q = head < H, terms = !qkv || is_q;
-              const int kh = is_q ? head / G : head < H + Hkv ? head - H : head - H - Hkv;
-              // (own: the CTA, how many tiles it holds, which of them this is)
-              const int at = !qkv ? a.at.sums + ((kind == kOut ? kvh : c) * (own >> 8 & 255) + (own & 255)) * 64 * R + qb * 256
-                           : is_q ? a.at.q + kRows + ((head - kh * G) * kParts + part) * TB + qb * 256
-                                  : a.at.kv + ((head < H + Hkv ? 0 : kParts) + part) * 32 * Rp + qb * 128;
-              const int first = qkv ? kh * S : own >> 16, last = qkv ? first + S : first + 1;
+              const int4 to_at = *reinterpret_cast<const int4*>(&job->at);
+              const bool whole = job->whole != 0;
               const uint8_t* from_st = mine + qb * 256;
 #pragma unroll 1
-              for (int p = first; p < last; ++p) {
+              for (int p = to_at.y; p < to_at.z; ++p) {
                 const uint32_t dst = peer(base, p);
 #pragma unroll 1
-                for (int i = lane; i < (terms ? 4 : 2) * rows; i += 32)
-                  send16(dst + at + 16 * i, *reinterpret_cast<const uint4*>(from_st + (terms ? 16 * i : (i >> 1) * 64 + (i & 1) * 16)), dst + bars + 8 * x);
+                for (int i = lane; i < to_at.w; i += 32)
+                  send16(dst + to_at.x + 16 * i, *reinterpret_cast<const uint4*>(from_st + (whole ? 16 * i : (i >> 1) * 64 + (i & 1) * 16)), dst + bars + 8 * x);
               }
             }
           }
         }
         // what comes next, once what others wait for is on its way
         tl += kWarps;
-        if (tl < jobs) ask_tile(turn, tl);
+        if (tl < jobs) {
+          __syncwarp();
+          if (lane == 0) describe(s_job + kLm + 1, kind, tl);
+          __syncwarp();
+          job = s_job + kLm + 1;
+          ask_for(turn, job, 0);
+        }
       } while (tl < jobs);
       if (kind == kQkv && attends) {
         // this warp's first block of cached keys, while the queries travel (behind the cached rows there may be anything: 0 x NaN is NaN)
@@ -847,7 +877,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
         Vg = Kg + k_half;
         if (kg * S + slice < nold) load_cached<DH>(kf, vf, Kg, Vg, (kg * S + slice) * 16, kv, g, t);
       }
-      if (kind != kLm && kind != kQkv) ask_tile(turn + 1, warp);   // (behind QKV the keys come first)
+      if (kind != kLm && kind != kQkv) ask_turn(turn + 1);     // (behind QKV the keys come first)
     }
     layers_done += a.n_layers;
     // the largest of `count` lists for a token, by 16 lanes
@@ -872,7 +902,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     __syncthreads();
     if (!silent(kXMax) && warp < NC && lane < Rp / 2)
       send16(to + (uint32_t)(a.at.misc + 8 * c * Rp + 16 * lane), *reinterpret_cast<const uint4*>(s_stage + 16 * lane), to + bars + 8 * kXMax);
-    asked = ask_tile(0, warp);
+    asked = ask_turn(0);
     wait(kXMax, step_parity);
     step_parity ^= 1u;
     // ------------------------------------------------------------------ acceptance (App. B.2) and append (App. B.3 step 4)
@@ -984,8 +1014,7 @@ bool small_shape(const cs_model_config& c, int R, int NC, int stride, SmallShape
   auto take = [&](long long bytes) { const long long at = off; off += (bytes + 15) & ~15ll; return (int)min(at, 1ll << 30); };
   out->at.xn = take(d / 16 * tile);
   out->at.at = take(G * parts * tile);
-  out->at.act = take(2 * cs_ceil_div(F / 32, NC) * tile);
-  out->at.po = take((long long)out->slice_bytes << out->log_slices);
+  out->at.act = take(max(2 * cs_ceil_div(F / 32, NC) * tile, (long long)out->slice_bytes << out->log_slices));
   out->at.sums = take(64ll * NC * out->own_d * R);
   out->at.stage = take(max(64ll * Rp * kWarps, (long long)out->slice_bytes));
   out->at.norm = take(out->own_d * tile);
@@ -997,12 +1026,11 @@ bool small_shape(const cs_model_config& c, int R, int NC, int stride, SmallShape
   out->at.gain0 = take(2ll * d);
   out->at.rope = take(4ll * Rp * c.head_dim);
   out->at.turn = take(16ll * (R + 2) * (c.head_dim / 2));
-  out->at.owner = take(4ll * (d / 16));
-  out->at.kinds = take(16 * 5);
+  out->at.jobs = take((long long)sizeof(Job) * 6 * kWarps);
   off = (off + 1023) & ~1023ll;       // (the copies' swizzle goes by the address)
   out->at.ring = take(2048ll * kRing * kWarps);
   out->at.hist = take(4ll * stride);
-  out->at.misc = take(8ll * (kMaxCluster + kWarps) * Rp + 8ll * (kExchanges + kWarps) + 12ll * Rp + 16);
+  out->at.misc = take(8ll * kMaxCluster * Rp + 8ll * (kExchanges + kWarps) + 12ll * Rp + 16);
   out->at.total = (int)min(off, 1ll << 30);
   return off <= 227 * 1024;
 }
@@ -1013,11 +1041,11 @@ bool small_shape(const cs_model_config& c, int R, int NC, int stride, SmallShape
 // heads of 64), and all sequences' clusters at once - of sixteen CTAs, or of eight where that is too many.  Calls of 6 to 8 steps, launch by
 // launch / here, us (sequences x rows, tokens of history):
 //                                        1 x 11, 512   1 x 1, 2000   1 x 11, 3500  4 x 11, 1000  8 x 4, 600   8 x 13, 600   14 x 7, 600   1 x 8, 8000
-//   2 layers of 2.0 MiB, heads of 32        659/357       607/321       729/450       644/289       608/285      783/388       790/321
-//   8 of them                              1870/1130     1729/1016     2115/1471     1940/895      1774/865     2445/1206     2442/1006
-//   2 of 1.2 MiB, heads of 64               695/479       611/417       725/613       632/389       628/357      785/528       800/494       555/646
-//   4 of 0.5 MiB (eight CTAs)              1079/648       918/514      1109/828       964/515       953/374     1292/544      1290/435       804/614
-//   2 of 2.0 MiB, LM head of 16 MiB         699/536       646/441       750/630       685/422       635/457      830/701       837/533       587/551
+//   2 layers of 2.0 MiB, heads of 32        671/323       618/301       730/415       657/264       617/263      789/343       795/296
+//   8 of them                              1865/1005     1727/940      2114/1349     1957/804      1784/783     2443/1040     2439/900
+//   2 of 1.2 MiB, heads of 64               706/456       619/401       729/591       641/369       633/341      799/508       807/405       552/557
+//   4 of 0.5 MiB (eight CTAs)              1089/593       923/486      1120/767       971/476       960/352     1298/482      1293/402       807/584
+//   2 of 2.0 MiB, LM head of 16 MiB         702/501       657/409       743/594       692/395       638/417      832/645       842/502       578/529
 // Sixteen CTAs stream a larger model from L2 slower than the chip does: 2 layers of 4.5 MiB with an LM head of 8 MiB 878/1352 for 16 x 7 rows, of 17 MiB
 // 768/1122 for one row.  Clusters that do not all run at once wait for one another: 16 sequences of 7 rows with the 16 MiB LM head 857/1025.
 cs_status cs_launch_small_loop(cs_ctx* ctx, bool* taken, cudaStream_t st) {
