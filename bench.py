@@ -772,12 +772,14 @@ def run_step_timeline(args, cs, inputs, dev, cfg):
     for i in range(1, S + 1):
         for j in range(nst):
             iv[j] += (ends[i, j] - (ends[i, j - 1] if j else ends[i - 1, nst - 1])) / S / 1e3
-    # launches of a step: search, set-up, embedding, then per layer QKV, attention, merge, O, gate/up, down, then LM head, acceptance, commit
-    per_layer = (nst - 6) // cfg.n_layers
-    if per_layer != 6:
-        raise RuntimeError(f"unexpected launch layout: {nst} launches for {cfg.n_layers} layers")
-    lay = iv[3:3 + 6 * cfg.n_layers].reshape(cfg.n_layers, 6)
+    # launches of a step: search, set-up, embedding, then per layer QKV, attention, merge (not where the keys are one slice), O, gate/up, down,
+    # then LM head, acceptance, commit
     names = ["qkv", "attention", "merge", "o", "gate_up", "down"]
+    if "merge" not in fams:
+        names.remove("merge")
+    if nst - 6 != len(names) * cfg.n_layers:
+        raise RuntimeError(f"unexpected launch layout: {nst} launches for {cfg.n_layers} layers")
+    lay = iv[3:3 + len(names) * cfg.n_layers].reshape(cfg.n_layers, len(names))
     line = {"metric": "step timeline", "value": float(iv.sum()), "unit": "us", "higher_is_better": False, "n_gpus": 1,
             "steps": S, "warmup": W, "ms_per_step": e0.elapsed_time(e1) / (S + 1), "dtype": "bf16", "data": "synthetic",
             "config": {"workload": "step_timeline", "batch": B, "k": k, "kv": args.kv, "layers": cfg.n_layers,

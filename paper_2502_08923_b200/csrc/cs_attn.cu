@@ -356,20 +356,20 @@ int cs_launch_attention(cs_ctx* ctx, const void* kv_cache, int layer, int B, int
   // head_dim 128 runs on the tcgen05 kernels.  The one with the query rows as M does a tile's work of
   // 128 rows whatever the block holds, but has the shorter chain; the one with keys and head dims as M does
   // only that of the real rows, and takes blocks of up to 48 rows per KV head whose CTAs walk many tiles.
-  // Measured per layer, rows as M / keys as M, attention and merge, 44 rows: 14 tiles 30.3 / 28.6 us, 17 tiles
-  // 34.5 / 31.9, 20 tiles 39.8 / 35.7, 28 tiles 50.7 / 44.3, 33 tiles 58.0 / 49.7, 65 tiles 113.8 / 89.8; 84 rows,
-  // 65 tiles: 120.2 / 173.9.  The line is older than these figures (K and V of the other kernel did not leave L2 first,
-  // 13 tiles were 32.4 / 33.2 and 16 tiles 36.1 / 37.2), and blocks of few rows would gain from that kernel sooner still: 4 rows, 5 tiles
-  // 18.0 / 18.1, 9 tiles 23.8 / 21.4, 17 tiles 35.0 / 30.8, 32 tiles 56.4 / 48.5; 16 rows, 5 tiles 20.2 / 18.7, 9 tiles
-  // 24.9 / 22.1, 14 tiles 32.4 / 29.1, 32 tiles 56.5 / 49.6; 28 rows, 9 tiles 25.0 / 25.1, 15 tiles 32.7 / 31.2.  The register-resident mma.sync kernel takes the other head sizes.
+  // Whole layers, rows as M / keys as M, us, with caches that are full - 44 rows: 9 tiles 139.8 / 140.2, 14 tiles 147.0 / 145.8, 20 tiles 155.8 /
+  // 152.0 (4 sequences); 28 rows: 9 tiles 140.3 / 141.5, 20 tiles 155.5 / 153.2 (8); 16 rows: 5 tiles 115.2 / 114.5, 9 tiles 120.4 / 118.3, 20 tiles
+  // 135.5 / 130.8 (4); 84 rows, 65 tiles, attention and merge alone: 120.2 / 173.9.  Full caches would gain from 7 tiles on with up to 16 rows
+  // and from 13 with up to 48, by 1 - 2 %.  But tiles are counted from the cache's size, and where it is mostly empty the second
+  // kernel's start, 2 - 4 us slower, is what counts: 44 rows over 500 or 4,000 keys in a cache of 40,000 106.6 / 110.5 and 108.4 / 112.5, 16 rows over
+  // 300 of 4,600 117.3 / 118.6; so the line stays where the walk is long.  The register-resident mma.sync kernel takes the other head sizes.
   // CS_ATTN_KERNEL=tc|tcw|mma, read when the context is created, forces one of them (tests run
   // them on the same inputs).
   int nsplit = 0;
   if (ctx->attn_force != 1) {
     const bool wide = ctx->attn_force == 3 || (ctx->attn_force == 0 && cs_attention_tc_tiles_per_cta(ctx, B, R) > 20 &&
                                                ctx->cfg.n_heads / ctx->cfg.n_kv_heads * R <= 48);
-    if (wide) nsplit = cs_launch_attention_tcw(ctx, kv_cache, layer, B, R, st);
-    if (nsplit == 0) nsplit = cs_launch_attention_tc(ctx, kv_cache, layer, B, R, st);
+    if (wide) nsplit = cs_launch_attention_tcw(ctx, kv_cache, layer, B, R, &merge, st);
+    if (nsplit == 0) nsplit = cs_launch_attention_tc(ctx, kv_cache, layer, B, R, &merge, st);
   }
   if (nsplit <= 0)
     switch (ctx->cfg.head_dim) {

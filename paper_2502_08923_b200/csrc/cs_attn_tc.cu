@@ -62,6 +62,7 @@ struct AttnArgs {
   float scale_log2e;
   float* out_o;
   float* out_ml;
+  __nv_bfloat16* whole;   // kWhole: the attention output, two bf16 terms
   int* status;
   unsigned long long wait_ns;
   unsigned long long* stamp;
@@ -140,6 +141,7 @@ __device__ __forceinline__ bool quarter_any(int quarter, bool pred) {
   return out != 0;
 }
 
+template <bool kWhole>   // one slice: what is written is the attention output itself, and there is nothing to merge
 __global__ void __launch_bounds__(kThreads, 1)
 k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmQ, AttnArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -451,13 +453,35 @@ k_attn_tc(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUte
     quarter_any(quarter, false);
     if (valid) {
       const size_t obase = ((size_t)split * a.rows + (b * R + r0 + q / G)) * a.H + (kvh * G + q % G);
-      float* dst = a.out_o + obase * kDh + 32 * part;
+      auto sum = [&]() { return have ? (s_x[q] + s_x[128 + q]) + (s_x[256 + q] + s_x[384 + q]) : 0.f; };
+      if constexpr (kWhole) {
+        // nothing to merge: normalised, as the next projection's operand (what k_attn_merge makes of one slice)
+        const float l = sum(), inv = l > 0.f ? 1.f / l : 0.f;
+        __nv_bfloat16* dst = a.whole + obase * kDh + 32 * part;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) store8(dst + 8 * j, o + 8 * j);   // (whole 32-byte sectors)
-      if (part == 0) {
-        constexpr float kLn2 = 0.6931471805599453f;
-        a.out_ml[obase * 2] = have ? m * kLn2 : -INFINITY;
-        a.out_ml[obase * 2 + 1] = have ? (s_x[q] + s_x[128 + q]) + (s_x[256 + q] + s_x[384 + q]) : 0.f;
+        for (int j = 0; j < 4; ++j) {
+          uint32_t h[4], w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float y0 = o[8 * j + 2 * e] * inv, y1 = o[8 * j + 2 * e + 1] * inv;
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(y0, y1);
+            const float2 f = __bfloat1622float2(hi);
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(y0 - f.x, y1 - f.y);
+            h[e] = *reinterpret_cast<const uint32_t*>(&hi);
+            w[e] = *reinterpret_cast<const uint32_t*>(&lo);
+          }
+          *reinterpret_cast<uint4*>(dst + 8 * j) = make_uint4(h[0], h[1], h[2], h[3]);
+          *reinterpret_cast<uint4*>(dst + (size_t)CS_MAX_ROWS * a.H * kDh + 8 * j) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+      } else {
+        float* dst = a.out_o + obase * kDh + 32 * part;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) store8(dst + 8 * j, o + 8 * j);   // (whole 32-byte sectors)
+        if (part == 0) {
+          constexpr float kLn2 = 0.6931471805599453f;
+          a.out_ml[obase * 2] = have ? m * kLn2 : -INFINITY;
+          a.out_ml[obase * 2 + 1] = sum();
+        }
       }
     }
     if (*s_abort && lane == 0) atomicOr(a.status, CS_DEV_TIMEOUT);
@@ -487,7 +511,7 @@ int cs_attention_tc_tiles_per_cta(const cs_ctx* ctx, int B, int R) {
   return cs_ceil_div(cs_ceil_div(c.max_seq, kTileKeys), nsplit);
 }
 
-int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, cudaStream_t st) {
+int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, bool* merge, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
   const int G = c.n_heads / c.n_kv_heads;
   if (c.head_dim != kDh || G > kNQMax || R < 1 || R > 256) return 0;
@@ -513,10 +537,12 @@ int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, 
   // rows of the softmax
   const size_t smem = 1024 + (size_t)kSlots * kSlotBytes + kCtlBytes + 4 * 128 * 4;
   int nsplit = ctx->num_sms / (B * c.n_kv_heads * ngroups);
+  const bool whole = *merge && nsplit <= 1;            // (a cache of one tile is one slice too, but not worth a path of its own)
   if (nsplit > ctx->attn_splits) nsplit = ctx->attn_splits;
   if (nsplit < 1) nsplit = 1;
   if (smem > ctx->attn_tc_smem_set) {
-    if (cudaFuncSetAttribute(k_attn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_attn_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_attn_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       snprintf(ctx->err, sizeof(ctx->err), "attention needs %zu bytes of shared memory", smem);
       return -1;
     }
@@ -529,12 +555,13 @@ int cs_launch_attention_tc(cs_ctx* ctx, const void* kv_cache, int layer, int B, 
   a.max_batch = c.max_batch; a.max_seq = c.max_seq; a.nsplit = nsplit; a.rows = B * R;
   a.smem_bytes = (int)smem;
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)kDh);
-  a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.status = ctx->d_status;
+  a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.whole = ctx->attn_out; a.status = ctx->d_status;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, CS_FAM_ATTENTION);
-  if (cs_launch_pdl(k_attn_tc, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
+  if (cs_launch_pdl(whole ? k_attn_tc<true> : k_attn_tc<false>, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
     snprintf(ctx->err, sizeof(ctx->err), "attention launch failed");
     return -1;
   }
+  if (whole) *merge = false;
   return nsplit;
 }

@@ -70,6 +70,7 @@ struct AttnArgs {
   float scale_log2e;
   float* out_o;
   float* out_ml;
+  __nv_bfloat16* whole;   // kWhole: the attention output, two bf16 terms
   int* status;
   unsigned long long wait_ns;   // limit of every bounded wait
   unsigned long long* stamp;    // step timeline slot of this launch, or NULL
@@ -161,6 +162,7 @@ __device__ __forceinline__ bool group_any(int id, bool pred) {
   return out != 0;
 }
 
+template <bool kWhole>   // one slice: what is written is the attention output itself, and there is nothing to merge
 __global__ void __launch_bounds__(kThreads, 1)
 k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmQ, AttnArgs a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -601,6 +603,33 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
       if (!ok) { *s_abort = 1; have = false; }
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    // the column sums: add the 128 key lanes' shares up (warp shuffle, then the four warps of the group).  A slice's output does not wait for them.
+    float* sum_w = s_red + warp * kCols;
+    const float* red = s_red + (grp * 4) * kCols;
+    auto add_up = [&]() {
+#pragma unroll
+      for (int c = 0; c < kCols / 8; ++c) {
+        if (c < nch) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float t, t_other;
+            if (j & 1) unpack2(lsum[(8 * c + j) >> 1], t_other, t); else unpack2(lsum[(8 * c + j) >> 1], t, t_other);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+            if (lane == 0) sum_w[8 * c + j] = t;
+          }
+        }
+      }
+      group_all(1 + grp, true);
+    };
+    if constexpr (kWhole) {
+      add_up();
+      if (lane < ncol) {                               // (every warp its own copy of its columns' 1 / sum)
+        const float l = have ? (red[lane] + red[kCols + lane]) + (red[2 * kCols + lane] + red[3 * kCols + lane]) : 0.f;
+        w_nme[lane] = l > 0.f ? 1.f / l : 0.f;
+      }
+      __syncwarp();
+    }
     // O^T: this thread holds head dim `row` of its columns; one 512-byte row of the partial output per column
 #pragma unroll
     for (int c = 0; c < kCols / 8; ++c) {
@@ -619,34 +648,37 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
 #pragma unroll
           for (int j = 0; j < 8; ++j) o[j] = 0.f;
         }
+        if constexpr (kWhole) {
+          // Nothing to merge: normalised, as the next projection's operand (what k_attn_merge makes of one slice).  Neighbouring lanes swap, so that
+          // each writes two dims of one of two columns.
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int q = q0 + 8 * c + j;
-          if (q < nq) {
-            const size_t obase = ((size_t)split * a.rows + (b * R + r0 + q / G)) * a.H + (kvh * G + q % G);
-            a.out_o[obase * kDh + row] = o[j];
+          for (int j = 0; j < 8; j += 2) {
+            const float y0 = o[j] * w_nme[8 * c + j], y1 = o[j + 1] * w_nme[8 * c + j + 1];
+            const float got = __shfl_xor_sync(0xffffffffu, lane & 1 ? y0 : y1, 1);
+            const float d0 = lane & 1 ? got : y0, d1 = lane & 1 ? y1 : got;
+            const int q = q0 + 8 * c + j + (lane & 1);
+            if (q < nq) {
+              const __nv_bfloat162 hi = __floats2bfloat162_rn(d0, d1);
+              const float2 f = __bfloat1622float2(hi);
+              __nv_bfloat16* dst = a.whole + ((size_t)(b * R + r0 + q / G) * a.H + (kvh * G + q % G)) * kDh + (row & ~1);
+              *reinterpret_cast<__nv_bfloat162*>(dst) = hi;
+              *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)CS_MAX_ROWS * a.H * kDh) = __floats2bfloat162_rn(d0 - f.x, d1 - f.y);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int q = q0 + 8 * c + j;
+            if (q < nq) {
+              const size_t obase = ((size_t)split * a.rows + (b * R + r0 + q / G)) * a.H + (kvh * G + q % G);
+              a.out_o[obase * kDh + row] = o[j];
+            }
           }
         }
       }
     }
-    // the column sums: add the 128 key lanes' shares up (warp shuffle, then the four warps of the group)
-    float* sum_w = s_red + warp * kCols;
-#pragma unroll
-    for (int c = 0; c < kCols / 8; ++c) {
-      if (c < nch) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          float t, t_other;
-          if (j & 1) unpack2(lsum[(8 * c + j) >> 1], t_other, t); else unpack2(lsum[(8 * c + j) >> 1], t, t_other);
-#pragma unroll
-          for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-          if (lane == 0) sum_w[8 * c + j] = t;
-        }
-      }
-    }
-    group_all(1 + grp, true);
-    if (wq == 0) {
-      const float* red = s_red + (grp * 4) * kCols;
+    if constexpr (!kWhole) add_up();
+    if (wq == 0 && !kWhole) {
       const float* m_fin = w_mo;                       // (warp 4 * grp: its own copy)
       constexpr float kLn2 = 0.6931471805599453f;
       for (int col = lane; col < ncol; col += 32) {
@@ -675,7 +707,7 @@ k_attn_tcw(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUt
 
 }  // namespace
 
-int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, cudaStream_t st) {
+int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B, int R, bool* merge, cudaStream_t st) {
   const cs_model_config& c = ctx->cfg;
   const int G = c.n_heads / c.n_kv_heads;
   if (c.head_dim != kDh || G > kNQMax || R < 1 || R > 256) return 0;
@@ -705,10 +737,12 @@ int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B,
   const size_t smem = 1024 + (size_t)4 * NQ * 128 + kPBufs * natoms * kHalfBytes + (size_t)2 * kStages * 2 * kHalfBytes +
                       kCtlBytes + kNQMax * 4 + kSoftWarps * 3 * kCols * 4 + 2 * kSoftWarps * kCols * 4;
   int nsplit = ctx->num_sms / (B * c.n_kv_heads * ngroups);
+  const bool whole = *merge && nsplit <= 1;            // (a cache of one tile is one slice too, but not worth a path of its own)
   if (nsplit > ctx->attn_splits) nsplit = ctx->attn_splits;
   if (nsplit < 1) nsplit = 1;
   if (smem > ctx->attn_tcw_smem_set) {
-    if (cudaFuncSetAttribute(k_attn_tcw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_attn_tcw<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k_attn_tcw<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       snprintf(ctx->err, sizeof(ctx->err), "attention needs %zu bytes of shared memory", smem);
       return -1;
     }
@@ -721,12 +755,13 @@ int cs_launch_attention_tcw(cs_ctx* ctx, const void* kv_cache, int layer, int B,
   a.max_batch = c.max_batch; a.max_seq = c.max_seq; a.nsplit = nsplit; a.NQ = NQ; a.rows = B * R;
   a.smem_bytes = (int)smem;
   a.scale_log2e = 1.4426950408889634f / sqrtf((float)kDh);
-  a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.status = ctx->d_status;
+  a.out_o = ctx->attn_o; a.out_ml = ctx->attn_ml; a.whole = ctx->attn_out; a.status = ctx->d_status;
   a.wait_ns = ctx->wait_limit_ns;
   a.stamp = cs_next_stamp(ctx, CS_FAM_ATTENTION);
-  if (cs_launch_pdl(k_attn_tcw, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
+  if (cs_launch_pdl(whole ? k_attn_tcw<true> : k_attn_tcw<false>, dim3(B * c.n_kv_heads, nsplit, ngroups), dim3(kThreads), smem, st, ctx->tmKV, ctx->tmQ, a) != cudaSuccess) {
     snprintf(ctx->err, sizeof(ctx->err), "attention launch failed");
     return -1;
   }
+  if (whole) *merge = false;
   return nsplit;
 }
