@@ -8,9 +8,10 @@
 // No global scratch memory, no global atomics, one launch, deterministic.
 //
 // Bound by a chain of latencies: length, tokens (through L2), cluster barrier, draft.  Launched back to back, us a search, with a load waited
-// for per group of candidates and two barriers of the whole cluster behind them / now: 1 x 4,097 tokens 3.02 / 2.89, 1 x 32,768
-// 3.77 / 3.03, 8 x 8,192 3.97 / 3.24, 64 x 4,096 3.97 / 3.52, 64 x 32,768 7.53 / 5.39, 64 x 131,072 18.3 / 11.9.  (The second four
-// tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and 13.5 for the last two.)
+// for per group of candidates, two barriers of the whole cluster behind them and rows off 16 bytes read token by token / now: 1 x 4,097 tokens 3.03 /
+// 2.67, 1 x 32,768 3.76 / 3.10, 8 x 5,003 6.13 / 3.08, 64 x 1,003 3.77 / 2.82, 32 x 20,002 6.95 / 4.3, 64 x 30,001 10.0 / 5.6, 64 x 32,768
+// 7.4 / 5.6, 64 x 131,072 18.2 / 12.2.  (The second four tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and
+// 13.5 for the last two.)
 #include <limits.h>
 
 #include "cs_common.cuh"
@@ -70,14 +71,16 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
     const int per = (((n_cand + nblk - 1) / nblk) + 3) & ~3;
     const int lo = rank * per;
     const int hi = min(n_cand, lo + per);
-    const bool vec_ok = ((reinterpret_cast<uintptr_t>(h) & 15) == 0) && gamma <= 5;
+    // Groups of four tokens begin on 16 bytes, `off` tokens ahead of the row where a row does not.  A group is loaded where it holds a token of the row.
+    const bool vec_ok = gamma <= 5;
+    const int off = vec_ok ? (int)(reinterpret_cast<uintptr_t>(h) >> 2 & 3) : 0;
     auto test = [&](const int4& u, const int4& v, int p) {
-      // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies past the
-      // accepted length only feeds candidates that `hi` masks off
+      // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies ahead of the row or past the
+      // accepted length only feeds candidates that are masked off
       const int t[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        bool eq = (p + i < hi);
+        bool eq = (unsigned)(p + i - lo) < (unsigned)(hi - lo);
 #pragma unroll
         for (int j = 0; j < 5; ++j)
           if (j < gamma) eq = eq && (t[i + j] == key[j]);
@@ -91,20 +94,21 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
         if (eq) best = latest ? max(best, p + i) : min(best, p + i);
       }
     };
-    for (int base = lo; base < hi; base += kGroups * kThreads * 4) {
+    for (int base = ((lo + off) & ~3) - off; base < hi; base += kGroups * kThreads * 4) {
       int4 u[kGroups], v[kGroups];
 #pragma unroll
       for (int q = 0; q < kGroups; ++q) {
         const int p = base + (q * kThreads + tid) * 4;
-        if (vec_ok && p < hi && p + 8 <= stride) {
+        if (vec_ok && p < hi) {
           u[q] = ld_int4(h + p);
-          v[q] = ld_int4(h + p + 4);
+          v[q] = ld_int4(h + (p + 4 < stride ? p + 4 : p));   // (behind the row's end nothing is wanted)
         }
       }
 #pragma unroll
       for (int q = 0; q < kGroups; ++q) {
         const int p = base + (q * kThreads + tid) * 4;
-        if (vec_ok && p + 8 <= stride) test(u[q], v[q], p);
+        if (base + q * kThreads * 4 >= hi) break;        // (short shares end in the first group)
+        if (vec_ok) test(u[q], v[q], p);
         else scan(p);
       }
     }
