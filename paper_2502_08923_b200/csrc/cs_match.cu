@@ -94,7 +94,8 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
         if (eq) best = latest ? max(best, p + i) : min(best, p + i);
       }
     };
-    for (int base = ((lo + off) & ~3) - off; base < hi; base += kGroups * kThreads * 4) {
+    // (An empty share, hi <= lo, has nothing to test: its first group may begin ahead of hi, and the mask in test() holds only where lo < hi.)
+    for (int base = lo < hi ? ((lo + off) & ~3) - off : hi; base < hi; base += kGroups * kThreads * 4) {
       int4 u[kGroups], v[kGroups];
 #pragma unroll
       for (int q = 0; q < kGroups; ++q) {
