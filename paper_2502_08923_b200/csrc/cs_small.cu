@@ -130,11 +130,6 @@ __device__ __noinline__ void wait_long(uint32_t bar, uint32_t parity, volatile i
       }
     }
 }
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 __device__ __forceinline__ void cluster_meet() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -593,14 +588,14 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
                 mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
                 const float n_lo = fmaxf(m_lo, mx_lo * a.scale_log2e), n_hi = fmaxf(m_hi, mx_hi * a.scale_log2e);
                 const float z_lo = n_lo == -INFINITY ? 0.f : n_lo, z_hi = n_hi == -INFINITY ? 0.f : n_hi;   // (a row may have no key here)
-                const float c_lo = ex2(m_lo - z_lo), c_hi = ex2(m_hi - z_hi);
+                const float c_lo = exp2f(m_lo - z_lo), c_hi = exp2f(m_hi - z_hi);
                 m_lo = n_lo; m_hi = n_hi;
                 s_lo *= c_lo; s_hi *= c_hi;
                 uint32_t ph[4], pl[4];
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                  const float e0 = ex2(fmaf(s[0][q][0], a.scale_log2e, -z_lo)), e1 = ex2(fmaf(s[0][q][1], a.scale_log2e, -z_lo));
-                  const float e2 = ex2(fmaf(s[0][q][2], a.scale_log2e, -z_hi)), e3 = ex2(fmaf(s[0][q][3], a.scale_log2e, -z_hi));
+                  const float e0 = exp2f(fmaf(s[0][q][0], a.scale_log2e, -z_lo)), e1 = exp2f(fmaf(s[0][q][1], a.scale_log2e, -z_lo));
+                  const float e2 = exp2f(fmaf(s[0][q][2], a.scale_log2e, -z_hi)), e3 = exp2f(fmaf(s[0][q][3], a.scale_log2e, -z_hi));
                   s_lo += e0 + e1;
                   s_hi += e2 + e3;
                   split2(e0, e1, ph[2 * q], pl[2 * q]);
@@ -644,7 +639,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
               float M = ml.x;
 #pragma unroll
               for (int off = 8; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-              const float f = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
+              const float f = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
               float sum = ml.y * f;
 #pragma unroll
               for (int off = 8; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
@@ -699,7 +694,7 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
 #pragma unroll 1
               for (int s = 0; s < S; ++s) {
                 const float2 ml = *reinterpret_cast<const float2*>(r + s * a.slice_bytes);
-                const float f = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
+                const float f = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M);
                 sum = fmaf(ml.y, f, sum);
 #pragma unroll
                 for (int x = 0; x < DH / 32; ++x) y[x] = fmaf(*reinterpret_cast<const float*>(s_po + s * a.slice_bytes + 4 * (q * DH + lane + 32 * x)), f, y[x]);
