@@ -16,8 +16,9 @@
 
 namespace {
 
+// (what vmap and other transforms hand in looks like a tensor, but has no memory of its own)
 bool plain(const at::Tensor& t, int64_t dim) {
-  return t.is_cuda() && t.scalar_type() == at::kInt && t.layout() == at::kStrided && t.dim() == dim && t.is_contiguous();
+  return t.has_storage() && t.is_cuda() && t.scalar_type() == at::kInt && t.layout() == at::kStrided && t.dim() == dim && t.is_contiguous();
 }
 
 // find_match(hist, hist_len, gamma, k, policy) -> (match_pos [B], draft [B][k], draft_len [B]), or the call's status where that
@@ -41,12 +42,16 @@ PyObject* find_match(PyObject*, PyObject* const* args, Py_ssize_t n_args) {
   const at::Tensor pos = at::detail::empty_cuda({B}, at::kInt, hist.device(), std::nullopt);
   const at::Tensor draft = at::detail::empty_cuda({B, k}, at::kInt, hist.device(), std::nullopt);
   const at::Tensor draft_len = at::detail::empty_cuda({B}, at::kInt, hist.device(), std::nullopt);
+  // (everything that may throw comes before the interpreter's lock is given up: the handler below needs it)
   void* const stream = c10::cuda::getCurrentCUDAStream().stream();
+  const int32_t* const h = static_cast<const int32_t*>(hist.const_data_ptr());
+  const int32_t* const n = static_cast<const int32_t*>(len.const_data_ptr());
+  int32_t* const out_pos = static_cast<int32_t*>(pos.mutable_data_ptr());
+  int32_t* const out_draft = k > 0 ? static_cast<int32_t*>(draft.mutable_data_ptr()) : nullptr;
+  int32_t* const out_len = static_cast<int32_t*>(draft_len.mutable_data_ptr());
   cs_status s;
   Py_BEGIN_ALLOW_THREADS
-  s = cs_find_match(static_cast<const int32_t*>(hist.const_data_ptr()), static_cast<const int32_t*>(len.const_data_ptr()), (int)B, (int)stride,
-                    (int)gamma, (int)k, (cs_match_policy)policy, static_cast<int32_t*>(pos.mutable_data_ptr()),
-                    k > 0 ? static_cast<int32_t*>(draft.mutable_data_ptr()) : nullptr, static_cast<int32_t*>(draft_len.mutable_data_ptr()), stream);
+  s = cs_find_match(h, n, (int)B, (int)stride, (int)gamma, (int)k, (cs_match_policy)policy, out_pos, out_draft, out_len, stream);
   Py_END_ALLOW_THREADS
   if (s != CS_OK) return PyLong_FromLong(s);
   PyObject* out = PyTuple_New(3);
