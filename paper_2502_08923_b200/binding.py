@@ -1,11 +1,14 @@
 """ctypes binding of libcopyspec.so: same names as the C ABI (include/copyspec.h),
 argument marshalling only.  PyTorch provides device memory and the current stream; every
 step of the path runs in the library's CUDA kernels.  There is no CPU fallback: if the
-library cannot be loaded, every call raises."""
+library cannot be loaded, every call raises.  (The search call also has its marshalling in native code;
+without that file, which goes by the versions of Python and torch, it takes the way of the other calls.)"""
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import warnings
 
 import torch
 
@@ -142,10 +145,22 @@ def load(build_if_missing: bool = True) -> C.CDLL:
     lib.cs_gram_index_status.argtypes = [vp, i, i, vp]
     lib.cs_linear.restype = i
     lib.cs_linear.argtypes = [vp, vp, vp, i, i, i, vp, vp]
-    from . import _native
-    _search = _native.find_match
+    _search = _native_search()
     _lib = lib
     return lib
+
+
+def _native_search():
+    """cs_find_match in native code, or, where there is none for this Python and torch, what leaves every call to the general path."""
+    path = _build.native_path()
+    try:
+        spec = importlib.util.spec_from_file_location(f"{__package__}._native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        return module.find_match
+    except ImportError as e:
+        warnings.warn(f"the search call's native side does not load, its general path takes all calls: {e}", RuntimeWarning)
+        return lambda *args: None
 
 
 # Addresses travel as plain integers: every pointer argument is declared c_void_p.
