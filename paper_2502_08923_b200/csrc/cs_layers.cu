@@ -426,7 +426,7 @@ __global__ void k_loop_init(const int* hist_len, const int* kv_len, int B, int s
   __syncthreads();
   for (int b = t; b < B; b += blockDim.x) {
     const int n = hist_len[b];
-    const bool fits = n >= 1 && n + max_new <= stride && n + max_new + k <= max_seq;
+    const bool fits = n >= 1 && (long long)n + max_new <= stride && (long long)n + max_new + k <= max_seq;
     const bool consistent = kv_len[b] == n - 1;
     emitted[b] = 0;
     int d = 0;
