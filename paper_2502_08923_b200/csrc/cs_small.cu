@@ -792,12 +792,14 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
           const int tile = job->tile, qb = job->quarter;
           const bool one = uniform((uint32_t)job->one) != 0;
           if (kind == kLm) {
-            // a tile of 16 ids: the largest sum of each token, and of the warp's tiles (1/rms scales all of a token's sums alike)
+            // a tile of 16 ids: the largest sum of each token, and of the warp's tiles (1/rms scales all of a token's sums alike; NaN and -inf are nobody's
+            // choice, as launch by launch)
             const int r0 = 16 * tile + row;
 #pragma unroll
             for (int q = 0; q < NT; ++q) {
-              float v = r0 < a.vocab ? acc[q][0] : -INFINITY;
-              int id = r0 < a.vocab ? r0 : INT_MAX;
+              float v = -INFINITY;
+              int id = INT_MAX;
+              if (r0 < a.vocab && acc[q][0] > v) { v = acc[q][0]; id = r0; }
               if (r0 + 8 < a.vocab && acc[q][1] > v) { v = acc[q][1]; id = r0 + 8; }
 #pragma unroll
               for (int off = 4; off < 32; off <<= 1) {
