@@ -9,9 +9,9 @@
 //
 // Bound by a chain of latencies: length, tokens (through L2), cluster barrier, draft.  Launched back to back, us a search, with a load waited
 // for per group of candidates, two barriers of the whole cluster behind them and rows off 16 bytes read token by token / now: 1 x 4,097 tokens 3.03 /
-// 2.67, 1 x 32,768 3.76 / 3.10, 8 x 5,003 6.13 / 3.08, 64 x 1,003 3.77 / 2.82, 32 x 20,002 6.95 / 4.3, 64 x 30,001 10.0 / 5.6, 64 x 32,768
-// 7.4 / 5.6, 64 x 131,072 18.2 / 12.2.  (The second four tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and
-// 13.5 for the last two.)
+// 2.26, 1 x 32,768 3.76 / 2.76, 8 x 5,003 6.13 / 2.67, 64 x 1,003 3.77 / 2.79, 32 x 20,002 6.95 / 4.1, 64 x 30,001 10.0 / 5.1, 64 x 32,768
+// 7.4 / 5.1, 64 x 131,072 18.2 / 10.8.  (The second four tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and
+// 13.5 for the last two, where the present loads took 5.5 and 12.)
 #include <limits.h>
 
 #include "cs_common.cuh"
@@ -35,7 +35,9 @@ __device__ __forceinline__ void cluster_wait() {
 }
 constexpr int kGroups = 4;             // groups of candidates whose tokens a thread has in flight
 
-__global__ void __launch_bounds__(kThreads)
+// Four CTAs an SM: 60 registers.  (72, as the compiler would have it, leave three: 64 x 32,768 tokens back to back 5.1 -> 6.7 us.  The keys are loaded where
+// they are used; ahead of that branch all eight took the registers that the tokens in flight need: 5.5.)
+__global__ void __launch_bounds__(kThreads, 4)
 k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
              int k, int policy, int* __restrict__ match_pos, int* __restrict__ draft,
              int* __restrict__ draft_len, int* __restrict__ last_tok,
@@ -58,61 +60,67 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
   const bool latest = (policy == CS_MATCH_LATEST);
   const int none = latest ? -1 : INT_MAX;
 
-  int key[CS_MAX_GAMMA];
-#pragma unroll
-  for (int j = 0; j < CS_MAX_GAMMA; ++j)
-    key[j] = (j < gamma && n >= gamma) ? __ldcg(h + n - gamma + j) : -1;
-
   if (tid == 0) s_best = none;
   __syncthreads();
 
   int best = none;
   if (n_cand > 0) {
-    const int per = (((n_cand + nblk - 1) / nblk) + 3) & ~3;
-    const int lo = rank * per;
-    const int hi = min(n_cand, lo + per);
-    // Groups of four tokens begin on 16 bytes, `off` tokens ahead of the row where a row does not.  A group is loaded where it holds a token of the row.
+    // This CTA's candidates are lo .. hi - 1 (none where lo = hi; unsigned, as lo + per may pass 2^31 in the longest rows).  From here on positions count
+    // from `first`, where the loads begin: c0 .. c1 - 1, and nothing that is added to them comes near 2^31.
+    const int log_nblk = __ffs(nblk) - 1;                // (a power of two)
+    const unsigned per = ((((unsigned)n_cand + nblk_u - 1) >> log_nblk) + 3) & ~3u;
+    const unsigned lo = min(rank_u * per, (unsigned)n_cand), hi = min(lo + per, (unsigned)n_cand);
+    // Four tokens at a time begin on 16 bytes, `off` tokens ahead of the row where a row does not.
     const bool vec_ok = gamma <= 5;
-    const int off = vec_ok ? (int)(reinterpret_cast<uintptr_t>(h) >> 2 & 3) : 0;
-    auto test = [&](const int4& u, const int4& v, int p) {
-      // tokens p .. p+7 cover candidates p .. p+3 for gamma <= 5; what lies ahead of the row or past the
-      // accepted length only feeds candidates that are masked off
-      const int t[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+    const unsigned off = vec_ok ? (unsigned)(reinterpret_cast<uintptr_t>(h) >> 2 & 3) : 0u;
+    const int first = (int)((lo + off) & ~3u) - (int)off, c0 = (int)lo - first, c1 = (int)hi - first;
+    const int* hs = h + first;
+    if (vec_ok) {
+      int key[5];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        bool eq = (unsigned)(p + i - lo) < (unsigned)(hi - lo);
+      for (int j = 0; j < 5; ++j) key[j] = j < gamma ? __ldcg(h + n - gamma + j) : -1;
+      const int room = c1 + min(stride - (int)hi, 8);    // tokens of the row from `first` on, as far as they matter
+      auto test = [&](const int4& u, const int4& v, int s) {
+        // tokens s .. s+7 cover candidates s .. s+3 for gamma <= 5; what lies ahead of the row or past the
+        // accepted length only feeds candidates that are masked off
+        const int t[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int j = 0; j < 5; ++j)
-          if (j < gamma) eq = eq && (t[i + j] == key[j]);
-        if (eq) best = latest ? max(best, p + i) : min(best, p + i);
-      }
-    };
-    auto scan = [&](int p) {
-      for (int i = 0; i < 4 && p + i < hi; ++i) {
-        bool eq = true;
-        for (int j = 0; j < gamma; ++j) eq = eq && (__ldcg(h + p + i + j) == key[j]);
-        if (eq) best = latest ? max(best, p + i) : min(best, p + i);
-      }
-    };
-    // (An empty share, hi <= lo, has nothing to test: its first group may begin ahead of hi, and the mask in test() holds only where lo < hi.)
-    for (int base = lo < hi ? ((lo + off) & ~3) - off : hi; base < hi; base += kGroups * kThreads * 4) {
-      int4 u[kGroups], v[kGroups];
+        for (int i = 0; i < 4; ++i) {
+          bool eq = (unsigned)(s + i - c0) < (unsigned)(c1 - c0);
 #pragma unroll
-      for (int q = 0; q < kGroups; ++q) {
-        const int p = base + (q * kThreads + tid) * 4;
-        if (vec_ok && p < hi) {
-          u[q] = ld_int4(h + p);
-          v[q] = ld_int4(h + (p + 4 < stride ? p + 4 : p));   // (behind the row's end nothing is wanted)
+          for (int j = 0; j < 5; ++j)
+            if (j < gamma) eq = eq && (t[i + j] == key[j]);
+          if (eq) best = latest ? max(best, s + i) : min(best, s + i);
+        }
+      };
+      for (int base = 0; base < c1; base += kGroups * kThreads * 4) {
+        int4 u[kGroups], v[kGroups];
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) {
+          const int s = base + (q * kThreads + tid) * 4;
+          if (s < c1) {
+            u[q] = ld_int4(hs + s);
+            v[q] = ld_int4(hs + (s + 4 < room ? s + 4 : s));   // (behind the row's end nothing is wanted)
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kGroups; ++q) {
+          if (base + q * kThreads * 4 >= c1) break;      // (short shares end in the first group)
+          test(u[q], v[q], base + (q * kThreads + tid) * 4);
         }
       }
+    } else {
+      int key[CS_MAX_GAMMA];
 #pragma unroll
-      for (int q = 0; q < kGroups; ++q) {
-        const int p = base + (q * kThreads + tid) * 4;
-        if (base + q * kThreads * 4 >= hi) break;        // (short shares end in the first group)
-        if (vec_ok) test(u[q], v[q], p);
-        else scan(p);
-      }
+      for (int j = 0; j < CS_MAX_GAMMA; ++j) key[j] = j < gamma ? __ldcg(h + n - gamma + j) : -1;
+      for (int s = tid * 4; s < c1; s += kThreads * 4)
+        for (int i = 0; i < 4 && s + i < c1; ++i) {
+          bool eq = true;
+          for (int j = 0; j < gamma; ++j) eq = eq && (__ldcg(hs + s + i + j) == key[j]);
+          if (eq) best = latest ? max(best, s + i) : min(best, s + i);
+        }
     }
+    if (best != none) best += first;
   }
   // warp vote, then one shared-memory atomic per warp
   best = latest ? __reduce_max_sync(0xffffffffu, best) : __reduce_min_sync(0xffffffffu, best);
@@ -156,8 +164,8 @@ cs_status cs_launch_find_match(const int32_t* hist, const int32_t* hist_len, int
   if (gamma < 1 || gamma > CS_MAX_GAMMA || (policy != CS_MATCH_LATEST && policy != CS_MATCH_FIRST) || k < 0 || B < 0)
     return CS_ERR_ARG;
   if (B == 0) return CS_OK;
-  // 4096 candidates per CTA keep every thread at >= 4 vector iterations on long
-  // histories; short ones use a single CTA per sequence
+  // 4,096 candidates are one round of a CTA's loads in flight: short histories use a single CTA per
+  // sequence, and only rows of more than 8 x 4,096 tokens take further rounds
   int cl = 1;
   while (cl < kMaxCluster && stride > cl * 4096) cl *= 2;
   cudaLaunchConfig_t lc = {};
