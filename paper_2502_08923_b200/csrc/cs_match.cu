@@ -9,8 +9,8 @@
 //
 // Bound by a chain of latencies: length, tokens (through L2), cluster barrier, draft.  Launched back to back, us a search, with a load waited
 // for per group of candidates, two barriers of the whole cluster behind them and rows off 16 bytes read token by token / now: 1 x 4,097 tokens 3.03 /
-// 2.26, 1 x 32,768 3.76 / 2.76, 8 x 5,003 6.13 / 2.67, 64 x 1,003 3.77 / 2.79, 32 x 20,002 6.95 / 4.1, 64 x 30,001 10.0 / 5.1, 64 x 32,768
-// 7.4 / 5.1, 64 x 131,072 18.2 / 10.8.  (The second four tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and
+// 2.31, 1 x 32,768 3.76 / 2.81, 8 x 5,003 6.13 / 2.74, 64 x 1,003 3.77 / 2.86, 32 x 20,002 6.95 / 4.0, 64 x 30,001 10.0 / 5.1, 64 x 32,768
+// 7.4 / 5.1, 64 x 131,072 18.2 / 10.6.  (The second four tokens of a thread from its neighbour by shuffles, half of the loads: 5.95 and
 // 13.5 for the last two, where the present loads took 5.5 and 12.)
 #include <limits.h>
 
@@ -79,33 +79,43 @@ k_find_match(const int* hist, const int* hist_len, int stride, int gamma,
       int key[5];
 #pragma unroll
       for (int j = 0; j < 5; ++j) key[j] = j < gamma ? __ldcg(h + n - gamma + j) : -1;
-      const int room = c1 + min(stride - (int)hi, 8);    // tokens of the row from `first` on, as far as they matter
+      // Candidates whose eight tokens lie in the caller's rows: w0 .. w1 - 1.  The others, at the rows' very ends, are looked at token by token.
+      const int room = c1 + min(stride - (int)hi, 8) + (b + 1 < (int)gridDim.y ? min(stride, 8) : 0);   // tokens from `first` on, as far as they matter
+      const int w0 = first < 0 && (b == 0 || stride < 3) ? min(4, c1) : c0, w1 = max(w0, min(c1, room < 8 ? 0 : (room - 4) & ~3));
       auto test = [&](const int4& u, const int4& v, int s) {
         // tokens s .. s+7 cover candidates s .. s+3 for gamma <= 5; what lies ahead of the row or past the
         // accepted length only feeds candidates that are masked off
         const int t[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          bool eq = (unsigned)(s + i - c0) < (unsigned)(c1 - c0);
+          bool eq = (unsigned)(s + i - w0) < (unsigned)(w1 - w0);
 #pragma unroll
           for (int j = 0; j < 5; ++j)
             if (j < gamma) eq = eq && (t[i + j] == key[j]);
           if (eq) best = latest ? max(best, s + i) : min(best, s + i);
         }
       };
-      for (int base = 0; base < c1; base += kGroups * kThreads * 4) {
+      const int e = tid - (kThreads - 32), p = e < w0 - c0 ? c0 + e : w1 + e - (w0 - c0);   // (ten at most; the last warp has the least else to do)
+      if (e >= 0 && p < c1) {
+        bool eq = true;
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (j < gamma) eq = eq & (__ldcg(hs + p + j) == key[j]);
+        if (eq) best = latest ? max(best, p) : min(best, p);
+      }
+      for (int base = w0 < w1 ? w0 & ~3 : w1; base < w1; base += kGroups * kThreads * 4) {
         int4 u[kGroups], v[kGroups];
 #pragma unroll
         for (int q = 0; q < kGroups; ++q) {
           const int s = base + (q * kThreads + tid) * 4;
-          if (s < c1) {
+          if (s < w1) {
             u[q] = ld_int4(hs + s);
-            v[q] = ld_int4(hs + (s + 4 < room ? s + 4 : s));   // (behind the row's end nothing is wanted)
+            v[q] = ld_int4(hs + s + 4);
           }
         }
 #pragma unroll
         for (int q = 0; q < kGroups; ++q) {
-          if (base + q * kThreads * 4 >= c1) break;      // (short shares end in the first group)
+          if (base + q * kThreads * 4 >= w1) break;      // (short shares end in the first group)
           test(u[q], v[q], base + (q * kThreads + tid) * 4);
         }
       }
