@@ -86,7 +86,7 @@ struct SmallArgs {
   __nv_bfloat16* kv;
   int B, stride, gamma, k, policy, max_new, eos_id;
   int log_slices, log_rows, own_d, slice_bytes;   // CTAs per KV head and tiles of 16 query rows per KV head (powers of two), tiles of the residual stream per CTA at most, an attention result
-  int *emitted, *done, *accept, *out, *argmax, *mpos, *dlen;
+  int *emitted, *done;
   unsigned long long* stats;
   int* status;
   unsigned long long *progress, *report;   // pinned: the word that the host waits for; status bits, then the image of cs_stats
@@ -458,9 +458,8 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     const int p0 = *s_best == INT_MAX ? -1 : *s_best;
     const int from = p0 + a.gamma, dl = p0 < 0 ? 0 : min(a.k, nn - from);
     const bool fits = kv >= 0 && kv + dl + 1 <= a.max_seq;
-    if (c == 0 && tid == kClerk) { a.mpos[b] = p0; a.dlen[b] = dl; }
-    if (!fits) {                                               // no room for the block: the sequence stops here
-      if (c == 0 && tid == 0) { atomicOr(a.status, CS_DEV_CAPACITY); a.accept[b] = -1; }
+    if (!fits) {                                               // no room for the block: the sequence stops here (none is let in that could come to this)
+      if (c == 0 && tid == 0) atomicOr(a.status, CS_DEV_CAPACITY);
       break;
     }
     // ---------------------------------------------------------------- embedding and first norm, all rows in every CTA.  Row r: the last accepted
@@ -911,7 +910,6 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
         const int tgt = tok > dl ? -1 : a.script != nullptr ? s_script[tok] : arg;
         s_tgt[tok] = tgt;
         if (tok < dl && s_hist[from + tok] != tgt) atomicMin(s_tau, tok);
-        if (c == 0) a.argmax[(size_t)b * R + tok] = arg;
       }
     }
     __syncthreads();
@@ -925,13 +923,9 @@ k_small_loop(const __grid_constant__ SmallMaps maps, const __grid_constant__ Sma
     }
     if (tid < cnt) s_hist[n + tid] = s_tgt[tid];
     if (c == 0) {
-      if (tid < R) {
-        a.out[(size_t)b * R + tid] = tid <= tau ? s_tgt[tid] : -1;
-        if (tid < cnt) h[n + tid] = s_tgt[tid];
-      }
+      if (tid < cnt) h[n + tid] = s_tgt[tid];
       if (tid == kClerk) {
         cs_stats* st = reinterpret_cast<cs_stats*>(a.stats);
-        a.accept[b] = tau;
         a.hist_len[b] = n + cnt;
         a.kv_len[b] = n + cnt - 1;
         a.emitted[b] = e + cnt;
@@ -1113,8 +1107,7 @@ cs_status cs_launch_small_loop(cs_ctx* ctx, bool* taken, cudaStream_t st) {
   a.hist = L.hist; a.hist_len = L.hist_len; a.kv_len = L.kv_len; a.script = L.script; a.kv = static_cast<__nv_bfloat16*>(L.kv_cache);
   a.B = L.B; a.stride = L.stride; a.gamma = L.gamma; a.k = L.k; a.policy = L.policy; a.max_new = L.max_new; a.eos_id = L.eos_id;
   a.log_slices = shape.log_slices; a.log_rows = shape.log_rows; a.own_d = shape.own_d; a.slice_bytes = shape.slice_bytes; a.at = shape.at;
-  a.emitted = ctx->loop_emitted; a.done = ctx->loop_done; a.accept = ctx->loop_accept; a.out = ctx->loop_out; a.argmax = ctx->loop_argmax;
-  a.mpos = ctx->loop_mpos; a.dlen = ctx->loop_dlen;
+  a.emitted = ctx->loop_emitted; a.done = ctx->loop_done;
   a.stats = ctx->loop_stats; a.status = ctx->d_status;
   a.progress = ctx->progress_dev; a.report = reinterpret_cast<unsigned long long*>(ctx->step_out_dev);
   a.wait_ns = ctx->wait_limit_ns;
