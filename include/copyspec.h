@@ -163,7 +163,8 @@ cs_status cs_sync_status(cs_ctx* ctx, void* stream);
  * the draft_len[b] = min(k, n - (p0 + gamma)) tokens that follow the match (0 without a
  * match); draft entries past draft_len[b] are set to -1.
  *   hist [B][stride] int32, hist_len [B] int32, match_pos [B], draft [B][k],
- *   draft_len [B].  1 <= gamma <= 8, 0 <= k, B >= 0 (B == 0 is a no-op).
+ *   draft_len [B].  1 <= gamma <= 8, 0 <= k, B >= 0 (B == 0 is a no-op).  Any alignment of an
+ *   int32; nothing outside the B * stride tokens is read.
  *   Needs no context and no scratch memory.  Errors: CS_ERR_ARG, CS_ERR_CUDA. */
 cs_status cs_find_match(const int32_t* hist, const int32_t* hist_len, int B, int stride,
                         int gamma, int k, cs_match_policy policy, int32_t* match_pos,

@@ -1,7 +1,7 @@
 // The search call for Python, in native code: marshalling of cs_find_match with its outputs made by the allocator directly.
 //
-// The search takes 3.5 to 6 us on the device, a call through ctypes 10.7: three tensors made from Python, eleven
-// arguments converted, two tensors looked at, the launch.  Here 4.9 for one history of 4,097 tokens, and 5.8 for 64 of 32,768, where the
+// The search takes 2.3 to 5.1 us on the device, a call through ctypes 10.7: three tensors made from Python, eleven
+// arguments converted, two tensors looked at, the launch.  Here 5.0 - 5.3 for one history of 4,097 tokens, and 5.3 - 5.5 for 64 of 32,768, where the
 // device sets the pace.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>

@@ -27,10 +27,14 @@
 // cluster barriers 980 (11,400 instructions a warp and step); with hand-overs counted on mbarriers and K split over the warps 555; with the SwiGLU output
 // multiplied where it was made, one turn of code for all projections and weights out of the registers 500; with weights by TMA and the
 // statistics kept by a warp that nobody waits for 475; with what a warp does for a tile worked out once and fragment loads that meet every bank once
-// 433.  What is left of 38 us a step: 17 turns or hand-overs of 1.5 - 2 us.
+// 433; now 426, with softmax weights by exp2f (3 more) and nothing stored that nobody reads (4 less).  What is left of 38 us a step: 17 turns or hand-overs of
+// 1.5 - 2 us.
 //
 // Arithmetic as in the other kernels: activations, queries and softmax weights enter products as two bf16 terms, sums, norms,
 // rotation and softmax are fp32; every RMSNorm is folded into the projection behind it (1/rms scales the sums).
+//
+// Heads of 64 want more than the 128 registers that 512 threads leave each: 450 - 490 bytes of spill stores a thread, where heads of 32 have none.  They gain
+// less than heads of 32 in the table at the launch.
 //
 // Waits are bounded as in the other kernels: after the limit a CTA raises the status bit, waits for nothing and sends nothing any
 // more, gives its copies time to land and meets the others at the cluster barrier in front of the exit, which all of them reach.
